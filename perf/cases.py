@@ -249,6 +249,115 @@ def run(state):
     return dict(logits=state["logits"], hidden=state["hidden"], tokens=tokens, len=lens, status=status)
 
 
+# ---------------------------------------------------------------------------------------------- the same in 64 bits
+def _philox_word0(c0, c1, c2, seed):
+    """First output word of Philox4x32-10 at counter (c0, c1, c2, 0); c0 an int64 tensor, the rest numbers."""
+    m = 0xFFFFFFFF
+    c1, c2, c3 = torch.full_like(c0, c1), torch.full_like(c0, c2), torch.zeros_like(c0)
+    k0, k1 = seed & m, seed >> 32
+    for _ in range(10):
+        # 32 x 32 bit products in two halves: a 64-bit one would not fit a signed number
+        p0, p1 = [((a >> 16) * f, (a & 0xFFFF) * f) for a, f in ((c0, 0xD2511F53), (c2, 0xCD9E8D57))]
+        (h0, l0), (h1, l1) = [((hi + (lo >> 16)) >> 16, ((hi << 16) + lo) & m) for hi, lo in (p0, p1)]
+        c0, c1, c2, c3 = h1 ^ c1 ^ k0, l1, h0 ^ c3 ^ k1, l0
+        k0, k1 = (k0 + 0x9E3779B9) & m, (k1 + 0xBB67AE85) & m
+    return c0
+
+
+def _choose(logits, t, temp):
+    """The t-th generated token of every row: the arg-max, or the draw at a temperature as the header defines it."""
+    if temp:
+        v = torch.arange(logits.shape[1], device=logits.device)
+        noise = []
+        for r in range(logits.shape[0]):
+            u = ((_philox_word0(v, t, r, 12345) >> 9).double() + 0.5) / 2.0 ** 23
+            noise.append(-torch.log(-torch.log(u)))
+        logits = logits / temp + torch.stack(noise)
+    return torch.argmax(logits, dim=1)
+
+
+def exact(case, seed):
+    """The decoder without any rounding, in plain torch: logits and hidden states of the last generated token."""
+    if case["kind"] == "group":
+        return None                                            # whole values only
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(int(seed))
+
+    def norm(x):                                               # the gains are ones
+        return x * torch.rsqrt(x.square().mean(-1, keepdim=True) + 1e-6)
+
+    if case["kind"] == "logits":
+        h = torch.empty(case["rows"], case["d"], dtype=torch.float32, device="cuda").normal_(0.0, 3.0, generator=gen)
+        w = torch.empty(case["vocab"], case["d"], dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.02, generator=gen)
+        return norm(h.double()) @ w.double().T
+    shape = _shape(case)
+    w = dict(_weights(case, shape, gen))
+    lens = _lengths(case)
+    ids, off = _prompts(shape, lens, seed)
+    B, H, D, d, L = case["rows"], shape.n_heads, shape.head_dim, shape.d_model, shape.n_layers
+    cap = case["steps"] if case["kind"] == "decode" else case["tokens"]
+    n_max = int(lens.max()) + cap
+    inv_freq = shape.rope_theta ** (-2.0 * torch.arange(D // 2, dtype=torch.float64, device="cuda") / D)
+
+    def rope(x, pos):                                          # x [T, H, D], pos [T]
+        ang = pos.double()[:, None, None] * inv_freq
+        a, b, cs, sn = x[..., :D // 2], x[..., D // 2:], ang.cos(), ang.sin()
+        return torch.cat((a * cs - b * sn, b * cs + a * sn), dim=-1)
+
+    def layer(l, h, pos, attend):
+        x = norm(h)
+        q, k, v = [(x @ w[f"l{l}.{n}"].double().T).view(-1, H, D) for n in ("wq", "wk", "wv")]
+        h = h + attend(l, rope(q, pos), rope(k, pos), v).reshape(-1, d) @ w[f"l{l}.wo"].double().T
+        x = norm(h)
+        g = torch.nn.functional.silu(x @ w[f"l{l}.w_gate"].double().T)
+        return h + (g * (x @ w[f"l{l}.w_up"].double().T)) @ w[f"l{l}.w_down"].double().T
+
+    cache = {}
+
+    def attend_prompt(l, q, k, v):
+        out = torch.empty_like(q)
+        if cap > 1:
+            cache[l] = [torch.zeros(B, H, n_max, D, dtype=torch.float64, device="cuda") for _ in range(2)]
+        for r in range(B):
+            s = slice(int(off[r]), int(off[r + 1]))
+            n = s.stop - s.start
+            kr, vr = k[s].transpose(0, 1), v[s].transpose(0, 1)
+            sc = (q[s].transpose(0, 1) @ kr.transpose(1, 2)) / math.sqrt(D)
+            sc.masked_fill_(torch.ones(n, n, dtype=torch.bool, device="cuda").triu(1), -math.inf)
+            out[s] = (torch.softmax(sc, dim=-1) @ vr).transpose(0, 1)
+            if cap > 1:
+                cache[l][0][r, :, :n], cache[l][1][r, :, :n] = kr, vr
+        return out
+
+    rows = torch.arange(B, device="cuda")
+    ctx = torch.tensor(lens, device="cuda").long()
+
+    def attend_cached(l, q, k, v):
+        cache[l][0][rows, :, ctx], cache[l][1][rows, :, ctx] = k, v
+        sc = (cache[l][0] @ q[..., None])[..., 0] / math.sqrt(D)
+        sc.masked_fill_(torch.arange(n_max, device="cuda")[None, None, :] > ctx[:, None, None], -math.inf)
+        return (torch.softmax(sc, dim=-1)[:, :, None, :] @ cache[l][1])[:, :, 0]
+
+    h = w["embed"][torch.tensor(ids, device="cuda").long()].double()
+    pos = torch.tensor(np.concatenate([np.arange(n) for n in lens]), device="cuda")
+    for l in range(L):
+        h = layer(l, h, pos, attend_prompt)
+    h = h[torch.tensor(off[1:] - 1, device="cuda").long()]
+    head = w["lm_head"].double().T
+    active = torch.ones(B, 1, dtype=torch.float64, device="cuda")
+    for t in range(1, cap + 1):
+        if t > 1:
+            h = w["embed"][tok].double()
+            for l in range(L):
+                h = layer(l, h, ctx, attend_cached)
+            ctx = ctx + 1
+        logits = norm(h) @ head
+        if t < cap:
+            tok = _choose(logits, t, case["temp"])
+            active = active * (tok != shape.eos_id)[:, None]   # a row that ended leaves its outputs as they were: zero
+    return dict(logits=logits * active, hidden=h * active, tokens=None, len=None, status=None)
+
+
 # ---------------------------------------------------------------------------------------------- what a pass needs
 def _params(shape):
     d, F = shape.d_model, shape.d_ffn
