@@ -40,23 +40,23 @@ EMBED_STD = {"tiny": 0.1, "7b": 1.0, "13b": 1.0, "h64": 0.5}
 def listed():
     return [
         # the evaluation's decode-step workload: one micro-batch of 16 at full depth, instruction prompts
-        dict(name="decode 7b x32, 16 rows", kind="decode", shape="7b", layers=32, rows=16, lo=100, hi=380, steps=8, temp=0.0),
+        dict(name="decode 7b x32 16 rows", kind="decode", shape="7b", layers=32, rows=16, lo=100, hi=380, steps=8, temp=0.0),
         # one request alone: latency per token
-        dict(name="decode 7b, 1 row", kind="decode", shape="7b", layers=8, rows=1, lo=173, hi=173, steps=8, temp=0.0),
+        dict(name="decode 7b 1 row", kind="decode", shape="7b", layers=8, rows=1, lo=173, hi=173, steps=8, temp=0.0),
         # a middle bin of the variable batch size, ragged, generating at the paper's temperature
-        dict(name="decode 7b, 45 rows", kind="decode", shape="7b", layers=8, rows=45, lo=70, hi=500, steps=6, temp=0.5),
+        dict(name="decode 7b 45 rows", kind="decode", shape="7b", layers=8, rows=45, lo=70, hi=500, steps=6, temp=0.5),
         # a short bin of the variable batch size: close to the largest micro-batch
-        dict(name="decode 7b, 200 rows", kind="decode", shape="7b", layers=8, rows=200, lo=64, hi=300, steps=6, temp=0.0),
+        dict(name="decode 7b 200 rows", kind="decode", shape="7b", layers=8, rows=200, lo=64, hi=300, steps=6, temp=0.0),
         # long responses on the larger shape: the key/value cache outweighs the weights
-        dict(name="decode 13b, 24 rows, long", kind="decode", shape="13b", layers=6, rows=24, lo=1000, hi=2400, steps=6, temp=0.0),
+        dict(name="decode 13b 24 rows long", kind="decode", shape="13b", layers=6, rows=24, lo=1000, hi=2400, steps=6, temp=0.0),
         # heads of 64, more rows than one token tile of the small-batch kernel
-        dict(name="decode h64, 96 rows", kind="decode", shape="h64", layers=8, rows=96, lo=200, hi=900, steps=6, temp=0.0),
+        dict(name="decode h64 96 rows", kind="decode", shape="h64", layers=8, rows=96, lo=200, hi=900, steps=6, temp=0.0),
         # the prompt pass of the batch of 16
-        dict(name="prompt 7b, 16 x 64-256", kind="prompt", shape="7b", layers=8, rows=16, lo=64, hi=256, tokens=1, temp=0.0),
+        dict(name="prompt 7b 16 x 64-256", kind="prompt", shape="7b", layers=8, rows=16, lo=64, hi=256, tokens=1, temp=0.0),
         # one short prompt: time to the first token
-        dict(name="prompt 7b, 1 x 61", kind="prompt", shape="7b", layers=8, rows=1, lo=61, hi=61, tokens=1, temp=0.0),
+        dict(name="prompt 7b 1 x 61", kind="prompt", shape="7b", layers=8, rows=1, lo=61, hi=61, tokens=1, temp=0.0),
         # the length-perception pass: many prompts with the instruction appended, three tokens generated
-        dict(name="prompt 7b, 100 x 96-288", kind="prompt", shape="7b", layers=8, rows=100, lo=96, hi=288, tokens=3, temp=0.0),
+        dict(name="prompt 7b 100 x 96-288", kind="prompt", shape="7b", layers=8, rows=100, lo=96, hi=288, tokens=3, temp=0.0),
         # the tiny configuration's whole group: nothing but launches and latency
         dict(name="group tiny", kind="group", shape="tiny", layers=2, queries=32, lo=8, hi=32, median=0, max_new=64, noise=8.0,
              bin=16, base=8, vbs=0, fcr=1, vanilla=0),
