@@ -21,6 +21,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 constexpr size_t kAlign = 1024;
+constexpr size_t kRowStateBytes = (size_t)kMaxBatch * 4 * 8;   // 7 row arrays and the scalars
 inline size_t align_up(size_t x, size_t a = kAlign) { return (x + a - 1) / a * a; }
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 inline int round_up(int a, int b) { return ceil_div(a, b) * b; }
@@ -149,6 +150,7 @@ struct ss_ctx {
   uint32_t* status = nullptr;
   RowState st{};
   KvLayout kv{};
+  int32_t* d_chunk = nullptr;      // a prompt chunk's arrays, packed: tokens, rows, positions, prefix sums, last tokens
   int32_t *d_tokens = nullptr, *d_tok_row = nullptr, *d_tok_pos = nullptr, *d_cu = nullptr, *d_last = nullptr;
   // prompt-pass activations (R rows)
   int R = 0;
@@ -199,6 +201,13 @@ struct ss_ctx {
   bool in_batch = false;
   std::vector<int32_t> prompt_len;
   int32_t* pinned = nullptr;     // [0] n_active, [1] status
+  // Page-locked staging for what a batch sends and fetches: a copy from or to pageable memory costs the host 5 to 10 us
+  // each, and a batch needed 2 to 7 on its way up and one per row on its way back (200 rows: 2.2 of 19.7 ms per batch of
+  // six steps).  Up: row state and block table as one copy, a chunk's token arrays as another.  Down: row state, tokens.
+  uint8_t *up = nullptr, *down = nullptr;
+  size_t up_chunk = 0;           // where the chunk arrays start inside `up`
+  size_t table_off = 0;          // where the block table starts behind the row state (device and staging alike)
+  cudaEvent_t up_ev[2] = {nullptr, nullptr};   // last copy out of the row part / the chunk part of `up`
   // ---- sampling (greedy while inv_temp == 0)
   SampleCfg sample{0.f, 0u, 0u};
   std::vector<int32_t> next_row_keys;   // keys of the next batch's rows; empty = 0, 1, 2, ...
@@ -387,7 +396,7 @@ void layout(const ss_model_cfg& m, const ss_runtime_cfg& rt, int n_sm, Offsets& 
   o.staging = a.take(o.staging_bytes);
   o.inv_freq = a.take(m.head_dim / 2 * sizeof(float));
   o.status = a.take(64);
-  o.rows = a.take((size_t)kMaxBatch * 4 * 8 + 64);           // 7 row arrays + scalars
+  o.rows = a.take(kRowStateBytes + 64);
   o.max_pages = ceil_div(rt.max_ctx, kPageTokens);
   o.block_table = a.take((size_t)kMaxBatch * o.max_pages * 4);
   o.out_tokens = a.take((size_t)kMaxBatch * rt.max_new_tokens * 4);
@@ -617,6 +626,33 @@ int enqueue_prefill_chunk(ss_ctx* c, int s0, int s1, const int32_t* cu, int T) {
   return SS_OK;
 }
 
+// ------------------------------------------------------------------------------------ staging
+void free_host(ss_ctx* c) {
+  if (c->pinned) cudaFreeHost(c->pinned);
+  for (auto& ev : c->up_ev)
+    if (ev) cudaEventDestroy(ev);
+}
+
+// A part of the staging area, free to be filled: an earlier copy out of it has run.
+cudaError_t staging_free(ss_ctx* c, int part) { return cudaEventSynchronize(c->up_ev[part]); }
+
+// Sends the row state and the block tables of B rows, filled in at c->up (row arrays first, tables at table_off).
+cudaError_t send_rows(ss_ctx* c, int B) {
+  cudaError_t e = cudaMemcpyAsync(c->st.ctx_len, c->up, c->table_off + (size_t)B * c->st.max_pages * 4, cudaMemcpyHostToDevice,
+                                  c->stream);
+  return e == cudaSuccess ? cudaEventRecord(c->up_ev[0], c->stream) : e;
+}
+
+// Row state and block table of a new batch of B rows in the staging area: everything zero, no pages.
+void clear_rows(ss_ctx* c, int B, int cap, int32_t** rows, int32_t** bt) {
+  *rows = (int32_t*)c->up;
+  *bt = (int32_t*)(c->up + c->table_off);
+  std::memset(*rows, 0, kRowStateBytes);
+  std::fill(*bt, *bt + (size_t)B * c->st.max_pages, -1);
+  (*rows)[7 * kMaxBatch + 0] = cap;
+  (*rows)[7 * kMaxBatch + 1] = B;
+}
+
 }  // namespace
 
 // ======================================================================================= C ABI
@@ -714,12 +750,8 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
   c->st.max_pages = o.max_pages;
   c->st.max_new = rt->max_new_tokens;
   c->R = o.R;
-  int32_t* tk = (int32_t*)(A + o.tok);
-  c->d_tokens = tk;
-  c->d_tok_row = tk + o.R;
-  c->d_tok_pos = tk + 2 * (size_t)o.R;
-  c->d_cu = tk + 3 * (size_t)o.R;
-  c->d_last = c->d_cu + kMaxBatch + 4;
+  c->d_chunk = (int32_t*)(A + o.tok);
+  c->table_off = o.block_table - o.rows;
   c->h = (float*)(A + o.h);
   c->x = (bf16*)(A + o.x);
   c->qkv = (bf16*)(A + o.qkv);
@@ -793,11 +825,21 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
     inv[i] = (float)std::pow((double)model->rope_theta, -2.0 * i / model->head_dim);
   cudaError_t e = cudaMemcpyAsync(c->inv_freq, inv.data(), inv.size() * 4, cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->status, 0, 64, c->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(rows, 0, (size_t)kMaxBatch * 4 * 8 + 64, c->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(rows, 0, kRowStateBytes + 64, c->stream);
   // activation operands must be finite wherever a TMA box may reach beyond the valid rows
   if (e == cudaSuccess) e = cudaMemsetAsync(A + o.h, 0, o.partial - o.h, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  if (e == cudaSuccess) e = cudaHostAlloc((void**)&c->pinned, 64, cudaHostAllocDefault);
+  // one page-locked allocation for all of it: each costs the host 1 to 2 ms, whatever its size
+  c->up_chunk = align_up(c->table_off + (size_t)rt->max_batch * o.max_pages * 4);
+  const size_t down_off = align_up(c->up_chunk + ((size_t)o.R * 3 + 2 * kMaxBatch + 8) * 4);
+  const size_t down_bytes = kRowStateBytes + (size_t)rt->max_batch * rt->max_new_tokens * 4;
+  if (e == cudaSuccess) e = cudaHostAlloc((void**)&c->pinned, kAlign + down_off + down_bytes, cudaHostAllocDefault);
+  if (e == cudaSuccess) {
+    c->up = (uint8_t*)c->pinned + kAlign;
+    c->down = c->up + down_off;
+  }
+  for (auto& ev : c->up_ev)
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(gemm_wx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess)
@@ -806,7 +848,7 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
     e = cudaFuncSetAttribute(mega_kernel_fn((v & 1) ? 128 : 64, (v & 2) != 0, (v & 4) != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
                              227 * 1024);
   if (e != cudaSuccess) {
-    c->last_cuda = (int)e;
+    free_host(c);
     delete c;
     return SS_ERR_CUDA;
   }
@@ -817,7 +859,7 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
 int ss_destroy(ss_ctx* c) {
   if (!c) return SS_ERR_ARG;
   cudaStreamSynchronize(c->stream);
-  if (c->pinned) cudaFreeHost(c->pinned);
+  free_host(c);
   delete c;
   return SS_OK;
 }
@@ -889,7 +931,9 @@ int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, c
     if (tokens[i] < 0 || tokens[i] >= m.vocab) return SS_ERR_ARG;
 
   // host-side batch state
-  std::vector<int32_t> bt((size_t)B * c->st.max_pages, -1);
+  SS_CUDA(c, staging_free(c, 0));
+  int32_t *rows, *bt;
+  clear_rows(c, B, cap, &rows, &bt);
   c->batch_pages.clear();
   c->prompt_len.assign(B, 0);
   c->row_pages.assign(B, {});
@@ -910,7 +954,6 @@ int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, c
   c->in_batch = true;
   c->B = B;
   c->cap = cap;
-  std::vector<int32_t> rows((size_t)kMaxBatch * 8, 0);
   for (int r = 0; r < B; ++r) {
     rows[0 * kMaxBatch + r] = c->prompt_len[r];   // ctx_len after the prompt pass
     rows[3 * kMaxBatch + r] = 1;                  // active
@@ -918,8 +961,6 @@ int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, c
     rows[6 * kMaxBatch + r] = r < (int)c->next_row_keys.size() ? c->next_row_keys[r] : r;
   }
   c->next_row_keys.clear();
-  rows[7 * kMaxBatch + 0] = cap;
-  rows[7 * kMaxBatch + 1] = B;
   int rc = SS_OK;
   auto bail = [&](int code) { ss_release_batch(c); return code; };
 #define SS_CUDA_B(expr)                                              \
@@ -927,36 +968,38 @@ int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, c
     cudaError_t _e = (expr);                                         \
     if (_e != cudaSuccess) { c->last_cuda = (int)_e; return bail(SS_ERR_CUDA); } \
   } while (0)
-  SS_CUDA_B(cudaMemcpyAsync(c->st.ctx_len, rows.data(), rows.size() * 4, cudaMemcpyHostToDevice, c->stream));
-  SS_CUDA_B(cudaMemcpyAsync(c->st.block_table, bt.data(), bt.size() * 4, cudaMemcpyHostToDevice, c->stream));
+  SS_CUDA_B(send_rows(c, B));
 
   // chunks of whole sequences
-  std::vector<int32_t> tok_row, tok_pos, cu_loc, last;
   int s0 = 0;
   while (s0 < B) {
     int s1 = s0, T = 0;
     while (s1 < B && T + (cu[s1 + 1] - cu[s1]) <= c->rt.max_prefill_tokens) { T += cu[s1 + 1] - cu[s1]; ++s1; }
-    tok_row.resize(T); tok_pos.resize(T); cu_loc.assign(1, 0); last.clear();
-    int t = 0;
-    for (int s = s0; s < s1; ++s) {
-      const int len = cu[s + 1] - cu[s];
-      for (int p = 0; p < len; ++p, ++t) { tok_row[t] = s; tok_pos[t] = p; }
-      cu_loc.push_back(t);
-      last.push_back(t - 1);
+    // the chunk's arrays, packed into one copy; the host runs ahead of the GPU by at most one chunk
+    SS_CUDA_B(staging_free(c, 1));
+    const int n_seq = s1 - s0;
+    int32_t* tok = (int32_t*)(c->up + c->up_chunk);
+    int32_t *tok_row = tok + T, *tok_pos = tok + 2 * (size_t)T, *cu_loc = tok + 3 * (size_t)T, *last = cu_loc + n_seq + 1;
+    std::copy(tokens + cu[s0], tokens + cu[s1], tok);
+    for (int s = s0, t = 0; s < s1; ++s) {
+      cu_loc[s - s0] = t;
+      for (int p = 0; p < cu[s + 1] - cu[s]; ++p, ++t) { tok_row[t] = s; tok_pos[t] = p; }
+      cu_loc[s - s0 + 1] = t;
+      last[s - s0] = t - 1;
     }
-    SS_CUDA_B(cudaMemcpyAsync(c->d_tokens, tokens + cu[s0], (size_t)T * 4, cudaMemcpyHostToDevice, c->stream));
-    SS_CUDA_B(cudaMemcpyAsync(c->d_tok_row, tok_row.data(), (size_t)T * 4, cudaMemcpyHostToDevice, c->stream));
-    SS_CUDA_B(cudaMemcpyAsync(c->d_tok_pos, tok_pos.data(), (size_t)T * 4, cudaMemcpyHostToDevice, c->stream));
-    SS_CUDA_B(cudaMemcpyAsync(c->d_cu, cu_loc.data(), cu_loc.size() * 4, cudaMemcpyHostToDevice, c->stream));
-    SS_CUDA_B(cudaMemcpyAsync(c->d_last, last.data(), last.size() * 4, cudaMemcpyHostToDevice, c->stream));
+    SS_CUDA_B(cudaMemcpyAsync(c->d_chunk, tok, (3 * (size_t)T + 2 * n_seq + 1) * 4, cudaMemcpyHostToDevice, c->stream));
+    SS_CUDA_B(cudaEventRecord(c->up_ev[1], c->stream));
+    c->d_tokens = c->d_chunk;
+    c->d_tok_row = c->d_chunk + T;
+    c->d_tok_pos = c->d_chunk + 2 * (size_t)T;
+    c->d_cu = c->d_chunk + 3 * (size_t)T;
+    c->d_last = c->d_cu + n_seq + 1;
     if ((rc = enqueue_prefill_chunk(c, s0, s1, cu, T))) return bail(rc);
     SS_CUDA_B(launch(c, gather_last_rmsnorm_kernel, dim3(s1 - s0), dim3(256), 0, (const float*)c->h,
                      (const int32_t*)c->d_last, c->h_dec + (size_t)s0 * m.d_model, (const bf16*)c->final_norm,
                      c->x_dec + (size_t)s0 * m.d_model,
                      (opts && opts->dump_hidden) ? opts->dump_hidden + (size_t)s0 * m.d_model : (float*)nullptr,
                      m.d_model, m.rms_eps));
-    // the host vectors above are reused by the next chunk
-    SS_CUDA_B(cudaStreamSynchronize(c->stream));
     s0 = s1;
   }
   // LM head on the last tokens, first generated token, bookkeeping
@@ -1040,8 +1083,9 @@ int ss_resume(ss_ctx* c, const int32_t* ids, int32_t B, const int32_t* eos_at, i
     need_pages += (size_t)ceil_div(len + cap, kPageTokens) - it->second.pages.size();
   }
   if (need_pages > c->free_pages.size()) return SS_ERR_KV_BUDGET;
-  std::vector<int32_t> bt((size_t)B * c->st.max_pages, -1);
-  std::vector<int32_t> rows((size_t)kMaxBatch * 8, 0);
+  SS_CUDA(c, staging_free(c, 0));
+  int32_t *rows, *bt;
+  clear_rows(c, B, cap, &rows, &bt);
   c->batch_pages.clear();
   c->batch_tokens.clear();
   c->batch_cu.clear();
@@ -1067,15 +1111,11 @@ int ss_resume(ss_ctx* c, const int32_t* ids, int32_t B, const int32_t* eos_at, i
     rows[6 * kMaxBatch + r] = r < (int)c->next_row_keys.size() ? c->next_row_keys[r] : r;
   }
   c->next_row_keys.clear();
-  rows[7 * kMaxBatch + 0] = cap;
-  rows[7 * kMaxBatch + 1] = B;
   c->in_batch = true;
   c->B = B;
   c->cap = cap;
   auto bail = [&](int code) { ss_release_batch(c); return code; };
-  cudaError_t e = cudaMemcpyAsync(c->st.ctx_len, rows.data(), rows.size() * 4, cudaMemcpyHostToDevice, c->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(c->st.block_table, bt.data(), bt.size() * 4, cudaMemcpyHostToDevice, c->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);          // the host vectors go out of scope
+  const cudaError_t e = send_rows(c, B);
   if (e != cudaSuccess) { c->last_cuda = (int)e; return bail(SS_ERR_CUDA); }
   int rc = enqueue_decode_step(c, opts, first_tokens);
   if (rc) return bail(rc);
@@ -1116,23 +1156,35 @@ int ss_read_batch(ss_ctx* c, int32_t* out_tokens, int32_t stride, int32_t* out_l
   if (!c || !out_len || !out_status || (out_tokens && stride < 1)) return SS_ERR_ARG;
   if (!c->in_batch) return SS_ERR_STATE;
   const int B = c->B;
-  std::vector<int32_t> gen(B), fin(B);
-  SS_CUDA(c, cudaMemcpyAsync(gen.data(), c->st.gen, (size_t)B * 4, cudaMemcpyDeviceToHost, c->stream));
-  SS_CUDA(c, cudaMemcpyAsync(fin.data(), c->st.finished, (size_t)B * 4, cudaMemcpyDeviceToHost, c->stream));
+  // row state and status come back together; the tokens (rows of the batch's cap) with them where that is little, else
+  // once it is known how many there are
+  int32_t* rows = (int32_t*)c->down;
+  int32_t* tok = (int32_t*)(c->down + kRowStateBytes);
+  auto fetch_tokens = [&](int n) {
+    return cudaMemcpy2DAsync(tok, (size_t)n * 4, c->st.out_tokens, (size_t)c->st.max_new * 4, (size_t)n * 4, B, cudaMemcpyDeviceToHost,
+                             c->stream);
+  };
+  int n_tok = out_tokens && (size_t)B * c->cap <= 16384 ? c->cap : 0;
+  SS_CUDA(c, cudaMemcpyAsync(rows, c->st.ctx_len, kRowStateBytes, cudaMemcpyDeviceToHost, c->stream));
   SS_CUDA(c, cudaMemcpyAsync(c->pinned + 1, c->status, 4, cudaMemcpyDeviceToHost, c->stream));
+  if (n_tok) SS_CUDA(c, fetch_tokens(n_tok));
   SS_CUDA(c, cudaStreamSynchronize(c->stream));
   if (c->pinned[1] != 0) return report_device_status(c, (uint32_t)c->pinned[1]);
+  const int32_t *gen = rows + 2 * kMaxBatch, *fin = rows + 4 * kMaxBatch;
+  int longest = 0;
   for (int r = 0; r < B; ++r) {
     if (out_tokens && gen[r] > stride) return SS_ERR_CAPACITY;
     out_len[r] = gen[r];
     out_status[r] = fin[r] ? 1 : 0;
+    longest = std::max(longest, gen[r]);
   }
-  if (out_tokens) {
-    for (int r = 0; r < B; ++r)
-      if (gen[r] > 0)
-        SS_CUDA(c, cudaMemcpyAsync(out_tokens + (size_t)r * stride, c->st.out_tokens + (size_t)r * c->st.max_new,
-                                   (size_t)gen[r] * 4, cudaMemcpyDeviceToHost, c->stream));
-    SS_CUDA(c, cudaStreamSynchronize(c->stream));
+  if (out_tokens && longest > 0) {
+    if (!n_tok) {
+      n_tok = longest;
+      SS_CUDA(c, fetch_tokens(n_tok));
+      SS_CUDA(c, cudaStreamSynchronize(c->stream));
+    }
+    for (int r = 0; r < B; ++r) std::copy(tok + (size_t)r * n_tok, tok + (size_t)r * n_tok + gen[r], out_tokens + (size_t)r * stride);
   }
   return SS_OK;
 }
