@@ -114,7 +114,6 @@ struct MegaSmem {
   volatile int act_epoch;          // projections whose activation operand is complete
   volatile int abort;
   int prefix[kMaxBatch + 1];
-  float inv_s[kMaxBatch];          // 1/rms of every row for the running stage
   __align__(16) float q_s[8][128]; // attention: per worker warp, rotated query (then the new token's value); read as float4
   __align__(16) float att_s[8][9][132];   // attention: [pair of the pass][partial: 8 warps + new token][acc[Dh], max, sum]
   int pair_id[8], pair_ustart[9], pair_n, pair_next, pair_lo, pair_hi;
@@ -127,7 +126,6 @@ struct MegaSmem {
   int4 seg_tab[kSegTabEntries];    // tile tables of the per-layer projections (when they fit)
   uint8_t active_s[kMaxBatch];     // rows active in this step
 };
-static_assert(sizeof(float) * 8 * 9 * 132 >= 2 * (2 * 4 * 64 * 4), "arg-max scratch aliases att_s");
 static_assert(sizeof(float) * 8 * 9 * 132 >= 8 * 32 * 36 * sizeof(float), "the drain's transposition scratch aliases att_s");
 
 __device__ __forceinline__ void named_bar_workers() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
@@ -329,44 +327,6 @@ __device__ void stage_residual(const MegaArgs& a, const MegaSmem* sm, int wtid, 
     ss = warp_sum(ss);
     if (lane == 0) a.rowss[(size_t)r * kMaxSlices + sl] = ss;
   }
-}
-
-// ---- helpers shared by the stages ----------------------------------------------------------------------
-// 1/rms of every active row into shared memory: warp w takes rows w, w+8, ... (four rows' loads in flight).
-// Split in two so that a stage can put its own loads in flight between the halves.
-struct InvRmsLoads { float v[4][2]; };
-__device__ __forceinline__ InvRmsLoads inv_rms_issue(const MegaArgs& a, const MegaSmem* sm, int r0, int lane) {
-  const int ns = (a.d + kRowSlice - 1) / kRowSlice;        // <= 64: two slices per lane
-  InvRmsLoads q;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int r = r0 + 8 * k;
-    const bool on = r < a.B && sm->active_s[r];
-    const float* p = a.rowss + (size_t)(on ? r : 0) * kMaxSlices;
-    q.v[k][0] = (on && lane < ns) ? ldcg_now(p + lane) : 0.f;
-    q.v[k][1] = (on && lane + 32 < ns) ? ldcg_now(p + lane + 32) : 0.f;
-  }
-  return q;
-}
-__device__ __forceinline__ void inv_rms_finish(const MegaArgs& a, MegaSmem* sm, const InvRmsLoads& q, int r0, int lane) {
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int r = r0 + 8 * k;
-    const float t = warp_sum(q.v[k][0] + q.v[k][1]);
-    if (r < a.B && lane == 0) sm->inv_s[r] = sm->active_s[r] ? rsqrtf(t / a.d + a.eps) : 0.f;
-  }
-}
-__device__ __forceinline__ void stage_inv_rms(const MegaArgs& a, MegaSmem* sm, int wtid) {
-  const int lane = wtid & 31, wid = wtid >> 5;
-  for (int r0 = wid; r0 < a.B; r0 += 32) {
-    const InvRmsLoads q = inv_rms_issue(a, sm, r0, lane);
-    inv_rms_finish(a, sm, q, r0, lane);
-  }
-  named_bar_workers();
-}
-
-__device__ __forceinline__ void group_bar(int id, int threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
 // ---- stage: q,k,v from partials + RoPE + cache append + paged attention ----------------------------------
@@ -1001,126 +961,84 @@ __device__ void stage_attention(const MegaArgs& a, MegaSmem* sm, int wtid, int l
 }
 
 // ---- stage: SwiGLU ----------------------------------------------------------------------------------
-// 8 consecutive features per thread (two 128-bit loads per partial segment, one 128-bit store).  The loads
-// for 1/rms and the first unit's partials are in flight together.
-__device__ __forceinline__ void gate_up_sums(const MegaArgs& a, const MegaSmem* sm, const MegaGemmShape& gs, int f0, int r, float (&gt)[8],
-                                             float (&up)[8]) {
-  const int4 tg = tile_seg(sm, gs, f0), tu = tile_seg(sm, gs, a.F + f0);
-  PartialLoads<8, 2> qg, qu;
-  partials_issue<8, 2>(a.partial, gs, a.NT, tg, f0, r, qg);
-  partials_issue<8, 2>(a.partial, gs, a.NT, tu, a.F + f0, r, qu);
-  partials_sum<8, 2>(a.partial, gs, a.NT, tg, f0, r, qg, gt);
-  partials_sum<8, 2>(a.partial, gs, a.NT, tu, a.F + f0, r, qu, up);
-}
-
-__device__ void stage_swiglu(const MegaArgs& a, MegaSmem* sm, int wtid) {
+// Work unit = (row, 256 features) per warp, 8 consecutive features per lane (two 128-bit loads per partial segment, one
+// 128-bit store); units are dealt round-robin over the CTAs.  The row is the warp's own, so its 1/rms is two more loads
+// beside the partials instead of a pass over all rows with a barrier behind it (200 rows: 19.3 -> 10.2 us).
+__device__ void stage_swiglu(const MegaArgs& a, const MegaSmem* sm, int wtid) {
   const MegaGemmShape& gs = a.shape[2];
   const int lane = wtid & 31, wid = wtid >> 5;
-  const int F8 = a.F >> 3;
-  const long long n = (long long)a.B * F8, stride = (long long)gridDim.x * kMegaWorkers;
-  long long e = (long long)blockIdx.x * kMegaWorkers + wtid;
-  const InvRmsLoads q = inv_rms_issue(a, sm, wid, lane);
-  float gt[8], up[8];
-  int r = 0, f0 = 0;
-  bool have = false;
-  if (e < n) {
-    r = (int)(e / F8);
-    f0 = (int)(e - (long long)r * F8) << 3;
-    have = sm->active_s[r] != 0;
-    if (have) gate_up_sums(a, sm, gs, f0, r, gt, up);
-  }
-  inv_rms_finish(a, sm, q, wid, lane);
-  for (int r0 = wid + 32; r0 < a.B; r0 += 32) {
-    const InvRmsLoads q2 = inv_rms_issue(a, sm, r0, lane);
-    inv_rms_finish(a, sm, q2, r0, lane);
-  }
-  named_bar_workers();
-  for (;;) {
-    if (have) {
-      const float inv = sm->inv_s[r];
-      __align__(16) bf16 ob[8];
+  const int nc = (a.F + 255) >> 8, n_units = a.B * nc;
+  for (int u = wid * gridDim.x + blockIdx.x; u < n_units; u += 8 * gridDim.x) {
+    const int r = u / nc, f0 = (u - r * nc) * 256 + lane * 8;
+    if (!sm->active_s[r]) continue;
+    const bool on = f0 < a.F;
+    const int fl = on ? f0 : 0;                           // lanes beyond the last feature read the first ones, store nothing
+    const int4 tg = tile_seg(sm, gs, fl), tu = tile_seg(sm, gs, a.F + fl);
+    PartialLoads<8, 2> qg, qu;
+    partials_issue<8, 2>(a.partial, gs, a.NT, tg, fl, r, qg);
+    partials_issue<8, 2>(a.partial, gs, a.NT, tu, a.F + fl, r, qu);
+    const float inv = warp_row_inv_rms(a, r, lane);
+    float gt[8], up[8];
+    partials_sum<8, 2>(a.partial, gs, a.NT, tg, fl, r, qg, gt);
+    partials_sum<8, 2>(a.partial, gs, a.NT, tu, a.F + fl, r, qu, up);
+    __align__(16) bf16 ob[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const float gv = gt[j] * inv;
-        ob[j] = __float2bfloat16_rn(__fdividef(gv, 1.f + __expf(-gv)) * (up[j] * inv));
-      }
-      *reinterpret_cast<uint4*>(a.act + (size_t)r * a.F + f0) = *reinterpret_cast<const uint4*>(ob);
+    for (int j = 0; j < 8; ++j) {
+      const float gv = gt[j] * inv;
+      ob[j] = __float2bfloat16_rn(__fdividef(gv, 1.f + __expf(-gv)) * (up[j] * inv));
     }
-    e += stride;
-    if (e >= n) break;
-    r = (int)(e / F8);
-    f0 = (int)(e - (long long)r * F8) << 3;
-    have = sm->active_s[r] != 0;
-    if (have) gate_up_sums(a, sm, gs, f0, r, gt, up);
+    if (on) *reinterpret_cast<uint4*>(a.act + (size_t)r * a.F + f0) = *reinterpret_cast<const uint4*>(ob);
   }
 }
 
 // ---- stage: per-tile arg-max of the logits --------------------------------------------------------------
-// One vocabulary tile per half of the workers (128 threads = the tile's rows).
-__device__ void stage_tile_argmax(const MegaArgs& a, MegaSmem* sm, int wtid) {
+// Work unit = (256-row vocabulary tile, two batch rows) per warp, 8 consecutive ids per lane: the decision among a
+// lane's ids needs no exchange, so a (tile, row) costs one warp reduction, and the units of many rows spread over
+// every warp of the chip.  Before, a tile's 128 ids sat on 128 threads that walked through all rows one after the other,
+// a reduction each, on half of the CTAs (16 / 45 sampled / 200 rows: 17.8 / 54.5 / 108 -> 11.3 / 40.0 / 47.7 us).
+__device__ void stage_tile_argmax(const MegaArgs& a, const MegaSmem* sm, int wtid) {
   const MegaGemmShape& gs = a.shape[4];
-  const int half_id = wtid >> 7, t128 = wtid & 127, lane = wtid & 31, w4 = t128 >> 5;
-  // scratch [tile half][4 warps][64 batch rows] of keys, then of ids, in the attention partials' space
-  uint32_t* s_key = reinterpret_cast<uint32_t*>(&sm->att_s[0][0][0]) + half_id * 256;
-  int* s_id = reinterpret_cast<int*>(&sm->att_s[0][0][0]) + 512 + half_id * 256;
-  stage_inv_rms(a, sm, wtid);
-  const size_t slot_stride = (size_t)a.NT * kTileN, cta_stride = slot_stride * gs.max_seg;
-  for (int tile0 = blockIdx.x * 2; tile0 < a.n_tiles_lm; tile0 += gridDim.x * 2) {
-    const int tile = tile0 + half_id;                   // 128 vocabulary rows: one half of a 256-row GEMM tile
-    const bool tile_ok = tile < a.n_tiles_lm;
-    const int v = tile * 128 + t128;
-    int4 ts = make_int4(0, 1, 0, 0);
-    if (tile_ok) ts = tile_seg(sm, gs, v);
-    for (int rb = 0; rb < a.B; rb += 64) {              // 64 batch rows at a time (scratch holds 4 x 64 per half)
-      const int rend = min(a.B, rb + 64);
-      for (int r0 = rb; r0 < rend; r0 += 8) {           // 8 rows' partial loads in flight together
-        float x0[8], x1[8], x2[8];
-        const size_t col = (size_t)(v % kTileN);
+  const int lane = wtid & 31, wid = wtid >> 5;
+  const int n_units = gs.n_tiles * ((a.B + 1) >> 1);
+  for (int u = wid * gridDim.x + blockIdx.x; u < n_units; u += 8 * gridDim.x) {
+    const int rg = u / gs.n_tiles, tile = u - rg * gs.n_tiles;
+    const int v0 = tile * kTileN + lane * 8;
+    const int4 ts = tile_seg(sm, gs, v0);
+    PartialLoads<8, 2> q[2];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int r = r0 + j;
-          const bool on = tile_ok && r < rend && sm->active_s[r] && v < a.V;
-          const size_t off = (size_t)(on ? r : 0) * kTileN + col;
-          x0[j] = on ? __ldcg(a.partial + (size_t)ts.x * slot_stride + off) : 0.f;
-          x1[j] = (on && ts.y <= ts.z) ? __ldcg(a.partial + (size_t)ts.y * cta_stride + off) : 0.f;
-          x2[j] = (on && ts.y + 1 <= ts.z) ? __ldcg(a.partial + (size_t)(ts.y + 1) * cta_stride + off) : 0.f;
-        }
+    for (int k = 0; k < 2; ++k) partials_issue<8, 2>(a.partial, gs, a.NT, ts, v0, min(2 * rg + k, a.B - 1), q[k]);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int r = r0 + j;
-          if (r >= rend) break;                           // uniform over the CTA
-          uint32_t key = 0;
-          if (tile_ok && sm->active_s[r] && v < a.V) {
-            float lg = x0[j] + x1[j] + x2[j];             // CTA order: slot0, c_next, c_next + 1, ...
-            const size_t off = (size_t)r * kTileN + col;
-            for (int c = ts.y + 2; c <= ts.z; ++c) lg += __ldcg(a.partial + (size_t)c * cta_stride + off);
-            lg *= sm->inv_s[r];
-            if (a.dump_logits) a.dump_logits[(size_t)r * a.V + v] = lg;
-            if (!(a.st.eos_at[r] > 0 && v == a.eos_id))
-              key = float_order_key(decision_value(lg, a.sample, v, a.st.gen[r] + 1, a.st.row_key[r]));
-          }
-          const uint32_t best = __reduce_max_sync(0xffffffffu, key);
-          const uint32_t who = __ballot_sync(0xffffffffu, key == best);
-          if (lane == 0) {
-            s_key[w4 * 64 + (r - rb)] = best;
-            s_id[w4 * 64 + (r - rb)] = tile * 128 + w4 * 32 + (__ffs(who) - 1);
+    for (int k = 0; k < 2; ++k) {
+      const int r = 2 * rg + k;
+      if (r >= a.B || !sm->active_s[r]) continue;         // warp-uniform
+      const float inv = warp_row_inv_rms(a, r, lane);
+      int gen = a.st.gen[r] + 1;
+      const int key_r = a.st.row_key[r];
+      const int skip = a.st.eos_at[r] > 0 ? a.eos_id : -1;
+      float lg[8];
+      partials_sum<8, 2>(a.partial, gs, a.NT, ts, v0, r, q[k], lg);
+      uint32_t bk = 0;                                    // below every real key
+      int bi = v0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        lg[j] *= inv;
+        const int v = v0 + j;
+        if (v < a.V) {
+          if (a.dump_logits) a.dump_logits[(size_t)r * a.V + v] = lg[j];
+          if (v != skip) {
+            const uint32_t key = float_order_key(decision_value(lg[j], a.sample, v, gen, key_r));
+            if (key > bk) { bk = key; bi = v; }           // ids ascend: '>' keeps the lowest
+            asm volatile("" : "+r"(gen) : "r"(bk));       // one draw after the other: eight at once do not fit the registers
           }
         }
       }
-      named_bar_workers();
-      if (tile_ok) {
-        for (int r = rb + t128; r < rend; r += 128) {
-          if (!sm->active_s[r]) continue;
-          uint32_t bk = s_key[r - rb];
-          int bi = s_id[r - rb];
-#pragma unroll
-          for (int w = 1; w < 4; ++w)
-            if (s_key[w * 64 + (r - rb)] > bk) { bk = s_key[w * 64 + (r - rb)]; bi = s_id[w * 64 + (r - rb)]; }
-          a.tile_val[(size_t)r * a.n_tiles_lm + tile] = __uint_as_float(bk);
-          a.tile_idx[(size_t)r * a.n_tiles_lm + tile] = bi;
-        }
+      const uint32_t best = __reduce_max_sync(0xffffffffu, bk);
+      const uint32_t who = __ballot_sync(0xffffffffu, bk == best);
+      bi = __shfl_sync(0xffffffffu, bi, __ffs(who) - 1);  // the lowest lane holds the lowest ids
+      if (lane == 0) {
+        a.tile_val[(size_t)r * a.n_tiles_lm + tile] = __uint_as_float(best);
+        a.tile_idx[(size_t)r * a.n_tiles_lm + tile] = bi;
       }
-      named_bar_workers();
     }
   }
 }
@@ -1133,7 +1051,7 @@ __device__ void stage_final(const MegaArgs& a, int wtid) {
     if (a.st.active[r]) {
       uint32_t bk = 0;
       int bi = 0x7fffffff;
-      for (int t = lane; t < a.n_tiles_lm; t += 32) {
+      for (int t = lane; t < a.shape[4].n_tiles; t += 32) {
         const uint32_t k = __float_as_uint(__ldcg(a.tile_val + (size_t)r * a.n_tiles_lm + t));
         const int id = __ldcg(a.tile_idx + (size_t)r * a.n_tiles_lm + t);
         if (k > bk || (k == bk && id < bi)) { bk = k; bi = id; }
