@@ -40,6 +40,9 @@ constexpr int kMegaMaxStages = 8;          // ring depth bound (shared memory ho
 constexpr int kSegTabEntries = 256;        // tile-table entries kept in shared memory (the four per-layer projections)
 constexpr int kRowSlice = 128;             // elements of a row handled by one residual work item (one warp, 4 per lane)
 constexpr int kMaxSlices = 64;             // d_model <= 8192
+constexpr int kKvPieceBytes = 4096;        // one bulk copy of the cache scan: the keys (or values) of one unit
+constexpr int kKvMaxPieces = 4;            // pieces in flight per worker warp, at most
+constexpr int kPgTab = 512;                // units whose page ids are kept in shared memory
 
 enum : uint32_t { kStatusGridBarrierTimeout = 5, kStatusFlagTimeout = 6 };
 
@@ -68,7 +71,7 @@ struct MegaArgs {
   const uint8_t* const* wptr;      // [4*L + 1] tiled weights in execution order (qkv, o, gate/up, down)*L, lm head
   const bf16* const* norm_ptr;     // [2*L + 1] gains: attn_norm(l), ffn_norm(l) ..., final
   const bf16* embed;
-  const float* inv_freq;
+  const float2* rope;              // [position][Dh / 2] (cos, sin)
   MegaGemmShape shape[5];          // qkv, o, gate/up, down, lm head
   // batch
   int B, NT, stages;
@@ -76,6 +79,9 @@ struct MegaArgs {
   int x_rows;                      // activation rows per TMA load (the tensor map's box height)
   RowState st;
   KvLayout kv;
+  int kv_pieces;                   // shared-memory pieces per worker warp for the cache scan
+  float* att_part;                 // [CTA][Dh + 2] (acc, max, sum) of the pair a CTA's range starts inside of
+  unsigned long long* att_flag;    // [CTA] set to the running barrier's number once att_part[CTA] is complete
   // activations (decode buffers)
   float* h;                        // [B][d] residual stream
   bf16 *x, *o, *act;               // GEMM operands: x' [B][d], attention out [B][d], SwiGLU out [B][F]
@@ -114,19 +120,36 @@ struct MegaSmem {
   volatile int act_epoch;          // projections whose activation operand is complete
   volatile int abort;
   int prefix[kMaxBatch + 1];
-  __align__(16) float q_s[8][128]; // attention: per worker warp, rotated query (then the new token's value); read as float4
-  __align__(16) float att_s[8][9][132];   // attention: [pair of the pass][partial: 8 warps + new token][acc[Dh], max, sum]
-  int pair_id[8], pair_ustart[9], pair_n, pair_next, pair_lo, pair_hi;
-  // per-step attention set-up that does not change from layer to layer (valid when att_single)
-  int att_single;                  // the CTA's pairs fit one pass: the lists above are built once per step
-  int att_warp_pairs;              // the CTA's run has many pairs: every warp takes whole pairs (attention_warp_pairs)
-  int pair_pos[8], pair_pgnew[8];  // per pass: new token's position and page
-  int unit_pg[8][8];               // per pass: ids of the first 8 pages of each warp's slice of the scan
-  float rope_c[8][128], rope_sn[8][128];   // cos / sin of the new position per pair, cooperative lane layout
+  // attention, set up once per step (the lengths do not change between layers): every warp's slice of the cache scan
+  int sl_begin[8], sl_n[8];        // its first unit and its units
+  int sl_r[8], sl_hd[8], sl_u0[8]; // its first unit's row, head and place in the pair
+  int sl_head[8];                  // pair the slice starts inside of, or -1
+  int sl_tail[8];                  // pair that starts in the slice and goes on behind it, or -1
+  int att_head;                    // pair the CTA's range starts inside of, or -1
+  int att_cut;                     // some pair is cut between warps (or CTAs): there is something to merge
+  int att_row0;                    // first row of the CTA's range: pg_tab holds the page of every unit from there on
+  int max_units;
+  int cost[kMaxBatch + 1];         // as prefix, in work: a row's units and kAttnPairCost
+  uint64_t kv_full[8][kKvMaxPieces];
+  int ctx_s[kMaxBatch];            // cached tokens of every row
+  int pg_tab[kPgTab];
   int4 seg_tab[kSegTabEntries];    // tile tables of the per-layer projections (when they fit)
   uint8_t active_s[kMaxBatch];     // rows active in this step
 };
-static_assert(sizeof(float) * 8 * 9 * 132 >= 8 * 32 * 36 * sizeof(float), "the drain's transposition scratch aliases att_s");
+// Scratch behind MegaSmem.  In the attention stage: every warp's rotated query, then two partials per warp.  In a drain:
+// the transposition of 16 outputs of a warp's tokens (16 in the kernel of the small batches, else 32; rows padded to 20).
+struct AttnScratch {
+  float q_s[8][128];
+  float slot[8][2][132];           // [warp][0: the pair it starts inside of, 1: the pair that goes on][acc[Dh], max, sum]
+};
+constexpr int kDrainPad = 20;
+__host__ __device__ constexpr int mega_scratch_bytes(bool wide) {
+  return wide ? 8 * 32 * kDrainPad * 4 : (int)sizeof(AttnScratch);
+}
+static_assert(sizeof(AttnScratch) >= 8 * 16 * kDrainPad * 4 && sizeof(AttnScratch) <= mega_scratch_bytes(true), "scratch");
+static_assert(sizeof(MegaSmem) % 16 == 0, "the scratch is read as float4");
+static_assert(sizeof(MegaSmem) + mega_scratch_bytes(true) + 1024 + 2 * (kBlockBytes + 2 * 128 * kTileK * 2) + 2 * 8 * kKvPieceBytes <= 227 * 1024,
+              "two ring stages and two pieces per warp fit beside the widest batch's scratch");
 
 __device__ __forceinline__ void named_bar_workers() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
@@ -275,14 +298,17 @@ __device__ __forceinline__ void sum_partials_cg(const MegaSmem* sm, const float*
   partials_sum<N, BATCH>(partial, s, NT, t, n0, tok, q, x);
 }
 
-// 1/rms of row r; warp-collective (every lane returns it).  Lane i reads slices i, i+32.
-__device__ __forceinline__ float warp_row_inv_rms(const MegaArgs& a, int r, int lane) {
+// 1/rms of row r; warp-collective (every lane returns it).  Lane i reads slices i, i+32; issue and finish are apart so
+// that a stage can put its own loads in between.
+__device__ __forceinline__ float row_ss_issue(const MegaArgs& a, int r, int lane) {
   const int ns = (a.d + kRowSlice - 1) / kRowSlice;        // <= 64
   const float* p = a.rowss + (size_t)r * kMaxSlices;
   const float v0 = lane < ns ? ldcg_now(p + lane) : 0.f;
   const float v1 = lane + 32 < ns ? ldcg_now(p + lane + 32) : 0.f;
-  return rsqrtf(warp_sum(v0 + v1) / a.d + a.eps);
+  return v0 + v1;
 }
+__device__ __forceinline__ float row_ss_inv_rms(const MegaArgs& a, float ss) { return rsqrtf(warp_sum(ss) / a.d + a.eps); }
+__device__ __forceinline__ float warp_row_inv_rms(const MegaArgs& a, int r, int lane) { return row_ss_inv_rms(a, row_ss_issue(a, r, lane)); }
 
 // ---- stage: embedding (or residual add) + lazy RMSNorm operand -------------------------------------
 // Work unit = (row, slice of 128 columns) per warp, 4 columns per lane; units are dealt round-robin over
@@ -330,94 +356,242 @@ __device__ void stage_residual(const MegaArgs& a, const MegaSmem* sm, int wtid, 
 }
 
 // ---- stage: q,k,v from partials + RoPE + cache append + paged attention ----------------------------------
-// Work is dealt in units of (row, head, one batch of loads = kAttnU load steps of cached tokens: 16 tokens
-// at head size 128, i.e. half a page).  Every CTA owns a contiguous run of (row, head) pairs holding
-// about 1/gridDim of all units (pairs are not split across CTAs, so their partial results meet in shared
-// memory).  A CTA works through its pairs in passes of up to 8:
-//   A  warp j builds pair j's rotated query (shared memory) and the new token's k,v: appended to the
-//      page, and entered as the pair's ninth partial (score, 1, v);
-//   B  the pass's units are cut into 8 equal contiguous slices, one per warp; a warp scans its units
-//      and leaves one (max, sum, acc) partial per pair it touched;
-//   C  warp j merges pair j's partials and writes the bf16 output.
-// Scan layout: a key row is Dh/8 chunks of 16 bytes; lane (g, gl) of the warp handles key g of the
-// load step and chunks gl, gl+GROUP, gl+2*GROUP, gl+3*GROUP, so each warp-wide load reads 64
-// contiguous bytes per key (full sectors).
-constexpr int kAttnPass = 8;               // pairs per pass (= worker warps)
-constexpr int kAttnU = 2;                  // load steps per work unit of the cache scan (one batch of loads in flight)
-constexpr int kAttnSlots = 9;              // partials per pair: one per warp + the new token
-constexpr int kAttnWarpPairsMin = 24;      // pairs in a CTA's run from which every warp takes whole pairs (at most 1/3 idle)
+// Work is counted in units of (row, head, 8 KiB of cache): 16 cached tokens at head size 128, 32 at 64; their keys and
+// their values are contiguous 4 KiB each.  All units of the step, in (row, head, token) order, are cut into one
+// contiguous range per CTA and that into one slice per worker warp, once per step.
+//
+// A warp streams its slice through its own few pieces of shared memory with bulk copies (keys and values of a unit are
+// one piece each): a piece is asked for as soon as the one before it in the same place has been read, across pairs and
+// -- the cache does not depend on this step's projections -- across layers, so a warp has its next pieces in flight
+// while it computes, sits in a barrier or builds a query.  Before, a warp held one unit's loads in registers and worked
+// on them before it asked for the next: the scan moved 4.2 to 4.7 TB/s (24 rows of 1700 cached tokens, 13B shape).
+//
+// A warp builds the query of every pair its slice touches (the warp with the pair's first unit also appends the new
+// token's key and value and starts from its score), so warps do not wait for one another; only pairs that are cut
+// between warps are merged at the end, through shared memory.  Ranges end between pairs unless some row is long
+// (kAttnCutUnits): then a pair may be cut between CTAs too, and the CTA that has its start collects the others'
+// partials from global memory, each announced by a flag.
+//
+// Scan layout: keys -- lane (g, gl) takes key g of a load step and a quarter (half at Dh 64) of its chunks, ordered so
+// that the eight lanes of a shared-memory phase hit different banks; values -- a lane owns four dimensions of every key
+// (every second key at Dh 64), so the running sum is four registers and needs no exchange at the end.
+constexpr int kAttnCutUnits = 40;          // units of the longest row from which pairs are cut between CTAs
+constexpr int kAttnPairCost = 2;           // what a pair costs beside its units (query, new token), in units
 
-// Tables of the pass whose pair list is in shared memory: the new tokens' positions and pages, the ids of the first
-// pages of every warp's slice of the scan (all requested together, so that the scan itself starts no chain of
-// dependent look-ups), and -- with_rope, for a CTA whose pairs fit one pass: once per step -- the rotations.
-template <int DH>
-__device__ __forceinline__ void attention_pass_tables(const MegaArgs& a, MegaSmem* sm, int wtid, bool with_rope) {
-  constexpr int EPL = DH / 32;
-  constexpr int UT = kAttnU * (32 / (DH / 32));
-  constexpr int UPP = kPageTokens / UT;
-  const int lane = wtid & 31, wid = wtid >> 5;
-  const int H = a.H;
-  const int np = sm->pair_n, U = sm->pair_ustart[np];
-  if (wid < np) {
-    const int p = sm->pair_id[wid];
-    const int r = p / H;
-    const int pos = a.st.ctx_len[r];
-    if (with_rope) {
-#pragma unroll
-      for (int j = 0; j < EPL; ++j) {
-        float sn, cs;
-        sincosf((float)pos * a.inv_freq[(lane & 15) * EPL + j], &sn, &cs);
-        sm->rope_c[wid][lane * EPL + j] = cs;
-        sm->rope_sn[wid][lane * EPL + j] = sn;
-      }
-    }
-    if (lane == 0) {
-      sm->pair_pos[wid] = pos;
-      sm->pair_pgnew[wid] = a.st.block_table[(size_t)r * a.st.max_pages + pos / kPageTokens];
-    }
-  }
-  // page ids of the first (up to 8) distinct pages of this warp's slice, in scan order
-  const int u0 = (int)((long long)wid * U / 8), u1 = (int)((long long)(wid + 1) * U / 8);
-  const int u = u0 + lane;
-  int j = 0, ui = 0;
-  bool newpage = false;
-  if (u < u1) {
-    while (j + 1 < np && sm->pair_ustart[j + 1] <= u) ++j;
-    ui = u - sm->pair_ustart[j];
-    newpage = lane == 0 || ui % UPP == 0;
-  }
-  const unsigned int starts = __ballot_sync(0xffffffffu, newpage);
-  const int ord = __popc(starts & (0xffffffffu >> (31 - lane))) - 1;
-  if (newpage && ord < 8)
-    sm->unit_pg[wid][ord] = a.st.block_table[(size_t)(sm->pair_id[j] / H) * a.st.max_pages + ui / UPP];
+template <int DH> struct AttnLayout {
+  static constexpr int GROUP = DH / 32;           // lanes per key
+  static constexpr int KPW = 32 / GROUP;          // keys per warp-wide load step
+  static constexpr int UT = 2 * KPW;              // cached tokens per unit
+  static constexpr int UPP = kPageTokens / UT;    // units per page (2 at Dh 128, 1 at Dh 64)
+  static constexpr int VK = 128 / DH;             // keys per value step (16 steps per unit)
+  static constexpr int EPL = DH / 32;             // cooperative layout: consecutive dimensions per lane
+};
+
+// Packed pairs of fp32: two fused multiply-adds per instruction.
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// Two bf16 in a word -> two fp32 (element 0 in the low half).
+__device__ __forceinline__ uint64_t bf16x2_to_f32x2(uint32_t u) {
+  return pack_f32x2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
 }
 
-// Once per step (the lengths do not change between layers): units per row, this CTA's run of pairs, and --
-// when the run fits one pass -- the pass list, the new tokens' positions/pages/rotations and the ids of
-// the first pages of every warp's slice.
-template <int DH, bool WIDE>
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint2 lds64(uint32_t addr) {
+  uint2 v;
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory");
+  return v;
+}
+
+// A warp's stream of cache pieces: where the next copy comes from, and the place of the next piece to be read.  The
+// pieces of a pair of t units follow in the order K0, K1, V0, K2, V1, .., V(t-1), the order in which they are read.
+// Lane i holds source and size of piece i of the current 32 and issues it: the search for a piece's pair, page and
+// position is done for 32 pieces at a time (and once per step where a slice has no more).
+struct KvStream {
+  uint32_t base;           // shared-memory address of the warp's pieces
+  uint64_t hint;
+  const bf16* src;         // this lane's piece: its place in layer 0, its bytes
+  uint32_t bytes;
+  int next, total, layer;  // piece of the slice to ask for next, pieces of the slice, layer
+  int in_slot, out_slot;   // place of the next copy / of the next piece to be read
+  uint32_t out_phase;
+  int flight;              // copies not read yet
+};
+
+// This lane's piece of the 32 from `first` on.
+template <int DH>
+__device__ __forceinline__ void kv_stream_locate(const MegaArgs& a, MegaSmem* sm, KvStream& k, int first, int wid, int lane) {
+  using L = AttnLayout<DH>;
+  const int i = first + lane;
+  k.src = a.kv.pool;
+  k.bytes = 0;
+  if (i >= k.total) return;
+  const int H = a.H, s0 = sm->sl_begin[wid], n = sm->sl_n[wid];
+  // row of the unit s0 + i / 2, by bisection of the rows' first units
+  const int x = s0 + (i >> 1);
+  int r = 0;
+#pragma unroll
+  for (int step = kMaxBatch / 2; step > 0; step >>= 1)
+    if (sm->prefix[r + step] * H <= x) r += step;
+  // (rows without units share their successor's first unit: the last of them is the row that has it)
+  const int row0 = sm->prefix[r] * H, npr = sm->prefix[r + 1] - sm->prefix[r];
+  const int hd = (x - row0) / npr;
+  const int p0 = row0 + hd * npr;                         // the pair's first unit
+  const int f = max(p0, s0), t = min(p0 + npr, s0 + n) - f, j = i - 2 * (f - s0);
+  const int part = j == 0 ? 0 : (j == 2 * t - 1 ? 1 : (j & 1) ^ 1);
+  const int u = j == 0 ? 0 : (j == 2 * t - 1 ? t - 1 : (j & 1) ? (j + 1) >> 1 : (j >> 1) - 1);
+  const int ui = f - p0 + u;                              // unit of the pair
+  const int at = sm->prefix[r] - sm->prefix[sm->att_row0] + ui;
+  int pg;
+  if (at < kPgTab) {
+    pg = sm->pg_tab[at];
+  } else {
+    pg = a.st.block_table[(size_t)r * a.st.max_pages + ui / L::UPP];
+    if (pg < 0 || pg >= a.kv.n_pages) { atomicCAS(a.status, 0u, (uint32_t)kStatusBadPage); pg = 0; }
+  }
+  const int tok = ui * L::UT;
+  k.src = a.kv.pool + (size_t)pg * a.kv.page_elems + ((size_t)(part * H + hd) * kPageTokens + tok % kPageTokens) * DH;
+  k.bytes = (uint32_t)min(L::UT, sm->ctx_s[r] - tok) * (DH * 2);          // cached tokens only
+}
+
+// Asks for the next piece; nothing after the last layer's slice.
+template <int DH>
+__device__ __forceinline__ void kv_stream_next(const MegaArgs& a, MegaSmem* sm, KvStream& k, int wid, int lane) {
+  if (k.layer >= a.n_layers || k.total == 0) return;
+  if (lane == (k.next & 31)) {
+    const uint32_t bar = smem_u32(&sm->kv_full[wid][k.in_slot]);
+    mbar_expect_tx(bar, k.bytes);
+    bulk_load(k.base + (uint32_t)k.in_slot * kKvPieceBytes, k.src + (size_t)k.layer * a.kv.layer_stride, k.bytes, bar, k.hint);
+  }
+  ++k.flight;
+  if (++k.in_slot == a.kv_pieces) k.in_slot = 0;
+  if (++k.next == k.total) { k.next = 0; ++k.layer; }
+  if ((k.next & 31) == 0 && k.total > 32) kv_stream_locate<DH>(a, sm, k, k.next, wid, lane);
+}
+
+template <int DH>
+__device__ __forceinline__ void kv_stream_start(const MegaArgs& a, MegaSmem* sm, KvStream& k, uint32_t kv0, int wid, int lane) {
+  k.base = kv0 + (uint32_t)(wid * a.kv_pieces) * kKvPieceBytes;
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(k.hint));
+  k.layer = k.next = k.in_slot = k.out_slot = k.flight = 0;
+  k.out_phase = 0;
+  k.total = 2 * sm->sl_n[wid];
+  kv_stream_locate<DH>(a, sm, k, 0, wid, lane);
+  for (int i = 0; i < a.kv_pieces; ++i) kv_stream_next<DH>(a, sm, k, wid, lane);
+}
+
+// Waits for the next piece; returns false (in every lane) if the CTA aborted.
+__device__ __forceinline__ bool kv_stream_wait(const MegaArgs& a, MegaSmem* sm, const KvStream& k, int wid) {
+  const bool ok = mega_wait(smem_u32(&sm->kv_full[wid][k.out_slot]), k.out_phase, sm, a.status, kStatusProducerTimeout, a.wait_limit);
+  return __all_sync(0xffffffffu, ok);
+}
+// The piece has been read by every lane: its place is free and the next copy may go there.
+template <int DH>
+__device__ __forceinline__ void kv_stream_done(const MegaArgs& a, MegaSmem* sm, KvStream& k, int wid, int lane) {
+  --k.flight;
+  kv_stream_next<DH>(a, sm, k, wid, lane);
+}
+__device__ __forceinline__ uint32_t kv_stream_advance(const MegaArgs& a, KvStream& k) {
+  const uint32_t at = k.base + (uint32_t)k.out_slot * kKvPieceBytes;
+  if (++k.out_slot == a.kv_pieces) { k.out_slot = 0; k.out_phase ^= 1u; }
+  return at;
+}
+// An abandoned step leaves copies in flight: they get a bounded time to land before the shared memory is given up.
+__device__ __forceinline__ void kv_stream_end(const MegaArgs& a, MegaSmem* sm, KvStream& k, int wid, int lane) {
+  for (; k.flight > 0; --k.flight) {
+    const long long t0 = clock64();
+    while (!mbar_try_wait(smem_u32(&sm->kv_full[wid][k.out_slot]), k.out_phase) && clock64() - t0 < 2000000LL) __nanosleep(100);
+    if (++k.out_slot == a.kv_pieces) { k.out_slot = 0; k.out_phase ^= 1u; }
+  }
+}
+
+// Row, head and unit of the pair at position x of the step's units (x below their number); warp-collective.
+__device__ __forceinline__ void locate_unit(const MegaSmem* sm, int H, int x, int lane, int& r, int& hd, int& ui) {
+  int n = 0;
+#pragma unroll
+  for (int j = 0; j < kMaxBatch / 32; ++j) n += sm->prefix[lane * (kMaxBatch / 32) + j + 1] * H <= x ? 1 : 0;
+  r = __reduce_add_sync(0xffffffffu, n);                  // rows that end before x
+  const int off = x - sm->prefix[r] * H, npr = sm->prefix[r + 1] - sm->prefix[r];
+  hd = off / npr;
+  ui = off - hd * npr;
+}
+
+// The step's work, a pair counting as its units and kAttnPairCost more, has positions of its own: row r begins at
+// cost[r] * H.  locate_work gives the pair at position x (below the total), the position inside it and its units.
+__device__ __forceinline__ void locate_work(const MegaSmem* sm, int H, int x, int lane, int& r, int& hd, int& in, int& npr) {
+  int n = 0;
+#pragma unroll
+  for (int j = 0; j < kMaxBatch / 32; ++j) n += sm->cost[lane * (kMaxBatch / 32) + j + 1] * H <= x ? 1 : 0;
+  r = __reduce_add_sync(0xffffffffu, n);
+  npr = sm->prefix[r + 1] - sm->prefix[r];
+  const int off = x - sm->cost[r] * H;
+  hd = off / (npr + kAttnPairCost);
+  in = off - hd * (npr + kAttnPairCost);
+}
+// Where CTA c's range begins, as a position of work: between pairs unless the step has long rows.
+__device__ __forceinline__ int range_begin(const MegaSmem* sm, int H, int c, int n_cta, int lane) {
+  const int total = sm->cost[kMaxBatch] * H;
+  const int x = (int)((long long)c * total / n_cta);
+  if (x >= total || sm->max_units >= kAttnCutUnits) return x;
+  int r, hd, in, npr;
+  locate_work(sm, H, x, lane, r, hd, in, npr);
+  return in ? x + npr + kAttnPairCost - in : x;
+}
+// The unit at a position of work (a pair's first unit for all of its extra cost).
+__device__ __forceinline__ int unit_at(const MegaSmem* sm, int H, int x, int lane) {
+  if (x >= sm->cost[kMaxBatch] * H) return sm->prefix[kMaxBatch] * H;
+  int r, hd, in, npr;
+  locate_work(sm, H, x, lane, r, hd, in, npr);
+  return sm->prefix[r] * H + hd * npr + max(0, in - kAttnPairCost);
+}
+
+// Once per step (the lengths do not change between layers): units per row, every warp's slice, page ids.
+template <int DH>
 __device__ void attention_setup(const MegaArgs& a, MegaSmem* sm, int wtid) {
-  constexpr int UT = kAttnU * (32 / (DH / 32));   // cached tokens per work unit (16 at Dh 128, 32 at Dh 64)
+  using L = AttnLayout<DH>;
   const int lane = wtid & 31, wid = wtid >> 5;
   const int H = a.H, B = a.B;
-  // ---- per-step copies in shared memory: which rows are active, and the per-layer tile tables
-  for (int r = wtid; r < kMaxBatch; r += kMegaWorkers) sm->active_s[r] = (r < B && a.st.active[r]) ? 1 : 0;
+  // ---- per-step copies in shared memory: row state, and the per-layer tile tables
+  for (int r = wtid; r < kMaxBatch; r += kMegaWorkers) {
+    sm->active_s[r] = (r < B && a.st.active[r]) ? 1 : 0;
+    sm->ctx_s[r] = r < B ? a.st.ctx_len[r] : 0;
+  }
   for (int t = 0; t < 4; ++t) {
     const MegaGemmShape& gs = a.shape[t];
     if (gs.smem_off < 0) continue;
     for (int i = wtid; i < gs.n_tiles; i += kMegaWorkers)
       sm->seg_tab[gs.smem_off + i] = __ldg(reinterpret_cast<const int4*>(gs.tiles) + i);
   }
-  // ---- pages per row (exclusive prefix, active rows only) and this CTA's run of pairs
+  // ---- units per row (exclusive prefix, active rows only)
   if (wid == 0) {
-    int cnt[8], loc = 0;
+    int cnt[8], loc = 0, most = 0;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int r = lane * 8 + j;
       int c = 0;
-      if (r < B && a.st.active[r]) c = (a.st.ctx_len[r] + UT - 1) / UT;
+      if (r < B && a.st.active[r]) c = (a.st.ctx_len[r] + L::UT - 1) / L::UT;
       cnt[j] = c;
       loc += c;
+      most = max(most, c);
     }
     int inc = loc;
 #pragma unroll
@@ -425,574 +599,425 @@ __device__ void attention_setup(const MegaArgs& a, MegaSmem* sm, int wtid) {
       const int t = __shfl_up_sync(0xffffffffu, inc, o);
       if (lane >= o) inc += t;
     }
-    int run = inc - loc;
+    most = __reduce_max_sync(0xffffffffu, most);
+    int here = 0;                                         // active rows among this lane's eight, and before them
+#pragma unroll
+    for (int j = 0; j < 8; ++j) here += cnt[j] > 0 ? 1 : 0;
+    int rows = here;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, rows, o);
+      if (lane >= o) rows += t;
+    }
+    int run = inc - loc, n_rows = rows - here;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       sm->prefix[lane * 8 + j] = run;
+      sm->cost[lane * 8 + j] = run + n_rows * kAttnPairCost;
       run += cnt[j];
+      n_rows += cnt[j] > 0 ? 1 : 0;
     }
-    if (lane == 31) sm->prefix[kMaxBatch] = inc;
-    if (lane == 0) { sm->pair_lo = 0x7fffffff; sm->pair_hi = -1; }
+    if (lane == 31) {
+      sm->prefix[kMaxBatch] = run;
+      sm->cost[kMaxBatch] = run + n_rows * kAttnPairCost;
+    }
+    if (lane == 0) { sm->att_cut = 0; sm->max_units = most; }
   }
   named_bar_workers();
+  // ---- this CTA's range, and the slice of every warp
+  const int w_lo = range_begin(sm, H, blockIdx.x, gridDim.x, lane), w_hi = range_begin(sm, H, blockIdx.x + 1, gridDim.x, lane);
+  const int lo = unit_at(sm, H, w_lo, lane), hi = unit_at(sm, H, w_hi, lane);
+  const int s0 = unit_at(sm, H, w_lo + (int)((long long)(w_hi - w_lo) * wid / 8), lane);
+  const int s1 = unit_at(sm, H, w_lo + (int)((long long)(w_hi - w_lo) * (wid + 1) / 8), lane);
+  int r0 = 0, r1 = 0, cta_head = -1;                      // rows the CTA's range touches; pair it starts inside of
+  if (hi > lo) {
+    int hd, ui;
+    locate_unit(sm, H, hi - 1, lane, r1, hd, ui);
+    locate_unit(sm, H, lo, lane, r0, hd, ui);
+    if (ui > 0) cta_head = r0 * H + hd;
+  }
   {
-    const long long T = (long long)sm->prefix[kMaxBatch] * H;        // all units
-    const long long lo = (long long)blockIdx.x * T / gridDim.x, hi = (long long)(blockIdx.x + 1) * T / gridDim.x;
-    int mylo = 0x7fffffff, myhi = -1;
-    for (int p = wtid; p < B * H; p += kMegaWorkers) {
-      const int r = p / H, hd = p - r * H;
-      const int npr = sm->prefix[r + 1] - sm->prefix[r];     // pages of this row (0 if inactive)
-      if (npr <= 0) continue;
-      const long long cum = (long long)sm->prefix[r] * H + (long long)hd * npr;   // units before this pair
-      if (cum >= lo && cum < hi) { mylo = min(mylo, p); myhi = max(myhi, p); }
+    int r = 0, hd = 0, ui = 0, head = -1, tail = -1;
+    if (s1 > s0) {
+      int re, hde, uie;
+      locate_unit(sm, H, s1 - 1, lane, re, hde, uie);
+      if (uie + 1 < sm->prefix[re + 1] - sm->prefix[re] && s1 - 1 - uie >= s0) tail = re * H + hde;
+      locate_unit(sm, H, s0, lane, r, hd, ui);
+      if (ui > 0) head = r * H + hd;
     }
-    if (mylo <= myhi) { atomicMin(&sm->pair_lo, mylo); atomicMax(&sm->pair_hi, myhi); }
-  }
-  named_bar_workers();
-  const int p_begin = sm->pair_lo, p_end = sm->pair_hi + 1;
-  if (wid == 0) {
-    int n = 0, p = p_begin, ustart = 0;
-    while (p < p_end && n < kAttnPass) {
-      const int r = p / H;
-      const int npr = sm->prefix[r + 1] - sm->prefix[r];
-      if (npr <= 0) { p = (r + 1) * H; continue; }
-      if (lane == 0) { sm->pair_id[n] = p; sm->pair_ustart[n] = ustart; }
-      ustart += npr;
-      ++n;
-      ++p;
-    }
-    // any pair with work left beyond the first eight?
-    bool more = false;
-    for (int q = p; q < p_end && !more; ) {
-      const int r = q / H;
-      if (sm->prefix[r + 1] - sm->prefix[r] > 0) more = true; else q = (r + 1) * H;
-    }
-    if (lane == 0) { sm->pair_n = n; sm->pair_next = p; sm->pair_ustart[n] = ustart; sm->att_single = more ? 0 : 1; }
-    if constexpr (WIDE) {
-      // pairs with work in the whole run
-      int cnt = 0;
-      for (int q = p_begin; q < p_end; ) {
-        const int r = q / H;
-        const int e = min(p_end, (r + 1) * H);
-        if (sm->prefix[r + 1] - sm->prefix[r] > 0) cnt += e - q;
-        q = e;
-      }
-      if (lane == 0) sm->att_warp_pairs = cnt >= kAttnWarpPairsMin ? 1 : 0;
+    if (lane == 0) {
+      sm->sl_r[wid] = r; sm->sl_hd[wid] = hd; sm->sl_u0[wid] = ui; sm->sl_n[wid] = s1 - s0;
+      sm->sl_begin[wid] = s0; sm->sl_head[wid] = head; sm->sl_tail[wid] = tail;
+      if (head >= 0 || tail >= 0) sm->att_cut = 1;
+      if (wid == 0) { sm->att_row0 = r0; sm->att_head = cta_head; }
     }
   }
-  named_bar_workers();
-  if (sm->att_single) attention_pass_tables<DH>(a, sm, wtid, true);
+  // ---- page of every unit of these rows, as far as the table goes
+  const int first = sm->prefix[r0], n_tab = hi > lo ? min(kPgTab, sm->prefix[r1 + 1] - first) : 0;
+  for (int r = r0; r <= r1; ++r) {
+    const int at = sm->prefix[r] - first, npr = sm->prefix[r + 1] - sm->prefix[r];
+    for (int u = wtid; u < npr && at + u < n_tab; u += kMegaWorkers) {
+      int pg = a.st.block_table[(size_t)r * a.st.max_pages + u / L::UPP];
+      if (pg < 0 || pg >= a.kv.n_pages) { atomicCAS(a.status, 0u, (uint32_t)kStatusBadPage); pg = 0; }
+      sm->pg_tab[at + u] = pg;
+    }
+  }
   named_bar_workers();
 }
 
-// ---- pieces of the attention stage, each run by one warp, as attention_warp_pairs puts them together ----------
-// (stage_attention below has the same steps written out in place: it is the path of the small batches, and its
-// register allocation is what the whole kernel's speed hangs on)
-template <int DH> struct AttnLayout {
-  static constexpr int GROUP = DH / 32;           // lanes per key in the cache scan
-  static constexpr int KPW = 32 / GROUP;          // keys per warp-wide load step
-  static constexpr int EPL = DH / 32;             // cooperative layout: consecutive dimensions per lane
-  static constexpr int U = kAttnU;                // load steps per work unit: one batch of loads
-  static constexpr int UPP = kPageTokens / (U * KPW);   // units per page (2 at Dh 128, 1 at Dh 64)
+// One running partial of a pair in the value layout: lane's four dimensions, the maximum and the sum of the weights.
+struct AttnPartial {
+  float acc[4], m, l;
 };
-
-// A: the pair's rotated, scaled query into qs[DH]; the new token's k, v appended to page pg at position pos and
-// entered as the partial ns[DH + 2] = (v, score, 1).  cs / sn: the rotation of this lane's dimensions.
+__device__ __forceinline__ void attn_merge(AttnPartial& p, const float4 acc, float m, float l) {
+  const float mn = fmaxf(p.m, m);
+  const float w0 = exp2f(p.m - mn), w1 = exp2f(m - mn);
+  p.acc[0] = p.acc[0] * w0 + acc.x * w1;
+  p.acc[1] = p.acc[1] * w0 + acc.y * w1;
+  p.acc[2] = p.acc[2] * w0 + acc.z * w1;
+  p.acc[3] = p.acc[3] * w0 + acc.w * w1;
+  p.l = p.l * w0 + l * w1;
+  p.m = mn;
+}
+// The pair's bf16 output (lanes of the first VK-th part hold the DH dimensions).
 template <int DH>
-__device__ __forceinline__ void attn_prepare_pair(const MegaArgs& a, const MegaSmem* sm, int layer, int lane, int r, int hd, int pos,
-                                                  int pg, const float (&cs)[DH / 32], const float (&sn)[DH / 32], float* qs, float* ns) {
-  constexpr int EPL = AttnLayout<DH>::EPL;
-  const int H = a.H, d = a.d;
-  const MegaGemmShape& gs = a.shape[0];
-  const float qscale = rsqrtf((float)DH) * 1.4426950408889634f;
-  const size_t v_off = (size_t)H * kPageTokens * DH;
-  const float inv = warp_row_inv_rms(a, r, lane);
-  const int e0 = lane * EPL;
-  float qx[EPL], kx[EPL], vx[EPL];
-  {
-    const int nq = hd * DH + e0, nk = d + nq, nv = 2 * d + nq;
-    const int4 tq = tile_seg(sm, gs, nq), tk = tile_seg(sm, gs, nk), tv = tile_seg(sm, gs, nv);
-    PartialLoads<EPL, 4> lq, lk, lv;
-    partials_issue<EPL, 4>(a.partial, gs, a.NT, tq, nq, r, lq);
-    partials_issue<EPL, 4>(a.partial, gs, a.NT, tk, nk, r, lk);
-    partials_issue<EPL, 4>(a.partial, gs, a.NT, tv, nv, r, lv);
-    partials_sum<EPL, 4>(a.partial, gs, a.NT, tq, nq, r, lq, qx);
-    partials_sum<EPL, 4>(a.partial, gs, a.NT, tk, nk, r, lk, kx);
-    partials_sum<EPL, 4>(a.partial, gs, a.NT, tv, nv, r, lv, vx);
-  }
-  if (pg < 0 || pg >= a.kv.n_pages) { atomicCAS(a.status, 0u, (uint32_t)kStatusBadPage); pg = -1; }
-  bf16* kdst = a.kv.pool + (size_t)layer * a.kv.layer_stride + (size_t)(pg < 0 ? 0 : pg) * a.kv.page_elems +
-               ((size_t)hd * kPageTokens + (pos % kPageTokens)) * DH + e0;
-  float dot = 0.f;
+__device__ __forceinline__ void attn_store(const MegaArgs& a, const AttnPartial& p, int r, int hd, int lane) {
+  if (lane * 4 >= DH) return;
+  const float il = 1.f / p.l;
+  __align__(8) bf16 ob[4];
 #pragma unroll
-  for (int j = 0; j < EPL; ++j) {
-    const float xq = qx[j] * inv, xk = kx[j] * inv;
-    const float pq = __shfl_xor_sync(0xffffffffu, xq, 16), pk = __shfl_xor_sync(0xffffffffu, xk, 16);
-    const float oq = (lane < 16) ? xq * cs[j] - pq * sn[j] : xq * cs[j] + pq * sn[j];
-    const float ok = (lane < 16) ? xk * cs[j] - pk * sn[j] : xk * cs[j] + pk * sn[j];
-    const float qf = oq * qscale;                     // the query is only ever an ALU operand: it stays fp32
-    const bf16 kb16 = __float2bfloat16_rn(ok), vb16 = __float2bfloat16_rn(vx[j] * inv);
-    if (pg >= 0) { kdst[j] = kb16; kdst[v_off + j] = vb16; }
-    qs[e0 + j] = qf;
-    ns[e0 + j] = __bfloat162float(vb16);
-    dot += qf * __bfloat162float(kb16);
-  }
-  dot = warp_sum(dot);
-  if (lane == 0) { ns[DH] = dot; ns[DH + 1] = 1.f; }
+  for (int j = 0; j < 4; ++j) ob[j] = __float2bfloat16_rn(p.acc[j] * il);
+  *reinterpret_cast<uint2*>(a.o + (size_t)r * a.d + hd * DH + lane * 4) = *reinterpret_cast<const uint2*>(ob);
 }
 
-// B: one unit (U load steps of KPW keys; kb = first key of the page's head, s0 = first load step, tcount = the
-// page's tokens) folded into the running (m, l, acc) of the lane's key slot.
 template <int DH>
-__device__ __forceinline__ void attn_scan_unit(const bf16* __restrict__ kb, size_t v_off, int s0, int tcount, const float* qs, int g, int gl,
-                                               float& m, float& l, float (&acc)[32]) {
-  constexpr int GROUP = AttnLayout<DH>::GROUP, KPW = AttnLayout<DH>::KPW, U = AttnLayout<DH>::U;
-  uint4 kk[U][4], vv[U][4];
-#pragma unroll
-  for (int uu = 0; uu < U; ++uu) {
-    const int t = (s0 + uu) * KPW + g;
-    if (t < tcount) {
-      const uint4* kp = reinterpret_cast<const uint4*>(kb + (size_t)t * DH);
-      const uint4* vp = reinterpret_cast<const uint4*>(kb + (size_t)t * DH + v_off);
-#pragma unroll
-      for (int c = 0; c < 4; ++c) { kk[uu][c] = __ldg(kp + c * GROUP + gl); vv[uu][c] = __ldg(vp + c * GROUP + gl); }
-    } else {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) { kk[uu][c] = make_uint4(0, 0, 0, 0); vv[uu][c] = kk[uu][c]; }
-    }
-  }
-  float sc_[U];
-#pragma unroll
-  for (int uu = 0; uu < U; ++uu) {
-    float dot = 0.f;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float kf[8];
-      unpack8(kk[uu][c], kf);
-      const float4 qa = *reinterpret_cast<const float4*>(qs + (c * GROUP + gl) * 8);
-      const float4 qb = *reinterpret_cast<const float4*>(qs + (c * GROUP + gl) * 8 + 4);
-      dot += qa.x * kf[0] + qa.y * kf[1] + qa.z * kf[2] + qa.w * kf[3] + qb.x * kf[4] + qb.y * kf[5] +
-             qb.z * kf[6] + qb.w * kf[7];
-    }
-#pragma unroll
-    for (int o = GROUP / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-    sc_[uu] = ((s0 + uu) * KPW + g < tcount) ? dot : -CUDART_INF_F;
-  }
-  float mn = m;
-#pragma unroll
-  for (int uu = 0; uu < U; ++uu) mn = fmaxf(mn, sc_[uu]);
-  if (mn != -CUDART_INF_F) {
-    if (mn != m) {
-      const float sc = exp2f(m - mn);
-      l *= sc;
-#pragma unroll
-      for (int e = 0; e < 32; ++e) acc[e] *= sc;
-      m = mn;
-    }
-#pragma unroll
-    for (int uu = 0; uu < U; ++uu) {
-      if (sc_[uu] != -CUDART_INF_F) {
-        const float pw = exp2f(sc_[uu] - mn);
-        l += pw;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          float vf[8];
-          unpack8(vv[uu][c], vf);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) acc[c * 8 + e] += pw * vf[e];
-        }
-      }
-    }
-  }
-}
-
-// The warp's KPW key slots merged, the result stored as the partial slot[DH + 2] = (acc, m, l); (m, l, acc) reset.
-template <int DH>
-__device__ __forceinline__ void attn_flush(float* slot, int g, int gl, float& m, float& l, float (&acc)[32]) {
-  constexpr int GROUP = AttnLayout<DH>::GROUP;
-#pragma unroll
-  for (int o = GROUP; o < 32; o <<= 1) {
-    const float om = __shfl_xor_sync(0xffffffffu, m, o);
-    const float ol = __shfl_xor_sync(0xffffffffu, l, o);
-    const float mn = fmaxf(m, om);
-    const float w0 = (m == -CUDART_INF_F) ? 0.f : exp2f(m - mn);
-    const float w1 = (om == -CUDART_INF_F) ? 0.f : exp2f(om - mn);
-    l = l * w0 + ol * w1;
-#pragma unroll
-    for (int e = 0; e < 32; ++e) {
-      const float oa = __shfl_xor_sync(0xffffffffu, acc[e], o);
-      acc[e] = acc[e] * w0 + oa * w1;
-    }
-    m = mn;
-  }
-  if (g == 0) {
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-      for (int e = 0; e < 8; ++e) slot[(c * GROUP + gl) * 8 + e] = acc[c * 8 + e];
-    if (gl == 0) { slot[DH] = m; slot[DH + 1] = l; }
-  }
-  m = -CUDART_INF_F;
-  l = 0.f;
-#pragma unroll
-  for (int e = 0; e < 32; ++e) acc[e] = 0.f;
-}
-
-// C: the pair's partials slots[0 .. kAttnSlots) merged and written as bf16 output of (row r, head hd).
-template <int DH>
-__device__ __forceinline__ void attn_merge_pair(const MegaArgs& a, const float (*slots)[132], int lane, int r, int hd) {
-  constexpr int EPL = AttnLayout<DH>::EPL;
-  const int e0 = lane * EPL;
-  float M = -CUDART_INF_F;
-  for (int k = 0; k < kAttnSlots; ++k) M = fmaxf(M, slots[k][DH]);
-  float L = 0.f, A[EPL];
-#pragma unroll
-  for (int j = 0; j < EPL; ++j) A[j] = 0.f;
-  for (int k = 0; k < kAttnSlots; ++k) {
-    const float mk = slots[k][DH];
-    if (mk == -CUDART_INF_F) continue;
-    const float wt = exp2f(mk - M);
-    L += slots[k][DH + 1] * wt;
-#pragma unroll
-    for (int j = 0; j < EPL; ++j) A[j] += slots[k][e0 + j] * wt;
-  }
-  const float il = 1.f / L;
-#pragma unroll
-  for (int j = 0; j < EPL; ++j) a.o[(size_t)r * a.d + hd * DH + e0 + j] = __float2bfloat16_rn(A[j] * il);
-}
-
-// Wide batches, where a CTA's run has many pairs: every warp takes whole pairs (the run's pairs with work, in turn)
-// and does all three steps for them by itself, so nothing is shared between the warps and nothing holds them in
-// step: while one warp builds a query, the others' loads are in flight.  The pair's page ids are looked up by the
-// lanes together (lane i: pages i and i + 32) and handed out by shuffle.
-template <int DH>
-__device__ void attention_warp_pairs(const MegaArgs& a, MegaSmem* sm, int wtid, int layer) {
+__device__ void stage_attention(const MegaArgs& a, MegaSmem* sm, AttnScratch* sc, KvStream& kvs, int wtid, int layer,
+                                unsigned long long ticket) {
   using L = AttnLayout<DH>;
-  constexpr int GROUP = L::GROUP, EPL = L::EPL, U = L::U, UPP = L::UPP;
+  constexpr int GROUP = L::GROUP, KPW = L::KPW, UT = L::UT, VK = L::VK, EPL = L::EPL;
   const int lane = wtid & 31, wid = wtid >> 5;
   const int gl = lane % GROUP, g = lane / GROUP;
-  const int H = a.H;
-  const bf16* kv_layer = a.kv.pool + (size_t)layer * a.kv.layer_stride;
-  const size_t v_off = (size_t)H * kPageTokens * DH;
-  const int p_begin = sm->pair_lo, p_end = sm->pair_hi + 1;
-  float (*slots)[132] = sm->att_s[wid];
-  float* qs = sm->q_s[wid];
-  int n = 0;
-  for (int p = p_begin; p < p_end; ) {
-    const int r = p / H;
-    const int npr = sm->prefix[r + 1] - sm->prefix[r];
-    if (npr <= 0) { p = (r + 1) * H; continue; }
-    if ((n++ & 7) != wid) { ++p; continue; }
-    const int hd = p - r * H;
-    const int pos = a.st.ctx_len[r];
-    const int last_page = pos / kPageTokens;            // the new token's page
-    const int32_t* bt = a.st.block_table + (size_t)r * a.st.max_pages;
-    const int pgs0 = lane <= last_page ? bt[lane] : 0;
-    const int pgs1 = lane + 32 <= last_page ? bt[lane + 32] : 0;
-    if (lane < kAttnSlots) slots[lane][DH] = -CUDART_INF_F;
-    float sn[EPL], cs[EPL];
-#pragma unroll
-    for (int j = 0; j < EPL; ++j) sincosf((float)pos * a.inv_freq[(lane & 15) * EPL + j], &sn[j], &cs[j]);
-    const int pg_new = last_page < 32 ? __shfl_sync(0xffffffffu, pgs0, last_page)
-                                      : (last_page < 64 ? __shfl_sync(0xffffffffu, pgs1, last_page - 32) : bt[last_page]);
-    __syncwarp();
-    attn_prepare_pair<DH>(a, sm, layer, lane, r, hd, pos, pg_new, cs, sn, qs, slots[kAttnSlots - 1]);
-    __syncwarp();
-    float m = -CUDART_INF_F, l = 0.f, acc[32];
-#pragma unroll
-    for (int e = 0; e < 32; ++e) acc[e] = 0.f;
-    int pg = 0;
-    for (int ui = 0; ui < npr; ++ui) {
-      const int pi = ui / UPP;
-      if (ui % UPP == 0) {
-        pg = pi < 32 ? __shfl_sync(0xffffffffu, pgs0, pi) : (pi < 64 ? __shfl_sync(0xffffffffu, pgs1, pi - 32) : bt[pi]);
-        if (pg < 0 || pg >= a.kv.n_pages) { atomicCAS(a.status, 0u, (uint32_t)kStatusBadPage); pg = 0; }
-      }
-      const int tcount = min(kPageTokens, pos - pi * kPageTokens);
-      const bf16* kb = kv_layer + (size_t)pg * a.kv.page_elems + (size_t)hd * kPageTokens * DH;
-      attn_scan_unit<DH>(kb, v_off, (ui % UPP) * U, tcount, qs, g, gl, m, l, acc);
-    }
-    attn_flush<DH>(slots[0], g, gl, m, l, acc);
-    __syncwarp();
-    attn_merge_pair<DH>(a, slots, lane, r, hd);
-    __syncwarp();
-    ++p;
-  }
-}
-
-template <int DH>
-__device__ void stage_attention(const MegaArgs& a, MegaSmem* sm, int wtid, int layer) {
-  constexpr int GROUP = DH / 32;           // lanes per key in the cache scan
-  constexpr int KPW = 32 / GROUP;          // keys per warp-wide load step
-  constexpr int EPL = DH / 32;             // cooperative layout: consecutive dimensions per lane
-  constexpr int U = kAttnU;                // load steps per work unit: one batch of loads
-  constexpr int UPP = kPageTokens / (U * KPW);   // units per page (2 at Dh 128, 1 at Dh 64)
-  const int lane = wtid & 31, wid = wtid >> 5;
-  const int gl = lane % GROUP, g = lane / GROUP;
+  const int sw = g & (4 / GROUP * 2 - 1) & 3;             // bank swizzle of the key chunks: g & 1 at Dh 128, g & 3 at Dh 64
+  const int dl = (lane * 4) % DH, vk = lane * 4 / DH;     // value layout: first of the lane's dimensions, key of a step
   const int H = a.H, d = a.d;
   const MegaGemmShape& gs = a.shape[0];
   const float qscale = rsqrtf((float)DH) * 1.4426950408889634f;
-  const bf16* kv_layer = a.kv.pool + (size_t)layer * a.kv.layer_stride;
   const size_t v_off = (size_t)H * kPageTokens * DH;
 
-  const int p_begin = sm->pair_lo, p_end = sm->pair_hi + 1;          // empty run: lo > hi
-  const bool single = sm->att_single != 0;
-
-  for (int pass0 = p_begin; pass0 < p_end; ) {
-    // ---- the pass: next (up to 8) pairs with work; pair_id / pair_pages / pair_ustart in shared memory
-    if (wid == 0 && !single) {
-      int n = 0, p = pass0, ustart = 0;
-      // lanes walk the pairs together (few iterations: rows without work are skipped by whole rows)
-      while (p < p_end && n < kAttnPass) {
-        const int r = p / H;
-        const int npr = sm->prefix[r + 1] - sm->prefix[r];
-        if (npr <= 0) { p = (r + 1) * H; continue; }
-        if (lane == 0) { sm->pair_id[n] = p; sm->pair_ustart[n] = ustart; }
-        ustart += npr;
-        ++n;
-        ++p;
-      }
-      if (lane == 0) { sm->pair_n = n; sm->pair_next = p; sm->pair_ustart[n] = ustart; }
-    }
-    for (int i = wtid; i < kAttnPass * kAttnSlots; i += kMegaWorkers) sm->att_s[i / kAttnSlots][i % kAttnSlots][DH] = -CUDART_INF_F;
-    named_bar_workers();
-    if (!single) {
-      // positions and page ids of this pass, looked up together (a CTA with one pass did this once per step)
-      attention_pass_tables<DH>(a, sm, wtid, false);
-      named_bar_workers();
-    }
-    const int np_pass = sm->pair_n;
-    const int U_pass = sm->pair_ustart[np_pass];
-
-    // ---- A: warp j prepares pair j
-    if (wid < np_pass) {
-      const int p = sm->pair_id[wid];
-      const int r = p / H, hd = p - r * H;
-      const int pos = sm->pair_pos[wid];
-      const float inv = warp_row_inv_rms(a, r, lane);
-      const int e0 = lane * EPL;
-      float sn[EPL], cs[EPL];
+  int r = sm->sl_r[wid], hd = sm->sl_hd[wid], ui = sm->sl_u0[wid], left = sm->sl_n[wid];
+  bool aborted = false;                                   // a wait ran out: this warp only keeps the barriers from here on
+  while (left > 0 && !aborted) {
+    const int npr = sm->prefix[r + 1] - sm->prefix[r], pos = sm->ctx_s[r];
+    const int take = min(npr - ui, left);
+    const bool own = ui == 0;                             // this warp has the pair's first unit: the new token is its
+    const bool whole = own && take == npr;
+    AttnPartial p;
+    uint64_t q2[16];
+    // ---- the rotated, scaled query; the new token's key and value
+    {
+      const int e0 = lane * EPL, nq = hd * DH + e0, nk = d + nq, nv = 2 * d + nq;
+      const int4 tq = tile_seg(sm, gs, nq), tk = tile_seg(sm, gs, nk), tv = tile_seg(sm, gs, nv);
+      PartialLoads<EPL, 4> lq, lk, lv;
+      partials_issue<EPL, 4>(a.partial, gs, a.NT, tq, nq, r, lq);
+      partials_issue<EPL, 4>(a.partial, gs, a.NT, tk, nk, r, lk);
+      partials_issue<EPL, 4>(a.partial, gs, a.NT, tv, nv, r, lv);
+      const float2* rp = a.rope + (size_t)pos * (DH / 2) + (lane & 15) * EPL;
+      float2 cs[EPL];
 #pragma unroll
-      for (int j = 0; j < EPL; ++j) {
-        if (single) { cs[j] = sm->rope_c[wid][e0 + j]; sn[j] = sm->rope_sn[wid][e0 + j]; }
-        else sincosf((float)pos * a.inv_freq[(lane & 15) * EPL + j], &sn[j], &cs[j]);
-      }
+      for (int j = 0; j < EPL; ++j) cs[j] = __ldg(rp + j);
+      int pg = own ? a.st.block_table[(size_t)r * a.st.max_pages + pos / kPageTokens] : 0;
+      const float inv = warp_row_inv_rms(a, r, lane);
       float qx[EPL], kx[EPL], vx[EPL];
-      {
-        const int nq = hd * DH + e0, nk = d + nq, nv = 2 * d + nq;
-        const int4 tq = tile_seg(sm, gs, nq), tk = tile_seg(sm, gs, nk), tv = tile_seg(sm, gs, nv);
-        PartialLoads<EPL, 4> lq, lk, lv;
-        partials_issue<EPL, 4>(a.partial, gs, a.NT, tq, nq, r, lq);
-        partials_issue<EPL, 4>(a.partial, gs, a.NT, tk, nk, r, lk);
-        partials_issue<EPL, 4>(a.partial, gs, a.NT, tv, nv, r, lv);
-        partials_sum<EPL, 4>(a.partial, gs, a.NT, tq, nq, r, lq, qx);
-        partials_sum<EPL, 4>(a.partial, gs, a.NT, tk, nk, r, lk, kx);
-        partials_sum<EPL, 4>(a.partial, gs, a.NT, tv, nv, r, lv, vx);
-      }
-      int pg = sm->pair_pgnew[wid];
+      partials_sum<EPL, 4>(a.partial, gs, a.NT, tq, nq, r, lq, qx);
+      partials_sum<EPL, 4>(a.partial, gs, a.NT, tk, nk, r, lk, kx);
+      partials_sum<EPL, 4>(a.partial, gs, a.NT, tv, nv, r, lv, vx);
       if (pg < 0 || pg >= a.kv.n_pages) { atomicCAS(a.status, 0u, (uint32_t)kStatusBadPage); pg = -1; }
-      bf16* kdst = a.kv.pool + (size_t)layer * a.kv.layer_stride + (size_t)(pg < 0 ? 0 : pg) * a.kv.page_elems +
-                   ((size_t)hd * kPageTokens + (pos % kPageTokens)) * DH + e0;
-      float dot = 0.f;
-      float* qs = sm->q_s[wid];
-      float* ns = sm->att_s[wid][kAttnSlots - 1];
+      __align__(8) bf16 kb[EPL], vb[EPL];
+      float qf[EPL], dot = 0.f;
 #pragma unroll
       for (int j = 0; j < EPL; ++j) {
         const float xq = qx[j] * inv, xk = kx[j] * inv;
         const float pq = __shfl_xor_sync(0xffffffffu, xq, 16), pk = __shfl_xor_sync(0xffffffffu, xk, 16);
-        const float oq = (lane < 16) ? xq * cs[j] - pq * sn[j] : xq * cs[j] + pq * sn[j];
-        const float ok = (lane < 16) ? xk * cs[j] - pk * sn[j] : xk * cs[j] + pk * sn[j];
-        const float qf = oq * qscale;                     // the query is only ever an ALU operand: it stays fp32
-        const bf16 kb16 = __float2bfloat16_rn(ok), vb16 = __float2bfloat16_rn(vx[j] * inv);
-        if (pg >= 0) { kdst[j] = kb16; kdst[v_off + j] = vb16; }
-        qs[e0 + j] = qf;
-        ns[e0 + j] = __bfloat162float(vb16);
-        dot += qf * __bfloat162float(kb16);
+        const float oq = (lane < 16) ? xq * cs[j].x - pq * cs[j].y : xq * cs[j].x + pq * cs[j].y;
+        const float ok = (lane < 16) ? xk * cs[j].x - pk * cs[j].y : xk * cs[j].x + pk * cs[j].y;
+        qf[j] = oq * qscale;                              // the query is only ever an ALU operand: it stays fp32
+        kb[j] = __float2bfloat16_rn(ok);
+        vb[j] = __float2bfloat16_rn(vx[j] * inv);
+        dot += qf[j] * __bfloat162float(kb[j]);
       }
+      float* qs = sc->q_s[wid];
+      __syncwarp();                                       // the warp has read the query before this one
+      if constexpr (EPL == 4) *reinterpret_cast<float4*>(qs + e0) = make_float4(qf[0], qf[1], qf[2], qf[3]);
+      else *reinterpret_cast<float2*>(qs + e0) = make_float2(qf[0], qf[1]);
       dot = warp_sum(dot);
-      if (lane == 0) { ns[DH] = dot; ns[DH + 1] = 1.f; }
+      if (own) {
+        if (pg >= 0) {
+          bf16* kdst = a.kv.pool + (size_t)layer * a.kv.layer_stride + (size_t)pg * a.kv.page_elems +
+                       ((size_t)hd * kPageTokens + (pos % kPageTokens)) * DH + e0;
+          if constexpr (EPL == 4) {
+            *reinterpret_cast<uint2*>(kdst) = *reinterpret_cast<const uint2*>(kb);
+            *reinterpret_cast<uint2*>(kdst + v_off) = *reinterpret_cast<const uint2*>(vb);
+          } else {
+            *reinterpret_cast<uint32_t*>(kdst) = *reinterpret_cast<const uint32_t*>(kb);
+            *reinterpret_cast<uint32_t*>(kdst + v_off) = *reinterpret_cast<const uint32_t*>(vb);
+          }
+        }
+        p.m = dot;
+        p.l = g == 0 ? 1.f : 0.f;                         // summed over the key slots at the end
+        if constexpr (EPL == 4) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) p.acc[j] = __bfloat162float(vb[j]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float t = __shfl_sync(0xffffffffu, __bfloat162float(vb[j & 1]), (dl + j) >> 1);
+            p.acc[j] = vk == 0 ? t : 0.f;
+          }
+        }
+      } else {
+        p.m = -CUDART_INF_F;
+        p.l = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) p.acc[j] = 0.f;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float4* qc = reinterpret_cast<const float4*>(qs + ((c ^ sw) * GROUP + gl) * 8);
+        const float4 q0 = qc[0], q1 = qc[1];
+        q2[c * 4 + 0] = pack_f32x2(q0.x, q0.y); q2[c * 4 + 1] = pack_f32x2(q0.z, q0.w);
+        q2[c * 4 + 2] = pack_f32x2(q1.x, q1.y); q2[c * 4 + 3] = pack_f32x2(q1.z, q1.w);
+      }
     }
-    named_bar_workers();
-
-    // ---- B: this warp's slice of the pass's units
+    uint64_t acc0 = pack_f32x2(p.acc[0], p.acc[1]), acc1 = pack_f32x2(p.acc[2], p.acc[3]);
+    // ---- the units of this pair in the slice: the values of one are summed beside the scores of the next
+    float s_[2];
+    uint4 kk[2][4];
+    uint2 vv[16];
+    auto load_keys = [&]() {
+      const uint32_t at = kv_stream_advance(a, kvs);
+#pragma unroll
+      for (int uu = 0; uu < 2; ++uu)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) kk[uu][c] = lds128(at + (uint32_t)((uu * KPW + g) * DH * 2 + ((c ^ sw) * GROUP + gl) * 16));
+    };
+    auto load_values = [&]() {
+      const uint32_t at = kv_stream_advance(a, kvs) + (uint32_t)lane * 8;
+#pragma unroll
+      for (int s = 0; s < 16; ++s) vv[s] = lds64(at + (uint32_t)s * 256);
+    };
+    auto scores = [&](int cnt) {                          // of the unit in kk; -inf behind its last token
+#pragma unroll
+      for (int uu = 0; uu < 2; ++uu) {
+        uint64_t d0 = 0, d1 = 0;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          d0 = fma_f32x2(bf16x2_to_f32x2(kk[uu][c].x), q2[c * 4 + 0], d0);
+          d1 = fma_f32x2(bf16x2_to_f32x2(kk[uu][c].y), q2[c * 4 + 1], d1);
+          d0 = fma_f32x2(bf16x2_to_f32x2(kk[uu][c].z), q2[c * 4 + 2], d0);
+          d1 = fma_f32x2(bf16x2_to_f32x2(kk[uu][c].w), q2[c * 4 + 3], d1);
+        }
+        float x0, x1, x2, x3;
+        unpack_f32x2(d0, x0, x1);
+        unpack_f32x2(d1, x2, x3);
+        float dot = (x0 + x1) + (x2 + x3);
+#pragma unroll
+        for (int o = GROUP / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+        s_[uu] = uu * KPW + g < cnt ? dot : -CUDART_INF_F;
+      }
+    };
+    float p0, p1;
+    auto weights = [&]() {                                // of the unit whose scores are in s_
+      float mn = fmaxf(s_[0], s_[1]);
+#pragma unroll
+      for (int o = GROUP; o < 32; o <<= 1) mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+      if (mn > p.m) {                                     // warp-uniform
+        const float w = exp2f(p.m - mn);
+        const uint64_t w2 = pack_f32x2(w, w);
+        p.l *= w;
+        acc0 = mul_f32x2(acc0, w2);
+        acc1 = mul_f32x2(acc1, w2);
+        p.m = mn;
+      }
+      const float mr = p.m == -CUDART_INF_F ? 0.f : p.m;  // no score above -inf so far: weights of 0, not NaN
+      p0 = exp2f(s_[0] - mr);
+      p1 = exp2f(s_[1] - mr);
+      p.l += p0 + p1;
+    };
+    auto add_value = [&](int s) {
+      const float pw = __shfl_sync(0xffffffffu, s < 8 ? p0 : p1, ((s * VK + vk) % KPW) * GROUP);
+      const uint64_t w2 = pack_f32x2(pw, pw);
+      acc0 = fma_f32x2(bf16x2_to_f32x2(vv[s].x), w2, acc0);
+      acc1 = fma_f32x2(bf16x2_to_f32x2(vv[s].y), w2, acc1);
+    };
+    if (!kv_stream_wait(a, sm, kvs, wid)) { aborted = true; break; }
+    load_keys();
+    __syncwarp();
+    kv_stream_done<DH>(a, sm, kvs, wid, lane);
+    scores(pos - ui * UT);
+    for (int k = 1; k < take; ++k) {
+      ++ui;
+      weights();
+      if (!kv_stream_wait(a, sm, kvs, wid)) { aborted = true; break; }
+      load_keys();
+      if (!kv_stream_wait(a, sm, kvs, wid)) { aborted = true; break; }
+      load_values();
+      __syncwarp();
+      kv_stream_done<DH>(a, sm, kvs, wid, lane);
+      kv_stream_done<DH>(a, sm, kvs, wid, lane);
+#pragma unroll
+      for (int s = 0; s < 16; ++s) add_value(s);          // every unit but a pair's last is full
+      scores(pos - ui * UT);
+    }
+    if (aborted) break;
     {
-      const int u0 = (int)((long long)wid * U_pass / 8), u1 = (int)((long long)(wid + 1) * U_pass / 8);
-      int j = 0;
-      while (j + 1 < np_pass && sm->pair_ustart[j + 1] <= u0) ++j;
-      float m = -CUDART_INF_F, l = 0.f, acc[32];
+      const int cnt = min(UT, pos - ui * UT);
+      weights();
+      if (!kv_stream_wait(a, sm, kvs, wid)) { aborted = true; break; }
+      load_values();
+      __syncwarp();
+      kv_stream_done<DH>(a, sm, kvs, wid, lane);
 #pragma unroll
-      for (int e = 0; e < 32; ++e) acc[e] = 0.f;
-      auto flush = [&](int jj) {
-        // merge the KPW key slots of the warp, then lanes of key slot 0 store the partial
-#pragma unroll
-        for (int o = GROUP; o < 32; o <<= 1) {
-          const float om = __shfl_xor_sync(0xffffffffu, m, o);
-          const float ol = __shfl_xor_sync(0xffffffffu, l, o);
-          const float mn = fmaxf(m, om);
-          const float w0 = (m == -CUDART_INF_F) ? 0.f : exp2f(m - mn);
-          const float w1 = (om == -CUDART_INF_F) ? 0.f : exp2f(om - mn);
-          l = l * w0 + ol * w1;
-#pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            const float oa = __shfl_xor_sync(0xffffffffu, acc[e], o);
-            acc[e] = acc[e] * w0 + oa * w1;
-          }
-          m = mn;
-        }
-        float* slot = sm->att_s[jj][wid];
-        if (g == 0) {
-#pragma unroll
-          for (int c = 0; c < 4; ++c)
-#pragma unroll
-            for (int e = 0; e < 8; ++e) slot[(c * GROUP + gl) * 8 + e] = acc[c * 8 + e];
-          if (gl == 0) { slot[DH] = m; slot[DH + 1] = l; }
-        }
-        m = -CUDART_INF_F;
-        l = 0.f;
-#pragma unroll
-        for (int e = 0; e < 32; ++e) acc[e] = 0.f;
-      };
-      int kpage = -1, pg = 0;                            // ordinal of the current page in this slice, its id
-      for (int u = u0; u < u1; ++u) {
-        if (u >= sm->pair_ustart[j + 1]) { flush(j); ++j; }
-        const int p = sm->pair_id[j];
-        const int r = p / H, hd = p - r * H;
-        const int ui = u - sm->pair_ustart[j];           // unit of the pair: page ui / UPP, batch ui % UPP of it
-        const int pi = ui / UPP;
-        const int pos = sm->pair_pos[j];
-        if (u == u0 || ui % UPP == 0) {
-          ++kpage;
-          pg = kpage < 8 ? sm->unit_pg[wid][kpage] : a.st.block_table[(size_t)r * a.st.max_pages + pi];
-          if (pg < 0 || pg >= a.kv.n_pages) { atomicCAS(a.status, 0u, (uint32_t)kStatusBadPage); pg = 0; }
-        }
-        const int tcount = min(kPageTokens, pos - pi * kPageTokens);
-        const bf16* kb = kv_layer + (size_t)pg * a.kv.page_elems + (size_t)hd * kPageTokens * DH;
-        const float* qs = sm->q_s[j];
-        {
-          const int s0 = (ui % UPP) * U;
-          uint4 kk[U][4], vv[U][4];
-#pragma unroll
-          for (int uu = 0; uu < U; ++uu) {
-            const int t = (s0 + uu) * KPW + g;
-            if (t < tcount) {
-              const uint4* kp = reinterpret_cast<const uint4*>(kb + (size_t)t * DH);
-              const uint4* vp = reinterpret_cast<const uint4*>(kb + (size_t)t * DH + v_off);
-#pragma unroll
-              for (int c = 0; c < 4; ++c) { kk[uu][c] = __ldg(kp + c * GROUP + gl); vv[uu][c] = __ldg(vp + c * GROUP + gl); }
-            } else {
-#pragma unroll
-              for (int c = 0; c < 4; ++c) { kk[uu][c] = make_uint4(0, 0, 0, 0); vv[uu][c] = kk[uu][c]; }
-            }
-          }
-          float sc_[U];
-#pragma unroll
-          for (int uu = 0; uu < U; ++uu) {
-            float dot = 0.f;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              float kf[8];
-              unpack8(kk[uu][c], kf);
-              const float4 qa = *reinterpret_cast<const float4*>(qs + (c * GROUP + gl) * 8);
-              const float4 qb = *reinterpret_cast<const float4*>(qs + (c * GROUP + gl) * 8 + 4);
-              dot += qa.x * kf[0] + qa.y * kf[1] + qa.z * kf[2] + qa.w * kf[3] + qb.x * kf[4] + qb.y * kf[5] +
-                     qb.z * kf[6] + qb.w * kf[7];
-            }
-#pragma unroll
-            for (int o = GROUP / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-            sc_[uu] = ((s0 + uu) * KPW + g < tcount) ? dot : -CUDART_INF_F;
-          }
-          float mn = m;
-#pragma unroll
-          for (int uu = 0; uu < U; ++uu) mn = fmaxf(mn, sc_[uu]);
-          if (mn != -CUDART_INF_F) {
-            if (mn != m) {
-              const float sc = exp2f(m - mn);
-              l *= sc;
-#pragma unroll
-              for (int e = 0; e < 32; ++e) acc[e] *= sc;
-              m = mn;
-            }
-#pragma unroll
-            for (int uu = 0; uu < U; ++uu) {
-              if (sc_[uu] != -CUDART_INF_F) {
-                const float pw = exp2f(sc_[uu] - mn);
-                l += pw;
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                  float vf[8];
-                  unpack8(vv[uu][c], vf);
-#pragma unroll
-                  for (int e = 0; e < 8; ++e) acc[c * 8 + e] += pw * vf[e];
-                }
-              }
-            }
-          }
+      for (int s = 0; s < 16; ++s) {
+        if (s * VK < cnt) {                               // warp-uniform; what lies behind the last token is not a number to use
+          if (VK == 2 && s * VK + vk >= cnt) vv[s] = make_uint2(0, 0);
+          add_value(s);
         }
       }
-      if (u1 > u0) flush(j);
+      ++ui;
     }
-    named_bar_workers();
+    left -= take;
+    // ---- the slice's partial of the pair
+#pragma unroll
+    for (int o = GROUP; o < 32; o <<= 1) p.l += __shfl_xor_sync(0xffffffffu, p.l, o);
+    unpack_f32x2(acc0, p.acc[0], p.acc[1]);
+    unpack_f32x2(acc1, p.acc[2], p.acc[3]);
+    if constexpr (VK == 2) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) p.acc[j] += __shfl_xor_sync(0xffffffffu, p.acc[j], 16);
+    }
+    if (whole) {
+      attn_store<DH>(a, p, r, hd, lane);
+    } else {
+      float* slot = sc->slot[wid][own ? 1 : 0];
+      if (vk == 0) *reinterpret_cast<float4*>(slot + dl) = make_float4(p.acc[0], p.acc[1], p.acc[2], p.acc[3]);
+      if (lane == 0) { slot[128] = p.m; slot[129] = p.l; }
+    }
+    if (left > 0) {
+      ui = 0;
+      if (++hd == H) {
+        hd = 0;
+        do ++r; while (sm->prefix[r + 1] == sm->prefix[r]);
+      }
+    }
+  }
+  if (!sm->att_cut) return;
 
-    // ---- C: warp j merges pair j
-    if (wid < np_pass) {
-      const int p = sm->pair_id[wid];
-      const int r = p / H, hd = p - r * H;
-      const int e0 = lane * EPL;
-      float M = -CUDART_INF_F;
-      for (int k = 0; k < kAttnSlots; ++k) M = fmaxf(M, sm->att_s[wid][k][DH]);
-      float L = 0.f, A[EPL];
+  // ---- pairs cut between warps or CTAs
+  named_bar_workers();
+  if (sm->abort) return;
+  auto add_slot = [&](AttnPartial& p, int w, int which) {
+    const float* slot = sc->slot[w][which];
+    attn_merge(p, *reinterpret_cast<const float4*>(slot + dl), slot[128], slot[129]);
+  };
+  AttnPartial zero;
+  zero.m = -CUDART_INF_F;
+  zero.l = 0.f;
 #pragma unroll
-      for (int j = 0; j < EPL; ++j) A[j] = 0.f;
-      for (int k = 0; k < kAttnSlots; ++k) {
-        const float mk = sm->att_s[wid][k][DH];
-        if (mk == -CUDART_INF_F) continue;
-        const float wt = exp2f(mk - M);
-        L += sm->att_s[wid][k][DH + 1] * wt;
-#pragma unroll
-        for (int j = 0; j < EPL; ++j) A[j] += sm->att_s[wid][k][e0 + j] * wt;
+  for (int j = 0; j < 4; ++j) zero.acc[j] = 0.f;
+  // the pair this CTA's range starts inside of: its owner is an earlier CTA
+  if (wid == 0 && sm->att_head >= 0) {
+    AttnPartial p = zero;
+    p.m = -3.0e38f;                                       // finite: an empty start leaves exp2f(m - max) at 0 and not at NaN
+    for (int w = 0; w < 8; ++w)
+      if (sm->sl_head[w] == sm->att_head) add_slot(p, w, 0);
+    float* out = a.att_part + (size_t)blockIdx.x * (DH + 4);
+    if (vk == 0) __stcg(reinterpret_cast<float4*>(out + dl), make_float4(p.acc[0], p.acc[1], p.acc[2], p.acc[3]));
+    if (lane == 0) { __stcg(out + DH, p.m); __stcg(out + DH + 1, p.l); }
+    __syncwarp();
+    if (lane == 0) asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(a.att_flag + blockIdx.x), "l"(ticket) : "memory");
+  }
+  const int pair = sm->sl_tail[wid];
+  if (pair >= 0) {
+    AttnPartial p = zero;
+    p.m = -3.0e38f;
+    add_slot(p, wid, 1);
+    for (int w = wid + 1; w < 8; ++w)
+      if (sm->sl_head[w] == pair) add_slot(p, w, 0);
+    const int pr = pair / H, ph = pair - pr * H;
+    const int end = sm->prefix[pr] * H + (ph + 1) * (sm->prefix[pr + 1] - sm->prefix[pr]);
+    bool ok = true;
+    // (ranges end between pairs in a step without long rows: then no other CTA starts before this pair's end)
+    if (sm->max_units >= kAttnCutUnits) {
+      for (int c = blockIdx.x + 1; c < (int)gridDim.x && ok; ++c) {
+        const int b0 = unit_at(sm, H, range_begin(sm, H, c, gridDim.x, lane), lane);
+        const int b1 = unit_at(sm, H, range_begin(sm, H, c + 1, gridDim.x, lane), lane);
+        if (b0 >= end) break;
+        if (b0 == b1) continue;                           // fewer units than CTAs
+        if (lane == 0) {
+          const long long t0 = clock64();
+          while (ld_acquire_u64(a.att_flag + c) != ticket) {
+            if (sm->abort) { ok = false; break; }
+            if (clock64() - t0 > a.wait_limit) {
+              atomicCAS(a.status, 0u, (uint32_t)kStatusFlagTimeout);
+              sm->abort = 1;
+              ok = false;
+              break;
+            }
+          }
+        }
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        const float* in = a.att_part + (size_t)c * (DH + 4);
+        attn_merge(p, __ldcg(reinterpret_cast<const float4*>(in + dl)), __ldcg(in + DH), __ldcg(in + DH + 1));
       }
-      const float il = 1.f / L;
-#pragma unroll
-      for (int j = 0; j < EPL; ++j) a.o[(size_t)r * d + hd * DH + e0 + j] = __float2bfloat16_rn(A[j] * il);
     }
-    pass0 = single ? p_end : sm->pair_next;       // a single pass covers the whole run
-    named_bar_workers();
+    if (!ok) return;
+    attn_store<DH>(a, p, pr, ph, lane);
   }
 }
 
 // ---- stage: SwiGLU ----------------------------------------------------------------------------------
-// Work unit = (row, 256 features) per warp, 8 consecutive features per lane (two 128-bit loads per partial segment, one
-// 128-bit store); units are dealt round-robin over the CTAs.  The row is the warp's own, so its 1/rms is two more loads
+// Work unit = (row, 256 features) per warp, two groups of 4 consecutive features per lane (a warp-wide load covers 512
+// contiguous bytes of a partial segment); units are dealt round-robin over the CTAs.  The row is the warp's own, so its 1/rms is two more loads
 // beside the partials instead of a pass over all rows with a barrier behind it (200 rows: 19.3 -> 10.2 us).
 __device__ void stage_swiglu(const MegaArgs& a, const MegaSmem* sm, int wtid) {
   const MegaGemmShape& gs = a.shape[2];
   const int lane = wtid & 31, wid = wtid >> 5;
   const int nc = (a.F + 255) >> 8, n_units = a.B * nc;
   for (int u = wid * gridDim.x + blockIdx.x; u < n_units; u += 8 * gridDim.x) {
-    const int r = u / nc, f0 = (u - r * nc) * 256 + lane * 8;
+    const int r = u / nc, c0 = (u - r * nc) * 256 + lane * 4;
     if (!sm->active_s[r]) continue;
-    const bool on = f0 < a.F;
-    const int fl = on ? f0 : 0;                           // lanes beyond the last feature read the first ones, store nothing
-    const int4 tg = tile_seg(sm, gs, fl), tu = tile_seg(sm, gs, a.F + fl);
-    PartialLoads<8, 2> qg, qu;
-    partials_issue<8, 2>(a.partial, gs, a.NT, tg, fl, r, qg);
-    partials_issue<8, 2>(a.partial, gs, a.NT, tu, a.F + fl, r, qu);
-    const float inv = warp_row_inv_rms(a, r, lane);
-    float gt[8], up[8];
-    partials_sum<8, 2>(a.partial, gs, a.NT, tg, fl, r, qg, gt);
-    partials_sum<8, 2>(a.partial, gs, a.NT, tu, a.F + fl, r, qu, up);
-    __align__(16) bf16 ob[8];
+    int f[2];
+    PartialLoads<4, 2> qg[2], qu[2];
+    int4 tg[2], tu[2];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float gv = gt[j] * inv;
-      ob[j] = __float2bfloat16_rn(__fdividef(gv, 1.f + __expf(-gv)) * (up[j] * inv));
+    for (int k = 0; k < 2; ++k) {
+      f[k] = c0 + 128 * k < a.F ? c0 + 128 * k : 0;       // lanes beyond the last feature read the first ones, store nothing
+      tg[k] = tile_seg(sm, gs, f[k]);
+      tu[k] = tile_seg(sm, gs, a.F + f[k]);
+      partials_issue<4, 2>(a.partial, gs, a.NT, tg[k], f[k], r, qg[k]);
+      partials_issue<4, 2>(a.partial, gs, a.NT, tu[k], a.F + f[k], r, qu[k]);
     }
-    if (on) *reinterpret_cast<uint4*>(a.act + (size_t)r * a.F + f0) = *reinterpret_cast<const uint4*>(ob);
+    const float inv = warp_row_inv_rms(a, r, lane);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      float gt[4], up[4];
+      partials_sum<4, 2>(a.partial, gs, a.NT, tg[k], f[k], r, qg[k], gt);
+      partials_sum<4, 2>(a.partial, gs, a.NT, tu[k], a.F + f[k], r, qu[k], up);
+      __align__(8) bf16 ob[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float gv = gt[j] * inv;
+        ob[j] = __float2bfloat16_rn(__fdividef(gv, 1.f + __expf(-gv)) * (up[j] * inv));
+      }
+      if (c0 + 128 * k < a.F) *reinterpret_cast<uint2*>(a.act + (size_t)r * a.F + f[k]) = *reinterpret_cast<const uint2*>(ob);
+    }
   }
 }
 
 // ---- stage: per-tile arg-max of the logits --------------------------------------------------------------
-// Work unit = (256-row vocabulary tile, two batch rows) per warp, 8 consecutive ids per lane: the decision among a
+// Work unit = (256-row vocabulary tile, two batch rows) per warp, 2 x 4 consecutive ids per lane: the decision among a
 // lane's ids needs no exchange, so a (tile, row) costs one warp reduction, and the units of many rows spread over
 // every warp of the chip.  Before, a tile's 128 ids sat on 128 threads that walked through all rows one after the other,
 // a reduction each, on half of the CTAs (16 / 45 sampled / 200 rows: 17.8 / 54.5 / 108 -> 11.3 / 40.0 / 47.7 us).
@@ -1002,39 +1027,51 @@ __device__ void stage_tile_argmax(const MegaArgs& a, const MegaSmem* sm, int wti
   const int n_units = gs.n_tiles * ((a.B + 1) >> 1);
   for (int u = wid * gridDim.x + blockIdx.x; u < n_units; u += 8 * gridDim.x) {
     const int rg = u / gs.n_tiles, tile = u - rg * gs.n_tiles;
-    const int v0 = tile * kTileN + lane * 8;
-    const int4 ts = tile_seg(sm, gs, v0);
-    PartialLoads<8, 2> q[2];
+    const int v0 = tile * kTileN + lane * 4;              // and 128 further: a warp-wide load covers 512 contiguous bytes
+    // everything the two rows need is asked for before the first use
+    float ss[2];
+    int gen[2], row_key[2], skip[2];
 #pragma unroll
-    for (int k = 0; k < 2; ++k) partials_issue<8, 2>(a.partial, gs, a.NT, ts, v0, min(2 * rg + k, a.B - 1), q[k]);
+    for (int k = 0; k < 2; ++k) {
+      const int r = min(2 * rg + k, a.B - 1);
+      ss[k] = row_ss_issue(a, r, lane);
+      gen[k] = a.st.gen[r] + 1;
+      row_key[k] = a.st.row_key[r];
+      skip[k] = a.st.eos_at[r] > 0 ? a.eos_id : -1;
+    }
+    const int4 ts = tile_seg(sm, gs, v0);
+    PartialLoads<4, 2> q[2][2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        partials_issue<4, 2>(a.partial, gs, a.NT, ts, v0 + 128 * h, min(2 * rg + k, a.B - 1), q[k][h]);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const int r = 2 * rg + k;
       if (r >= a.B || !sm->active_s[r]) continue;         // warp-uniform
-      const float inv = warp_row_inv_rms(a, r, lane);
-      int gen = a.st.gen[r] + 1;
-      const int key_r = a.st.row_key[r];
-      const int skip = a.st.eos_at[r] > 0 ? a.eos_id : -1;
-      float lg[8];
-      partials_sum<8, 2>(a.partial, gs, a.NT, ts, v0, r, q[k], lg);
+      const float inv = row_ss_inv_rms(a, ss[k]);
       uint32_t bk = 0;                                    // below every real key
-      int bi = v0;
+      int bi = 0x7fffffff;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        lg[j] *= inv;
-        const int v = v0 + j;
-        if (v < a.V) {
-          if (a.dump_logits) a.dump_logits[(size_t)r * a.V + v] = lg[j];
-          if (v != skip) {
-            const uint32_t key = float_order_key(decision_value(lg[j], a.sample, v, gen, key_r));
-            if (key > bk) { bk = key; bi = v; }           // ids ascend: '>' keeps the lowest
-            asm volatile("" : "+r"(gen) : "r"(bk));       // one draw after the other: eight at once do not fit the registers
+      for (int h = 0; h < 2; ++h) {
+        float lg[4];
+        partials_sum<4, 2>(a.partial, gs, a.NT, ts, v0 + 128 * h, r, q[k][h], lg);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          lg[j] *= inv;
+          const int v = v0 + 128 * h + j;
+          if (v < a.V) {
+            if (a.dump_logits) a.dump_logits[(size_t)r * a.V + v] = lg[j];
+            if (v != skip[k]) {
+              const uint32_t key = float_order_key(decision_value(lg[j], a.sample, v, gen[k], row_key[k]));
+              if (key > bk) { bk = key; bi = v; }         // ids ascend: '>' keeps the lowest
+            }
           }
         }
       }
       const uint32_t best = __reduce_max_sync(0xffffffffu, bk);
-      const uint32_t who = __ballot_sync(0xffffffffu, bk == best);
-      bi = __shfl_sync(0xffffffffu, bi, __ffs(who) - 1);  // the lowest lane holds the lowest ids
+      bi = (int)__reduce_min_sync(0xffffffffu, bk == best ? (unsigned int)bi : 0x7fffffffu);
       if (lane == 0) {
         a.tile_val[(size_t)r * a.n_tiles_lm + tile] = __uint_as_float(best);
         a.tile_idx[(size_t)r * a.n_tiles_lm + tile] = bi;
@@ -1083,9 +1120,7 @@ __device__ void stage_final(const MegaArgs& a, int wtid) {
 }
 
 // ------------------------------------------------------------------------------------ the kernel
-// WIDE: the variant for batches of more than 64 rows, which adds attention_warp_pairs.  It is an instantiation of
-// its own because the batches up to 64 rows live on this kernel's register allocation: the same code with the
-// extra path compiled in ran the 16-row step 2.5 % slower.
+// WIDE: the variant for batches of more than 64 rows (128 token lanes per instruction, one or two token tiles).
 // TRACE: with the stage-boundary time stamps of CTA 0 (ss_set_trace); the timed paths run the variant without them.
 template <int DH, bool WIDE, bool TRACE>
 __global__ void __launch_bounds__(kMegaThreads, 1)
@@ -1095,7 +1130,8 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
   MegaSmem* sm = reinterpret_cast<MegaSmem*>(smem_raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cta = blockIdx.x;
-  const uint32_t stage0 = (smem_u32(smem_raw) + (uint32_t)sizeof(MegaSmem) + 1023u) & ~1023u;
+  float* scratch = reinterpret_cast<float*>(smem_raw + sizeof(MegaSmem));
+  const uint32_t stage0 = (smem_u32(smem_raw) + (uint32_t)(sizeof(MegaSmem) + mega_scratch_bytes(WIDE)) + 1023u) & ~1023u;
   // ring: S activation blocks first, then S weight blocks.  A token tile shorter than 128 rows is read
   // by the tensor core as 128 rows anyway; the surplus rows fall on the blocks that follow.
   // the batches up to 64 rows always have one token tile, computed with the 64-lane instruction
@@ -1105,6 +1141,7 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
   const uint32_t stage_tx = (uint32_t)kBlockBytes + x_bytes;
   const int S = a.stages;
   const uint32_t x0 = stage0, w0 = stage0 + (uint32_t)S * x_bytes;
+  const uint32_t kv0 = w0 + (uint32_t)S * kBlockBytes;     // the worker warps' pieces of the cache scan
   const int acc_bufs = m_tiles == 1 ? 2 : 1;         // 512 columns: two buffers of 256, or one of 2 x 256
   constexpr uint32_t kTmemCols = 512;
   const int n_gemm = 4 * a.n_layers + 1;
@@ -1118,6 +1155,7 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
       mbar_init(smem_u32(&sm->acc_full[b]), 1);
       mbar_init(smem_u32(&sm->acc_empty[b]), 8);
     }
+    for (int b = 0; b < 8 * kKvMaxPieces; ++b) mbar_init(smem_u32(&sm->kv_full[0][0] + b), 1);
     sm->w_issued = 0;
     sm->act_epoch = 0;
     sm->abort = 0;
@@ -1283,7 +1321,9 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
     int tr = 0;
     if (tracer) a.trace[tr++] = global_timer_ns();
     if (cta == 0 && wtid == 0) a.st.scalars[1] = 0;   // rows still active after this step (counted in the last stage)
-    attention_setup<DH, WIDE>(a, sm, wtid);
+    attention_setup<DH>(a, sm, wtid);
+    KvStream kvs;
+    kv_stream_start<DH>(a, sm, kvs, kv0, wid, lane);
     stage_residual(a, sm, wtid, 0, nullptr, a.norm_ptr[0], a.n_layers == 0);
     ok = grid_barrier(a, sm, epoch, wtid, true);
     if (ok && wtid == 0) { __threadfence_block(); sm->act_epoch = 1; }
@@ -1332,23 +1372,26 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
             } else {
               // many rows: a lane holds one token's outputs, so direct 128-bit stores put every lane's 16 bytes
               // into a sector of its own, 1 KiB apart, and the drain is bound by the sectors it writes.  The
-              // warp turns 32 outputs at a time through shared memory (rows padded to 36 floats: both
-              // directions free of bank conflicts) and stores whole 128-byte lines, four tokens per instruction.
-              float* tr = &sm->att_s[0][0][0] + wid * (32 * 36);
-              const int t_hi = lane >> 3, cg = lane & 7;
+              // warp turns 16 outputs at a time through shared memory and stores 64-byte runs, eight tokens per
+              // instruction.
+              float* tr = scratch + wid * (per_q * kDrainPad);
+              const int t_hi = lane >> 2, cg = lane & 3;
 #pragma unroll
-              for (int sub = 0; sub < 2; ++sub) {
+              for (int sub = 0; sub < 4; ++sub) {
+                if (lane < per_q) {
 #pragma unroll
-                for (int j = 0; j < 32; j += 4)
-                  *reinterpret_cast<uint4*>(tr + lane * 36 + j) =
-                      make_uint4(v[sub * 32 + j], v[sub * 32 + j + 1], v[sub * 32 + j + 2], v[sub * 32 + j + 3]);
+                  for (int j = 0; j < 16; j += 4)
+                    *reinterpret_cast<uint4*>(tr + lane * kDrainPad + j) =
+                        make_uint4(v[sub * 16 + j], v[sub * 16 + j + 1], v[sub * 16 + j + 2], v[sub * 16 + j + 3]);
+                }
                 __syncwarp();
-                for (int i = 0; i < per_q / 4; ++i) {
-                  const int tl = 4 * i + t_hi;
+#pragma unroll
+                for (int i = 0; i < per_q / 8; ++i) {
+                  const int tl = 8 * i + t_hi;
                   const int tg = mt * 128 + quarter * per_q + tl;
                   if (tg < a.B)
-                    *reinterpret_cast<uint4*>(a.partial + (slot * a.NT + tg) * kTileN + colhalf * 128 + c + sub * 32 + 4 * cg) =
-                        *reinterpret_cast<const uint4*>(tr + tl * 36 + 4 * cg);
+                    *reinterpret_cast<uint4*>(a.partial + (slot * a.NT + tg) * kTileN + colhalf * 128 + c + sub * 16 + 4 * cg) =
+                        *reinterpret_cast<const uint4*>(tr + tl * kDrainPad + 4 * cg);
                 }
                 __syncwarp();
               }
@@ -1369,12 +1412,7 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
       if (tracer) a.trace[tr++] = global_timer_ns();       // every CTA's partials visible
       // ---- the stage that consumes the projection
       if (type == 0) {
-        if constexpr (WIDE) {
-          if (sm->att_warp_pairs) attention_warp_pairs<DH>(a, sm, wtid, layer);
-          else stage_attention<DH>(a, sm, wtid, layer);
-        } else {
-          stage_attention<DH>(a, sm, wtid, layer);
-        }
+        stage_attention<DH>(a, sm, reinterpret_cast<AttnScratch*>(scratch), kvs, wtid, layer, a.grid_base + epoch);
       } else if (type == 1) {
         stage_residual(a, sm, wtid, 1, &a.shape[1], a.norm_ptr[2 * layer + 1], false);
       } else if (type == 2) {
@@ -1391,6 +1429,7 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
       if (type == 4) stage_final(a, wtid);
       else if (wtid == 0) { __threadfence_block(); sm->act_epoch = gm + 2; }
     }
+    kv_stream_end(a, sm, kvs, wid, lane);
   }
 
   tc_fence_before();

@@ -80,6 +80,15 @@ repack_weights_kernel(const uint4* __restrict__ src, long long rows, int K, uint
   *reinterpret_cast<uint4*>(blk + r * 128 + ((c ^ (r & 7)) << 4)) = src[id];
 }
 
+// ------------------------------------------------------------------------------------ rotations
+// rope[pos][i] = (cos, sin) of pos * inv_freq[i]: grid (positions), block Dh / 2.  Filled once per context; the kernels
+// that rotate read it instead of evaluating a sine and a cosine per (token, head, pair).
+__global__ void rope_table_kernel(const float* __restrict__ inv_freq, float2* __restrict__ rope) {
+  float sn, cs;
+  sincosf((float)blockIdx.x * inv_freq[threadIdx.x], &sn, &cs);
+  rope[(size_t)blockIdx.x * blockDim.x + threadIdx.x] = make_float2(cs, sn);
+}
+
 // ------------------------------------------------------------------------------------ embedding + first norm
 // h[row] = E[token]; x[row] = RMSNorm(h[row]) * g   (rows: decode B rows or T prompt tokens)
 __global__ void __launch_bounds__(256)

@@ -147,6 +147,7 @@ struct ss_ctx {
   int n_loaded = 0, n_expected = 0;
   // misc device
   float* inv_freq = nullptr;
+  float2* rope = nullptr;          // [max_ctx][Dh / 2] (cos, sin)
   uint32_t* status = nullptr;
   RowState st{};
   KvLayout kv{};
@@ -166,6 +167,8 @@ struct ss_ctx {
   TileSeg* tbl_lm_prompt = nullptr;                                  // LM head after the prompt pass (128-row tiles)
   float* rowss = nullptr;          // [kMaxBatch][kMaxSlices]
   unsigned long long* grid_ctr = nullptr;
+  float* att_part = nullptr;       // decode attention: partial results that cross CTAs, and their flags
+  unsigned long long* att_flag = nullptr;
   unsigned long long* trace = nullptr;  // stage-boundary time stamps of the last decode step
   int trace_len = 0;
   unsigned long long grid_epochs = 0;   // grid barriers passed by all launches so far
@@ -355,7 +358,7 @@ struct ArenaPlan {
 struct Offsets {
   size_t embed, lm_head, final_norm, staging, staging_bytes, weights_end;
   std::vector<size_t> attn_norm, wqkv, wo, ffn_norm, wgu, wdown;
-  size_t inv_freq, status, rows, block_table, out_tokens, tok, h, x, qkv, qkv_f, attn_o, gu, act;
+  size_t inv_freq, rope, att_part, att_flag, status, rows, block_table, out_tokens, tok, h, x, qkv, qkv_f, attn_o, gu, act;
   size_t h_dec, x_dec, o_dec, act_dec, partial, kv;
   size_t tbl[5], tbl_lm_prompt, tile_val, tile_idx, rowss, grid_ctr, wptr, norm_ptr, trace;
   size_t partial_bytes;
@@ -395,6 +398,9 @@ void layout(const ss_model_cfg& m, const ss_runtime_cfg& rt, int n_sm, Offsets& 
   o.staging_bytes = std::max(std::max(V * d, F * d), d * d) * 2;
   o.staging = a.take(o.staging_bytes);
   o.inv_freq = a.take(m.head_dim / 2 * sizeof(float));
+  o.rope = a.take((size_t)rt.max_ctx * (m.head_dim / 2) * sizeof(float2));
+  o.att_part = a.take((size_t)n_sm * (m.head_dim + 4) * sizeof(float));
+  o.att_flag = a.take((size_t)n_sm * 8);
   o.status = a.take(64);
   o.rows = a.take(kRowStateBytes + 64);
   o.max_pages = ceil_div(rt.max_ctx, kPageTokens);
@@ -489,14 +495,20 @@ int weight_slot(const ss_ctx* c, const std::string& name, WeightSlot* out) {
   return SS_ERR_ARG;
 }
 
+// Grid-barrier counter and attention flags (which hold barrier numbers) back to zero.
+void reset_grid(ss_ctx* c) {
+  cudaMemsetAsync(c->grid_ctr, 0, 8, c->stream);
+  cudaMemsetAsync(c->att_flag, 0, (size_t)c->n_sm * 8, c->stream);
+  cudaStreamSynchronize(c->stream);
+  c->grid_epochs = 0;
+}
+
 // A non-zero status word: the step that set it was abandoned half way.  The error is reported once; the word
 // and the grid-barrier counter (left in an unknown state by the abort) are cleared so that the context can
 // start a new batch.
 int report_device_status(ss_ctx* c, uint32_t word) {
-  cudaMemsetAsync(c->grid_ctr, 0, 8, c->stream);
   cudaMemsetAsync(c->status, 0, 4, c->stream);
-  cudaStreamSynchronize(c->stream);
-  c->grid_epochs = 0;
+  reset_grid(c);
   return word == (uint32_t)kStatusBadPage ? SS_ERR_STATE : SS_ERR_DEVICE_TIMEOUT;
 }
 
@@ -532,7 +544,7 @@ int enqueue_decode_step(ss_ctx* c, const ss_step_opts* opts, int32_t* next_token
   a.wptr = c->wptr_dev;
   a.norm_ptr = c->norm_dev;
   a.embed = c->embed;
-  a.inv_freq = c->inv_freq;
+  a.rope = c->rope;
   const int shp[5][2] = {{3 * d, d}, {d, d}, {2 * F, d}, {d, F}, {V, d}};
   size_t need_partial = 0;
   int tab_entries = 0;
@@ -549,10 +561,16 @@ int enqueue_decode_step(ss_ctx* c, const ss_step_opts* opts, int32_t* next_token
   a.B = B; a.NT = NT;
   a.m_tiles = NT > 128 ? 2 : 1;
   a.x_rows = NT > 128 ? 128 : NT;
+  const bool wide = NT > 64;
   const int stage_bytes = kBlockBytes + a.m_tiles * a.x_rows * kTileK * 2;
-  const int header = (int)sizeof(MegaSmem) + 1024;
-  a.stages = std::max(2, std::min(kMegaMaxStages, (227 * 1024 - header) / stage_bytes));
-  const size_t smem = (size_t)header + (size_t)a.stages * stage_bytes;
+  // shared memory left behind the header is shared out between the weight ring and the pieces of the cache scan
+  const int header = (int)sizeof(MegaSmem) + mega_scratch_bytes(wide) + 1024, piece_set = 8 * kKvPieceBytes;
+  const int room = 227 * 1024 - header;
+  a.stages = std::max(2, std::min(kMegaMaxStages, (room - 2 * piece_set) / stage_bytes));
+  a.kv_pieces = std::min(kKvMaxPieces, (room - a.stages * stage_bytes) / piece_set);
+  const size_t smem = (size_t)header + (size_t)a.stages * stage_bytes + (size_t)a.kv_pieces * piece_set;
+  a.att_part = c->att_part;
+  a.att_flag = c->att_flag;
   a.st = c->st; a.kv = c->kv;
   a.h = c->h_dec; a.x = c->x_dec; a.o = c->o_dec; a.act = c->act_dec;
   a.rowss = c->rowss; a.partial = c->partial;
@@ -569,7 +587,6 @@ int enqueue_decode_step(ss_ctx* c, const ss_step_opts* opts, int32_t* next_token
   a.trace = c->trace_on ? c->trace : nullptr;
   a.wait_limit = c->wait_limit;
   void* args[4] = {(void*)mx, (void*)mo, (void*)ma, (void*)&a};
-  const bool wide = NT > 64;
   const void* fn = mega_kernel_fn(m.head_dim, wide, a.trace != nullptr);
   SS_CUDA(c, cudaLaunchCooperativeKernel(fn, dim3(c->n_sm), dim3(kMegaThreads), args, smem, c->stream));
   c->grid_epochs += 1 + 2 * (unsigned long long)(4 * m.n_layers + 1);
@@ -735,6 +752,9 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
   c->n_expected = 3 + 9 * model->n_layers;
   c->loaded.assign(c->n_expected, 0);
   c->inv_freq = (float*)(A + o.inv_freq);
+  c->rope = (float2*)(A + o.rope);
+  c->att_part = (float*)(A + o.att_part);
+  c->att_flag = (unsigned long long*)(A + o.att_flag);
   c->status = (uint32_t*)(A + o.status);
   int32_t* rows = (int32_t*)(A + o.rows);
   c->st.ctx_len = rows + 0 * kMaxBatch;
@@ -824,6 +844,11 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
   for (int i = 0; i < model->head_dim / 2; ++i)
     inv[i] = (float)std::pow((double)model->rope_theta, -2.0 * i / model->head_dim);
   cudaError_t e = cudaMemcpyAsync(c->inv_freq, inv.data(), inv.size() * 4, cudaMemcpyHostToDevice, c->stream);
+  if (e == cudaSuccess) {
+    rope_table_kernel<<<(unsigned)rt->max_ctx, model->head_dim / 2, 0, c->stream>>>(c->inv_freq, c->rope);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->att_flag, 0, (size_t)n_sm * 8, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->status, 0, 64, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(rows, 0, kRowStateBytes + 64, c->stream);
   // activation operands must be finite wherever a TMA box may reach beyond the valid rows
@@ -1241,9 +1266,7 @@ int ss_selftest_wait_timeout(ss_ctx* c, int32_t limit_us) {
   SS_CUDA(c, cudaStreamSynchronize(c->stream));
   if (c->pinned[1] != 0) return report_device_status(c, (uint32_t)c->pinned[1]);
   // the wait came through although an arrival was missing: the counter no longer matches the epochs
-  cudaMemsetAsync(c->grid_ctr, 0, 8, c->stream);
-  cudaStreamSynchronize(c->stream);
-  c->grid_epochs = 0;
+  reset_grid(c);
   return SS_OK;
 }
 

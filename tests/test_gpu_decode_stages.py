@@ -1,0 +1,72 @@
+"""The decode step's stages at the edges of their work splits, against the oracle (teacher-forced) and, for a context too
+long for it, against the prompt pass over the same tokens.  Tolerances as everywhere (parity_util)."""
+import numpy as np
+import pytest
+
+from paper_2305_13144_b200 import synth
+from parity_util import HIDDEN_TOL, LOGIT_TOL, engine, teacher_forced
+
+pytestmark = pytest.mark.gpu
+
+
+def _shape(heads, head_dim, ffn=256, vocab=300, layers=2):
+    return synth.ModelShape(n_layers=layers, d_model=heads * head_dim, n_heads=heads, head_dim=head_dim, d_ffn=ffn, vocab=vocab)
+
+
+@pytest.mark.parametrize("heads,head_dim,lens", [
+    # one unit of the cache scan is 16 tokens at head size 128, 32 at 64: contexts around its multiples, rows without cut pairs
+    (3, 128, [1, 15, 16, 17, 31, 32, 33, 47, 48, 49]),
+    (5, 64, [1, 31, 32, 33, 63, 64, 65, 95, 97]),
+    # a row of 40 units or more: its pairs are cut between CTAs; fewer units than CTAs, so some CTAs have none
+    (1, 128, [700, 3, 17]),
+    (2, 64, [1500, 40]),
+    # cut pairs with every CTA at work, a long row beside short ones
+    (8, 128, [900, 12, 333, 641]),
+    # wide batches: two pieces per warp, rows of very different lengths (a pair costs more than its units)
+    (4, 64, [1 + (7 * i) % 90 for i in range(70)]),
+    (2, 128, [2 + (13 * i) % 120 for i in range(131)]),
+])
+def test_cache_scan_splits(heads, head_dim, lens):
+    shape = _shape(heads, head_dim)
+    w = synth.make_weights(shape, seed=21)
+    rng = np.random.default_rng(3)
+    prompts = [rng.integers(3, shape.vocab, size=n).tolist() for n in lens]
+    targets = [2 + i % 4 for i in range(len(lens))]        # rows leave the batch while it runs: the split changes from step to step
+    follow = list(range(len(lens))) if len(lens) <= 16 else [0, 1, 2, 3, 5, 8, 31, 64, len(lens) - 1]
+    el, eh, _ = teacher_forced(shape, w, prompts, targets, cap=5, follow=follow, max_batch=max(16, len(lens)), max_ctx=max(lens) + 6,
+                               max_prefill=max(512, max(lens)), kv_tokens=sum(lens) + 64 * len(lens))
+    assert el <= LOGIT_TOL and eh <= HIDDEN_TOL, (el, eh)
+
+
+@pytest.mark.parametrize("ffn,vocab,rows", [(264, 257, 1), (8, 511, 3), (520, 1000, 17), (1000, 33, 65)])
+def test_swiglu_and_argmax_units(ffn, vocab, rows):
+    """Feature and vocabulary counts that end inside a 256-wide unit, odd row counts (the arg-max takes rows in pairs)."""
+    shape = _shape(2, 64, ffn=ffn, vocab=vocab)
+    w = synth.make_weights(shape, seed=22)
+    rng = np.random.default_rng(4)
+    prompts = [rng.integers(3, vocab, size=int(n)).tolist() for n in rng.integers(2, 20, size=rows)]
+    el, eh, _ = teacher_forced(shape, w, prompts, [4] * rows, cap=4, follow=sorted({0, rows // 2, rows - 1}), max_batch=max(16, rows),
+                               max_prefill=2048, kv_tokens=8192)
+    assert el <= LOGIT_TOL and eh <= HIDDEN_TOL, (el, eh)
+
+
+def test_context_beyond_the_page_table_in_shared_memory():
+    """8300 cached tokens are 519 units, more than the page table in shared memory holds (512): the decode step over token
+    8301 gives the logits that the prompt pass over 8301 tokens gives."""
+    import torch
+    from paper_2305_13144_b200 import api
+    shape = _shape(1, 128)
+    w = synth.make_weights(shape, seed=23)
+    ids = np.random.default_rng(5).integers(3, shape.vocab, size=8301).astype(np.int32)
+    eng = engine(shape, w, max_batch=2, max_ctx=8400, max_prefill=8301, max_new=4, kv_tokens=2 * 8400)
+    out = [torch.zeros(1, shape.vocab, dtype=torch.float32, device="cuda") for _ in range(2)]
+    api.ss_prefill(eng, ids, np.array([0, 8301], dtype=np.int32), None, 2, dump_logits=out[0])
+    api.ss_read_batch(eng, 1, 2)
+    api.ss_release_batch(eng)
+    api.ss_prefill(eng, ids[:8300], np.array([0, 8300], dtype=np.int32), None, 3,
+                   forced_tokens=torch.tensor(ids[8300:], dtype=torch.int32, device="cuda"))
+    api.ss_decode_step(eng, dump_logits=out[1])
+    _, lens, _ = api.ss_read_batch(eng, 1, 3)
+    api.ss_release_batch(eng)
+    a, b = (t.cpu().numpy()[0] for t in out)
+    assert lens[0] == 2 and np.max(np.abs(a - b)) <= LOGIT_TOL * np.max(np.abs(a))
