@@ -441,63 +441,14 @@ gemm_wx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       if (!ok) break;
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * p.NT);
-      const int n = tile * kTileM + row;            // output feature
-      if (a.mode == kGemmPartial) {
-        const size_t slot = (size_t)cta * p.max_seg + seg;
-        float* dst = a.partial + slot * p.NT * 128 + row;
-        for (int c = 0; c < p.NT; c += 8) {
-          float v[8];
-          tmem_ld8(taddr + c, v);
+      const size_t slot = (size_t)cta * p.max_seg + seg;
+      float* dst = a.partial + slot * p.NT * 128 + row;
+      for (int c = 0; c < p.NT; c += 8) {
+        float v[8];
+        tmem_ld8(taddr + c, v);
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            if (c + j < n_valid) dst[(size_t)(c + j) * 128] = v[j];
-        }
-      } else if (a.mode == kGemmDirectBf16) {
-        __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(a.out_bf16);
-        for (int c = 0; c < p.NT; c += 8) {
-          float v[8];
-          tmem_ld8(taddr + c, v);
-          if (n < p.n_out) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-              if (c + j < n_valid) out[(size_t)(tok0 + c + j) * a.ld_out + n] = __float2bfloat16_rn(v[j]);
-          }
-        }
-      } else if (a.mode == kGemmDirectF32) {
-        // plain fp32 store: the consumer (RoPE, SwiGLU) rounds once, after its own arithmetic
-        for (int c = 0; c < p.NT; c += 8) {
-          float v[8];
-          tmem_ld8(taddr + c, v);
-          if (n < p.n_out) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-              if (c + j < n_valid) a.out_f32[(size_t)(tok0 + c + j) * a.ld_out + n] = v[j];
-          }
-        }
-      } else if (p.NT % 32 == 0) {
-        // read-modify-write of the fp32 residual: 32 tokens' loads in flight per round trip
-        for (int c = 0; c < p.NT; c += 32) {
-          float v[32], h[32];
-          tmem_ld32(taddr + c, v);
-          if (n < p.n_out) {
-            float* o = a.out_f32 + (size_t)(tok0 + c) * a.ld_out + n;
-#pragma unroll
-            for (int j = 0; j < 32; ++j) h[j] = (c + j < n_valid) ? __ldcg(o + (size_t)j * a.ld_out) : 0.f;
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (c + j < n_valid) o[(size_t)j * a.ld_out] = h[j] + v[j];
-          }
-        }
-      } else {
-        for (int c = 0; c < p.NT; c += 8) {
-          float v[8];
-          tmem_ld8(taddr + c, v);
-          if (n < p.n_out) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-              if (c + j < n_valid) a.out_f32[(size_t)(tok0 + c + j) * a.ld_out + n] += v[j];
-          }
-        }
+        for (int j = 0; j < 8; ++j)
+          if (c + j < n_valid) dst[(size_t)(c + j) * 128] = v[j];
       }
       tc_fence_before();
       __syncwarp();
@@ -529,6 +480,76 @@ constexpr int kPairTokens = 256;                                 // token tile o
 // Remote arrival on the first CTA's copy of a barrier (used by the partner's epilogue warps).
 __device__ __forceinline__ void mbar_arrive_leader(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar & kPairLeaderMask) : "memory");
+}
+
+// ---- epilogues that finish a projection.  Weight rows that belong together (the two dimensions of a rotation, gate and
+// up of a feature, neighbouring value dimensions) are neighbours in the tiled layout, i.e. on neighbouring lanes of the
+// accumulator.  Of 32 tokens the even lane of two takes the first 16 and the odd lane the others: each hands the other
+// lane the values it needs, 16 shuffles for 32 values, and then holds both rows of its 16 tokens.
+// Writing the fp32 accumulators out for a kernel of its own to rotate (or gate) cost, per layer of 16281 tokens at the
+// 7B shape, 222 (258) us of that kernel beside the write: at the copy bandwidth, so it had to go, not to be tuned.
+__device__ __forceinline__ void pair_rows(const float (&v)[32], int lane, float (&lo)[16], float (&hi)[16]) {
+  const bool odd = lane & 1;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const float got = __shfl_xor_sync(0xffffffffu, odd ? v[j] : v[16 + j], 1);
+    lo[j] = odd ? got : v[j];
+    hi[j] = odd ? v[16 + j] : got;
+  }
+}
+__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+// q, k, v: rotation (q, k), one rounding; operand of the prompt-pass attention, and keys and values into the pages.
+__device__ __forceinline__ void epilogue_qkv(const GemmArgs& a, uint32_t taddr, int n, int tok0, int n_valid, int lane) {
+  const int sec = n / a.d, in = n - sec * a.d, hd = in / a.Dh, e = (in - hd * a.Dh) & ~1;      // sec, hd: warp-uniform
+  const int first = (lane & 1) * 16;
+  __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(a.out) + (size_t)sec * a.d + hd * a.Dh + e;
+  __nv_bfloat16* kv = reinterpret_cast<__nv_bfloat16*>(a.kv_layer) + (size_t)((max(sec, 1) - 1) * a.H + hd) * kPageTokens * a.Dh + e;
+  for (int c = 0; c < n_valid; c += 32) {
+    const int mine = tok0 + min(c + lane, n_valid - 1);
+    const int pos_l = __ldg(a.tok_pos + mine), slot_l = __ldg(a.tok_slot + mine);
+    float v[32], lo[16], hi[16];
+    tmem_ld32(taddr + c, v);
+    pair_rows(v, lane, lo, hi);
+    if (sec < 2) {
+      const float2* rope = a.rope + (e >> 1);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const int pos = __shfl_sync(0xffffffffu, pos_l, first + j);
+        const float2 cs = __ldg(rope + (size_t)pos * (a.Dh >> 1));
+        const float x0 = lo[j], x1 = hi[j];
+        lo[j] = x0 * cs.x - x1 * cs.y;
+        hi[j] = x1 * cs.x + x0 * cs.y;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const int slot = __shfl_sync(0xffffffffu, slot_l, first + j);
+      if (c + first + j < n_valid) {
+        const uint32_t w = pack_bf16x2(lo[j], hi[j]);
+        *reinterpret_cast<uint32_t*>(out + (size_t)(tok0 + c + first + j) * 3 * a.d) = w;
+        if (sec > 0) *reinterpret_cast<uint32_t*>(kv + (size_t)(slot / kPageTokens) * a.page_elems + (slot % kPageTokens) * a.Dh) = w;
+      }
+    }
+  }
+}
+
+// silu(gate) * up, one rounding.
+__device__ __forceinline__ void epilogue_swiglu(const GemmArgs& a, uint32_t taddr, int n, int tok0, int n_valid, int lane) {
+  const int F = a.p.n_out >> 1, f = n >> 1, first = (lane & 1) * 16;
+  __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(a.out) + (size_t)tok0 * F + f;
+  for (int c = 0; c < n_valid; c += 32) {
+    float v[32], gate[16], up[16];
+    tmem_ld32(taddr + c, v);
+    pair_rows(v, lane, gate, up);
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (f < F && c + first + j < n_valid)
+        out[(size_t)(c + first + j) * F] = __float2bfloat16_rn(gate[j] / (1.f + __expf(-gate[j])) * up[j]);
+  }
 }
 
 // Persistent: gridDim.x / 2 pairs walk the (pair of weight tiles, token tile) units pair, pair + P, pair + 2 P, ...
@@ -652,39 +673,22 @@ gemm_wx_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * kPairTokens);
       const int n = (2 * wt + (int)rank) * kTileM + row;
-      if (a.mode == kGemmDirectF32) {
-        for (int c = 0; c < kPairTokens; c += 32) {
-          float v[32];
-          tmem_ld32(taddr + c, v);
-          if (n < p.n_out) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (c + j < n_valid) a.out_f32[(size_t)(tok0 + c + j) * a.ld_out + n] = v[j];
-          }
-        }
-      } else if (a.mode == kGemmDirectBf16) {
-        __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(a.out_bf16);
-        for (int c = 0; c < kPairTokens; c += 32) {
-          float v[32];
-          tmem_ld32(taddr + c, v);
-          if (n < p.n_out) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (c + j < n_valid) out[(size_t)(tok0 + c + j) * a.ld_out + n] = __float2bfloat16_rn(v[j]);
-          }
-        }
+      if (a.mode == kGemmQkv) {
+        if (n < p.n_out) epilogue_qkv(a, taddr, n, tok0, n_valid, lane);        // warp-uniform: d is a multiple of 64
+      } else if (a.mode == kGemmSwiglu) {
+        epilogue_swiglu(a, taddr, n, tok0, n_valid, lane);
       } else {
         // read-modify-write of the fp32 residual: 32 tokens' loads in flight per round trip
-        for (int c = 0; c < kPairTokens; c += 32) {
+        for (int c = 0; c < n_valid; c += 32) {
           float v[32], h[32];
           tmem_ld32(taddr + c, v);
           if (n < p.n_out) {
-            float* o = a.out_f32 + (size_t)(tok0 + c) * a.ld_out + n;
+            float* o = a.residual + (size_t)(tok0 + c) * p.n_out + n;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) h[j] = (c + j < n_valid) ? __ldcg(o + (size_t)j * a.ld_out) : 0.f;
+            for (int j = 0; j < 32; ++j) h[j] = (c + j < n_valid) ? __ldcg(o + (size_t)j * p.n_out) : 0.f;
 #pragma unroll
             for (int j = 0; j < 32; ++j)
-              if (c + j < n_valid) o[(size_t)j * a.ld_out] = h[j] + v[j];
+              if (c + j < n_valid) o[(size_t)j * p.n_out] = h[j] + v[j];
           }
         }
       }

@@ -3,6 +3,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <vector_types.h>
 #include <vector>
 
 #include "seqsched.h"
@@ -35,11 +36,12 @@ enum : uint32_t {
 };
 
 // ---- GEMM:  D[n_out, tok] = W[n_out, K] . X[tok, K]^T  -------------------------------------
-// The tile-iteration space (n_tiles x kb) is cut into `gridx` equal contiguous ranges, one per
-// CTA (split along K where a range ends inside a tile).  In kGemmPartial mode every (CTA,
-// tile) segment is written as an fp32 partial; the consumer kernel adds the segments of a tile
-// in CTA order, so the result does not depend on timing.
-enum GemmMode : int { kGemmPartial = 0, kGemmDirectBf16 = 1, kGemmDirectF32Add = 2, kGemmDirectF32 = 3 };
+// kGemmPartial (gemm_wx_kernel): the tile-iteration space (n_tiles x kb) is cut into `gridx` equal contiguous ranges,
+// one per CTA (split along K where a range ends inside a tile); every (CTA, tile) segment is written as an fp32 partial
+// and the consumer kernel adds the segments of a tile in CTA order, so the result does not depend on timing.
+// The others (gemm_wx_pair_kernel) finish a tile in its epilogue: added to the fp32 residual; rotated and written as
+// bf16 q, k, v operand and cache entries; or gated (SwiGLU) and written as bf16 operand.
+enum GemmMode : int { kGemmPartial = 0, kGemmResidual = 1, kGemmQkv = 2, kGemmSwiglu = 3 };
 
 struct GemmPlan {
   int n_out, K, n_tiles, kb;
@@ -57,9 +59,15 @@ struct GemmArgs {
   int mode;
   int n_tok;           // valid tokens
   float* partial;      // [gridx*max_seg][NT][128]
-  void* out_bf16;      // [tok][ld_out]
-  float* out_f32;
-  int ld_out;
+  float* residual;     // kGemmResidual: [tok][n_out]
+  void* out;           // kGemmQkv: bf16 [tok][3 d]; kGemmSwiglu: bf16 [tok][n_out / 2]
+  // kGemmQkv
+  int d, H, Dh;
+  const float2* rope;          // [position][Dh / 2] (cos, sin)
+  const int32_t* tok_pos;      // [tok] position in its row
+  const int32_t* tok_slot;     // [tok] page * kPageTokens + place in the page
+  void* kv_layer;              // the layer's pages
+  size_t page_elems;
   uint32_t* status;
 };
 

@@ -1,9 +1,10 @@
 // Kernels of the prompt pass, the weight repacking and the batch's first arg-max (sm_100a).
 //
 // Prompt pass (all prompt tokens of a chunk at once):
-//   embed_rmsnorm -> [ qkv GEMM -> rope_append_prefill -> attn_prefill -> o GEMM (+= residual) ->
-//   rmsnorm -> gate/up GEMM -> swiglu -> down GEMM (+= residual) -> rmsnorm ] x layers ->
+//   embed_rmsnorm -> [ qkv GEMM (rotates, fills the cache) -> attn_prefill -> o GEMM (+= residual) ->
+//   rmsnorm -> gate/up GEMM (SwiGLU) -> down GEMM (+= residual) -> rmsnorm ] x layers ->
 //   gather_last_rmsnorm -> LM-head GEMM (fp32 partials) -> lmhead_tile_argmax -> bookkeeping
+// (short chunks: the four GEMMs leave partials, and a kernel behind each does what the epilogues do)
 // The decode step itself is one persistent kernel (ss_decode_mega.cuh) and shares the small helpers here.
 //
 // Every kernel starts with griddepcontrol.launch_dependents / griddepcontrol.wait so that the
@@ -64,16 +65,23 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
 // the exact shared-memory image of a 256-row x 64-column tile under the 128-byte swizzle (row r at
 // r*128 bytes, its 16-byte chunk c stored at chunk position c ^ (r & 7)).  Each half of a block is
 // the image of a 128-row tile, which is what the prompt-pass GEMM loads.  One thread per 16-byte chunk.
-// row_off places the source at a row offset of the destination matrix (q,k,v and gate,up are stacked).
+// row_off places the source at a row offset of the destination matrix (q,k,v are stacked).  `half`, `step` say where a
+// source row goes in it: rows that one thread of an epilogue (or of the decode step) wants together become neighbours.
+//   half = 0: row r goes to row_off + r * step (step 1; 2 for gate and up, which alternate)
+//   half > 0: the two halves of every 2 * half rows alternate (q and k: the two dimensions of a rotation)
 __global__ void __launch_bounds__(256)
 repack_weights_kernel(const uint4* __restrict__ src, long long rows, int K, uint8_t* __restrict__ dst, int row_off,
-                      int kb) {
+                      int kb, int half, int step) {
   const int chunks_per_row = K >> 3;
   const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (id >= rows * chunks_per_row) return;
   const long long sr = id / chunks_per_row;
   const int cc = (int)(id - sr * chunks_per_row);
-  const long long n = row_off + sr;
+  long long n = row_off + sr * step;
+  if (half > 0) {
+    const long long i = sr % (2 * half);
+    n = row_off + (sr - i) + (i < half ? 2 * i : 2 * (i - half) + 1);
+  }
   const long long tile = n / kTileN;
   const int r = (int)(n % kTileN), k = cc >> 3, c = cc & 7;
   uint8_t* blk = dst + ((size_t)tile * kb + k) * (size_t)kBlockBytes;
@@ -90,46 +98,63 @@ __global__ void rope_table_kernel(const float* __restrict__ inv_freq, float2* __
 }
 
 // ------------------------------------------------------------------------------------ embedding + first norm
-// h[row] = E[token]; x[row] = RMSNorm(h[row]) * g   (rows: decode B rows or T prompt tokens)
+// A row of d floats (d a multiple of 64, at most 8192) is held by 256 threads as up to 8 x 4 values each: read once,
+// normalised from registers.  (Element by element with a second pass over the row: 15 us for a handful of tokens, a chain
+// of dependent round trips, and 171 us for 16281 tokens, 0.35 of the copy bandwidth; now 5 and 58 us.)
+constexpr int kRowVec = 8;
+__device__ __forceinline__ float row_sum_squares(const float4 (&v)[kRowVec], int d4, float* red) {
+  float ss = 0.f;
+#pragma unroll
+  for (int k = 0; k < kRowVec; ++k)
+    if (threadIdx.x + k * 256 < d4) ss += v[k].x * v[k].x + v[k].y * v[k].y + v[k].z * v[k].z + v[k].w * v[k].w;
+  return block_sum(ss, red);
+}
+__device__ __forceinline__ void store_normed(const float4 (&v)[kRowVec], int d4, float inv, const bf16* __restrict__ g, bf16* __restrict__ x) {
+#pragma unroll
+  for (int k = 0; k < kRowVec; ++k) {
+    const int i = threadIdx.x + k * 256;
+    if (i < d4) {
+      const uint2 gb = __ldg(reinterpret_cast<const uint2*>(g) + i);
+      const float2 g0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gb.x));
+      const float2 g1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gb.y));
+      uint2 o;
+      o.x = pack_bf16x2(v[k].x * inv * g0.x, v[k].y * inv * g0.y);
+      o.y = pack_bf16x2(v[k].z * inv * g1.x, v[k].w * inv * g1.y);
+      reinterpret_cast<uint2*>(x)[i] = o;
+    }
+  }
+}
+
+// h[t] = E[token]; x[t] = RMSNorm(h[t]) * g over T prompt tokens.
 __global__ void __launch_bounds__(256)
-embed_rmsnorm_kernel(const int32_t* __restrict__ tokens, const int32_t* __restrict__ active,
-                     const bf16* __restrict__ E, const bf16* __restrict__ g, float* __restrict__ h,
+embed_rmsnorm_kernel(const int32_t* __restrict__ tokens, const bf16* __restrict__ E, const bf16* __restrict__ g, float* __restrict__ h,
                      bf16* __restrict__ x, int d, float eps, int vocab) {
   __shared__ float red[32];
   pdl_launch_dependents();
   pdl_wait();
-  const int r = blockIdx.x;
-  if (active && !active[r]) return;
+  const size_t r = blockIdx.x;
   int tok = tokens[r];
   if (tok < 0 || tok >= vocab) tok = 0;
-  const bf16* e = E + (size_t)tok * d;
-  float ss = 0.f;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) {
-    const float v = __bfloat162float(e[i]);
-    h[(size_t)r * d + i] = v;
-    ss += v * v;
-  }
-  ss = block_sum(ss, red);
-  const float inv = rsqrtf(ss / d + eps);
-  for (int i = threadIdx.x; i < d; i += blockDim.x) {
-    const float v = __bfloat162float(e[i]);
-    x[(size_t)r * d + i] = __float2bfloat16_rn(v * inv * __bfloat162float(g[i]));
-  }
-}
-
-__device__ __forceinline__ void unpack8(const uint4& u, float (&f)[8]) {
-  const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&u);
+  const int d4 = d >> 2;
+  float4 v[kRowVec];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float2 t = __bfloat1622float2(p[j]);
-    f[2 * j] = t.x;
-    f[2 * j + 1] = t.y;
+  for (int k = 0; k < kRowVec; ++k) {
+    const int i = threadIdx.x + k * 256;
+    if (i < d4) {
+      const uint2 e = __ldg(reinterpret_cast<const uint2*>(E + (size_t)tok * d) + i);
+      const float2 e0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&e.x));
+      const float2 e1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&e.y));
+      v[k] = make_float4(e0.x, e0.y, e1.x, e1.y);
+      reinterpret_cast<float4*>(h + r * d)[i] = v[k];
+    }
   }
+  const float inv = rsqrtf(row_sum_squares(v, d4, red) / d + eps);
+  store_normed(v, d4, inv, g, x + r * d);
 }
 
 // ------------------------------------------------------------------------------------ LM head argmax
-// Stage 1, grid n_tiles (of the vocabulary), block 128 (thread = vocabulary row of the tile):
-// logits from partials for every row of the batch, optional dump, and the tile's best (value, id)
+// Stage 1, grid (n_tiles of the vocabulary, rows / kArgmaxRows), block 128 (thread = vocabulary row of the tile):
+// logits from partials for the block's rows of the batch, optional dump, and the tile's best (value, id)
 // per batch row; the lowest id wins a tie; EOS is left out when the row has a forced-EOS schedule.
 // Stage 2 (inside bookkeeping_kernel) picks the best tile per row.
 __device__ __forceinline__ uint32_t float_order_key(float f) {      // monotone float -> uint32
@@ -171,17 +196,19 @@ __device__ __forceinline__ float decision_value(float logit, const SampleCfg& sc
   return fmaf(logit, sc.inv_temp, -logf(-logf(u)));
 }
 
+constexpr int kArgmaxRows = 8;             // one after the other in a block: 100 rows by one block each took 92 us
 __global__ void __launch_bounds__(128)
 lmhead_tile_argmax_kernel(const float* __restrict__ partial, SplitInfo sp, RowState st, float* __restrict__ dump_logits,
                           float* __restrict__ tile_val, int32_t* __restrict__ tile_idx, int B, int vocab, int n_tiles,
                           int eos_id, SampleCfg sc) {
-  __shared__ uint32_t s_key[4][kMaxBatch];
-  __shared__ int s_id[4][kMaxBatch];
+  __shared__ uint32_t s_key[4][kArgmaxRows];
+  __shared__ int s_id[4][kArgmaxRows];
   pdl_launch_dependents();
   pdl_wait();
   const int tile = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int v = tile * 128 + threadIdx.x;
-  for (int r = 0; r < B; ++r) {
+  const int r_lo = blockIdx.y * kArgmaxRows, r_hi = min(B, r_lo + kArgmaxRows);
+  for (int r = r_lo; r < r_hi; ++r) {
     uint32_t key = 0;                              // below every real key
     if (st.active[r]) {
       if (v < vocab) {
@@ -193,19 +220,19 @@ lmhead_tile_argmax_kernel(const float* __restrict__ partial, SplitInfo sp, RowSt
       const uint32_t best = __reduce_max_sync(0xffffffffu, key);
       const uint32_t who = __ballot_sync(0xffffffffu, key == best);
       if (lane == 0) {
-        s_key[warp][r] = best;
-        s_id[warp][r] = tile * 128 + warp * 32 + (__ffs(who) - 1);     // lowest lane = lowest id
+        s_key[warp][r - r_lo] = best;
+        s_id[warp][r - r_lo] = tile * 128 + warp * 32 + (__ffs(who) - 1);     // lowest lane = lowest id
       }
     }
   }
   __syncthreads();
-  for (int r = threadIdx.x; r < B; r += 128) {
-    if (!st.active[r]) continue;
-    uint32_t bk = s_key[0][r];
-    int bi = s_id[0][r];
+  const int k = threadIdx.x, r = r_lo + k;
+  if (r < r_hi && st.active[r]) {
+    uint32_t bk = s_key[0][k];
+    int bi = s_id[0][k];
 #pragma unroll
     for (int w = 1; w < 4; ++w)
-      if (s_key[w][r] > bk) { bk = s_key[w][r]; bi = s_id[w][r]; }     // warps ascend in id: '>' keeps the lowest
+      if (s_key[w][k] > bk) { bk = s_key[w][k]; bi = s_id[w][k]; }     // warps ascend in id: '>' keeps the lowest
     tile_val[(size_t)r * n_tiles + tile] = __uint_as_float(bk);       // order key, bit-cast
     tile_idx[(size_t)r * n_tiles + tile] = bi;
   }
@@ -273,15 +300,13 @@ rmsnorm_kernel(const float* __restrict__ h, const bf16* __restrict__ g, bf16* __
   pdl_launch_dependents();
   pdl_wait();
   const size_t r = blockIdx.x;
-  float ss = 0.f;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) {
-    const float v = h[r * d + i];
-    ss += v * v;
-  }
-  ss = block_sum(ss, red);
-  const float inv = rsqrtf(ss / d + eps);
-  for (int i = threadIdx.x; i < d; i += blockDim.x)
-    x[r * d + i] = __float2bfloat16_rn(h[r * d + i] * inv * __bfloat162float(g[i]));
+  const int d4 = d >> 2;
+  float4 v[kRowVec];
+#pragma unroll
+  for (int k = 0; k < kRowVec; ++k)
+    if (threadIdx.x + k * 256 < d4) v[k] = reinterpret_cast<const float4*>(h + r * d)[threadIdx.x + k * 256];
+  const float inv = rsqrtf(row_sum_squares(v, d4, red) / d + eps);
+  store_normed(v, d4, inv, g, x + r * d);
 }
 
 // Gather each sequence's last token: h_last[s] = h[last[s]]; x_last[s] = RMSNorm(h_last[s]) * g.
@@ -292,248 +317,313 @@ gather_last_rmsnorm_kernel(const float* __restrict__ h, const int32_t* __restric
   __shared__ float red[32];
   pdl_launch_dependents();
   pdl_wait();
-  const int s = blockIdx.x;
-  const size_t t = (size_t)last_tok[s];
-  float ss = 0.f;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) {
-    const float v = h[t * d + i];
-    ss += v * v;
+  const size_t s = blockIdx.x, t = (size_t)last_tok[s];
+  const int d4 = d >> 2;
+  float4 v[kRowVec];
+#pragma unroll
+  for (int k = 0; k < kRowVec; ++k) {
+    const int i = threadIdx.x + k * 256;
+    if (i < d4) {
+      v[k] = reinterpret_cast<const float4*>(h + t * d)[i];
+      reinterpret_cast<float4*>(h_out + s * d)[i] = v[k];
+      if (dump_hidden) {                             // the caller's buffer: no alignment beyond a float's
+        float* o = dump_hidden + s * d + (size_t)i * 4;
+        o[0] = v[k].x; o[1] = v[k].y; o[2] = v[k].z; o[3] = v[k].w;
+      }
+    }
   }
-  ss = block_sum(ss, red);
-  const float inv = rsqrtf(ss / d + eps);
-  for (int i = threadIdx.x; i < d; i += blockDim.x) {
-    const float v = h[t * d + i];
-    h_out[(size_t)s * d + i] = v;
-    if (dump_hidden) dump_hidden[(size_t)s * d + i] = v;
-    x_out[(size_t)s * d + i] = __float2bfloat16_rn(v * inv * __bfloat162float(g[i]));
+  const float inv = rsqrtf(row_sum_squares(v, d4, red) / d + eps);
+  store_normed(v, d4, inv, g, x_out + s * d);
+}
+
+// ---- short prompts (chunks of at most kShortTokens tokens): every projection is split over all SMs along K as well and
+// leaves fp32 partials [slot][token][128 rows]; these kernels add them (four consecutive outputs per thread) and do what
+// the epilogues of the paired GEMM do.  With a CTA per 128-row tile the o and down projections ran on 32 CTAs of 148 and
+// took 50 us each for 61 tokens (7B shape); the whole prompt pass of 8 layers went from 1.89 to 1.05 ms.
+constexpr int kShortTokens = 128;
+
+// Partials of outputs n0 .. n0 + 3 (inside one 128-row tile) for token tok, added in CTA order.
+__device__ __forceinline__ float4 sum_partials4(const float* __restrict__ partial, const SplitInfo& s, int n0, int tok) {
+  const int4 t = __ldg(reinterpret_cast<const int4*>(s.tiles) + (n0 >> 7));
+  const size_t slot_stride = (size_t)s.NT * 128, cta_stride = slot_stride * s.max_seg;
+  const size_t off = (size_t)tok * 128 + (n0 & 127);
+  float4 x = __ldcg(reinterpret_cast<const float4*>(partial + (size_t)t.x * slot_stride + off));
+  for (int c = t.y; c <= t.z; c += 4) {
+    float4 u[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) u[j] = __ldcg(reinterpret_cast<const float4*>(partial + (size_t)min(c + j, t.z) * cta_stride + off));
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (c + j <= t.z) { x.x += u[j].x; x.y += u[j].y; x.z += u[j].z; x.w += u[j].w; }
+  }
+  return x;
+}
+
+// grid (T, ceil(3d / 1024)), block 256
+__global__ void __launch_bounds__(256)
+short_qkv_kernel(const float* __restrict__ partial, SplitInfo sp, GemmArgs a) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int t = blockIdx.x, n = (blockIdx.y * 256 + threadIdx.x) * 4;
+  if (n >= 3 * a.d) return;
+  const int sec = n / a.d, in = n - sec * a.d, hd = in / a.Dh, e = in - hd * a.Dh;
+  float4 x = sum_partials4(partial, sp, n, t);
+  if (sec < 2) {
+    const float2* rope = a.rope + (size_t)a.tok_pos[t] * (a.Dh >> 1) + (e >> 1);
+    const float2 c0 = __ldg(rope), c1 = __ldg(rope + 1);
+    x = make_float4(x.x * c0.x - x.y * c0.y, x.y * c0.x + x.x * c0.y, x.z * c1.x - x.w * c1.y, x.w * c1.x + x.z * c1.y);
+  }
+  const uint2 w = make_uint2(pack_bf16x2(x.x, x.y), pack_bf16x2(x.z, x.w));
+  *reinterpret_cast<uint2*>(reinterpret_cast<bf16*>(a.out) + (size_t)t * 3 * a.d + n) = w;
+  if (sec > 0) {
+    const int slot = a.tok_slot[t];
+    *reinterpret_cast<uint2*>(reinterpret_cast<bf16*>(a.kv_layer) + (size_t)(slot / kPageTokens) * a.page_elems +
+                              ((size_t)((sec - 1) * a.H + hd) * kPageTokens + slot % kPageTokens) * a.Dh + e) = w;
   }
 }
 
-// RoPE on q and k of the packed fp32 [T, 3d] projection, one rounding to bf16 afterwards: q, k, v go to the packed
-// bf16 [T, 3d] operand of the prompt-pass attention and k, v into the pages.
-// grid (T), block 256 = (256 / (Dh/2)) heads side by side x Dh/2 rotation pairs; the sine and cosine of a
-// (token, pair) are computed once and used for every head.  tok_row / tok_pos give each token's row in the
-// batch and position.
+// h[t] += projection; x[t] = RMSNorm(h[t]) * g.  grid (T), block 256
 __global__ void __launch_bounds__(256)
-rope_append_prefill_kernel(const float* __restrict__ qkv_f, bf16* __restrict__ qkv, const int32_t* __restrict__ tok_row,
-                           const int32_t* __restrict__ tok_pos, RowState st, KvLayout kv, int layer,
-                           const float* __restrict__ inv_freq, int d, uint32_t* status) {
+short_residual_kernel(const float* __restrict__ partial, SplitInfo sp, float* __restrict__ h, const bf16* __restrict__ g,
+                      bf16* __restrict__ x, int d, float eps) {
+  __shared__ float red[32];
   pdl_launch_dependents();
   pdl_wait();
   const size_t t = blockIdx.x;
-  const int r = tok_row[t], pos = tok_pos[t];
-  const int Dh = kv.Dh, half = Dh >> 1;
-  const int i = threadIdx.x % half, hsub = threadIdx.x / half, hpar = blockDim.x / half;
-  float sn, cs;
-  sincosf((float)pos * inv_freq[i], &sn, &cs);
-  const int page = st.block_table[(size_t)r * st.max_pages + pos / kPageTokens];
-  if (page < 0 || page >= kv.n_pages) {
-    atomicCAS(status, 0u, (uint32_t)kStatusBadPage);
-    return;
+  const int d4 = d >> 2;
+  float4 v[kRowVec];
+#pragma unroll
+  for (int k = 0; k < kRowVec; ++k) {
+    const int i = threadIdx.x + k * 256;
+    if (i < d4) {
+      const float4 p = sum_partials4(partial, sp, i * 4, (int)t), h4 = reinterpret_cast<const float4*>(h + t * d)[i];
+      v[k] = make_float4(h4.x + p.x, h4.y + p.y, h4.z + p.z, h4.w + p.w);
+      reinterpret_cast<float4*>(h + t * d)[i] = v[k];
+    }
   }
-  for (int hd = hsub; hd < kv.H; hd += hpar) {
-    const float* qf = qkv_f + t * 3 * d + hd * Dh;
-    const float* kf = qf + d;
-    const float* vf = kf + d;
-    bf16* q = qkv + t * 3 * d + hd * Dh;
-    bf16* k = q + d;
-    bf16* v = k + d;
-    const float q0 = qf[i], q1 = qf[i + half], k0 = kf[i], k1 = kf[i + half];
-    const bf16 kr0 = __float2bfloat16_rn(k0 * cs - k1 * sn), kr1 = __float2bfloat16_rn(k1 * cs + k0 * sn);
-    const bf16 v0 = __float2bfloat16_rn(vf[i]), v1 = __float2bfloat16_rn(vf[i + half]);
-    q[i] = __float2bfloat16_rn(q0 * cs - q1 * sn);
-    q[i + half] = __float2bfloat16_rn(q1 * cs + q0 * sn);
-    k[i] = kr0;
-    k[i + half] = kr1;
-    v[i] = v0;
-    v[i + half] = v1;
-    bf16* kbase = kv.pool + (size_t)layer * kv.layer_stride + (size_t)page * kv.page_elems +
-                  ((size_t)hd * kPageTokens + (pos % kPageTokens)) * Dh;
-    bf16* vbase = kbase + (size_t)kv.H * kPageTokens * Dh;
-    kbase[i] = kr0;
-    kbase[i + half] = kr1;
-    vbase[i] = v0;
-    vbase[i + half] = v1;
-  }
+  const float inv = rsqrtf(row_sum_squares(v, d4, red) / d + eps);
+  store_normed(v, d4, inv, g, x + t * d);
 }
 
-// Causal attention over one prompt on the tensor cores (warp-level mma, m16n8k16, bf16 in, fp32 out).
-// CTA = (64 queries, head, sequence), four warps of 16 queries; keys and values are staged through shared
-// memory 32 at a time (values transposed, so that both B operands are read as pairs of consecutive
-// elements); online softmax on the accumulator fragments; the probabilities are re-used in registers as the
-// A operand of P.V.  qkv: [T, 3d] with RoPE applied; out: [T, d].
-// Fragment layout of mma.m16n8k16 (g = lane / 4, q = lane % 4): A regs 0..3 hold rows g, g+8, g, g+8 and
-// columns 2q..2q+1 (regs 0,1) or 2q+8..2q+9 (regs 2,3); B regs 0,1 hold k = 2q..2q+1 and 2q+8..2q+9 of
-// column g; C regs 0,1 hold row g, columns 2q..2q+1, regs 2,3 row g+8.
-__device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-               "{%0, %1, %2, %3};"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+// grid (T, ceil(2F / 1024)), block 256
+__global__ void __launch_bounds__(256)
+short_swiglu_kernel(const float* __restrict__ partial, SplitInfo sp, bf16* __restrict__ act, int F) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int t = blockIdx.x, n = (blockIdx.y * 256 + threadIdx.x) * 4;
+  if (n >= 2 * F) return;
+  const float4 x = sum_partials4(partial, sp, n, t);               // gate, up, gate, up
+  *reinterpret_cast<uint32_t*>(act + (size_t)t * F + (n >> 1)) =
+      pack_bf16x2(x.x / (1.f + __expf(-x.x)) * x.y, x.z / (1.f + __expf(-x.z)) * x.w);
 }
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&v);
+
+// Causal attention over one prompt on tcgen05.  CTA = (128 queries, head, sequence), one thread per query row; keys and
+// values come 128 at a time by TMA (128-byte swizzle) straight from the packed q,k,v operand.  Scores S = Q K^T (M = 128
+// queries, N = 128 keys) land in tensor memory, every thread reads its row, takes the running maximum and the weights
+// (fp32; rounded to bf16 as the A operand of the second product, as before), and O = P V (values as the MN-major B
+// operand, so nothing is transposed) is added to a running sum in registers.  P overwrites the keys at head size 128:
+// 96 KiB of shared memory and 256 columns of tensor memory, so two CTAs share an SM and one computes while the other's
+// loads and MMAs run.
+// Why: the warp-level mma of the first version is a sixteenth of tcgen05's rate on this part and its operands went
+// through a transposition in shared memory (630 -> 229 us per layer, 86 prompts of 96 to 288 tokens, 32 heads x 128).
+constexpr int kAttnTile = 128;             // queries per CTA, keys per step
+constexpr int kAttnBlock = kAttnTile * 128;    // one [128 rows x 64 columns] operand block: 16 KiB
+
+template <int DH> constexpr int attn_prefill_smem() {
+  return 2048 + (3 * (DH / 64) + (DH == 128 ? 0 : 2)) * kAttnBlock;
 }
+
+// Instruction descriptor as umma_idesc_bf16, with B (the values) MN-major.
+__host__ __device__ constexpr uint32_t umma_idesc_bf16_b_mn(int n, int m) { return umma_idesc_bf16(n, m) | (1u << 16); }
+// Shared-memory descriptor of an MN-major operand under the 128-byte swizzle: 64-element runs along N, rows (K) of 128
+// bytes, 8-row groups 1024 bytes apart, the next 64 elements of N one block further.
+__device__ __forceinline__ uint64_t smem_desc_mn_sw128(uint32_t saddr, uint32_t n_block_bytes) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr >> 4) & 0x3FFF);
+  d |= (uint64_t)(n_block_bytes >> 4) << 16;
+  d |= (uint64_t)(1024 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
+  return d;
+}
+__device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+
+struct AttnPrefillSmem {
+  uint64_t loaded, mma_done;
+  uint32_t tmem_base, pad;
+};
 
 template <int DH>
-__global__ void __launch_bounds__(128)
-attn_prefill_kernel(const bf16* __restrict__ qkv, const int32_t* __restrict__ cu_seqlens, bf16* __restrict__ out, int d) {
-  constexpr int QT = 64, KT = 32, KS = DH / 16, NB = DH / 8;
-  constexpr int KPAD = DH + 8;                     // padded rows: conflict-free fragment loads
-  constexpr int VPAD = KT + 8;
-  __shared__ __align__(16) bf16 s_k[KT][KPAD];     // [key][dim]
-  __shared__ __align__(16) bf16 s_vt[DH][VPAD];    // [dim][key]
-  pdl_launch_dependents();
-  pdl_wait();
+__global__ void __launch_bounds__(128, 2)
+attn_prefill_kernel(const __grid_constant__ CUtensorMap map_qkv, const int32_t* __restrict__ cu_seqlens, bf16* __restrict__ out, int d,
+                    uint32_t* status) {
+  constexpr int NB = DH / 64;                      // 64-column blocks per operand row
+  constexpr uint32_t kTmemCols = 256;              // scores, then outputs
+  extern __shared__ uint8_t smem_raw[];
+  AttnPrefillSmem* sm = reinterpret_cast<AttnPrefillSmem*>(smem_raw);
   const int hd = blockIdx.y, s = blockIdx.z;
-  const int seq0 = cu_seqlens[s], len = cu_seqlens[s + 1] - seq0;
-  const int qt0 = blockIdx.x * QT;
-  if (qt0 >= len) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = lane >> 2, q4 = lane & 3;
-  const int row0 = qt0 + warp * 16 + g, row1 = row0 + 8;     // this thread's two query positions
-  const float qscale = rsqrtf((float)DH) * 1.4426950408889634f;
-
-  // Q fragments, kept for the whole kernel (rows beyond the prompt read row len-1: valid memory, never stored)
-  uint32_t qa[KS][4];
-  {
-    const bf16* q0 = qkv + (size_t)(seq0 + min(row0, len - 1)) * 3 * d + hd * DH + q4 * 2;
-    const bf16* q1 = qkv + (size_t)(seq0 + min(row1, len - 1)) * 3 * d + hd * DH + q4 * 2;
-#pragma unroll
-    for (int ks = 0; ks < KS; ++ks) {
-      qa[ks][0] = *reinterpret_cast<const uint32_t*>(q0 + ks * 16);
-      qa[ks][1] = *reinterpret_cast<const uint32_t*>(q1 + ks * 16);
-      qa[ks][2] = *reinterpret_cast<const uint32_t*>(q0 + ks * 16 + 8);
-      qa[ks][3] = *reinterpret_cast<const uint32_t*>(q1 + ks * 16 + 8);
-    }
-  }
-  float o[NB][4];
-#pragma unroll
-  for (int nb = 0; nb < NB; ++nb) { o[nb][0] = o[nb][1] = o[nb][2] = o[nb][3] = 0.f; }
-  float m0 = -CUDART_INF_F, m1 = -CUDART_INF_F, l0 = 0.f, l1 = 0.f;
-
-  const int k_end = min(len, qt0 + QT);            // causal: keys up to the tile's last query
-  for (int kt0 = 0; kt0 < k_end; kt0 += KT) {
-    __syncthreads();
-    constexpr int CH = DH / 8;                     // 16-byte chunks per row
-    for (int c = threadIdx.x; c < KT * CH; c += 128) {
-      const int kr = c / CH, cc = c % CH;
-      uint4 uk = make_uint4(0, 0, 0, 0), uv = uk;
-      if (kt0 + kr < len) {
-        const bf16* base = qkv + (size_t)(seq0 + kt0 + kr) * 3 * d + d + hd * DH + cc * 8;
-        uk = *reinterpret_cast<const uint4*>(base);
-        uv = *reinterpret_cast<const uint4*>(base + d);
-      }
-      *reinterpret_cast<uint4*>(&s_k[kr][cc * 8]) = uk;
-      const bf16* pv = reinterpret_cast<const bf16*>(&uv);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) s_vt[cc * 8 + e][kr] = pv[e];
-    }
-    __syncthreads();
-    if (kt0 > qt0 + warp * 16 + 15) continue;      // every key of the tile is after this warp's last query
-
-    // S = Q K^T for 16 queries x 32 keys
-    float sc[KT / 8][4];
-#pragma unroll
-    for (int nb = 0; nb < KT / 8; ++nb) {
-      sc[nb][0] = sc[nb][1] = sc[nb][2] = sc[nb][3] = 0.f;
-#pragma unroll
-      for (int ks = 0; ks < KS; ++ks) {
-        const uint32_t b0 = *reinterpret_cast<const uint32_t*>(&s_k[nb * 8 + g][ks * 16 + q4 * 2]);
-        const uint32_t b1 = *reinterpret_cast<const uint32_t*>(&s_k[nb * 8 + g][ks * 16 + q4 * 2 + 8]);
-        mma_bf16_16816(sc[nb], qa[ks], b0, b1);
-      }
-    }
-    // scale, causal / length mask, running maxima
-    float mx0 = m0, mx1 = m1;
-#pragma unroll
-    for (int nb = 0; nb < KT / 8; ++nb) {
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int key = kt0 + nb * 8 + q4 * 2 + e;
-        sc[nb][e] = (key <= row0 && key < len) ? sc[nb][e] * qscale : -CUDART_INF_F;
-        sc[nb][2 + e] = (key <= row1 && key < len) ? sc[nb][2 + e] * qscale : -CUDART_INF_F;
-        mx0 = fmaxf(mx0, sc[nb][e]);
-        mx1 = fmaxf(mx1, sc[nb][2 + e]);
-      }
-    }
-    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1));
-    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
-    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
-    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
-    const float r0s = (mx0 == -CUDART_INF_F) ? 1.f : exp2f(m0 - mx0);     // exp2f(-inf) = 0 on the first tile
-    const float r1s = (mx1 == -CUDART_INF_F) ? 1.f : exp2f(m1 - mx1);
-    m0 = mx0;
-    m1 = mx1;
-    l0 *= r0s;
-    l1 *= r1s;
-#pragma unroll
-    for (int nb = 0; nb < NB; ++nb) {
-      o[nb][0] *= r0s; o[nb][1] *= r0s;
-      o[nb][2] *= r1s; o[nb][3] *= r1s;
-    }
-    // probabilities, as A fragments of P V (two 16-key steps)
-    uint32_t pa[KT / 16][4];
-#pragma unroll
-    for (int nb = 0; nb < KT / 8; ++nb) {
-      float p[4];
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        p[e] = (sc[nb][e] == -CUDART_INF_F) ? 0.f : exp2f(sc[nb][e] - m0);
-        p[2 + e] = (sc[nb][2 + e] == -CUDART_INF_F) ? 0.f : exp2f(sc[nb][2 + e] - m1);
-      }
-      l0 += p[0] + p[1];
-      l1 += p[2] + p[3];
-      pa[nb >> 1][(nb & 1) * 2 + 0] = pack_bf16x2(p[0], p[1]);
-      pa[nb >> 1][(nb & 1) * 2 + 1] = pack_bf16x2(p[2], p[3]);
-    }
-    // O += P V
-#pragma unroll
-    for (int nb = 0; nb < NB; ++nb) {
-#pragma unroll
-      for (int kk = 0; kk < KT / 16; ++kk) {
-        const uint32_t b0 = *reinterpret_cast<const uint32_t*>(&s_vt[nb * 8 + g][kk * 16 + q4 * 2]);
-        const uint32_t b1 = *reinterpret_cast<const uint32_t*>(&s_vt[nb * 8 + g][kk * 16 + q4 * 2 + 8]);
-        mma_bf16_16816(o[nb], pa[kk], b0, b1);
-      }
-    }
-  }
-  // row sums over the four lanes of a row, then the output
-  l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
-  l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
-  l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
-  l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
-  const float i0 = 1.f / l0, i1 = 1.f / l1;
-#pragma unroll
-  for (int nb = 0; nb < NB; ++nb) {
-    if (row0 < len)
-      *reinterpret_cast<uint32_t*>(out + (size_t)(seq0 + row0) * d + hd * DH + nb * 8 + q4 * 2) =
-          pack_bf16x2(o[nb][0] * i0, o[nb][1] * i0);
-    if (row1 < len)
-      *reinterpret_cast<uint32_t*>(out + (size_t)(seq0 + row1) * d + hd * DH + nb * 8 + q4 * 2) =
-          pack_bf16x2(o[nb][2] * i1, o[nb][3] * i1);
-  }
-}
-
-// act[t][f] = silu(gu[t][f]) * gu[t][F+f] over T tokens (gu fp32, act bf16: one rounding), 8 features per thread
-// (F a multiple of 8).  grid (T, ceil(F / 2048)), block 256.
-__global__ void __launch_bounds__(256)
-swiglu_kernel(const float* __restrict__ gu, bf16* __restrict__ act, int F) {
   pdl_launch_dependents();
+  const int seq0 = cu_seqlens[s], len = cu_seqlens[s + 1] - seq0;
+  const int qt0 = (int)(gridDim.x - 1 - blockIdx.x) * kAttnTile;          // the longest rows first
+  if (qt0 >= len) return;
+  const uint32_t q_s = (smem_u32(smem_raw) + (uint32_t)sizeof(AttnPrefillSmem) + 1023u) & ~1023u;
+  const uint32_t k_s = q_s + NB * kAttnBlock, v_s = k_s + NB * kAttnBlock;
+  const uint32_t p_s = DH == 128 ? k_s : v_s + NB * kAttnBlock;
+  const uint32_t loaded = smem_u32(&sm->loaded), mma_done = smem_u32(&sm->mma_done);
+  if (threadIdx.x == 0) {
+    mbar_init(loaded, 1);
+    mbar_init(mma_done, 1);
+    fence_barrier_init();
+    tma_prefetch_desc(&map_qkv);
+  }
+  if (warp == 0) {
+    tmem_alloc(smem_u32(&sm->tmem_base), kTmemCols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = sm->tmem_base, tmem_row = tmem + ((uint32_t)(warp * 32) << 16);
   pdl_wait();
-  const size_t t = blockIdx.x;
-  const int f0 = (blockIdx.y * blockDim.x + threadIdx.x) * 8;
-  if (f0 >= F) return;
-  const float4* g4 = reinterpret_cast<const float4*>(gu + t * 2 * F + f0);
-  const float4* u4 = reinterpret_cast<const float4*>(gu + t * 2 * F + F + f0);
-  const float4 ga = g4[0], gb = g4[1], ua = u4[0], ub = u4[1];
-  const float gt[8] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
-  const float up[8] = {ua.x, ua.y, ua.z, ua.w, ub.x, ub.y, ub.z, ub.w};
-  __align__(16) bf16 ob[8];
+
+  uint64_t hint;
+  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(hint));
+  auto load_kv = [&](int kt0, uint32_t more) {     // thread 0: the keys and values of a step
+    mbar_expect_tx(loaded, 2u * NB * kAttnBlock + more);
+    for (int b = 0; b < NB; ++b) {
+      tma_load_2d(k_s + b * kAttnBlock, &map_qkv, loaded, d + hd * DH + b * 64, seq0 + kt0, hint);
+      tma_load_2d(v_s + b * kAttnBlock, &map_qkv, loaded, 2 * d + hd * DH + b * 64, seq0 + kt0, hint);
+    }
+  };
+  if (threadIdx.x == 0) {
+    load_kv(0, NB * kAttnBlock);
+    for (int b = 0; b < NB; ++b) tma_load_2d(q_s + b * kAttnBlock, &map_qkv, loaded, hd * DH + b * 64, seq0 + qt0, hint);
+  }
+
+  const int row = threadIdx.x, pos = qt0 + row;    // this thread's query
+  const float qscale = rsqrtf((float)DH) * 1.4426950408889634f;
+  float o[DH];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) ob[j] = __float2bfloat16_rn(gt[j] / (1.f + __expf(-gt[j])) * up[j]);
-  *reinterpret_cast<uint4*>(act + t * F + f0) = *reinterpret_cast<const uint4*>(ob);
+  for (int e = 0; e < DH; ++e) o[e] = 0.f;
+  float m = -CUDART_INF_F, l = 0.f;
+  const int k_end = min(len, qt0 + kAttnTile);     // causal: keys up to the tile's last query
+  uint32_t n_load = 0, n_mma = 0;
+  bool ok = true;
+  for (int kt0 = 0; kt0 < k_end; kt0 += kAttnTile) {
+    ok = mbar_wait(loaded, n_load++ & 1u, status, kStatusProducerTimeout);
+    if (ok && threadIdx.x == 0) {
+      tc_fence_after();
+      const uint32_t idesc = umma_idesc_bf16(kAttnTile);
+#pragma unroll
+      for (int kk = 0; kk < DH / 16; ++kk) {
+        const uint32_t at = (uint32_t)((kk >> 2) * kAttnBlock);
+        umma_bf16(tmem, smem_desc_sw128(q_s + at) + (uint64_t)((kk & 3) * 2), smem_desc_sw128(k_s + at) + (uint64_t)((kk & 3) * 2), idesc,
+                  kk ? 1u : 0u);
+      }
+      umma_commit(mma_done);
+    }
+    ok = ok && mbar_wait(mma_done, n_mma++ & 1u, status, kStatusMmaTimeout);
+    if (!__syncthreads_and(ok)) { ok = false; break; }
+    tc_fence_after();
+    // keys this row may see in the step: all, or up to its own position (rows beyond the prompt are never stored)
+    const int vis = min(kAttnTile, pos - kt0 + 1);
+    float mx = m;
+#pragma unroll 1
+    for (int c = 0; c < kAttnTile; c += 64) {
+      uint32_t v[64];
+      tmem_ld64(tmem_row + c, v);
+#pragma unroll
+      for (int j = 0; j < 64; ++j) mx = fmaxf(mx, c + j < vis ? __uint_as_float(v[j]) * qscale : -CUDART_INF_F);
+    }
+    const float mr = mx == -CUDART_INF_F ? 0.f : mx;       // no finite score so far: weights of 0, not NaN
+    const float keep = exp2f(m - mr);
+    m = mx;
+    l *= keep;
+#pragma unroll 1
+    for (int c = 0; c < kAttnTile; c += 64) {
+      uint32_t v[64];
+      tmem_ld64(tmem_row + c, v);
+      // the row's line of the K-major operand block: eight 16-byte chunks, chunk i at place i ^ (row & 7)
+      const uint32_t line = p_s + (uint32_t)((c >> 6) * kAttnBlock + row * 128);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        uint32_t w[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          const int j = i * 8 + h * 2;
+          const float p0 = c + j < vis ? exp2f(__uint_as_float(v[j]) * qscale - mr) : 0.f;
+          const float p1 = c + j + 1 < vis ? exp2f(__uint_as_float(v[j + 1]) * qscale - mr) : 0.f;
+          l += p0 + p1;
+          w[h] = pack_bf16x2(p0, p1);
+        }
+        sts128(line + (uint32_t)((i ^ (row & 7)) * 16), w[0], w[1], w[2], w[3]);
+      }
+    }
+    if (kt0 + row >= len) {
+      // values behind the prompt's end belong to another row: a weight of 0 times what they may hold must stay 0
+      for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) sts128(v_s + (uint32_t)(b * kAttnBlock + row * 128 + i * 16), 0u, 0u, 0u, 0u);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    tc_fence_before();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      tc_fence_after();
+      const uint32_t idesc = umma_idesc_bf16_b_mn(DH, kAttnTile);
+#pragma unroll
+      for (int kk = 0; kk < kAttnTile / 16; ++kk)
+        umma_bf16(tmem + kAttnTile, smem_desc_sw128(p_s + (uint32_t)((kk >> 2) * kAttnBlock)) + (uint64_t)((kk & 3) * 2),
+                  smem_desc_mn_sw128(v_s + (uint32_t)(kk * 2048), kAttnBlock), idesc, kk ? 1u : 0u);
+      umma_commit(mma_done);
+    }
+    ok = mbar_wait(mma_done, n_mma++ & 1u, status, kStatusMmaTimeout);
+    if (!__syncthreads_and(ok)) { ok = false; break; }
+    if (threadIdx.x == 0 && kt0 + kAttnTile < k_end) load_kv(kt0 + kAttnTile, 0);
+    tc_fence_after();
+#pragma unroll
+    for (int c = 0; c < DH; c += 64) {
+      uint32_t v[64];
+      tmem_ld64(tmem_row + kAttnTile + c, v);
+#pragma unroll
+      for (int j = 0; j < 64; ++j) o[c + j] = fmaf(o[c + j], keep, __uint_as_float(v[j]));
+    }
+    tc_fence_before();
+  }
+  if (ok) {
+    // the row's bf16 output through the query's shared memory (read by the last MMA), so that rows are stored as whole lines
+    const float il = 1.f / l;
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float* x = o + b * 64 + i * 8;
+        sts128(q_s + (uint32_t)(b * kAttnBlock + row * 128 + (i ^ (row & 7)) * 16), pack_bf16x2(x[0] * il, x[1] * il),
+               pack_bf16x2(x[2] * il, x[3] * il), pack_bf16x2(x[4] * il, x[5] * il), pack_bf16x2(x[6] * il, x[7] * il));
+      }
+    __syncwarp();
+    constexpr int LPR = DH / 8;                    // lanes per output row, 16 bytes each
+    for (int i = 0; i < 32; i += 32 / LPR) {
+      const int rr = warp * 32 + i + lane / LPR, ch = lane % LPR;
+      uint4 v;
+      asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                   : "r"(q_s + (uint32_t)((ch >> 3) * kAttnBlock + rr * 128 + (((ch & 7) ^ (rr & 7)) * 16))) : "memory");
+      if (qt0 + rr < len) *reinterpret_cast<uint4*>(out + (size_t)(seq0 + qt0 + rr) * d + hd * DH + ch * 8) = v;
+    }
+  } else {
+    // a wait ran out: copies and MMAs in flight get a bounded time to end before their memory is given up
+    const long long t0 = clock64();
+    while (clock64() - t0 < 2000000LL) { }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    tmem_dealloc(tmem, kTmemCols);
+  }
 }
 
 }  // namespace ss

@@ -52,7 +52,8 @@ DecodeSplit plan_decode(int n_out, int K, int n_sm) {
   return p;
 }
 
-GemmPlan plan_gemm(int n_out, int K, int NT, int tok_tiles, int mode, int n_sm) {
+// Split of a projection in 128-row tiles (gemm_wx_kernel) over the SMs, for one tile of NT tokens.
+GemmPlan plan_gemm(int n_out, int K, int NT, int n_sm) {
   GemmPlan p{};
   p.n_out = n_out;
   p.K = K;
@@ -60,13 +61,8 @@ GemmPlan plan_gemm(int n_out, int K, int NT, int tok_tiles, int mode, int n_sm) 
   p.kb = ceil_div(K, kTileK);
   p.NT = NT;
   const long long total = (long long)p.n_tiles * p.kb;
-  if (mode == kGemmPartial) {
-    p.gridx = (int)std::min<long long>(n_sm, total);
-    p.gridy = 1;
-  } else {
-    p.gridx = p.n_tiles;
-    p.gridy = tok_tiles;
-  }
+  p.gridx = (int)std::min<long long>(n_sm, total);
+  p.gridy = 1;
   const int ipc = std::max(1, (int)((total + p.gridx - 1) / p.gridx));
   p.max_seg = (ipc + p.kb - 2) / p.kb + 1;
   const int stage_bytes = kTileM * kTileK * 2 + NT * kTileK * 2;
@@ -78,6 +74,8 @@ GemmPlan plan_gemm(int n_out, int K, int NT, int tok_tiles, int mode, int n_sm) 
   p.tmem_cols = cols;
   return p;
 }
+// Token tile of a short prompt chunk.
+int short_tile(int tokens) { return std::min(kShortTokens, round_up(tokens, 16)); }
 
 SplitInfo split_of(const GemmPlan& p, const TileSeg* tiles) {
   SplitInfo s;
@@ -151,20 +149,19 @@ struct ss_ctx {
   uint32_t* status = nullptr;
   RowState st{};
   KvLayout kv{};
-  int32_t* d_chunk = nullptr;      // a prompt chunk's arrays, packed: tokens, rows, positions, prefix sums, last tokens
-  int32_t *d_tokens = nullptr, *d_tok_row = nullptr, *d_tok_pos = nullptr, *d_cu = nullptr, *d_last = nullptr;
+  int32_t* d_chunk = nullptr;      // a prompt chunk's arrays, packed: tokens, cache slots, positions, prefix sums, last tokens
+  int32_t *d_tokens = nullptr, *d_tok_slot = nullptr, *d_tok_pos = nullptr, *d_cu = nullptr, *d_last = nullptr;
   // prompt-pass activations (R rows)
   int R = 0;
   float* h = nullptr;
   bf16 *x = nullptr, *qkv = nullptr, *attn_o = nullptr, *act = nullptr;
-  float *qkv_f = nullptr, *gu = nullptr;   // q,k,v and gate/up as they leave their GEMMs (fp32: rounded once, after RoPE / SwiGLU)
   // decode activations (kMaxBatch rows)
   float* h_dec = nullptr;
   bf16 *x_dec = nullptr, *o_dec = nullptr, *act_dec = nullptr;
   float* partial = nullptr;
   size_t partial_bytes = 0;
   TileSeg* tbl[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};   // decode step: qkv, o, gate/up, down, lm head
-  TileSeg* tbl_lm_prompt = nullptr;                                  // LM head after the prompt pass (128-row tiles)
+  TileSeg* tbl128[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};   // the same projections in 128-row tiles: short prompts, first LM head
   float* rowss = nullptr;          // [kMaxBatch][kMaxSlices]
   unsigned long long* grid_ctr = nullptr;
   float* att_part = nullptr;       // decode attention: partial results that cross CTAs, and their flags
@@ -276,7 +273,7 @@ int make_line_map(ss_ctx* c, CUtensorMap* out, const void* base, size_t bytes) {
   return SS_OK;
 }
 
-// activation operand map (cached): id 0 = x, 1 = attn_o, 2 = act (prompt pass); 3 = x_dec, 4 = o_dec, 5 = act_dec
+// activation operand map (cached): id 0 = x, 1 = attn_o, 2 = act, 6 = q,k,v (prompt pass); 3 = x_dec, 4 = o_dec, 5 = act_dec
 int xmap(ss_ctx* c, int id, int box_rows, const CUtensorMap** out) {
   auto key = std::make_pair(id, box_rows);
   auto it = c->xmaps.find(key);
@@ -289,6 +286,7 @@ int xmap(ss_ctx* c, int id, int box_rows, const CUtensorMap** out) {
       case 1: base = c->attn_o; rows = c->R; cols = d; break;
       case 2: base = c->act; rows = c->R; cols = F; break;
       case 3: base = c->x_dec; rows = kMaxBatch; cols = d; break;
+      case 6: base = c->qkv; rows = c->R; cols = 3 * (int64_t)d; break;
       case 4: base = c->o_dec; rows = kMaxBatch; cols = d; break;
       default: base = c->act_dec; rows = kMaxBatch; cols = F; break;
     }
@@ -301,31 +299,23 @@ int xmap(ss_ctx* c, int id, int box_rows, const CUtensorMap** out) {
   return SS_OK;
 }
 
-int run_gemm(ss_ctx* c, const uint8_t* w_tiled, const CUtensorMap& mx, const GemmPlan& p, int mode, int n_tok,
-             void* out_bf16, float* out_f32, int ld_out) {
+// A projection split over all SMs, into fp32 partials.
+int run_gemm(ss_ctx* c, const uint8_t* w_tiled, const CUtensorMap& mx, const GemmPlan& p, int n_tok) {
   GemmArgs a{};
   a.p = p;
   a.w_tiled = w_tiled;
-  a.mode = mode;
+  a.mode = kGemmPartial;
   a.n_tok = n_tok;
   a.partial = c->partial;
-  a.out_bf16 = out_bf16;
-  a.out_f32 = out_f32;
-  a.ld_out = ld_out;
   a.status = c->status;
-  if (mode == kGemmPartial) {
-    const size_t need = (size_t)p.gridx * p.max_seg * p.NT * 128 * sizeof(float);
-    if (need > c->partial_bytes) return SS_ERR_CAPACITY;
-  }
+  if ((size_t)p.gridx * p.max_seg * p.NT * 128 * sizeof(float) > c->partial_bytes) return SS_ERR_CAPACITY;
   // the weight tensor map is unused with tiled weights; the activation map stands in for it
-  SS_CUDA(c, launch(c, gemm_wx_kernel, dim3(p.gridy, p.gridx), dim3(kGemmThreads), (size_t)p.smem_bytes, mx, mx, a));
+  SS_CUDA(c, launch(c, gemm_wx_kernel, dim3(1, p.gridx), dim3(kGemmThreads), (size_t)p.smem_bytes, mx, mx, a));
   return SS_OK;
 }
 
-// The same product on pairs of CTAs (gemm_wx_pair_kernel): token tiles of 256, direct epilogues only.
-int run_gemm_pair(ss_ctx* c, const CUtensorMap& mw, const CUtensorMap& mx, int n_out, int K, int mode, int n_tok,
-                  void* out_bf16, float* out_f32, int ld_out) {
-  GemmArgs a{};
+// The same product on pairs of CTAs (gemm_wx_pair_kernel): token tiles of 256, finished in the epilogue that `a` asks for.
+int run_gemm_pair(ss_ctx* c, const CUtensorMap& mw, const CUtensorMap& mx, int n_out, int K, GemmArgs a) {
   a.p.n_out = n_out;
   a.p.K = K;
   a.p.n_tiles = 2 * ceil_div(n_out, kTileN);
@@ -333,13 +323,7 @@ int run_gemm_pair(ss_ctx* c, const CUtensorMap& mw, const CUtensorMap& mx, int n
   a.p.NT = kPairTokens;
   a.p.stages = std::min(kGemmMaxStages, (227 * 1024 - 2048) / kPairStageBytes);
   a.p.smem_bytes = 2048 + a.p.stages * kPairStageBytes;
-  a.mode = mode;
-  a.n_tok = n_tok;
-  a.out_bf16 = out_bf16;
-  a.out_f32 = out_f32;
-  a.ld_out = ld_out;
-  a.status = c->status;
-  a.p.gridy = ceil_div(n_tok, kPairTokens);                          // token tiles
+  a.p.gridy = ceil_div(a.n_tok, kPairTokens);                        // token tiles
   const int n_units = (a.p.n_tiles / 2) * a.p.gridy;
   a.p.gridx = std::min(n_units, c->n_sm / 2);                        // pairs of CTAs, each walking its units
   SS_CUDA(c, launch(c, gemm_wx_pair_kernel, dim3(2 * a.p.gridx), dim3(kGemmThreads), (size_t)a.p.smem_bytes, mw, mx, a));
@@ -358,9 +342,9 @@ struct ArenaPlan {
 struct Offsets {
   size_t embed, lm_head, final_norm, staging, staging_bytes, weights_end;
   std::vector<size_t> attn_norm, wqkv, wo, ffn_norm, wgu, wdown;
-  size_t inv_freq, rope, att_part, att_flag, status, rows, block_table, out_tokens, tok, h, x, qkv, qkv_f, attn_o, gu, act;
+  size_t inv_freq, rope, att_part, att_flag, status, rows, block_table, out_tokens, tok, h, x, qkv, attn_o, act;
   size_t h_dec, x_dec, o_dec, act_dec, partial, kv;
-  size_t tbl[5], tbl_lm_prompt, tile_val, tile_idx, rowss, grid_ctr, wptr, norm_ptr, trace;
+  size_t tbl[5], tbl128[5], tile_val, tile_idx, rowss, grid_ctr, wptr, norm_ptr, trace;
   size_t partial_bytes;
   int R, max_pages, n_pages;
   size_t total;
@@ -411,9 +395,7 @@ void layout(const ss_model_cfg& m, const ss_runtime_cfg& rt, int n_sm, Offsets& 
   o.h = a.take((size_t)o.R * d * 4);
   o.x = a.take((size_t)o.R * d * 2);
   o.qkv = a.take((size_t)o.R * 3 * d * 2);
-  o.qkv_f = a.take((size_t)o.R * 3 * d * 4);
   o.attn_o = a.take((size_t)o.R * d * 2);
-  o.gu = a.take((size_t)o.R * 2 * F * 4);
   o.act = a.take((size_t)o.R * F * 2);
   o.h_dec = a.take((size_t)kMaxBatch * d * 4);
   o.x_dec = a.take((size_t)kMaxBatch * d * 2);
@@ -426,9 +408,11 @@ void layout(const ss_model_cfg& m, const ss_runtime_cfg& rt, int n_sm, Offsets& 
   for (auto& s : shapes) {
     const DecodeSplit p = plan_decode(s[0], s[1], n_sm);
     pb = std::max(pb, (size_t)p.gsplit * p.max_seg * NTmax * kTileN * sizeof(float));
+    const GemmPlan q = plan_gemm(s[0], s[1], short_tile(rt.max_prefill_tokens), n_sm);
+    pb = std::max(pb, (size_t)q.gridx * q.max_seg * q.NT * 128 * sizeof(float));
   }
   {
-    const GemmPlan p = plan_gemm((int)V, (int)d, NTmax, 1, kGemmPartial, n_sm);
+    const GemmPlan p = plan_gemm((int)V, (int)d, NTmax, n_sm);
     pb = std::max(pb, (size_t)p.gridx * p.max_seg * p.NT * 128 * sizeof(float));
   }
   o.partial_bytes = pb;
@@ -439,7 +423,7 @@ void layout(const ss_model_cfg& m, const ss_runtime_cfg& rt, int n_sm, Offsets& 
   o.norm_ptr = a.take((size_t)(2 * m.n_layers + 1) * sizeof(void*));
   o.trace = a.take((size_t)(2 + 4 * (4 * m.n_layers + 1)) * 8);
   for (int i = 0; i < 5; ++i) o.tbl[i] = a.take((size_t)ceil_div(shapes[i][0], kTileN) * sizeof(TileSeg));
-  o.tbl_lm_prompt = a.take((size_t)ceil_div((int)V, kTileM) * sizeof(TileSeg));
+  for (int i = 0; i < 5; ++i) o.tbl128[i] = a.take((size_t)ceil_div(shapes[i][0], kTileM) * sizeof(TileSeg));
   o.tile_val = a.take((size_t)kMaxBatch * ceil_div((int)V, kTileM) * 4);
   o.tile_idx = a.take((size_t)kMaxBatch * ceil_div((int)V, kTileM) * 4);
   o.n_pages = (int)((rt.kv_pool_tokens + kPageTokens - 1) / kPageTokens) + rt.max_batch;
@@ -465,12 +449,17 @@ struct WeightSlot {
   int slot;
   bool tiled;
   int row_off;        // tiled: row offset inside the stacked matrix
+  int half, step;     // tiled: placement of the rows (repack_weights_kernel)
 };
 
 int weight_slot(const ss_ctx* c, const std::string& name, WeightSlot* out) {
   const int64_t d = c->m.d_model, F = c->m.d_ffn, V = c->m.vocab;
-  auto plain = [&](void* p, int64_t r, int64_t cc, int s) { *out = {p, r, cc, s, false, 0}; return SS_OK; };
-  auto tiled = [&](void* p, int64_t r, int64_t cc, int s, int64_t off) { *out = {p, r, cc, s, true, (int)off}; return SS_OK; };
+  auto plain = [&](void* p, int64_t r, int64_t cc, int s) { *out = {p, r, cc, s, false, 0, 0, 1}; return SS_OK; };
+  auto tiled = [&](void* p, int64_t r, int64_t cc, int s, int64_t off, int half = 0, int step = 1) {
+    *out = {p, r, cc, s, true, (int)off, half, step};
+    return SS_OK;
+  };
+  const int rot = c->m.head_dim / 2;      // the two dimensions of a rotation become neighbouring rows
   if (name == "embed") return plain(c->embed, V, d, 0);
   if (name == "lm_head") return tiled(c->lm_head, V, d, 1, 0);
   if (name == "final_norm") return plain(c->final_norm, 1, d, 2);
@@ -483,13 +472,13 @@ int weight_slot(const ss_ctx* c, const std::string& name, WeightSlot* out) {
     const LayerWeights& w = c->layers[l];
     const int base = 3 + l * 9;
     if (k == "attn_norm") return plain(w.attn_norm, 1, d, base + 0);
-    if (k == "wq") return tiled(w.wqkv, d, d, base + 1, 0);
-    if (k == "wk") return tiled(w.wqkv, d, d, base + 2, d);
+    if (k == "wq") return tiled(w.wqkv, d, d, base + 1, 0, rot);
+    if (k == "wk") return tiled(w.wqkv, d, d, base + 2, d, rot);
     if (k == "wv") return tiled(w.wqkv, d, d, base + 3, 2 * d);
     if (k == "wo") return tiled(w.wo, d, d, base + 4, 0);
     if (k == "ffn_norm") return plain(w.ffn_norm, 1, d, base + 5);
-    if (k == "w_gate") return tiled(w.wgu, F, d, base + 6, 0);
-    if (k == "w_up") return tiled(w.wgu, F, d, base + 7, F);
+    if (k == "w_gate") return tiled(w.wgu, F, d, base + 6, 0, 0, 2);
+    if (k == "w_up") return tiled(w.wgu, F, d, base + 7, 1, 0, 2);
     if (k == "w_down") return tiled(w.wdown, d, F, base + 8, 0);
   }
   return SS_ERR_ARG;
@@ -601,44 +590,74 @@ int enqueue_prefill_chunk(ss_ctx* c, int s0, int s1, const int32_t* cu, int T) {
   const int nseq = s1 - s0;
   int max_len = 0;
   for (int s = s0; s < s1; ++s) max_len = std::max(max_len, cu[s + 1] - cu[s]);
-  // more than half a pair's token tile: the paired kernel (token tiles of 256, two CTAs per 256 x 256 tile)
-  const bool pair = T > kPairTokens / 2;
-  const int NT = pair ? kPairTokens / 2 : std::min(256, round_up(T, 16));
-  const int tok_tiles = ceil_div(T, NT);
-  const CUtensorMap *mx, *mo, *ma;
+  const CUtensorMap *mx, *mo, *ma, *mq;
   int rc;
+  if ((rc = xmap(c, 6, kAttnTile, &mq))) return rc;
+  // what the q,k,v projection does behind the sum, whichever kernel does it
+  GemmArgs qkv{};
+  qkv.mode = kGemmQkv;
+  qkv.n_tok = T;
+  qkv.out = c->qkv;
+  qkv.d = d; qkv.H = H; qkv.Dh = Dh;
+  qkv.rope = c->rope;
+  qkv.tok_pos = c->d_tok_pos;
+  qkv.tok_slot = c->d_tok_slot;
+  qkv.page_elems = c->kv.page_elems;
+  qkv.status = c->status;
+  GemmArgs res{}, glu{};
+  res.mode = kGemmResidual;
+  res.n_tok = T;
+  res.residual = c->h;
+  res.status = c->status;
+  glu.mode = kGemmSwiglu;
+  glu.n_tok = T;
+  glu.out = c->act;
+  glu.status = c->status;
+  // more than half a pair's token tile: the paired kernel; below, the projections are split over the SMs along K too
+  const bool pair = T > kShortTokens;
+  const int NT = pair ? kPairTokens / 2 : short_tile(T);
   if ((rc = xmap(c, 0, NT, &mx)) || (rc = xmap(c, 1, NT, &mo)) || (rc = xmap(c, 2, NT, &ma))) return rc;
-  const GemmPlan p_qkv = plan_gemm(3 * d, d, NT, tok_tiles, kGemmDirectF32, c->n_sm);
-  const GemmPlan p_o = plan_gemm(d, d, NT, tok_tiles, kGemmDirectF32Add, c->n_sm);
-  const GemmPlan p_gu = plan_gemm(2 * F, d, NT, tok_tiles, kGemmDirectF32, c->n_sm);
-  const GemmPlan p_dn = plan_gemm(d, F, NT, tok_tiles, kGemmDirectF32Add, c->n_sm);
-  // one projection: on pairs of CTAs, or one CTA per tile for short chunks
-  auto project = [&](int l, int type, const uint8_t* w, const CUtensorMap& act, const GemmPlan& pl, int n_out, int K,
-                     int mode, float* out, int ld) -> int {
-    if (pair) return run_gemm_pair(c, c->wmaps[4 * l + type], act, n_out, K, mode, T, nullptr, out, ld);
-    return run_gemm(c, w, act, pl, mode, T, nullptr, out, ld);
+  const int shp[4][2] = {{3 * d, d}, {d, d}, {2 * F, d}, {d, F}};
+  GemmPlan plan[4];
+  SplitInfo split[4];
+  for (int i = 0; i < 4; ++i) {
+    plan[i] = plan_gemm(shp[i][0], shp[i][1], NT, c->n_sm);
+    split[i] = split_of(plan[i], c->tbl128[i]);
+  }
+  auto attend = [&]() -> int {
+    const dim3 ag(ceil_div(max_len, kAttnTile), H, nseq);
+    if (Dh == 128)
+      SS_CUDA(c, launch(c, attn_prefill_kernel<128>, ag, dim3(128), (size_t)attn_prefill_smem<128>(), *mq, (const int32_t*)c->d_cu, c->attn_o, d, c->status));
+    else
+      SS_CUDA(c, launch(c, attn_prefill_kernel<64>, ag, dim3(128), (size_t)attn_prefill_smem<64>(), *mq, (const int32_t*)c->d_cu, c->attn_o, d, c->status));
+    return SS_OK;
   };
   const bf16* first_norm = m.n_layers ? c->layers[0].attn_norm : c->final_norm;
-  SS_CUDA(c, launch(c, embed_rmsnorm_kernel, dim3(T), dim3(256), 0, (const int32_t*)c->d_tokens, (const int32_t*)nullptr,
+  SS_CUDA(c, launch(c, embed_rmsnorm_kernel, dim3(T), dim3(256), 0, (const int32_t*)c->d_tokens,
                     (const bf16*)c->embed, first_norm, c->h, c->x, d, m.rms_eps, V));
   for (int l = 0; l < m.n_layers; ++l) {
     const LayerWeights& w = c->layers[l];
-    if ((rc = project(l, 0, w.wqkv, *mx, p_qkv, 3 * d, d, kGemmDirectF32, c->qkv_f, 3 * d))) return rc;
-    SS_CUDA(c, launch(c, rope_append_prefill_kernel, dim3(T), dim3(256), 0, (const float*)c->qkv_f, c->qkv, (const int32_t*)c->d_tok_row,
-                      (const int32_t*)c->d_tok_pos, c->st, c->kv, l, (const float*)c->inv_freq, d, c->status));
-    const dim3 ag(ceil_div(max_len, 64), H, nseq);
-    if (Dh == 128)
-      SS_CUDA(c, launch(c, attn_prefill_kernel<128>, ag, dim3(128), 0, (const bf16*)c->qkv, (const int32_t*)c->d_cu, c->attn_o, d));
-    else
-      SS_CUDA(c, launch(c, attn_prefill_kernel<64>, ag, dim3(128), 0, (const bf16*)c->qkv, (const int32_t*)c->d_cu, c->attn_o, d));
-    if ((rc = project(l, 1, w.wo, *mo, p_o, d, d, kGemmDirectF32Add, c->h, d))) return rc;
-    SS_CUDA(c, launch(c, rmsnorm_kernel, dim3(T), dim3(256), 0, (const float*)c->h, (const bf16*)w.ffn_norm, c->x, d, m.rms_eps));
-    if ((rc = project(l, 2, w.wgu, *mx, p_gu, 2 * F, d, kGemmDirectF32, c->gu, 2 * F))) return rc;
-    SS_CUDA(c, launch(c, swiglu_kernel, dim3(T, ceil_div(F, 2048)), dim3(256), 0, (const float*)c->gu, c->act, F));
-    if ((rc = project(l, 3, w.wdown, *ma, p_dn, d, F, kGemmDirectF32Add, c->h, d))) return rc;
-    if (l + 1 < m.n_layers)
-      SS_CUDA(c, launch(c, rmsnorm_kernel, dim3(T), dim3(256), 0, (const float*)c->h,
-                        (const bf16*)c->layers[l + 1].attn_norm, c->x, d, m.rms_eps));
+    const bf16* next_norm = l + 1 < m.n_layers ? c->layers[l + 1].attn_norm : c->final_norm;
+    qkv.kv_layer = c->kv.pool + (size_t)l * c->kv.layer_stride;
+    if (pair) {
+      if ((rc = run_gemm_pair(c, c->wmaps[4 * l + 0], *mx, 3 * d, d, qkv)) || (rc = attend()) ||
+          (rc = run_gemm_pair(c, c->wmaps[4 * l + 1], *mo, d, d, res))) return rc;
+      SS_CUDA(c, launch(c, rmsnorm_kernel, dim3(T), dim3(256), 0, (const float*)c->h, (const bf16*)w.ffn_norm, c->x, d, m.rms_eps));
+      if ((rc = run_gemm_pair(c, c->wmaps[4 * l + 2], *mx, 2 * F, d, glu)) ||
+          (rc = run_gemm_pair(c, c->wmaps[4 * l + 3], *ma, d, F, res))) return rc;
+      if (l + 1 < m.n_layers)
+        SS_CUDA(c, launch(c, rmsnorm_kernel, dim3(T), dim3(256), 0, (const float*)c->h, next_norm, c->x, d, m.rms_eps));
+    } else {
+      const float* part = c->partial;
+      if ((rc = run_gemm(c, w.wqkv, *mx, plan[0], T))) return rc;
+      SS_CUDA(c, launch(c, short_qkv_kernel, dim3(T, ceil_div(3 * d, 1024)), dim3(256), 0, part, split[0], qkv));
+      if ((rc = attend()) || (rc = run_gemm(c, w.wo, *mo, plan[1], T))) return rc;
+      SS_CUDA(c, launch(c, short_residual_kernel, dim3(T), dim3(256), 0, part, split[1], c->h, (const bf16*)w.ffn_norm, c->x, d, m.rms_eps));
+      if ((rc = run_gemm(c, w.wgu, *mx, plan[2], T))) return rc;
+      SS_CUDA(c, launch(c, short_swiglu_kernel, dim3(T, ceil_div(2 * F, 1024)), dim3(256), 0, part, split[2], c->act, F));
+      if ((rc = run_gemm(c, w.wdown, *ma, plan[3], T))) return rc;
+      SS_CUDA(c, launch(c, short_residual_kernel, dim3(T), dim3(256), 0, part, split[3], c->h, next_norm, c->x, d, m.rms_eps));
+    }
   }
   return SS_OK;
 }
@@ -776,8 +795,6 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
   c->x = (bf16*)(A + o.x);
   c->qkv = (bf16*)(A + o.qkv);
   c->attn_o = (bf16*)(A + o.attn_o);
-  c->gu = (float*)(A + o.gu);
-  c->qkv_f = (float*)(A + o.qkv_f);
   c->act = (bf16*)(A + o.act);
   c->h_dec = (float*)(A + o.h_dec);
   c->x_dec = (bf16*)(A + o.x_dec);
@@ -825,10 +842,12 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
       if (cudaMemcpy(c->tbl[i], t.data(), t.size() * sizeof(TileSeg), cudaMemcpyHostToDevice) != cudaSuccess)
         return fail(SS_ERR_CUDA);
     }
-    c->tbl_lm_prompt = (TileSeg*)(A + o.tbl_lm_prompt);
-    const std::vector<TileSeg> t = tile_table(plan_gemm((int)V, (int)d, 16, 1, kGemmPartial, c->n_sm));
-    if (cudaMemcpy(c->tbl_lm_prompt, t.data(), t.size() * sizeof(TileSeg), cudaMemcpyHostToDevice) != cudaSuccess)
-      return fail(SS_ERR_CUDA);
+    for (int i = 0; i < 5; ++i) {
+      c->tbl128[i] = (TileSeg*)(A + o.tbl128[i]);
+      const std::vector<TileSeg> t = tile_table(plan_gemm(shp[i][0], shp[i][1], 16, c->n_sm));
+      if (cudaMemcpy(c->tbl128[i], t.data(), t.size() * sizeof(TileSeg), cudaMemcpyHostToDevice) != cudaSuccess)
+        return fail(SS_ERR_CUDA);
+    }
   }
   c->kv.pool = (bf16*)(A + o.kv);
   c->kv.page_elems = (size_t)2 * model->n_heads * kPageTokens * model->head_dim;
@@ -869,6 +888,10 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
     e = cudaFuncSetAttribute(gemm_wx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(gemm_wx_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(attn_prefill_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_prefill_smem<128>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(attn_prefill_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_prefill_smem<64>());
   for (int v = 0; v < 8 && e == cudaSuccess; ++v)
     e = cudaFuncSetAttribute(mega_kernel_fn((v & 1) ? 128 : 64, (v & 2) != 0, (v & 4) != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
                              227 * 1024);
@@ -912,7 +935,7 @@ int ss_load_weights(ss_ctx* c, const ss_tensor_desc* t, int32_t n) {
       }
       const long long chunks = (long long)ws.rows * (ws.cols / 8);
       repack_weights_kernel<<<(unsigned)((chunks + 255) / 256), 256, 0, c->stream>>>(
-          (const uint4*)src, ws.rows, (int)ws.cols, (uint8_t*)ws.dst, ws.row_off, ceil_div((int)ws.cols, kTileK));
+          (const uint4*)src, ws.rows, (int)ws.cols, (uint8_t*)ws.dst, ws.row_off, ceil_div((int)ws.cols, kTileK), ws.half, ws.step);
       SS_CUDA(c, cudaGetLastError());
       c->launches++;
       // the staging buffer (or the caller's tensor) is free again once the repack has run
@@ -1004,18 +1027,21 @@ int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, c
     SS_CUDA_B(staging_free(c, 1));
     const int n_seq = s1 - s0;
     int32_t* tok = (int32_t*)(c->up + c->up_chunk);
-    int32_t *tok_row = tok + T, *tok_pos = tok + 2 * (size_t)T, *cu_loc = tok + 3 * (size_t)T, *last = cu_loc + n_seq + 1;
+    int32_t *tok_slot = tok + T, *tok_pos = tok + 2 * (size_t)T, *cu_loc = tok + 3 * (size_t)T, *last = cu_loc + n_seq + 1;
     std::copy(tokens + cu[s0], tokens + cu[s1], tok);
     for (int s = s0, t = 0; s < s1; ++s) {
       cu_loc[s - s0] = t;
-      for (int p = 0; p < cu[s + 1] - cu[s]; ++p, ++t) { tok_row[t] = s; tok_pos[t] = p; }
+      for (int p = 0; p < cu[s + 1] - cu[s]; ++p, ++t) {
+        tok_slot[t] = c->row_pages[s][p / kPageTokens] * kPageTokens + p % kPageTokens;
+        tok_pos[t] = p;
+      }
       cu_loc[s - s0 + 1] = t;
       last[s - s0] = t - 1;
     }
     SS_CUDA_B(cudaMemcpyAsync(c->d_chunk, tok, (3 * (size_t)T + 2 * n_seq + 1) * 4, cudaMemcpyHostToDevice, c->stream));
     SS_CUDA_B(cudaEventRecord(c->up_ev[1], c->stream));
     c->d_tokens = c->d_chunk;
-    c->d_tok_row = c->d_chunk + T;
+    c->d_tok_slot = c->d_chunk + T;
     c->d_tok_pos = c->d_chunk + 2 * (size_t)T;
     c->d_cu = c->d_chunk + 3 * (size_t)T;
     c->d_last = c->d_cu + n_seq + 1;
@@ -1031,10 +1057,10 @@ int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, c
   const int NT = round_up(B, 16);
   const CUtensorMap* mx;
   if ((rc = xmap(c, 3, NT, &mx))) return bail(rc);
-  const GemmPlan p_lm = plan_gemm(m.vocab, m.d_model, NT, 1, kGemmPartial, c->n_sm);
-  if ((rc = run_gemm(c, c->lm_head, *mx, p_lm, kGemmPartial, B, nullptr, nullptr, 0))) return bail(rc);
-  SS_CUDA_B(launch(c, lmhead_tile_argmax_kernel, dim3(c->n_tiles_lm), dim3(128), 0, (const float*)c->partial,
-                   split_of(p_lm, c->tbl_lm_prompt), c->st, opts ? opts->dump_logits : (float*)nullptr, c->tile_val,
+  const GemmPlan p_lm = plan_gemm(m.vocab, m.d_model, NT, c->n_sm);
+  if ((rc = run_gemm(c, c->lm_head, *mx, p_lm, B))) return bail(rc);
+  SS_CUDA_B(launch(c, lmhead_tile_argmax_kernel, dim3(c->n_tiles_lm, ceil_div(B, kArgmaxRows)), dim3(128), 0, (const float*)c->partial,
+                   split_of(p_lm, c->tbl128[4]), c->st, opts ? opts->dump_logits : (float*)nullptr, c->tile_val,
                    c->tile_idx, B, m.vocab, c->n_tiles_lm, m.eos_id, c->sample));
   SS_CUDA_B(launch(c, bookkeeping_kernel, dim3(1), dim3(1024), 0, c->st, (const float*)c->tile_val,
                    (const int32_t*)c->tile_idx, c->n_tiles_lm, opts ? opts->forced_tokens : (const int32_t*)nullptr,
