@@ -40,20 +40,30 @@ std::mutex g_mu;
 DeviceSetup g_dev[kMaxDevices];
 EncodeTiledFn g_encode = nullptr;
 
-// x[r] = RMSNorm(h[r]) * g as bf16; rows r >= n_rows of the 16-row operand are zeroed.
+// x[r] = RMSNorm(h[r]) * g as bf16; rows r >= n_rows of the 16-row operand are zeroed; the status word starts at zero.
+// One pass: 256 threads hold the row (d a multiple of 64, at most 8192) as 8 x 4 values each.  `vec`: h is 16-byte and g
+// 8-byte aligned (the caller's pointers need not be).
 __global__ void __launch_bounds__(256)
 noalloc_rmsnorm_kernel(const float* __restrict__ h, const __nv_bfloat16* __restrict__ g, __nv_bfloat16* __restrict__ x,
-                       int n_rows, int d, float eps) {
+                       int n_rows, int d, float eps, int vec, uint32_t* status) {
   __shared__ float red[8];
-  const int r = blockIdx.x;
+  pdl_launch_dependents();
+  const int r = blockIdx.x, d4 = d >> 2;
+  if (r == 0 && threadIdx.x == 0) *status = 0u;
+  uint2* out = reinterpret_cast<uint2*>(x + (size_t)r * d);
   if (r >= n_rows) {
-    for (int i = threadIdx.x; i < d; i += blockDim.x) x[(size_t)r * d + i] = __float2bfloat16_rn(0.f);
+    for (int i = threadIdx.x; i < d4; i += 256) out[i] = make_uint2(0u, 0u);
     return;
   }
+  const float* hr = h + (size_t)r * d;
+  float4 v[8];
   float ss = 0.f;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) {
-    const float v = h[(size_t)r * d + i];
-    ss += v * v;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int i = threadIdx.x + k * 256;
+    v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i < d4) v[k] = vec ? __ldg(reinterpret_cast<const float4*>(hr) + i) : make_float4(hr[4 * i], hr[4 * i + 1], hr[4 * i + 2], hr[4 * i + 3]);
+    ss += v[k].x * v[k].x + v[k].y * v[k].y + v[k].z * v[k].z + v[k].w * v[k].w;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
@@ -63,20 +73,75 @@ noalloc_rmsnorm_kernel(const float* __restrict__ h, const __nv_bfloat16* __restr
 #pragma unroll
   for (int w = 0; w < 8; ++w) tot += red[w];
   const float inv = rsqrtf(tot / d + eps);
-  for (int i = threadIdx.x; i < d; i += blockDim.x)
-    x[(size_t)r * d + i] = __float2bfloat16_rn(h[(size_t)r * d + i] * inv * __bfloat162float(g[i]));
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int i = threadIdx.x + k * 256;
+    if (i < d4) {
+      __nv_bfloat162 g01, g23;
+      if (vec) {
+        const uint2 gb = __ldg(reinterpret_cast<const uint2*>(g) + i);
+        g01 = *reinterpret_cast<const __nv_bfloat162*>(&gb.x);
+        g23 = *reinterpret_cast<const __nv_bfloat162*>(&gb.y);
+      } else {
+        g01 = __nv_bfloat162(g[4 * i], g[4 * i + 1]);
+        g23 = __nv_bfloat162(g[4 * i + 2], g[4 * i + 3]);
+      }
+      const float2 a = __bfloat1622float2(g01), b = __bfloat1622float2(g23);
+      out[i] = make_uint2(pack_bf16x2(v[k].x * inv * a.x, v[k].y * inv * a.y), pack_bf16x2(v[k].z * inv * b.x, v[k].w * inv * b.y));
+    }
+  }
 }
 
 // logits[r][v] = sum of the partials of output row v for token r, in CTA order.  If a bounded wait of the
 // projection gave up (status word non-zero) the partials are not all there: the whole output becomes NaN,
 // which is how this call, having already returned, reports the failure.
-__global__ void __launch_bounds__(256)
-noalloc_reduce_kernel(const float* __restrict__ partial, SplitInfo sp, float* __restrict__ logits, int V,
+// grid (128-row tiles, rows / kReduceRows), block 128 (thread = vocabulary row of the tile).  The tile's segments follow from
+// the split arithmetic, 32-bit here: (CTAs + 1) x (tiles x k-blocks) is far below 2^31 for every size the array holds.
+constexpr int kReduceRows = 4;
+__global__ void __launch_bounds__(128)
+noalloc_reduce_kernel(const float* __restrict__ partial, SplitInfo sp, float* __restrict__ logits, int V, int n_rows,
                       const uint32_t* __restrict__ status) {
-  const int r = blockIdx.y, v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= V) return;
+  const int tile = blockIdx.x, v = tile * 128 + threadIdx.x, total = (int)sp.total;
+  auto begin = [&](int c) { return c * total / sp.gridx; };
+  auto owner = [&](int x) {
+    int c = (int)((unsigned int)x * (unsigned int)sp.gridx / (unsigned int)total);
+    while (c + 1 < sp.gridx && begin(c + 1) <= x) ++c;
+    return c;
+  };
+  const int c0 = owner(tile * sp.kb), c1 = owner(tile * sp.kb + sp.kb - 1);
+  const int slot0 = c0 * sp.max_seg + tile - begin(c0) / sp.kb;
+  const size_t slot_stride = (size_t)sp.NT * 128, cta_stride = slot_stride * sp.max_seg;
+  pdl_wait();
   const bool failed = *status != 0u;
-  logits[(size_t)r * V + v] = failed ? __int_as_float(0x7fc00000) : sum_partials_derived(partial, sp, v, r);
+  const int r0 = blockIdx.y * kReduceRows;
+  float acc[kReduceRows];
+#pragma unroll
+  for (int j = 0; j < kReduceRows; ++j)
+    acc[j] = r0 + j < n_rows ? __ldcg(partial + (size_t)slot0 * slot_stride + (size_t)(r0 + j) * 128 + threadIdx.x) : 0.f;
+  for (int c = c0 + 1; c <= c1; ++c)
+#pragma unroll
+    for (int j = 0; j < kReduceRows; ++j)
+      if (r0 + j < n_rows) acc[j] += __ldcg(partial + (size_t)c * cta_stride + (size_t)(r0 + j) * 128 + threadIdx.x);
+  if (v >= V) return;
+#pragma unroll
+  for (int j = 0; j < kReduceRows; ++j)
+    if (r0 + j < n_rows) logits[(size_t)(r0 + j) * V + v] = failed ? __int_as_float(0x7fc00000) : acc[j];
+}
+
+// A launch that may start before the kernel in front of it has finished; it waits for it itself (griddepcontrol.wait).
+template <class... KArgs, class... Args>
+cudaError_t launch_early(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
 }
 
 int setup_device(int dev, DeviceSetup** out) {
@@ -159,19 +224,20 @@ extern "C" int ss_logits_noalloc(const float* hidden, const void* norm_gain, con
   CUtensorMap mw, mx;
   if (encode_map(&mw, lm_head, vocab, d_model, kTileM) || encode_map(&mx, x, kNoAllocMaxRows, d_model, p.NT))
     return SS_ERR_CUDA;
-  // the status word must start at zero; x and the partials are rewritten below
-  if (cudaMemsetAsync(status, 0, 256, st) != cudaSuccess) return SS_ERR_CUDA;
-  noalloc_rmsnorm_kernel<<<kNoAllocMaxRows, 256, 0, st>>>(hidden, (const __nv_bfloat16*)norm_gain, x, n_rows, d_model,
-                                                          rms_eps);
+  // The first kernel starts when the stream's earlier work has finished; the projection may start beside it and fetch its
+  // first weights (which are older than the first kernel), the summing kernel beside the projection.
+  const int vec = ((uintptr_t)hidden & 15) == 0 && ((uintptr_t)norm_gain & 7) == 0;
+  noalloc_rmsnorm_kernel<<<kNoAllocMaxRows, 256, 0, st>>>(hidden, (const __nv_bfloat16*)norm_gain, x, n_rows, d_model, rms_eps, vec, status);
   GemmArgs a{};
   a.p = p;
   a.mode = kGemmPartial;
   a.n_tok = n_rows;
   a.partial = partial;
   a.status = status;
-  gemm_wx_kernel<<<dim3(1, p.gridx), kGemmThreads, p.smem_bytes, st>>>(mw, mx, a);
+  if (launch_early(gemm_wx_kernel, dim3(1, p.gridx), dim3(kGemmThreads), (size_t)p.smem_bytes, st, mw, mx, a) != cudaSuccess) return SS_ERR_CUDA;
   SplitInfo sp;
   sp.gridx = p.gridx; sp.kb = p.kb; sp.max_seg = p.max_seg; sp.NT = p.NT; sp.total = total; sp.tiles = nullptr;
-  noalloc_reduce_kernel<<<dim3((vocab + 255) / 256, n_rows), 256, 0, st>>>(partial, sp, logits, vocab, status);
+  if (launch_early(noalloc_reduce_kernel, dim3(p.n_tiles, (n_rows + kReduceRows - 1) / kReduceRows), dim3(128), 0, st, (const float*)partial, sp, logits,
+                   vocab, n_rows, (const uint32_t*)status) != cudaSuccess) return SS_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? SS_OK : SS_ERR_CUDA;
 }

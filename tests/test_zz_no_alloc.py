@@ -63,3 +63,25 @@ def test_noalloc_rejects_sizes_beyond_its_array():
     with pytest.raises(api.SSError) as e:
         api.ss_logits_noalloc(h, gain, head, 1e-6, out)              # 17 rows > 16
     assert e.value.code == api.SS_ERR_CAPACITY
+
+
+@pytest.mark.parametrize("rows,d,vocab,offset", [(1, 64, 130, 0), (5, 192, 1000, 1), (16, 4096, 4097, 0), (3, 8192, 129, 3)])
+def test_noalloc_sizes_and_alignments(rows, d, vocab, offset):
+    """Rows that do not fill the summing kernel's groups, vocabularies that end inside a tile, inputs that begin `offset`
+    elements behind a 16-byte boundary, against fp64.  The normalised input is rounded once (2^-9 at most, relative), so
+    the result is off by no more than that in the 2-norm but for the fp32 sums: 3e-3."""
+    import torch
+    from paper_2305_13144_b200 import api
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(rows + d)
+    h = torch.empty(rows * d + offset, device="cuda").normal_(0.0, 2.0, generator=gen)[offset:].view(rows, d)
+    gain = torch.empty(d + offset, device="cuda").uniform_(0.5, 1.5, generator=gen).to(torch.bfloat16)[offset:]
+    head = torch.empty(vocab, d, device="cuda").normal_(0.0, 0.02, generator=gen).to(torch.bfloat16)
+    out = torch.full((rows, vocab), float("nan"), device="cuda")
+    torch.cuda.synchronize()
+    for _ in range(2):
+        api.ss_logits_noalloc(h, gain, head, 1e-6, out)
+    torch.cuda.synchronize()
+    x = h.double() * torch.rsqrt(h.double().square().mean(1, keepdim=True) + 1e-6) * gain.double()
+    ref = x @ head.double().T
+    assert float((out.double() - ref).norm() / ref.norm()) <= 3e-3
