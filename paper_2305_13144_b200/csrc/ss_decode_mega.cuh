@@ -1014,64 +1014,72 @@ __device__ void stage_swiglu(const MegaArgs& a, const MegaSmem* sm, int wtid) {
 }
 
 // ---- stage: per-tile arg-max of the logits --------------------------------------------------------------
-// Work unit = (256-row vocabulary tile, two batch rows) per warp, 2 x 4 consecutive ids per lane: the decision among a
-// lane's ids needs no exchange, so a (tile, row) costs one warp reduction, and the units of many rows spread over
-// every warp of the chip.  Before, a tile's 128 ids sat on 128 threads that walked through all rows one after the other,
-// a reduction each, on half of the CTAs (16 / 45 sampled / 200 rows: 17.8 / 54.5 / 108 -> 11.3 / 40.0 / 47.7 us).
+// A warp has one 256-row vocabulary tile (so its table entry is looked up once) and takes batch rows two at a time, in
+// turn with the other warps of the tile; 2 x 4 consecutive ids per lane: the decision among a lane's ids needs no
+// exchange, so a (tile, row) costs one warp reduction, and many rows spread over every warp of the chip.  At first a
+// tile's 128 ids sat on 128 threads that walked through all rows one after the other, a reduction each, on half of the
+// CTAs (16 / 96 / 200 rows: 17.8 / 56.8 / 108 us); units of (tile, two rows) with a look-up each: 8.8 / 25.1 / 43.7;
+// now 4.7 / 11.9 / 24.8.
 __device__ void stage_tile_argmax(const MegaArgs& a, const MegaSmem* sm, int wtid) {
   const MegaGemmShape& gs = a.shape[4];
   const int lane = wtid & 31, wid = wtid >> 5;
-  const int n_units = gs.n_tiles * ((a.B + 1) >> 1);
-  for (int u = wid * gridDim.x + blockIdx.x; u < n_units; u += 8 * gridDim.x) {
-    const int rg = u / gs.n_tiles, tile = u - rg * gs.n_tiles;
+  const int n_warps = 8 * gridDim.x, n_pairs = (a.B + 1) >> 1;
+  const int n_groups = max(1, min(n_pairs, n_warps / gs.n_tiles));       // warps that share a tile
+  const bool sampled = a.sample.inv_temp != 0.f;
+  for (int u = wid * gridDim.x + blockIdx.x; u < gs.n_tiles * n_groups; u += n_warps) {
+    const int group = u / gs.n_tiles, tile = u - group * gs.n_tiles;
     const int v0 = tile * kTileN + lane * 4;              // and 128 further: a warp-wide load covers 512 contiguous bytes
-    // everything the two rows need is asked for before the first use
-    float ss[2];
-    int gen[2], row_key[2], skip[2];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int r = min(2 * rg + k, a.B - 1);
-      ss[k] = row_ss_issue(a, r, lane);
-      gen[k] = a.st.gen[r] + 1;
-      row_key[k] = a.st.row_key[r];
-      skip[k] = a.st.eos_at[r] > 0 ? a.eos_id : -1;
-    }
     const int4 ts = tile_seg(sm, gs, v0);
-    PartialLoads<4, 2> q[2][2];
+    for (int rg = group; rg < n_pairs; rg += n_groups) {
+      // everything the two rows need is asked for before the first use
+      float ss[2];
+      int gen[2], row_key[2], skip[2];
+      PartialLoads<4, 2> q[2][2];
 #pragma unroll
-    for (int k = 0; k < 2; ++k)
+      for (int k = 0; k < 2; ++k) {
+        const int r = min(2 * rg + k, a.B - 1);
+        ss[k] = row_ss_issue(a, r, lane);
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-        partials_issue<4, 2>(a.partial, gs, a.NT, ts, v0 + 128 * h, min(2 * rg + k, a.B - 1), q[k][h]);
+        for (int h = 0; h < 2; ++h) partials_issue<4, 2>(a.partial, gs, a.NT, ts, v0 + 128 * h, r, q[k][h]);
+        gen[k] = a.st.gen[r] + 1;
+        row_key[k] = a.st.row_key[r];
+        skip[k] = a.st.eos_at[r] > 0 ? a.eos_id : -1;
+      }
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int r = 2 * rg + k;
-      if (r >= a.B || !sm->active_s[r]) continue;         // warp-uniform
-      const float inv = row_ss_inv_rms(a, ss[k]);
-      uint32_t bk = 0;                                    // below every real key
-      int bi = 0x7fffffff;
+      for (int k = 0; k < 2; ++k) {
+        const int r = 2 * rg + k;
+        if (r >= a.B || !sm->active_s[r]) continue;       // warp-uniform
+        const float inv = row_ss_inv_rms(a, ss[k]);
+        uint32_t bk = 0;                                  // below every real key
+        int bi = 0x7fffffff;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        float lg[4];
-        partials_sum<4, 2>(a.partial, gs, a.NT, ts, v0 + 128 * h, r, q[k][h], lg);
+        for (int h = 0; h < 2; ++h) {
+          float lg[4];
+          partials_sum<4, 2>(a.partial, gs, a.NT, ts, v0 + 128 * h, r, q[k][h], lg);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          lg[j] *= inv;
-          const int v = v0 + 128 * h + j;
-          if (v < a.V) {
-            if (a.dump_logits) a.dump_logits[(size_t)r * a.V + v] = lg[j];
-            if (v != skip[k]) {
-              const uint32_t key = float_order_key(decision_value(lg[j], a.sample, v, gen[k], row_key[k]));
-              if (key > bk) { bk = key; bi = v; }         // ids ascend: '>' keeps the lowest
-            }
+          for (int j = 0; j < 4; ++j) lg[j] *= inv;
+          if (a.dump_logits) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (v0 + 128 * h + j < a.V) a.dump_logits[(size_t)r * a.V + v0 + 128 * h + j] = lg[j];
+          }
+          if (sampled) {                                  // four draws side by side: each is a chain of ten rounds
+#pragma unroll
+            for (int j = 0; j < 4; ++j) lg[j] = sampled_value(lg[j], a.sample, v0 + 128 * h + j, gen[k], row_key[k]);
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int v = v0 + 128 * h + j;
+            const uint32_t key = v < a.V && v != skip[k] ? float_order_key(lg[j]) : 0u;
+            if (key > bk) { bk = key; bi = v; }           // ids ascend: '>' keeps the lowest
           }
         }
-      }
-      const uint32_t best = __reduce_max_sync(0xffffffffu, bk);
-      bi = (int)__reduce_min_sync(0xffffffffu, bk == best ? (unsigned int)bi : 0x7fffffffu);
-      if (lane == 0) {
-        a.tile_val[(size_t)r * a.n_tiles_lm + tile] = __uint_as_float(best);
-        a.tile_idx[(size_t)r * a.n_tiles_lm + tile] = bi;
+        const uint32_t best = __reduce_max_sync(0xffffffffu, bk);
+        bi = (int)__reduce_min_sync(0xffffffffu, bk == best ? (unsigned int)bi : 0x7fffffffu);
+        if (lane == 0) {
+          a.tile_val[(size_t)r * a.n_tiles_lm + tile] = __uint_as_float(best);
+          a.tile_idx[(size_t)r * a.n_tiles_lm + tile] = bi;
+        }
       }
     }
   }

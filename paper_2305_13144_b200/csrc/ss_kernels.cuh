@@ -188,12 +188,14 @@ __device__ __forceinline__ uint32_t philox4x32_10_word0(uint32_t c0, uint32_t c1
   }
   return c0;
 }
-// The value whose arg-max decides the token: the logit itself (greedy) or logit / T + Gumbel noise.
-__device__ __forceinline__ float decision_value(float logit, const SampleCfg& sc, int v, int gen_index, int row_key) {
-  if (sc.inv_temp == 0.f) return logit;
+// The value whose arg-max decides the token: logit / T + Gumbel noise, or the logit itself (greedy).
+__device__ __forceinline__ float sampled_value(float logit, const SampleCfg& sc, int v, int gen_index, int row_key) {
   const uint32_t w = philox4x32_10_word0((uint32_t)v, (uint32_t)gen_index, (uint32_t)row_key, 0u, sc.seed_lo, sc.seed_hi);
   const float u = ((float)(w >> 9) + 0.5f) * (1.0f / 8388608.0f);      // 24 significant bits, never 0 or 1
   return fmaf(logit, sc.inv_temp, -logf(-logf(u)));
+}
+__device__ __forceinline__ float decision_value(float logit, const SampleCfg& sc, int v, int gen_index, int row_key) {
+  return sc.inv_temp == 0.f ? logit : sampled_value(logit, sc, v, gen_index, row_key);
 }
 
 constexpr int kArgmaxRows = 8;             // one after the other in a block: 100 rows by one block each took 92 us
@@ -343,8 +345,8 @@ gather_last_rmsnorm_kernel(const float* __restrict__ h, const int32_t* __restric
 constexpr int kShortTokens = 128;
 
 // Partials of outputs n0 .. n0 + 3 (inside one 128-row tile) for token tok, added in CTA order.
-__device__ __forceinline__ float4 sum_partials4(const float* __restrict__ partial, const SplitInfo& s, int n0, int tok) {
-  const int4 t = __ldg(reinterpret_cast<const int4*>(s.tiles) + (n0 >> 7));
+// t: the tile's table entry.
+__device__ __forceinline__ float4 sum_partials4(const float* __restrict__ partial, const SplitInfo& s, const int4 t, int n0, int tok) {
   const size_t slot_stride = (size_t)s.NT * 128, cta_stride = slot_stride * s.max_seg;
   const size_t off = (size_t)tok * 128 + (n0 & 127);
   float4 x = __ldcg(reinterpret_cast<const float4*>(partial + (size_t)t.x * slot_stride + off));
@@ -363,11 +365,12 @@ __device__ __forceinline__ float4 sum_partials4(const float* __restrict__ partia
 __global__ void __launch_bounds__(256)
 short_qkv_kernel(const float* __restrict__ partial, SplitInfo sp, GemmArgs a) {
   pdl_launch_dependents();
-  pdl_wait();
   const int t = blockIdx.x, n = (blockIdx.y * 256 + threadIdx.x) * 4;
   if (n >= 3 * a.d) return;
   const int sec = n / a.d, in = n - sec * a.d, hd = in / a.Dh, e = in - hd * a.Dh;
-  float4 x = sum_partials4(partial, sp, n, t);
+  const int4 seg = __ldg(reinterpret_cast<const int4*>(sp.tiles) + (n >> 7));
+  pdl_wait();
+  float4 x = sum_partials4(partial, sp, seg, n, t);
   if (sec < 2) {
     const float2* rope = a.rope + (size_t)a.tok_pos[t] * (a.Dh >> 1) + (e >> 1);
     const float2 c0 = __ldg(rope), c1 = __ldg(rope + 1);
@@ -382,37 +385,58 @@ short_qkv_kernel(const float* __restrict__ partial, SplitInfo sp, GemmArgs a) {
   }
 }
 
-// h[t] += projection; x[t] = RMSNorm(h[t]) * g.  grid (T), block 256
-__global__ void __launch_bounds__(256)
+// h[t] += projection; x[t] = RMSNorm(h[t]) * g.  grid (T), block 1024: few blocks, so every thread has only one or two
+// groups of four outputs, and what does not depend on the projection is read before the wait for it.
+__global__ void __launch_bounds__(1024)
 short_residual_kernel(const float* __restrict__ partial, SplitInfo sp, float* __restrict__ h, const bf16* __restrict__ g,
                       bf16* __restrict__ x, int d, float eps) {
   __shared__ float red[32];
   pdl_launch_dependents();
-  pdl_wait();
   const size_t t = blockIdx.x;
   const int d4 = d >> 2;
-  float4 v[kRowVec];
+  uint2 gb[2];
+  int4 seg[2];
 #pragma unroll
-  for (int k = 0; k < kRowVec; ++k) {
-    const int i = threadIdx.x + k * 256;
+  for (int k = 0; k < 2; ++k) {
+    const int i = min((int)threadIdx.x + k * 1024, d4 - 1);
+    gb[k] = __ldg(reinterpret_cast<const uint2*>(g) + i);
+    seg[k] = __ldg(reinterpret_cast<const int4*>(sp.tiles) + (i >> 5));
+  }
+  pdl_wait();
+  float4 v[2];
+  float ss = 0.f;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int i = threadIdx.x + k * 1024;
     if (i < d4) {
-      const float4 p = sum_partials4(partial, sp, i * 4, (int)t), h4 = reinterpret_cast<const float4*>(h + t * d)[i];
+      const float4 h4 = __ldcg(reinterpret_cast<const float4*>(h + t * d) + i), p = sum_partials4(partial, sp, seg[k], i * 4, (int)t);
       v[k] = make_float4(h4.x + p.x, h4.y + p.y, h4.z + p.z, h4.w + p.w);
       reinterpret_cast<float4*>(h + t * d)[i] = v[k];
+      ss += v[k].x * v[k].x + v[k].y * v[k].y + v[k].z * v[k].z + v[k].w * v[k].w;
     }
   }
-  const float inv = rsqrtf(row_sum_squares(v, d4, red) / d + eps);
-  store_normed(v, d4, inv, g, x + t * d);
+  const float inv = rsqrtf(block_sum(ss, red) / d + eps);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int i = threadIdx.x + k * 1024;
+    if (i < d4) {
+      const float2 g0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gb[k].x));
+      const float2 g1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gb[k].y));
+      reinterpret_cast<uint2*>(x + t * d)[i] = make_uint2(pack_bf16x2(v[k].x * inv * g0.x, v[k].y * inv * g0.y),
+                                                          pack_bf16x2(v[k].z * inv * g1.x, v[k].w * inv * g1.y));
+    }
+  }
 }
 
 // grid (T, ceil(2F / 1024)), block 256
 __global__ void __launch_bounds__(256)
 short_swiglu_kernel(const float* __restrict__ partial, SplitInfo sp, bf16* __restrict__ act, int F) {
   pdl_launch_dependents();
-  pdl_wait();
   const int t = blockIdx.x, n = (blockIdx.y * 256 + threadIdx.x) * 4;
   if (n >= 2 * F) return;
-  const float4 x = sum_partials4(partial, sp, n, t);               // gate, up, gate, up
+  const int4 seg = __ldg(reinterpret_cast<const int4*>(sp.tiles) + (n >> 7));
+  pdl_wait();
+  const float4 x = sum_partials4(partial, sp, seg, n, t);               // gate, up, gate, up
   *reinterpret_cast<uint32_t*>(act + (size_t)t * F + (n >> 1)) =
       pack_bf16x2(x.x / (1.f + __expf(-x.x)) * x.y, x.z / (1.f + __expf(-x.z)) * x.w);
 }

@@ -652,11 +652,11 @@ int enqueue_prefill_chunk(ss_ctx* c, int s0, int s1, const int32_t* cu, int T) {
       if ((rc = run_gemm(c, w.wqkv, *mx, plan[0], T))) return rc;
       SS_CUDA(c, launch(c, short_qkv_kernel, dim3(T, ceil_div(3 * d, 1024)), dim3(256), 0, part, split[0], qkv));
       if ((rc = attend()) || (rc = run_gemm(c, w.wo, *mo, plan[1], T))) return rc;
-      SS_CUDA(c, launch(c, short_residual_kernel, dim3(T), dim3(256), 0, part, split[1], c->h, (const bf16*)w.ffn_norm, c->x, d, m.rms_eps));
+      SS_CUDA(c, launch(c, short_residual_kernel, dim3(T), dim3(1024), 0, part, split[1], c->h, (const bf16*)w.ffn_norm, c->x, d, m.rms_eps));
       if ((rc = run_gemm(c, w.wgu, *mx, plan[2], T))) return rc;
       SS_CUDA(c, launch(c, short_swiglu_kernel, dim3(T, ceil_div(2 * F, 1024)), dim3(256), 0, part, split[2], c->act, F));
       if ((rc = run_gemm(c, w.wdown, *ma, plan[3], T))) return rc;
-      SS_CUDA(c, launch(c, short_residual_kernel, dim3(T), dim3(256), 0, part, split[3], c->h, next_norm, c->x, d, m.rms_eps));
+      SS_CUDA(c, launch(c, short_residual_kernel, dim3(T), dim3(1024), 0, part, split[3], c->h, next_norm, c->x, d, m.rms_eps));
     }
   }
   return SS_OK;
