@@ -36,7 +36,7 @@ namespace ss {
 
 constexpr int kMegaThreads = 352;
 constexpr int kMegaWorkers = 256;          // warps 3..10
-constexpr int kMegaMaxStages = 8;          // ring depth bound (shared memory holds 5 at batch 16)
+constexpr int kMegaMaxStages = 8;          // ring depth bound (shared memory holds 4 at batch 16)
 constexpr int kSegTabEntries = 256;        // tile-table entries kept in shared memory (the four per-layer projections)
 constexpr int kRowSlice = 128;             // elements of a row handled by one residual work item (one warp, 4 per lane)
 constexpr int kMaxSlices = 64;             // d_model <= 8192
@@ -375,8 +375,12 @@ __device__ void stage_residual(const MegaArgs& a, const MegaSmem* sm, int wtid, 
 // Scan layout: keys -- lane (g, gl) takes key g of a load step and a quarter (half at Dh 64) of its chunks, ordered so
 // that the eight lanes of a shared-memory phase hit different banks; values -- a lane owns four dimensions of every key
 // (every second key at Dh 64), so the running sum is four registers and needs no exchange at the end.
-constexpr int kAttnCutUnits = 40;          // units of the longest row from which pairs are cut between CTAs
-constexpr int kAttnPairCost = 2;           // what a pair costs beside its units (query, new token), in units
+// Units of the longest row from which pairs are cut between CTAs: a cut costs a flag and a merge behind the scan (about 2.5 us),
+// a pair that is not cut leaves its CTA up to its whole length over the others.  7B shape, 8 layers, cut from 8 / 20 / 40
+// units on: 16 rows of 100-380 tokens 852 / 851 / 844 us a step, 4 rows of 300-600 792 / 792 / 775, one row of 173 tokens
+// 779 / 731 / 731, one of 1500 822 / 822 / 821.
+constexpr int kAttnCutUnits = 40;
+constexpr int kAttnPairCost = 2;           // what a pair costs beside its units, in units (0 / 2 / 4: 200 rows 2502 / 2419 / 2431 us a step)
 
 template <int DH> struct AttnLayout {
   static constexpr int GROUP = DH / 32;           // lanes per key

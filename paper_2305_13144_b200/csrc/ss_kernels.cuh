@@ -341,8 +341,10 @@ gather_last_rmsnorm_kernel(const float* __restrict__ h, const int32_t* __restric
 // ---- short prompts (chunks of at most kShortTokens tokens): every projection is split over all SMs along K as well and
 // leaves fp32 partials [slot][token][128 rows]; these kernels add them (four consecutive outputs per thread) and do what
 // the epilogues of the paired GEMM do.  With a CTA per 128-row tile the o and down projections ran on 32 CTAs of 148 and
-// took 50 us each for 61 tokens (7B shape); the whole prompt pass of 8 layers went from 1.89 to 1.05 ms.
-constexpr int kShortTokens = 128;
+// took 50 us each for 61 tokens (7B shape); the whole prompt pass of 8 layers went from 1.89 to 0.91 ms.  Up to 256 tokens the
+// paired GEMM has one token tile, so 16 to 86 units for 74 pairs: 150 / 200 / 256 tokens, 6 layers, 842 / 888 / 981
+// against 1306 / 1357 / 1406 us (300 tokens paired: 1591).
+constexpr int kShortTokens = 256;
 
 // Partials of outputs n0 .. n0 + 3 (inside one 128-row tile) for token tok, added in CTA order.
 // t: the tile's table entry.

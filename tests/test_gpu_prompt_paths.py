@@ -1,0 +1,30 @@
+"""The prompt pass at the edges of its paths, teacher-forced against the oracle: chunks of up to 256 tokens (projections split
+along K, finished by kernels of their own) and above (pairs of CTAs, finished in the epilogue), and prompts around the
+attention's 128 x 128 tiles.  The decode steps behind it read the cache that each path filled."""
+import numpy as np
+import pytest
+
+from paper_2305_13144_b200 import synth
+from parity_util import HIDDEN_TOL, LOGIT_TOL, teacher_forced
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("heads,head_dim,ffn,lens", [
+    (2, 128, 264, [1]),
+    (2, 128, 264, [16, 1, 15]),                  # 32 tokens: the token tile is full
+    (3, 64, 520, [127, 2]),                      # 129 tokens
+    (2, 128, 256, [128, 127]),
+    (4, 64, 1000, [256]),                        # the longest chunk of the split path, two query tiles
+    (2, 128, 264, [257]),                        # the shortest of the paired path, a query tile with one row
+    (3, 64, 520, [129, 128, 1, 255]),            # 513 tokens: a third token tile with one
+    (1, 128, 8, [300, 385, 64]),
+])
+def test_prompt_lengths_and_paths(heads, head_dim, ffn, lens):
+    shape = synth.ModelShape(n_layers=2, d_model=heads * head_dim, n_heads=heads, head_dim=head_dim, d_ffn=ffn, vocab=300)
+    w = synth.make_weights(shape, seed=31)
+    rng = np.random.default_rng(6)
+    prompts = [rng.integers(3, shape.vocab, size=n).tolist() for n in lens]
+    el, eh, _ = teacher_forced(shape, w, prompts, [3] * len(lens), cap=3, max_ctx=max(lens) + 4, max_prefill=max(256, sum(lens)),
+                               kv_tokens=sum(lens) + 64 * len(lens))
+    assert el <= LOGIT_TOL and eh <= HIDDEN_TOL, (el, eh)
