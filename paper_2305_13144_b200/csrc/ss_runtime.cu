@@ -201,13 +201,13 @@ struct ss_ctx {
   bool in_batch = false;
   std::vector<int32_t> prompt_len;
   int32_t* pinned = nullptr;     // [0] n_active, [1] status
-  // Page-locked staging for what a batch sends and fetches: a copy from or to pageable memory costs the host 5 to 10 us
-  // each, and a batch needed 2 to 7 on its way up and one per row on its way back (200 rows: 2.2 of 19.7 ms per batch of
-  // six steps).  Up: row state and block table as one copy, a chunk's token arrays as another.  Down: row state, tokens.
-  uint8_t *up = nullptr, *down = nullptr;
+  // Staging for what a batch sends and fetches: a copy costs the host 5 to 10 us each, and a batch needed 2 to 7 on its way
+  // up and one per row on its way back (200 rows: 2.2 of 19.7 ms per batch of six steps).  Up: row state and block table
+  // as one copy, a chunk's token arrays as another.  Down: row state, tokens.  Ordinary memory: a copy from it
+  // returns when the source may be changed again, and page-locked memory with events to guard it was no faster.
+  std::vector<uint8_t> up, down;
   size_t up_chunk = 0;           // where the chunk arrays start inside `up`
   size_t table_off = 0;          // where the block table starts behind the row state (device and staging alike)
-  cudaEvent_t up_ev[2] = {nullptr, nullptr};   // last copy out of the row part / the chunk part of `up`
   // ---- sampling (greedy while inv_temp == 0)
   SampleCfg sample{0.f, 0u, 0u};
   std::vector<int32_t> next_row_keys;   // keys of the next batch's rows; empty = 0, 1, 2, ...
@@ -663,26 +663,15 @@ int enqueue_prefill_chunk(ss_ctx* c, int s0, int s1, const int32_t* cu, int T) {
 }
 
 // ------------------------------------------------------------------------------------ staging
-void free_host(ss_ctx* c) {
-  if (c->pinned) cudaFreeHost(c->pinned);
-  for (auto& ev : c->up_ev)
-    if (ev) cudaEventDestroy(ev);
-}
-
-// A part of the staging area, free to be filled: an earlier copy out of it has run.
-cudaError_t staging_free(ss_ctx* c, int part) { return cudaEventSynchronize(c->up_ev[part]); }
-
 // Sends the row state and the block tables of B rows, filled in at c->up (row arrays first, tables at table_off).
 cudaError_t send_rows(ss_ctx* c, int B) {
-  cudaError_t e = cudaMemcpyAsync(c->st.ctx_len, c->up, c->table_off + (size_t)B * c->st.max_pages * 4, cudaMemcpyHostToDevice,
-                                  c->stream);
-  return e == cudaSuccess ? cudaEventRecord(c->up_ev[0], c->stream) : e;
+  return cudaMemcpyAsync(c->st.ctx_len, c->up.data(), c->table_off + (size_t)B * c->st.max_pages * 4, cudaMemcpyHostToDevice, c->stream);
 }
 
 // Row state and block table of a new batch of B rows in the staging area: everything zero, no pages.
 void clear_rows(ss_ctx* c, int B, int cap, int32_t** rows, int32_t** bt) {
-  *rows = (int32_t*)c->up;
-  *bt = (int32_t*)(c->up + c->table_off);
+  *rows = (int32_t*)c->up.data();
+  *bt = (int32_t*)(c->up.data() + c->table_off);
   std::memset(*rows, 0, kRowStateBytes);
   std::fill(*bt, *bt + (size_t)B * c->st.max_pages, -1);
   (*rows)[7 * kMaxBatch + 0] = cap;
@@ -873,17 +862,10 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
   // activation operands must be finite wherever a TMA box may reach beyond the valid rows
   if (e == cudaSuccess) e = cudaMemsetAsync(A + o.h, 0, o.partial - o.h, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  // one page-locked allocation for all of it: each costs the host 1 to 2 ms, whatever its size
+  if (e == cudaSuccess) e = cudaHostAlloc((void**)&c->pinned, 64, cudaHostAllocDefault);
   c->up_chunk = align_up(c->table_off + (size_t)rt->max_batch * o.max_pages * 4);
-  const size_t down_off = align_up(c->up_chunk + ((size_t)o.R * 3 + 2 * kMaxBatch + 8) * 4);
-  const size_t down_bytes = kRowStateBytes + (size_t)rt->max_batch * rt->max_new_tokens * 4;
-  if (e == cudaSuccess) e = cudaHostAlloc((void**)&c->pinned, kAlign + down_off + down_bytes, cudaHostAllocDefault);
-  if (e == cudaSuccess) {
-    c->up = (uint8_t*)c->pinned + kAlign;
-    c->down = c->up + down_off;
-  }
-  for (auto& ev : c->up_ev)
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+  c->up.resize(c->up_chunk + ((size_t)o.R * 3 + 2 * kMaxBatch + 8) * 4);
+  c->down.resize(kRowStateBytes + (size_t)rt->max_batch * rt->max_new_tokens * 4);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(gemm_wx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess)
@@ -896,7 +878,7 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
     e = cudaFuncSetAttribute(mega_kernel_fn((v & 1) ? 128 : 64, (v & 2) != 0, (v & 4) != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
                              227 * 1024);
   if (e != cudaSuccess) {
-    free_host(c);
+    if (c->pinned) cudaFreeHost(c->pinned);
     delete c;
     return SS_ERR_CUDA;
   }
@@ -907,7 +889,7 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
 int ss_destroy(ss_ctx* c) {
   if (!c) return SS_ERR_ARG;
   cudaStreamSynchronize(c->stream);
-  free_host(c);
+  if (c->pinned) cudaFreeHost(c->pinned);
   delete c;
   return SS_OK;
 }
@@ -979,7 +961,6 @@ int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, c
     if (tokens[i] < 0 || tokens[i] >= m.vocab) return SS_ERR_ARG;
 
   // host-side batch state
-  SS_CUDA(c, staging_free(c, 0));
   int32_t *rows, *bt;
   clear_rows(c, B, cap, &rows, &bt);
   c->batch_pages.clear();
@@ -1023,10 +1004,9 @@ int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, c
   while (s0 < B) {
     int s1 = s0, T = 0;
     while (s1 < B && T + (cu[s1 + 1] - cu[s1]) <= c->rt.max_prefill_tokens) { T += cu[s1 + 1] - cu[s1]; ++s1; }
-    // the chunk's arrays, packed into one copy; the host runs ahead of the GPU by at most one chunk
-    SS_CUDA_B(staging_free(c, 1));
+    // the chunk's arrays, packed into one copy
     const int n_seq = s1 - s0;
-    int32_t* tok = (int32_t*)(c->up + c->up_chunk);
+    int32_t* tok = (int32_t*)(c->up.data() + c->up_chunk);
     int32_t *tok_slot = tok + T, *tok_pos = tok + 2 * (size_t)T, *cu_loc = tok + 3 * (size_t)T, *last = cu_loc + n_seq + 1;
     std::copy(tokens + cu[s0], tokens + cu[s1], tok);
     for (int s = s0, t = 0; s < s1; ++s) {
@@ -1039,7 +1019,6 @@ int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, c
       last[s - s0] = t - 1;
     }
     SS_CUDA_B(cudaMemcpyAsync(c->d_chunk, tok, (3 * (size_t)T + 2 * n_seq + 1) * 4, cudaMemcpyHostToDevice, c->stream));
-    SS_CUDA_B(cudaEventRecord(c->up_ev[1], c->stream));
     c->d_tokens = c->d_chunk;
     c->d_tok_slot = c->d_chunk + T;
     c->d_tok_pos = c->d_chunk + 2 * (size_t)T;
@@ -1134,7 +1113,6 @@ int ss_resume(ss_ctx* c, const int32_t* ids, int32_t B, const int32_t* eos_at, i
     need_pages += (size_t)ceil_div(len + cap, kPageTokens) - it->second.pages.size();
   }
   if (need_pages > c->free_pages.size()) return SS_ERR_KV_BUDGET;
-  SS_CUDA(c, staging_free(c, 0));
   int32_t *rows, *bt;
   clear_rows(c, B, cap, &rows, &bt);
   c->batch_pages.clear();
@@ -1209,8 +1187,8 @@ int ss_read_batch(ss_ctx* c, int32_t* out_tokens, int32_t stride, int32_t* out_l
   const int B = c->B;
   // row state and status come back together; the tokens (rows of the batch's cap) with them where that is little, else
   // once it is known how many there are
-  int32_t* rows = (int32_t*)c->down;
-  int32_t* tok = (int32_t*)(c->down + kRowStateBytes);
+  int32_t* rows = (int32_t*)c->down.data();
+  int32_t* tok = (int32_t*)(c->down.data() + kRowStateBytes);
   auto fetch_tokens = [&](int n) {
     return cudaMemcpy2DAsync(tok, (size_t)n * 4, c->st.out_tokens, (size_t)c->st.max_new * 4, (size_t)n * 4, B, cudaMemcpyDeviceToHost,
                              c->stream);
