@@ -203,9 +203,11 @@ struct ss_ctx {
   int32_t* pinned = nullptr;     // [0] n_active, [1] status
   // Staging for what a batch sends and fetches: a copy costs the host 5 to 10 us each, and a batch needed 2 to 7 on its way
   // up and one per row on its way back (200 rows: 2.2 of 19.7 ms per batch of six steps).  Up: row state and block table
-  // as one copy, a chunk's token arrays as another.  Down: row state, tokens.  Ordinary memory: a copy from it
-  // returns when the source may be changed again, and page-locked memory with events to guard it was no faster.
+  // as one copy, a chunk's token arrays as another.  Down: row state, tokens.  Page-locked memory was no faster.  A copy
+  // from ordinary memory may still be reading its source when the call returns, so `up` is filled again only behind
+  // `up_sent`, which is recorded after every copy out of it.
   std::vector<uint8_t> up, down;
+  cudaEvent_t up_sent = nullptr;
   size_t up_chunk = 0;           // where the chunk arrays start inside `up`
   size_t table_off = 0;          // where the block table starts behind the row state (device and staging alike)
   // ---- sampling (greedy while inv_temp == 0)
@@ -663,9 +665,19 @@ int enqueue_prefill_chunk(ss_ctx* c, int s0, int s1, const int32_t* cu, int T) {
 }
 
 // ------------------------------------------------------------------------------------ staging
+// Copies n bytes out of the staging area.
+cudaError_t send_up(ss_ctx* c, void* dst, const void* src, size_t n) {
+  const cudaError_t e = cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, c->stream);
+  const cudaError_t r = cudaEventRecord(c->up_sent, c->stream);
+  if (r != cudaSuccess) cudaStreamSynchronize(c->stream);
+  return e != cudaSuccess ? e : r;
+}
+// The staging area may be filled again: every copy out of it has run.
+cudaError_t wait_up(ss_ctx* c) { return cudaEventSynchronize(c->up_sent); }
+
 // Sends the row state and the block tables of B rows, filled in at c->up (row arrays first, tables at table_off).
 cudaError_t send_rows(ss_ctx* c, int B) {
-  return cudaMemcpyAsync(c->st.ctx_len, c->up.data(), c->table_off + (size_t)B * c->st.max_pages * 4, cudaMemcpyHostToDevice, c->stream);
+  return send_up(c, c->st.ctx_len, c->up.data(), c->table_off + (size_t)B * c->st.max_pages * 4);
 }
 
 // Row state and block table of a new batch of B rows in the staging area: everything zero, no pages.
@@ -863,6 +875,7 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
   if (e == cudaSuccess) e = cudaMemsetAsync(A + o.h, 0, o.partial - o.h, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e == cudaSuccess) e = cudaHostAlloc((void**)&c->pinned, 64, cudaHostAllocDefault);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->up_sent, cudaEventDisableTiming);
   c->up_chunk = align_up(c->table_off + (size_t)rt->max_batch * o.max_pages * 4);
   c->up.resize(c->up_chunk + ((size_t)o.R * 3 + 2 * kMaxBatch + 8) * 4);
   c->down.resize(kRowStateBytes + (size_t)rt->max_batch * rt->max_new_tokens * 4);
@@ -879,6 +892,7 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
                              227 * 1024);
   if (e != cudaSuccess) {
     if (c->pinned) cudaFreeHost(c->pinned);
+    if (c->up_sent) cudaEventDestroy(c->up_sent);
     delete c;
     return SS_ERR_CUDA;
   }
@@ -890,6 +904,7 @@ int ss_destroy(ss_ctx* c) {
   if (!c) return SS_ERR_ARG;
   cudaStreamSynchronize(c->stream);
   if (c->pinned) cudaFreeHost(c->pinned);
+  cudaEventDestroy(c->up_sent);
   delete c;
   return SS_OK;
 }
@@ -962,6 +977,7 @@ int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, c
 
   // host-side batch state
   int32_t *rows, *bt;
+  SS_CUDA(c, wait_up(c));
   clear_rows(c, B, cap, &rows, &bt);
   c->batch_pages.clear();
   c->prompt_len.assign(B, 0);
@@ -1004,7 +1020,8 @@ int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, c
   while (s0 < B) {
     int s1 = s0, T = 0;
     while (s1 < B && T + (cu[s1 + 1] - cu[s1]) <= c->rt.max_prefill_tokens) { T += cu[s1 + 1] - cu[s1]; ++s1; }
-    // the chunk's arrays, packed into one copy
+    // the chunk's arrays, packed into one copy (filled while the chunk before runs)
+    if (s0 > 0) SS_CUDA_B(wait_up(c));
     const int n_seq = s1 - s0;
     int32_t* tok = (int32_t*)(c->up.data() + c->up_chunk);
     int32_t *tok_slot = tok + T, *tok_pos = tok + 2 * (size_t)T, *cu_loc = tok + 3 * (size_t)T, *last = cu_loc + n_seq + 1;
@@ -1018,7 +1035,7 @@ int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, c
       cu_loc[s - s0 + 1] = t;
       last[s - s0] = t - 1;
     }
-    SS_CUDA_B(cudaMemcpyAsync(c->d_chunk, tok, (3 * (size_t)T + 2 * n_seq + 1) * 4, cudaMemcpyHostToDevice, c->stream));
+    SS_CUDA_B(send_up(c, c->d_chunk, tok, (3 * (size_t)T + 2 * n_seq + 1) * 4));
     c->d_tokens = c->d_chunk;
     c->d_tok_slot = c->d_chunk + T;
     c->d_tok_pos = c->d_chunk + 2 * (size_t)T;
@@ -1114,6 +1131,7 @@ int ss_resume(ss_ctx* c, const int32_t* ids, int32_t B, const int32_t* eos_at, i
   }
   if (need_pages > c->free_pages.size()) return SS_ERR_KV_BUDGET;
   int32_t *rows, *bt;
+  SS_CUDA(c, wait_up(c));
   clear_rows(c, B, cap, &rows, &bt);
   c->batch_pages.clear();
   c->batch_tokens.clear();

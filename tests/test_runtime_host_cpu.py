@@ -1,0 +1,70 @@
+"""Host code of the runtime without a GPU: the library's own sources, linked with a stand-in for the CUDA runtime that runs
+every queued copy as late as it may (tests/fake_cudart.cpp)."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2305_13144_b200 import api, build, synth
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    if not os.path.exists(nvcc):
+        pytest.skip("no nvcc")
+    lib = str(tmp_path_factory.mktemp("fake") / "libseqsched_fake.so")
+    subprocess.run([nvcc, "-gencode", "arch=compute_100a,code=compute_100a", "-std=c++17", "-shared", "-cudart", "none", "-Xcompiler", "-fPIC",
+                    "-Xlinker", "-Bsymbolic", "-I", os.path.join(build.ROOT, "include"), "-I", build.CSRC,
+                    *(os.path.join(build.CSRC, s) for s in build.SOURCES), os.path.join(HERE, "fake_cudart.cpp"), "-o", lib],
+                   check=True, capture_output=True)
+    with pytest.MonkeyPatch.context() as mp:
+        mp.setattr(api, "LIB_PATH", lib)
+        mp.setattr(api, "_lib_handle", None)
+        L = api.lib()
+        L.fake_changed_sources.restype = L.fake_pending.restype = C.c_int64
+        L.fake_pending.argtypes = [C.c_char_p]
+        yield L
+
+
+def _engine(L, max_prefill=32, max_new=8):
+    """An engine over host memory; its weights are loaded (and read as zeros by nobody)."""
+    shape = synth.ModelShape(n_layers=1, d_model=64, n_heads=1, head_dim=64, d_ffn=64, vocab=64)
+    m, rt = api.model_cfg(shape), api.runtime_cfg(16, 64, max_prefill, max_new, 2048)
+    arena = np.empty(api.ss_arena_bytes(m, rt) + 1024, dtype=np.uint8)
+    base = arena.ctypes.data + (-arena.ctypes.data) % 1024
+    h = C.c_void_p()
+    assert L.ss_create(C.byref(m), C.byref(rt), C.c_void_p(base), arena.size - 1024, None, C.byref(h)) == api.SS_OK
+    eng = api.Ctx(h, arena, None, m, rt)
+    api.ss_load_weights(eng, {k: synth.to_bf16_bits(v) for k, v in synth.make_weights(shape, seed=1).items()})
+    return eng
+
+
+def _batch(seed, lens):
+    rng = np.random.default_rng(seed)
+    cu = np.zeros(len(lens) + 1, dtype=np.int32)
+    cu[1:] = np.cumsum(lens)
+    return rng.integers(3, 64, size=int(cu[-1])).astype(np.int32), cu
+
+
+def test_staging_is_not_refilled_before_its_copies_have_run(fake):
+    """Prompt chunks and batches one behind the other, nothing waited for by the caller: what a copy reads is what it was given."""
+    eng = _engine(fake)
+    before = fake.fake_changed_sources()
+    for seed in range(3):
+        toks, cu = _batch(seed, [20, 17, 30, 5, 9])        # 32 tokens a chunk: four chunks
+        api.ss_prefill(eng, toks, cu, None, 4)
+        api.ss_keep_prompts(eng, np.arange(5) + 5 * (seed % 2), cu[1:] - cu[:-1])
+        api.ss_decode_steps(eng, 2)
+        api.ss_release_batch(eng)
+        for ids in ([0, 3], [2]):
+            api.ss_resume(eng, ids, None, 4)
+            api.ss_decode_steps(eng, 1)
+            api.ss_release_batch(eng)
+    api.ss_last_device_status(eng)                         # everything that is queued runs
+    assert fake.fake_changed_sources() == before
+    api.ss_destroy(eng)
