@@ -164,6 +164,9 @@ int ss_schedule(const ss_sched_cfg* cfg, const int32_t* prompt_len, const int32_
  *               generated token (1-based) is overwritten with eos_id.
  *   cap         most tokens a row may generate in this batch, the first one included
  *   first_tokens device int32 [B] or NULL
+ * Returns once the layers have run: opts->dump_hidden is complete.  The LM head and the choice of the first token may
+ * still be running, so opts->forced_tokens, the other outputs of opts and first_tokens must stay valid until the stream
+ * has been synchronised (ss_read_batch() does), as for a decode step.
  * A batch in flight must be released before the next ss_prefill(). */
 int ss_prefill(ss_ctx* ctx, const int32_t* tokens, const int32_t* cu_seqlens, int32_t B,
                const int32_t* eos_at, int32_t cap, const ss_step_opts* opts, int32_t* first_tokens);

@@ -252,6 +252,8 @@ def _opts(forced_tokens=None, dump_logits=None, dump_hidden=None, dump_choice=No
 
 def ss_prefill(ctx: Ctx, tokens, cu_seqlens, eos_at, cap: int, *, forced_tokens=None, dump_logits=None,
                dump_hidden=None, dump_choice=None, first_tokens=None) -> None:
+    """Returns once the layers have run (dump_hidden is complete); the LM head may still be running, so the other tensors
+    must be kept until the engine's stream has been synchronised."""
     tk, cu, ea = _np(tokens, np.int32), _np(cu_seqlens, np.int32), _np(eos_at, np.int32)
     o = _opts(forced_tokens, dump_logits, dump_hidden, dump_choice)
     _check(lib().ss_prefill(ctx.handle, _hp(tk), _hp(cu), int(cu.shape[0]) - 1, _hp(ea), int(cap),

@@ -208,6 +208,7 @@ struct ss_ctx {
   // `up_sent`, which is recorded after every copy out of it.
   std::vector<uint8_t> up, down;
   cudaEvent_t up_sent = nullptr;
+  cudaEvent_t layers_done = nullptr;   // behind the last layer of a prompt pass
   size_t up_chunk = 0;           // where the chunk arrays start inside `up`
   size_t table_off = 0;          // where the block table starts behind the row state (device and staging alike)
   // ---- sampling (greedy while inv_temp == 0)
@@ -876,6 +877,7 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e == cudaSuccess) e = cudaHostAlloc((void**)&c->pinned, 64, cudaHostAllocDefault);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->up_sent, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->layers_done, cudaEventDisableTiming);
   c->up_chunk = align_up(c->table_off + (size_t)rt->max_batch * o.max_pages * 4);
   c->up.resize(c->up_chunk + ((size_t)o.R * 3 + 2 * kMaxBatch + 8) * 4);
   c->down.resize(kRowStateBytes + (size_t)rt->max_batch * rt->max_new_tokens * 4);
@@ -893,6 +895,7 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
   if (e != cudaSuccess) {
     if (c->pinned) cudaFreeHost(c->pinned);
     if (c->up_sent) cudaEventDestroy(c->up_sent);
+    if (c->layers_done) cudaEventDestroy(c->layers_done);
     delete c;
     return SS_ERR_CUDA;
   }
@@ -905,6 +908,7 @@ int ss_destroy(ss_ctx* c) {
   cudaStreamSynchronize(c->stream);
   if (c->pinned) cudaFreeHost(c->pinned);
   cudaEventDestroy(c->up_sent);
+  cudaEventDestroy(c->layers_done);
   delete c;
   return SS_OK;
 }
@@ -954,8 +958,11 @@ int ss_release_batch(ss_ctx* c) {
   return SS_OK;
 }
 
-int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, const int32_t* eos_at, int32_t cap,
-               const ss_step_opts* opts, int32_t* first_tokens) {
+}  // extern "C"
+
+// ss_prefill() without the wait at its end.
+static int start_batch(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, const int32_t* eos_at, int32_t cap,
+                       const ss_step_opts* opts, int32_t* first_tokens) {
   if (!c || !tokens || !cu || B < 1 || cap < 1) return SS_ERR_ARG;
   if (c->n_loaded != c->n_expected || c->in_batch) return SS_ERR_STATE;
   if (B > c->rt.max_batch || cap > c->rt.max_new_tokens) return SS_ERR_CAPACITY;
@@ -1049,6 +1056,7 @@ int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, c
                      m.d_model, m.rms_eps));
     s0 = s1;
   }
+  SS_CUDA_B(cudaEventRecord(c->layers_done, c->stream));
   // LM head on the last tokens, first generated token, bookkeeping
   const int NT = round_up(B, 16);
   const CUtensorMap* mx;
@@ -1062,6 +1070,17 @@ int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, c
                    (const int32_t*)c->tile_idx, c->n_tiles_lm, opts ? opts->forced_tokens : (const int32_t*)nullptr,
                    first_tokens, opts ? opts->dump_choice : (int32_t*)nullptr, B, m.eos_id, 1));
 #undef SS_CUDA_B
+  return SS_OK;
+}
+
+extern "C" {
+
+int ss_prefill(ss_ctx* c, const int32_t* tokens, const int32_t* cu, int32_t B, const int32_t* eos_at, int32_t cap,
+               const ss_step_opts* opts, int32_t* first_tokens) {
+  if (int rc = start_batch(c, tokens, cu, B, eos_at, cap, opts, first_tokens)) return rc;
+  // the caller may read dump_hidden and reuse its inputs; the LM head, queued already, keeps the GPU busy meanwhile
+  const cudaError_t e = cudaEventSynchronize(c->layers_done);
+  if (e != cudaSuccess) { ss_release_batch(c); return cuda_fail(c, e); }
   return SS_OK;
 }
 
@@ -1361,7 +1380,7 @@ static int run_batch_list(ss_ctx* c, const ss_sched_cfg* cfg, const int32_t* pro
     for (int r = 0; r < B && resume; ++r) resume = c->kept.count(rows_src[r]) != 0;
     SS_CUDA_G(cudaEventRecord(ev[0], c->stream));
     if (resume) rc = ss_resume(c, rows_src, B, eos_at ? eos_b.data() : nullptr, b.cap, nullptr, nullptr);
-    else rc = ss_prefill(c, toks.data(), cu.data(), B, eos_at ? eos_b.data() : nullptr, b.cap, nullptr, nullptr);
+    else rc = start_batch(c, toks.data(), cu.data(), B, eos_at ? eos_b.data() : nullptr, b.cap, nullptr, nullptr);
     if (rc) return cleanup(rc);
     if (c->prompt_cache_mode == 1 && !resume) {
       std::vector<int32_t> kl(B);

@@ -30,7 +30,8 @@ struct Event {
 std::deque<Op> queue;
 uint64_t enqueued = 0, executed = 0;
 int64_t changed_sources = 0;
-cudaError_t next_wait = cudaSuccess;      // what the next wait returns
+std::string bad_kernel;                   // the kernel (part of its name) whose execution fails, once, and how
+cudaError_t bad_kernel_error = cudaSuccess, pending_error = cudaSuccess;
 std::map<const void*, std::string>& kernel_names() {      // filled while other objects are still being constructed
   static std::map<const void*, std::string> names;
   return names;
@@ -47,6 +48,12 @@ void execute(const Op& op) {
         std::memcpy((char*)op.dst + r * op.dpitch, (const char*)op.src + r * op.spitch, op.n);
       break;
     case Op::kSet: std::memset(op.dst, op.value, op.n); break;
+    case Op::kKernel:
+      if (!bad_kernel.empty() && op.name.find(bad_kernel) != std::string::npos) {
+        pending_error = bad_kernel_error;
+        bad_kernel.clear();
+      }
+      break;
     default: break;
   }
 }
@@ -57,9 +64,9 @@ void run_until(uint64_t at) {
     ++executed;
   }
 }
-cudaError_t waited() {
-  const cudaError_t e = next_wait;
-  next_wait = cudaSuccess;
+cudaError_t waited() {                    // the next wait reports an error, once
+  const cudaError_t e = pending_error;
+  pending_error = cudaSuccess;
   return e;
 }
 void add(Op op) { queue.push_back(std::move(op)); ++enqueued; }
@@ -74,7 +81,7 @@ int encode_tiled(...) { return 0; }
 extern "C" {
 // ---- what a test asks
 int64_t fake_changed_sources() { return changed_sources; }
-void fake_next_wait(int error) { next_wait = (cudaError_t)error; }
+void fake_fail_wait_behind(const char* part, int error) { bad_kernel = part; bad_kernel_error = (cudaError_t)error; }
 // Launches of kernels whose (mangled) name contains `part` that have not been executed.
 int64_t fake_pending(const char* part) {
   int64_t n = 0;

@@ -28,6 +28,7 @@ def fake(tmp_path_factory):
         L = api.lib()
         L.fake_changed_sources.restype = L.fake_pending.restype = C.c_int64
         L.fake_pending.argtypes = [C.c_char_p]
+        L.fake_fail_wait_behind.argtypes = [C.c_char_p, C.c_int]
         yield L
 
 
@@ -67,4 +68,22 @@ def test_staging_is_not_refilled_before_its_copies_have_run(fake):
             api.ss_release_batch(eng)
     api.ss_last_device_status(eng)                         # everything that is queued runs
     assert fake.fake_changed_sources() == before
+    api.ss_destroy(eng)
+
+
+def test_prompt_pass_returns_behind_its_layers(fake):
+    """When ss_prefill returns, the hidden states that it hands out are there and an error of the layers has been reported."""
+    eng = _engine(fake)
+    toks, cu = _batch(1, [20, 17, 30])
+    api.ss_prefill(eng, toks, cu, None, 4)
+    assert fake.fake_pending(b"gather_last_rmsnorm") == 0
+    assert fake.fake_pending(b"lmhead_tile_argmax") == 1   # nothing is gained by waiting for these
+    api.ss_release_batch(eng)
+    api.ss_last_device_status(eng)
+    fake.fake_fail_wait_behind(b"gather_last_rmsnorm", 719)       # cudaErrorLaunchFailure
+    with pytest.raises(api.SSError) as e:
+        api.ss_prefill(eng, toks, cu, None, 4)
+    assert e.value.code == api.SS_ERR_CUDA and api.ss_last_cuda_error(eng) == 719
+    api.ss_prefill(eng, toks, cu, None, 4)                 # the failed batch was released
+    api.ss_release_batch(eng)
     api.ss_destroy(eng)
