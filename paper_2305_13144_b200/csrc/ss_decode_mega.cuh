@@ -342,8 +342,10 @@ __device__ void stage_residual(const MegaArgs& a, const MegaSmem* sm, int wtid, 
       const float2 g0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gb.x));
       const float2 g1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gb.y));
       *reinterpret_cast<float4*>(a.h + (size_t)r * a.d + c) = make_float4(v[0], v[1], v[2], v[3]);
-      if (dump && a.dump_hidden)
-        *reinterpret_cast<float4*>(a.dump_hidden + (size_t)r * a.d + c) = make_float4(v[0], v[1], v[2], v[3]);
+      if (dump && a.dump_hidden) {                     // the caller's buffer: no alignment beyond a float's
+        float* o = a.dump_hidden + (size_t)r * a.d + c;
+        o[0] = v[0]; o[1] = v[1]; o[2] = v[2]; o[3] = v[3];
+      }
       __align__(8) bf16 xb[4];
       xb[0] = __float2bfloat16_rn(v[0] * g0.x); xb[1] = __float2bfloat16_rn(v[1] * g0.y);
       xb[2] = __float2bfloat16_rn(v[2] * g1.x); xb[3] = __float2bfloat16_rn(v[3] * g1.y);

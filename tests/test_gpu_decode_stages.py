@@ -70,3 +70,35 @@ def test_context_beyond_the_page_table_in_shared_memory():
     api.ss_release_batch(eng)
     a, b = (t.cpu().numpy()[0] for t in out)
     assert lens[0] == 2 and np.max(np.abs(a - b)) <= LOGIT_TOL * np.max(np.abs(a))
+
+
+@pytest.mark.parametrize("offset", [1, 2, 3])
+def test_outputs_at_any_float(offset):
+    """dump_hidden and dump_logits that begin `offset` floats behind a 16-byte boundary, in the prompt pass, a decode step and a
+    resumed batch: the same numbers as at the boundary."""
+    import torch
+    from paper_2305_13144_b200 import api
+    shape = _shape(2, 64, vocab=301)
+    eng = engine(shape, synth.make_weights(shape, seed=24))
+    rng = np.random.default_rng(6)
+    lens = [5, 33, 17]
+    cu = np.cumsum([0] + lens).astype(np.int32)
+    ids = rng.integers(3, shape.vocab, size=cu[-1]).astype(np.int32)
+
+    def dump(off):
+        sizes = dict(dump_hidden=3 * shape.d_model, dump_logits=3 * shape.vocab)
+        bufs = {k: [torch.zeros(n + 4, device="cuda")[off:off + n] for _ in range(3)] for k, n in sizes.items()}
+        out = [{k: b[i] for k, b in bufs.items()} for i in range(3)]
+        torch.cuda.synchronize()
+        api.ss_prefill(eng, ids, cu, None, 4, **out[0])
+        api.ss_keep_prompts(eng, [0, 1, 2], lens)
+        api.ss_decode_step(eng, **out[1])
+        api.ss_release_batch(eng)
+        api.ss_resume(eng, [0, 1, 2], None, 2, **out[2])
+        api.ss_release_batch(eng)
+        torch.cuda.synchronize()
+        assert api.ss_last_device_status(eng) == 0
+        return [t.cpu() for o in out for t in o.values()]
+
+    for a, b in zip(dump(0), dump(offset)):
+        assert torch.isfinite(a).all() and a.abs().max() > 0 and torch.equal(a, b)
