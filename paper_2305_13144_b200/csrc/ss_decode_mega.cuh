@@ -976,6 +976,7 @@ __device__ void stage_attention(const MegaArgs& a, MegaSmem* sm, AttnScratch* sc
         }
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
+        __syncwarp();                                     // lane 0's acquire holds for every lane's reads (a vote orders no memory)
         const float* in = a.att_part + (size_t)c * (DH + 4);
         attn_merge(p, __ldcg(reinterpret_cast<const float4*>(in + dl)), __ldcg(in + DH), __ldcg(in + DH + 1));
       }

@@ -38,6 +38,31 @@ def test_cache_scan_splits(heads, head_dim, lens):
     assert el <= LOGIT_TOL and eh <= HIDDEN_TOL, (el, eh)
 
 
+@pytest.mark.parametrize("heads,head_dim,lens", [(1, 128, [1500, 700]), (2, 64, [2300]), (8, 128, [900, 12, 333, 641])])
+def test_cut_pairs_give_the_same_bits_every_time(heads, head_dim, lens):
+    """Pairs that are cut between CTAs are merged in CTA order from partials that a flag announces: the batch started again
+    from the same kept prompts gives the same logits to the last bit, as it would not if a partial were read too early."""
+    import torch
+    from paper_2305_13144_b200 import api
+    shape = _shape(heads, head_dim)
+    eng = engine(shape, synth.make_weights(shape, seed=25), max_ctx=max(lens) + 8, max_prefill=sum(lens), kv_tokens=sum(lens) + 64 * len(lens))
+    cu = np.cumsum([0] + lens).astype(np.int32)
+    ids = np.random.default_rng(7).integers(3, shape.vocab, size=cu[-1]).astype(np.int32)
+    api.ss_prefill(eng, ids, cu, None, 4)
+    api.ss_keep_prompts(eng, np.arange(len(lens)), lens)
+    api.ss_release_batch(eng)
+    out = [torch.zeros(len(lens), shape.vocab, device="cuda") for _ in range(20)]
+    torch.cuda.synchronize()
+    for o in out:
+        api.ss_resume(eng, np.arange(len(lens)), None, 4)
+        api.ss_decode_step(eng)
+        api.ss_decode_step(eng, dump_logits=o)
+        api.ss_release_batch(eng)
+    torch.cuda.synchronize()
+    assert api.ss_last_device_status(eng) == 0 and out[0].abs().max() > 0
+    assert all(torch.equal(o, out[0]) for o in out[1:])
+
+
 @pytest.mark.parametrize("ffn,vocab,rows", [(264, 257, 1), (8, 511, 3), (520, 1000, 17), (1000, 33, 65)])
 def test_swiglu_and_argmax_units(ffn, vocab, rows):
     """Feature and vocabulary counts that end inside a 256-wide unit, odd row counts (the arg-max takes rows in pairs)."""
