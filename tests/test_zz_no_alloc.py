@@ -85,3 +85,43 @@ def test_noalloc_sizes_and_alignments(rows, d, vocab, offset):
     x = h.double() * torch.rsqrt(h.double().square().mean(1, keepdim=True) + 1e-6) * gain.double()
     ref = x @ head.double().T
     assert float((out.double() - ref).norm() / ref.norm()) <= 3e-3
+
+
+def test_noalloc_inside_a_graph_capture():
+    """What the call exists for: captured beside other work, replayed with other inputs, the results of a plain call.  The
+    captured launches depend on one another in the plain way, so that a framework can read the graph's edges with the calls
+    that know no other (cudaGraphGetEdges fails on edges that carry data of their own)."""
+    import ctypes
+    import torch
+    from paper_2305_13144_b200 import api
+    n, d, V = 7, 512, 1000
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(9)
+    head = torch.empty(V, d, device="cuda").normal_(0.0, 0.02, generator=gen).to(torch.bfloat16)
+    gain = torch.ones(d, device="cuda", dtype=torch.bfloat16)
+    src, h, out, after = (torch.zeros(n, k, device="cuda") for k in (d, d, V, V))
+    api.ss_logits_noalloc(h, gain, head, 1e-6, out)                      # the first call on a device, outside of a capture
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        h.copy_(src)
+        api.ss_logits_noalloc(h, gain, head, 1e-6, out)
+        after.copy_(out)
+        api.ss_logits_noalloc(h, gain, head, 1e-6, out)
+    rt = ctypes.CDLL("libcudart.so.12")
+    nodes, edges = ctypes.c_size_t(0), ctypes.c_size_t(0)
+    raw = ctypes.c_void_p(graph.raw_cuda_graph())
+    assert rt.cudaGraphGetNodes(raw, None, ctypes.byref(nodes)) == 0 and nodes.value >= 8
+    frm, to = ((ctypes.c_void_p * 64)() for _ in range(2))
+    edges.value = 64
+    assert rt.cudaGraphGetEdges(raw, frm, to, ctypes.byref(edges)) == 0
+    assert edges.value == nodes.value - 1                                 # a chain
+    graph.instantiate()
+    for seed in range(3):
+        src.normal_(0.0, 2.0, generator=gen)
+        want = torch.zeros(n, V, device="cuda")
+        api.ss_logits_noalloc(src, gain, head, 1e-6, want)
+        out.zero_(), after.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert want.abs().max() > 0 and torch.equal(out, want) and torch.equal(after, want)
