@@ -228,7 +228,7 @@ extern "C" int ss_logits_noalloc(const float* hidden, const void* norm_gain, con
   // The first kernel starts when the stream's earlier work has finished; the projection may start beside it and fetch its
   // first weights (which are older than the first kernel), the summing kernel beside the projection.
   // Not inside a capture: the graph would hold edges with data of their own, which a framework cannot read with the calls
-  // that know plain ones only (7 rows x 512 x 1000 captured: 6.8 us a call with such edges, 8.6 us without; 16 x 4096 x 32000: 48.3 and 50.9).
+  // that know plain ones only (5 rows x 512 x 1000 captured: 6.8 us a call with such edges, 8.6 us without; 16 x 4096 x 32000: 48.3 and 50.9).
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) {
     (void)cudaGetLastError();   // the launches report what is wrong with the stream

@@ -7,6 +7,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -206,7 +207,8 @@ struct ss_ctx {
   // as one copy, a chunk's token arrays as another.  Down: row state, tokens.  Page-locked memory was no faster.  A copy
   // from ordinary memory may still be reading its source when the call returns, so `up` is filled again only behind
   // `up_sent`, which is recorded after every copy out of it.
-  std::vector<uint8_t> up, down;
+  std::vector<uint8_t> up;
+  std::vector<int32_t> down_rows, down_tokens;   // tokens: as many as a batch has brought back so far
   cudaEvent_t up_sent = nullptr;
   cudaEvent_t layers_done = nullptr;   // behind the last layer of a prompt pass
   size_t up_chunk = 0;           // where the chunk arrays start inside `up`
@@ -879,8 +881,12 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->up_sent, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->layers_done, cudaEventDisableTiming);
   c->up_chunk = align_up(c->table_off + (size_t)rt->max_batch * o.max_pages * 4);
-  c->up.resize(c->up_chunk + ((size_t)o.R * 3 + 2 * kMaxBatch + 8) * 4);
-  c->down.resize(kRowStateBytes + (size_t)rt->max_batch * rt->max_new_tokens * 4);
+  try {
+    c->up.resize(c->up_chunk + ((size_t)o.R * 3 + 2 * kMaxBatch + 8) * 4);
+    c->down_rows.resize(kRowStateBytes / 4);
+  } catch (const std::bad_alloc&) {
+    e = cudaErrorMemoryAllocation;
+  }
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(gemm_wx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e == cudaSuccess)
@@ -1224,10 +1230,14 @@ int ss_read_batch(ss_ctx* c, int32_t* out_tokens, int32_t stride, int32_t* out_l
   const int B = c->B;
   // row state and status come back together; the tokens (rows of the batch's cap) with them where that is little, else
   // once it is known how many there are
-  int32_t* rows = (int32_t*)c->down.data();
-  int32_t* tok = (int32_t*)(c->down.data() + kRowStateBytes);
-  auto fetch_tokens = [&](int n) {
-    return cudaMemcpy2DAsync(tok, (size_t)n * 4, c->st.out_tokens, (size_t)c->st.max_new * 4, (size_t)n * 4, B, cudaMemcpyDeviceToHost,
+  int32_t* rows = c->down_rows.data();
+  auto fetch_tokens = [&](int n) -> cudaError_t {
+    try {
+      if (c->down_tokens.size() < (size_t)B * n) c->down_tokens.resize((size_t)B * n);
+    } catch (const std::bad_alloc&) {
+      return cudaErrorMemoryAllocation;
+    }
+    return cudaMemcpy2DAsync(c->down_tokens.data(), (size_t)n * 4, c->st.out_tokens, (size_t)c->st.max_new * 4, (size_t)n * 4, B, cudaMemcpyDeviceToHost,
                              c->stream);
   };
   int n_tok = out_tokens && (size_t)B * c->cap <= 16384 ? c->cap : 0;
@@ -1250,6 +1260,7 @@ int ss_read_batch(ss_ctx* c, int32_t* out_tokens, int32_t stride, int32_t* out_l
       SS_CUDA(c, fetch_tokens(n_tok));
       SS_CUDA(c, cudaStreamSynchronize(c->stream));
     }
+    const int32_t* tok = c->down_tokens.data();
     for (int r = 0; r < B; ++r) std::copy(tok + (size_t)r * n_tok, tok + (size_t)r * n_tok + gen[r], out_tokens + (size_t)r * stride);
   }
   return SS_OK;

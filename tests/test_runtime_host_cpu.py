@@ -32,10 +32,10 @@ def fake(tmp_path_factory):
         yield L
 
 
-def _engine(L, max_prefill=32, max_new=8):
+def _engine(L, max_prefill=32, max_new=8, max_batch=16):
     """An engine over host memory; its weights are loaded (and read as zeros by nobody)."""
     shape = synth.ModelShape(n_layers=1, d_model=64, n_heads=1, head_dim=64, d_ffn=64, vocab=64)
-    m, rt = api.model_cfg(shape), api.runtime_cfg(16, 64, max_prefill, max_new, 2048)
+    m, rt = api.model_cfg(shape), api.runtime_cfg(max_batch, 64, max_prefill, max_new, 2048)
     arena = np.empty(api.ss_arena_bytes(m, rt) + 1024, dtype=np.uint8)
     base = arena.ctypes.data + (-arena.ctypes.data) % 1024
     h = C.c_void_p()
@@ -86,4 +86,21 @@ def test_prompt_pass_returns_behind_its_layers(fake):
     assert e.value.code == api.SS_ERR_CUDA and api.ss_last_cuda_error(eng) == 719
     api.ss_prefill(eng, toks, cu, None, 4)                 # the failed batch was released
     api.ss_release_batch(eng)
+    api.ss_destroy(eng)
+
+
+def _resident():
+    return int(open("/proc/self/statm").read().split()[1]) * os.sysconf("SC_PAGE_SIZE")
+
+
+def test_host_memory_follows_the_batch_and_not_the_limits(fake):
+    """A context for 256 rows of up to a million tokens: its host memory grows with what a batch brings back."""
+    before = _resident()
+    eng = _engine(fake, max_batch=256, max_new=1 << 20)
+    assert _resident() - before < 64 << 20
+    toks, cu = _batch(3, [20, 17, 30])
+    api.ss_prefill(eng, toks, cu, None, 30)
+    out, lens, _ = api.ss_read_batch(eng, 3, 30)           # no kernel ran, so no token was generated
+    assert lens.tolist() == [0, 0, 0]
+    assert _resident() - before < 64 << 20
     api.ss_destroy(eng)
