@@ -406,19 +406,16 @@ void layout(const ss_model_cfg& m, const ss_runtime_cfg& rt, int n_sm, Offsets& 
   o.x_dec = a.take((size_t)kMaxBatch * d * 2);
   o.o_dec = a.take((size_t)kMaxBatch * d * 2);
   o.act_dec = a.take((size_t)kMaxBatch * F * 2);
-  // partial work space: the largest decode GEMM at the widest token tile
+  // partial work space: the largest split projection at its widest token tile
   const int NTmax = round_up(rt.max_batch, 16);
   size_t pb = 0;
   const int shapes[5][2] = {{(int)(3 * d), (int)d}, {(int)d, (int)d}, {(int)(2 * F), (int)d}, {(int)d, (int)F}, {(int)V, (int)d}};
-  for (auto& s : shapes) {
-    const DecodeSplit p = plan_decode(s[0], s[1], n_sm);
+  for (int i = 0; i < 5; ++i) {
+    const DecodeSplit p = plan_decode(shapes[i][0], shapes[i][1], n_sm);
     pb = std::max(pb, (size_t)p.gsplit * p.max_seg * NTmax * kTileN * sizeof(float));
-    const GemmPlan q = plan_gemm(s[0], s[1], short_tile(rt.max_prefill_tokens), n_sm);
+    // split prompt pass: the layers' projections over a short chunk, the LM head over the batch's rows
+    const GemmPlan q = plan_gemm(shapes[i][0], shapes[i][1], i < 4 ? short_tile(rt.max_prefill_tokens) : NTmax, n_sm);
     pb = std::max(pb, (size_t)q.gridx * q.max_seg * q.NT * 128 * sizeof(float));
-  }
-  {
-    const GemmPlan p = plan_gemm((int)V, (int)d, NTmax, n_sm);
-    pb = std::max(pb, (size_t)p.gridx * p.max_seg * p.NT * 128 * sizeof(float));
   }
   o.partial_bytes = pb;
   o.partial = a.take(pb);

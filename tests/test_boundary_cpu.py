@@ -112,3 +112,15 @@ def test_schedule_empty_group_and_capacity():
     rc = L.ss_schedule(ctypes.byref(cfg), pl.ctypes.data, pl.ctypes.data, None, 4, order.ctypes.data, b, 2,
                        ctypes.byref(nb))
     assert rc == api.SS_ERR_CAPACITY and nb.value == 4
+
+
+def test_arena_holds_no_split_sums_for_calls_that_do_not_happen():
+    """The LM head runs over the rows of a batch, never over the 256 tokens of a short prompt chunk: a large vocabulary costs its
+    weights (embedding, LM head, staging) and the partial sums of max_batch rows."""
+    def arena(vocab):
+        shape = synth.ModelShape(n_layers=1, d_model=64, n_heads=1, head_dim=64, d_ffn=64, vocab=vocab)
+        return api.ss_arena_bytes(api.model_cfg(shape), api.runtime_cfg(16, 64, 256, 8, 1024))
+    v = 128000
+    weights = 3 * v * 64 * 2
+    sums = 148 * 8 * 16 * 256 * 4            # CTAs x segments x rows x tile, rounded up: twice what either split needs
+    assert arena(v) - arena(128) < weights + sums + 4 * 2**20        # and a few MB of tables
