@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 from paper_2305_13144_b200 import synth
-from parity_util import HIDDEN_TOL, LOGIT_TOL, engine, teacher_forced
+from parity_util import HIDDEN_TOL, LOGIT_TOL, engine, large_shape_tol, teacher_forced
 
 pytestmark = pytest.mark.gpu
 
@@ -36,6 +36,69 @@ def test_cache_scan_splits(heads, head_dim, lens):
     el, eh, _ = teacher_forced(shape, w, prompts, targets, cap=5, follow=follow, max_batch=max(16, len(lens)), max_ctx=max(lens) + 6,
                                max_prefill=max(512, max(lens)), kv_tokens=sum(lens) + 64 * len(lens))
     assert el <= LOGIT_TOL and eh <= HIDDEN_TOL, (el, eh)
+
+
+@pytest.mark.parametrize("heads,head_dim,lens", [
+    # units per warp of 148 CTAs; a unit is two pieces, and a warp looks the pieces up 32 at a time and again in every layer
+    (8, 128, [700 + (37 * i) % 600 for i in range(40)]),       # 15 to 18: just below, at and above one look-up; pairs cut between CTAs
+    (8, 128, [1100 + (13 * i) % 180 for i in range(64)]),      # 31 to 34: two look-ups, some slices of exactly 64 pieces
+    (20, 128, [150 + (29 * i) % 220 for i in range(64)]),      # 14 to 22, whole pairs among them, slices that cross rows
+    (32, 64, [200 + (53 * i) % 300 for i in range(64)]),       # 15 to 23, up to two whole pairs
+    (16, 128, [10 + (31 * i) % 260 for i in range(150)]),      # the wide kernel: 7 to 23, three whole pairs and more
+    (16, 64, [20 + (41 * i) % 480 for i in range(200)]),       # 9 to 29
+])
+def test_cache_scan_refills(heads, head_dim, lens):
+    """Slices of more pieces than a warp looks up at once, over two layers (at the second the stream starts again at the slice's
+    first piece while the last ones of the first are being read).  Widths of 1024 and more: the tolerance of the large shapes."""
+    shape = _shape(heads, head_dim)
+    w = synth.make_weights(shape, seed=26)
+    rng = np.random.default_rng(8)
+    prompts = [rng.integers(3, shape.vocab, size=n).tolist() for n in lens]
+    follow = [0, len(lens) // 2, len(lens) - 1]
+    targets = [2 + i % 4 for i in range(len(lens))]
+    tol = large_shape_tol(shape.n_layers)
+    el, eh, _ = teacher_forced(shape, w, prompts, targets, cap=4, follow=follow, dtype=np.float32, max_batch=len(lens), max_ctx=max(lens) + 6,
+                               max_prefill=4096, kv_tokens=sum(lens) + 64 * len(lens))
+    assert el <= tol and eh <= tol, (el, eh)
+
+
+def test_not_a_number_stays_in_its_row():
+    """Rows whose keys and values are NaN share warps, cache pieces and prompt chunks with sound rows.  What such a row leaves
+    behind a sound row's last token -- in the same chunk, in a piece of shared memory, in a page used again -- carries weight 0 there
+    and must not be multiplied: the sound rows' logits are those of a batch without NaN, to the last bit."""
+    import torch
+    from paper_2305_13144_b200 import api
+    shape = _shape(4, 128)
+    w = synth.make_weights(shape, seed=27)
+    w["embed"][5] = np.nan                                 # token 5 is in the bad rows' prompts only
+    lens = [17, 300, 33, 129, 47, 260, 15, 64, 5, 90]
+    bad = [1, 3, 5, 7]
+    cu = np.cumsum([0] + lens).astype(np.int32)
+    rng = np.random.default_rng(9)
+    clean = rng.integers(6, shape.vocab, size=cu[-1]).astype(np.int32)
+    poisoned = clean.copy()
+    for r in bad:
+        poisoned[cu[r]:cu[r + 1]] = 5
+    sound = [r for r in range(len(lens)) if r not in bad]
+
+    def run(eng, ids):
+        out = [torch.zeros(len(lens), shape.vocab, device="cuda") for _ in range(3)]
+        forced = torch.full((len(lens),), 7, dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        api.ss_prefill(eng, ids, cu, None, 4, forced_tokens=forced, dump_logits=out[0])
+        for o in out[1:]:
+            api.ss_decode_step(eng, forced_tokens=forced, dump_logits=o)
+        api.ss_read_batch(eng, len(lens), 4)
+        api.ss_release_batch(eng)
+        return [o.cpu() for o in out]
+
+    eng = engine(shape, w, max_ctx=320, max_prefill=2048, kv_tokens=sum(lens) + 64 * len(lens))
+    want = run(eng, clean)
+    got = run(eng, poisoned)
+    again = run(eng, clean)                                # pages and operands that NaN was written to
+    for a, b, c in zip(want, got, again):
+        assert torch.isfinite(a).all() and a.abs().max() > 0
+        assert torch.isnan(b[bad]).all() and torch.equal(a[sound], b[sound]) and torch.equal(a, c)
 
 
 @pytest.mark.parametrize("heads,head_dim,lens", [(1, 128, [1500, 700]), (2, 64, [2300]), (8, 128, [900, 12, 333, 641])])
@@ -85,11 +148,12 @@ def test_context_beyond_the_page_table_in_shared_memory():
     ids = np.random.default_rng(5).integers(3, shape.vocab, size=8301).astype(np.int32)
     eng = engine(shape, w, max_batch=2, max_ctx=8400, max_prefill=8301, max_new=4, kv_tokens=2 * 8400)
     out = [torch.zeros(1, shape.vocab, dtype=torch.float32, device="cuda") for _ in range(2)]
+    forced = torch.tensor(ids[8300:], dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()                               # the engine's stream does not wait for torch's
     api.ss_prefill(eng, ids, np.array([0, 8301], dtype=np.int32), None, 2, dump_logits=out[0])
     api.ss_read_batch(eng, 1, 2)
     api.ss_release_batch(eng)
-    api.ss_prefill(eng, ids[:8300], np.array([0, 8300], dtype=np.int32), None, 3,
-                   forced_tokens=torch.tensor(ids[8300:], dtype=torch.int32, device="cuda"))
+    api.ss_prefill(eng, ids[:8300], np.array([0, 8300], dtype=np.int32), None, 3, forced_tokens=forced)
     api.ss_decode_step(eng, dump_logits=out[1])
     _, lens, _ = api.ss_read_batch(eng, 1, 3)
     api.ss_release_batch(eng)

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 from paper_2305_13144_b200 import synth
-from parity_util import HIDDEN_TOL, LOGIT_TOL, teacher_forced
+from parity_util import HIDDEN_TOL, LOGIT_TOL, engine, teacher_forced
 
 pytestmark = pytest.mark.gpu
 
@@ -28,3 +28,33 @@ def test_prompt_lengths_and_paths(heads, head_dim, ffn, lens):
     el, eh, _ = teacher_forced(shape, w, prompts, [3] * len(lens), cap=3, max_ctx=max(lens) + 4, max_prefill=max(256, sum(lens)),
                                kv_tokens=sum(lens) + 64 * len(lens))
     assert el <= LOGIT_TOL and eh <= HIDDEN_TOL, (el, eh)
+
+
+@pytest.mark.parametrize("lens", [[280, 100, 120, 30], [100, 120, 30, 300], [300, 299, 1]])
+def test_chunks_of_both_paths_in_one_batch(lens):
+    """Chunks of at most 300 tokens: some run on pairs of CTAs, some with their projections split along K."""
+    shape = synth.ModelShape(n_layers=2, d_model=256, n_heads=2, head_dim=128, d_ffn=264, vocab=300)
+    w = synth.make_weights(shape, seed=32)
+    rng = np.random.default_rng(10)
+    prompts = [rng.integers(3, shape.vocab, size=n).tolist() for n in lens]
+    el, eh, _ = teacher_forced(shape, w, prompts, [3] * len(lens), cap=3, max_ctx=max(lens) + 4, max_prefill=300,
+                               kv_tokens=sum(lens) + 64 * len(lens))
+    assert el <= LOGIT_TOL and eh <= HIDDEN_TOL, (el, eh)
+
+
+def test_hidden_states_are_there_when_the_call_returns():
+    """dump_hidden read on another stream right behind ss_prefill, without waiting for the engine's."""
+    import torch
+    from paper_2305_13144_b200 import api
+    shape = synth.ModelShape(n_layers=8, d_model=2048, n_heads=16, head_dim=128, d_ffn=4096, vocab=300)
+    eng = engine(shape, synth.make_weights(shape, seed=33), max_ctx=1100, max_prefill=2048, kv_tokens=9000)
+    cu = np.arange(9, dtype=np.int32) * 1000               # four chunks
+    ids = np.random.default_rng(11).integers(3, shape.vocab, size=8000).astype(np.int32)
+    for _ in range(3):
+        dh = torch.zeros(8, shape.d_model, device="cuda")
+        torch.cuda.synchronize()
+        api.ss_prefill(eng, ids, cu, None, 2, dump_hidden=dh)
+        at_return = dh.cpu()                               # torch's stream, not the engine's
+        torch.cuda.synchronize()
+        api.ss_release_batch(eng)
+        assert torch.equal(at_return, dh.cpu()) and (at_return.abs().amax(dim=1) > 0).all()
