@@ -80,7 +80,7 @@ struct MegaArgs {
   RowState st;
   KvLayout kv;
   int kv_pieces;                   // shared-memory pieces per worker warp for the cache scan
-  float* att_part;                 // [CTA][Dh + 2] (acc, max, sum) of the pair a CTA's range starts inside of
+  float* att_part;                 // [CTA][Dh + 4] (acc, max, sum, two unused) of the pair a CTA's range starts inside of
   unsigned long long* att_flag;    // [CTA] set to the running barrier's number once att_part[CTA] is complete
   // activations (decode buffers)
   float* h;                        // [B][d] residual stream
@@ -988,8 +988,9 @@ __device__ void stage_attention(const MegaArgs& a, MegaSmem* sm, AttnScratch* sc
 
 // ---- stage: SwiGLU ----------------------------------------------------------------------------------
 // Work unit = (row, 256 features) per warp: gate and up rows alternate in the weights, so a lane's four loads of four
-// consecutive outputs are two features each (and a warp-wide load covers 512 contiguous bytes of a partial segment); units are dealt round-robin over the CTAs.  The row is the warp's own, so its 1/rms is two more loads
-// beside the partials instead of a pass over all rows with a barrier behind it (200 rows: 19.3 -> 10.2 us).
+// consecutive outputs are two features each (and a warp-wide load covers 512 contiguous bytes of a partial segment); units
+// are dealt round-robin over the CTAs.  The row is the warp's own, so its 1/rms is two more loads beside the partials
+// instead of a pass over all rows with a barrier behind it (200 rows: 19.3 -> 10.2 us).
 __device__ void stage_swiglu(const MegaArgs& a, const MegaSmem* sm, int wtid) {
   const MegaGemmShape& gs = a.shape[2];
   const int lane = wtid & 31, wid = wtid >> 5;
@@ -1347,7 +1348,7 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
       const MegaGemmShape& gs = a.shape[type];
       // ---- drain this CTA's segments of projection gm into fp32 partials
       long long it0, it1;
-        mega_range(gs, cta, it0, it1);
+      mega_range(gs, cta, it0, it1);
       long long it = it0;
       int seg_local = 0;
       while (it < it1 && ok) {

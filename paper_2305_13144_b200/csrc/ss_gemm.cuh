@@ -1,14 +1,15 @@
 // Weight-streaming GEMM for sm_100a:  D[n_out, tok] = W[n_out, K] . X[tok, K]^T   (bf16 in, fp32 accumulate)
 //
-// The weight matrix is the tcgen05 "A" operand (128 rows per tile), the activations are "B"
-// (16..256 tokens per tile), so a decode step with a handful of rows still fills the 128-lane
-// tensor-memory accumulator while every weight byte crosses HBM exactly once.  Both operands
-// arrive by TMA (128-byte swizzle) into a multi-stage shared-memory ring; one elected thread
-// issues tcgen05.mma; four warps drain the accumulator from tensor memory.
+// gemm_wx_kernel: for few tokens (the LM head behind a prompt pass, short prompt chunks, ss_logits_noalloc; the decode
+// step has a GEMM of its own).  The weight matrix is the tcgen05 "A" operand (128 rows per tile), the activations are "B"
+// (one tile of 16..256 tokens), so a handful of tokens still fills the 128-lane tensor-memory accumulator while every
+// weight byte crosses HBM exactly once.  Both operands arrive by TMA (128-byte swizzle) into a multi-stage shared-memory
+// ring; one elected thread issues tcgen05.mma; four warps drain the accumulator from tensor memory.
+// Work decomposition: the (tile, k-block) iteration space is cut into gridDim.x equal contiguous ranges.  A range that ends
+// inside a tile produces a partial sum; all segments are written as fp32 partials which the consumer kernel adds in CTA
+// order.
 //
-// Work decomposition: the (tile, k-block) iteration space is cut into gridDim.y equal
-// contiguous ranges.  A range that ends inside a tile produces a partial sum; in kGemmPartial
-// mode all segments are written as fp32 partials which the consumer kernel adds in CTA order.
+// gemm_wx_pair_kernel: for more tokens than one tile, on pairs of CTAs; it finishes the projection in its epilogue.
 //
 // Programmatic dependent launch: weights never depend on the previous kernel, so the producer
 // fills the ring with weight tiles BEFORE griddepcontrol.wait and only then loads activations.
@@ -272,7 +273,7 @@ gemm_wx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   extern __shared__ uint8_t smem_raw[];
   const GemmPlan& p = a.p;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int cta = blockIdx.y, tok_tile = blockIdx.x;
+  const int cta = blockIdx.x;
 
   // carve shared memory: header, then 1024-byte aligned stages
   GemmSmemHeader* hdr = reinterpret_cast<GemmSmemHeader*>(smem_raw);
@@ -337,8 +338,7 @@ gemm_wx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       for (int i = 0; i < pre; ++i) {
         const long long it = it0 + i;
         const int kblk = (int)(it % p.kb);
-        tma_load_2d(stage0 + i * stage_bytes + a_bytes, &map_x, smem_u32(&hdr->full[i]), kblk * kTileK,
-                    tok_tile * p.NT, hint_x);
+        tma_load_2d(stage0 + i * stage_bytes + a_bytes, &map_x, smem_u32(&hdr->full[i]), kblk * kTileK, 0, hint_x);
       }
       // phase 2: steady state (second and later passes over the ring)
       int stage = 0, issued = pre;
@@ -351,7 +351,7 @@ gemm_wx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         mbar_expect_tx(full, stage_bytes);
         if (w_tiled) bulk_load(stage0 + stage * stage_bytes, w_block(tile, kblk), a_bytes, full, hint_w);
         else tma_load_2d(stage0 + stage * stage_bytes, &map_w, full, kblk * kTileK, tile * kTileM, hint_w);
-        tma_load_2d(stage0 + stage * stage_bytes + a_bytes, &map_x, full, kblk * kTileK, tok_tile * p.NT, hint_x);
+        tma_load_2d(stage0 + stage * stage_bytes + a_bytes, &map_x, full, kblk * kTileK, 0, hint_x);
         if (++stage == p.stages) { stage = 0; phase ^= 1u; }
         ++issued;
       }
@@ -414,9 +414,7 @@ gemm_wx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     const int row = quarter * 32 + lane;          // row inside the 128-row tile
     int seg = 0;
     long long it = it0;
-    const int tok0 = tok_tile * p.NT;
-    int n_valid = a.n_tok - tok0;
-    if (n_valid > p.NT) n_valid = p.NT;
+    const int n_valid = a.n_tok < p.NT ? a.n_tok : p.NT;
     while (it < it1) {
       const int tile = (int)(it / p.kb);
       long long seg_end = (long long)(tile + 1) * p.kb;
@@ -549,7 +547,7 @@ gemm_wx_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_cta_rank();          // 0: issues the MMAs; 1: its partner
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-  const int tok_tiles = p.gridy;                     // token tiles of 256
+  const int tok_tiles = p.tok_tiles;                 // of 256
   const int n_units = (p.n_tiles >> 1) * tok_tiles;
   GemmSmemHeader* hdr = reinterpret_cast<GemmSmemHeader*>(smem_raw);
   const uint32_t stage0 = (smem_u32(smem_raw) + (uint32_t)sizeof(GemmSmemHeader) + 1023u) & ~1023u;

@@ -36,17 +36,18 @@ enum : uint32_t {
 };
 
 // ---- GEMM:  D[n_out, tok] = W[n_out, K] . X[tok, K]^T  -------------------------------------
-// kGemmPartial (gemm_wx_kernel): the tile-iteration space (n_tiles x kb) is cut into `gridx` equal contiguous ranges,
-// one per CTA (split along K where a range ends inside a tile); every (CTA, tile) segment is written as an fp32 partial
-// and the consumer kernel adds the segments of a tile in CTA order, so the result does not depend on timing.
-// The others (gemm_wx_pair_kernel) finish a tile in its epilogue: added to the fp32 residual; rotated and written as
-// bf16 q, k, v operand and cache entries; or gated (SwiGLU) and written as bf16 operand.
-enum GemmMode : int { kGemmPartial = 0, kGemmResidual = 1, kGemmQkv = 2, kGemmSwiglu = 3 };
+// gemm_wx_kernel: the tile-iteration space (n_tiles x kb) is cut into `gridx` equal contiguous ranges, one per CTA (split
+// along K where a range ends inside a tile); every (CTA, tile) segment is written as an fp32 partial and the consumer
+// kernel adds the segments of a tile in CTA order, so the result does not depend on timing.
+// gemm_wx_pair_kernel finishes a tile in its epilogue: added to the fp32 residual; rotated and written as bf16 q, k, v
+// operand and cache entries; or gated (SwiGLU) and written as bf16 operand.
+enum GemmMode : int { kGemmResidual = 1, kGemmQkv = 2, kGemmSwiglu = 3 };
 
 struct GemmPlan {
   int n_out, K, n_tiles, kb;
   int NT;              // token tile (tcgen05 N), multiple of 16, <= 256
-  int gridx, gridy;    // CTAs along the iteration space / token tiles
+  int gridx;           // CTAs (pairs of CTAs in gemm_wx_pair_kernel)
+  int tok_tiles;       // gemm_wx_pair_kernel: token tiles
   int max_seg;         // partial slots per CTA
   int stages;
   int smem_bytes;
@@ -56,9 +57,9 @@ struct GemmPlan {
 struct GemmArgs {
   GemmPlan p;
   const void* w_tiled; // weights repacked as contiguous 32 KiB (256-row tile, k-block) images, or null (row-major via TMA)
-  int mode;
+  int mode;            // gemm_wx_pair_kernel: GemmMode
   int n_tok;           // valid tokens
-  float* partial;      // [gridx*max_seg][NT][128]
+  float* partial;      // gemm_wx_kernel: [gridx*max_seg][NT][128]
   float* residual;     // kGemmResidual: [tok][n_out]
   void* out;           // kGemmQkv: bf16 [tok][3 d]; kGemmSwiglu: bf16 [tok][n_out / 2]
   // kGemmQkv
@@ -81,7 +82,7 @@ struct TileSeg {
 struct SplitInfo {
   int gridx, kb, max_seg, NT;
   long long total;          // n_tiles * kb
-  const TileSeg* tiles;     // device table [n_tiles], or null (then the consumers derive it)
+  const TileSeg* tiles;     // device table [n_tiles], or null (noalloc_reduce_kernel derives the segments itself)
 };
 
 }  // namespace ss

@@ -206,7 +206,6 @@ extern "C" int ss_logits_noalloc(const float* hidden, const void* norm_gain, con
   p.NT = kNoAllocMaxRows;
   const long long total = (long long)p.n_tiles * p.kb;
   p.gridx = (int)(total < s->n_sm ? total : s->n_sm);
-  p.gridy = 1;
   const int ipc = (int)((total + p.gridx - 1) / p.gridx);
   p.max_seg = (ipc + p.kb - 2) / p.kb + 1;
   const int stage_bytes = kTileM * kTileK * 2 + p.NT * kTileK * 2;
@@ -228,7 +227,8 @@ extern "C" int ss_logits_noalloc(const float* hidden, const void* norm_gain, con
   // The first kernel starts when the stream's earlier work has finished; the projection may start beside it and fetch its
   // first weights (which are older than the first kernel), the summing kernel beside the projection.
   // Not inside a capture: the graph would hold edges with data of their own, which a framework cannot read with the calls
-  // that know plain ones only (5 rows x 512 x 1000 captured: 6.8 us a call with such edges, 8.6 us without; 16 x 4096 x 32000: 48.3 and 50.9).
+  // that know plain ones only (captured, us a call with such edges and without: 5 rows x 512 x 1000 6.8 and 8.6, 16 x 4096 x
+  // 32000 48.3 and 50.9).
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) {
     (void)cudaGetLastError();   // the launches report what is wrong with the stream
@@ -239,11 +239,10 @@ extern "C" int ss_logits_noalloc(const float* hidden, const void* norm_gain, con
   noalloc_rmsnorm_kernel<<<kNoAllocMaxRows, 256, 0, st>>>(hidden, (const __nv_bfloat16*)norm_gain, x, n_rows, d_model, rms_eps, vec, status);
   GemmArgs a{};
   a.p = p;
-  a.mode = kGemmPartial;
   a.n_tok = n_rows;
   a.partial = partial;
   a.status = status;
-  if (launch_after(early, gemm_wx_kernel, dim3(1, p.gridx), dim3(kGemmThreads), (size_t)p.smem_bytes, st, mw, mx, a) != cudaSuccess) return SS_ERR_CUDA;
+  if (launch_after(early, gemm_wx_kernel, dim3(p.gridx), dim3(kGemmThreads), (size_t)p.smem_bytes, st, mw, mx, a) != cudaSuccess) return SS_ERR_CUDA;
   SplitInfo sp;
   sp.gridx = p.gridx; sp.kb = p.kb; sp.max_seg = p.max_seg; sp.NT = p.NT; sp.total = total; sp.tiles = nullptr;
   if (launch_after(early, noalloc_reduce_kernel, dim3(p.n_tiles, (n_rows + kReduceRows - 1) / kReduceRows), dim3(128), 0, st, (const float*)partial, sp, logits,

@@ -63,7 +63,6 @@ GemmPlan plan_gemm(int n_out, int K, int NT, int n_sm) {
   p.NT = NT;
   const long long total = (long long)p.n_tiles * p.kb;
   p.gridx = (int)std::min<long long>(n_sm, total);
-  p.gridy = 1;
   const int ipc = std::max(1, (int)((total + p.gridx - 1) / p.gridx));
   p.max_seg = (ipc + p.kb - 2) / p.kb + 1;
   const int stage_bytes = kTileM * kTileK * 2 + NT * kTileK * 2;
@@ -309,13 +308,12 @@ int run_gemm(ss_ctx* c, const uint8_t* w_tiled, const CUtensorMap& mx, const Gem
   GemmArgs a{};
   a.p = p;
   a.w_tiled = w_tiled;
-  a.mode = kGemmPartial;
   a.n_tok = n_tok;
   a.partial = c->partial;
   a.status = c->status;
   if ((size_t)p.gridx * p.max_seg * p.NT * 128 * sizeof(float) > c->partial_bytes) return SS_ERR_CAPACITY;
   // the weight tensor map is unused with tiled weights; the activation map stands in for it
-  SS_CUDA(c, launch(c, gemm_wx_kernel, dim3(1, p.gridx), dim3(kGemmThreads), (size_t)p.smem_bytes, mx, mx, a));
+  SS_CUDA(c, launch(c, gemm_wx_kernel, dim3(p.gridx), dim3(kGemmThreads), (size_t)p.smem_bytes, mx, mx, a));
   return SS_OK;
 }
 
@@ -328,8 +326,8 @@ int run_gemm_pair(ss_ctx* c, const CUtensorMap& mw, const CUtensorMap& mx, int n
   a.p.NT = kPairTokens;
   a.p.stages = std::min(kGemmMaxStages, (227 * 1024 - 2048) / kPairStageBytes);
   a.p.smem_bytes = 2048 + a.p.stages * kPairStageBytes;
-  a.p.gridy = ceil_div(a.n_tok, kPairTokens);                        // token tiles
-  const int n_units = (a.p.n_tiles / 2) * a.p.gridy;
+  a.p.tok_tiles = ceil_div(a.n_tok, kPairTokens);
+  const int n_units = (a.p.n_tiles / 2) * a.p.tok_tiles;
   a.p.gridx = std::min(n_units, c->n_sm / 2);                        // pairs of CTAs, each walking its units
   SS_CUDA(c, launch(c, gemm_wx_pair_kernel, dim3(2 * a.p.gridx), dim3(kGemmThreads), (size_t)a.p.smem_bytes, mw, mx, a));
   return SS_OK;
@@ -615,14 +613,14 @@ int enqueue_prefill_chunk(ss_ctx* c, int s0, int s1, const int32_t* cu, int T) {
   glu.n_tok = T;
   glu.out = c->act;
   glu.status = c->status;
-  // more than half a pair's token tile: the paired kernel; below, the projections are split over the SMs along K too
+  // more than one token tile of a pair: the paired kernel; up to it, the projections are split over the SMs along K too
   const bool pair = T > kShortTokens;
   const int NT = pair ? kPairTokens / 2 : short_tile(T);
   if ((rc = xmap(c, 0, NT, &mx)) || (rc = xmap(c, 1, NT, &mo)) || (rc = xmap(c, 2, NT, &ma))) return rc;
   const int shp[4][2] = {{3 * d, d}, {d, d}, {2 * F, d}, {d, F}};
   GemmPlan plan[4];
   SplitInfo split[4];
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < 4 && !pair; ++i) {
     plan[i] = plan_gemm(shp[i][0], shp[i][1], NT, c->n_sm);
     split[i] = split_of(plan[i], c->tbl128[i]);
   }
