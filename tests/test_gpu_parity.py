@@ -58,7 +58,7 @@ def test_tiny_ragged_batch_sizes_and_page_boundaries():
 
 
 def test_very_short_prompts_leave_attention_groups_without_keys():
-    """Fewer cached tokens than key groups in the decode-attention CTA (prompts of 1, 2, 5 tokens)."""
+    """Fewer cached tokens than a warp takes in one load step of the cache scan (prompts of 1, 2, 5 tokens)."""
     shape = synth.TINY
     w = synth.make_weights(shape, seed=1234)
     rng = np.random.default_rng(11)
@@ -67,8 +67,8 @@ def test_very_short_prompts_leave_attention_groups_without_keys():
     assert el <= LOGIT_TOL and eh <= HIDDEN_TOL, (el, eh)
 
 
-def test_long_context_spans_attention_chunks():
-    """A prompt longer than one attention work item (256 tokens) and one prompt-pass query tile."""
+def test_long_context_spans_attention_tiles():
+    """Prompts of two and three query tiles of the prompt pass (128 tokens) and of about ten units of the cache scan."""
     shape = synth.TINY.with_layers(1)
     w = synth.make_weights(shape, seed=77)
     rng = np.random.default_rng(9)
@@ -165,8 +165,8 @@ def test_errors_before_launch():
 @pytest.mark.parametrize("B", [40, 64, 100, 130])
 def test_wide_batches_span_several_token_tiles(B):
     """Batches wider than 16 rows: token tiles of 48 and 64 (64-lane accumulator, all four lane quarters),
-    112 (one 128-lane accumulator tile) and 144 (two 128-lane tiles); the per-tile arg-max in groups of 64
-    rows; attention passes of more than 8 (row, head) pairs per CTA."""
+    112 (one 128-lane accumulator tile) and 144 (two 128-lane tiles); the per-tile arg-max by (vocabulary tile,
+    two rows); contexts of one to three units of the cache scan, fewer pairs than warps for most."""
     shape = synth.TINY.with_layers(1)
     w = synth.make_weights(shape, seed=21)
     rng = np.random.default_rng(B)

@@ -61,11 +61,11 @@ def test_13b_shape_two_layers_batch16():
 
 
 @pytest.mark.parametrize("B", [48, 80])
-def test_13b_shape_two_layers_attention_in_several_passes(B):
-    """40 heads x 48 or 80 rows are 13 or 22 (row, head) pairs per CTA of a 148-SM part: more than the eight of one
-    pass, fewer than the 24 from which every warp takes whole pairs.  48 rows run in the kernel of the batches up
-    to 64 rows, 80 rows in the one for wide batches; prompts of 20 to 90 tokens, so rows differ in pages; two of
-    the followed rows end early."""
+def test_13b_shape_two_layers_attention_slices_of_several_pairs(B):
+    """40 heads x 48 or 80 rows of 20 to 90 prompt tokens, i.e. 2 to 6 units of 16 cached tokens: on a 148-SM part a warp's
+    slice of the cache scan has 4 to 9 (48 rows) or 8 to 13 units (80 rows), with one to three whole (row, head) pairs and
+    pairs that are cut between warps, none between CTAs.  48 rows run in the kernel of the batches up to 64 rows, 80 rows
+    in the one for wide batches; two of the followed rows end early."""
     shape = synth.LLAMA_13B.with_layers(2)
     w = synth.make_weights(shape, seed=13)
     rng = np.random.default_rng(1000 + B)
@@ -83,8 +83,8 @@ def test_13b_shape_two_layers_attention_in_several_passes(B):
 
 def test_13b_shape_two_layers_wide_batch():
     """The variable-batch-size arm's launch configuration at the 13B shape: 136 rows (two 128-lane token
-    tiles, the second with 8 rows), short prompts; the oracle follows six rows spread over both tiles.  A CTA's run
-    has about 37 pairs here, so every warp takes whole pairs."""
+    tiles, the second with 8 rows), short prompts; the oracle follows six rows spread over both tiles.  Pairs have one to
+    three units here and every warp's slice three whole pairs or more, some of two rows."""
     shape = synth.LLAMA_13B.with_layers(2)
     w = synth.make_weights(shape, seed=13)
     rng = np.random.default_rng(136)
@@ -100,10 +100,10 @@ def test_13b_shape_two_layers_wide_batch():
     assert el <= large_shape_tol(2) and eh <= large_shape_tol(2), (el, eh)
 
 
-def test_many_heads_long_contexts_pages_beyond_the_first_64():
-    """A one-layer decoder with 32 heads x 64 and 120 rows whose prompts all have 2050 to 2110 tokens: 26 (row,
-    head) pairs per CTA, so every warp takes whole pairs, and 65 or 66 pages per row, so the scan goes through the
-    page ids a warp's lanes hold (pages 0..31 and 32..63) and the ones it looks up one by one beyond them."""
+def test_many_heads_long_contexts_hundreds_of_units_per_warp():
+    """A one-layer decoder with 32 heads x 64 and 120 rows whose prompts all have 2050 to 2110 tokens: 65 or 66 pages, and
+    units of 32 tokens, per row; a warp's slice has 210 to 213 units, i.e. 14 look-ups of 32 cache pieces, over two or three
+    whole (row, head) pairs and the ends of others, and pairs are cut between CTAs.  The prompts are 40 chunks."""
     shape = synth.ModelShape(n_layers=1, d_model=2048, n_heads=32, head_dim=64, d_ffn=512, vocab=1024)
     w = synth.make_weights(shape, seed=21)
     rng = np.random.default_rng(2100)
