@@ -724,8 +724,11 @@ def main():
         peaks, which = measured_peaks()
         peak = float(peaks["hbm_gbs"])
         achieved = model_bytes / decode_s / 1e9
-        h2d = int(g.prompt_tokens.nbytes + 4 * (g.n + 1) + 4 * g.n + 8 * 4 * 256 + 4 * 16 * 24 + 3 * g.prompt_tokens.nbytes)
-        d2h = int(tokens * 4 + 2 * 4 * g.n + 4)
+        # up: tokens, cache slots and positions of the prompt tokens, prefix sums and last tokens; row state (with what lies
+        # between it and the block table in the arena) and 24 block-table entries per row.  Down: row state, every row's
+        # slot of 512 tokens, the status word.
+        h2d = int(3 * g.prompt_tokens.nbytes + 4 * (2 * g.n + 1) + 9216 + 4 * 24 * g.n)
+        d2h = int(8192 + 4 * 512 * g.n + 4)
         traffic = measured_traffic_bytes() if shape.n_layers == 32 else None
         line = {
             "metric": METRIC, "value": tok_all / dev_all, "unit": "tokens/s", "n_gpus": world,
