@@ -29,7 +29,8 @@
 // rsqrt(mean h^2 + eps).  This lets a row be split over many CTAs without a cross-CTA reduction.
 //
 // Every wait (mbarrier, grid barrier, flag) is bounded; on expiry the kernel records a status word,
-// raises a CTA-wide abort flag and all roles leave.
+// raises a CTA-wide abort flag and all roles leave.  The worker warps leave together, behind a grid barrier: they meet in
+// barriers of the CTA, which have no limit of their own, so none of them goes by the abort flag alone.
 #pragma once
 
 #include "ss_kernels.cuh"
@@ -119,6 +120,7 @@ struct MegaSmem {
   volatile int w_issued;           // ring iterations armed by the weight producer
   volatile int act_epoch;          // projections whose activation operand is complete
   volatile int abort;
+  volatile int leave;              // set behind a grid barrier that found the flag up, or that nobody answered: the workers leave
   int prefix[kMaxBatch + 1];
   // attention, set up once per step (the lengths do not change between layers): every warp's slice of the cache scan
   int sl_begin[8], sl_n[8];        // its first unit and its units
@@ -178,22 +180,26 @@ __device__ __forceinline__ bool mega_wait(uint32_t bar, uint32_t parity, MegaSme
 }
 
 // Arrival on a grid-wide counter and the bounded poll for `target` arrivals, as one thread of a CTA does them.
-// Returns false when the limit ran out (or the CTA's abort flag went up) before the counter got there.
+// Returns false when the limit ran out before the counter got there, or the CTA's abort flag was up at the last look.
 __device__ __forceinline__ bool arrive_and_poll(unsigned long long* ctr, unsigned long long target, long long limit,
                                                 const volatile int* abort_flag) {
   // arrive: release-add without waiting for the old value (the writes of the whole CTA, made visible to this
   // thread by the bar.sync in front, are ordered before it); then poll with acquire loads
   asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(ctr), "l"(1ULL) : "memory");
   const long long t0 = clock64();
-  while (ld_acquire_u64(ctr) < target) {
-    if (abort_flag && *abort_flag) return false;
+  for (;;) {
+    const int aborted = abort_flag ? *abort_flag : 0;     // beside the poll: no latency of its own
+    const bool there = ld_acquire_u64(ctr) >= target;
+    if (aborted) return false;
+    if (there) return true;
     if (clock64() - t0 > limit) return false;
   }
-  return true;
 }
 
-// Workers only.  Returns false if the CTA aborted.  `wrote_operand`: this CTA wrote activations that other
-// CTAs read with TMA after the barrier, so its global writes are ordered before the async proxy's reads.
+// Workers only.  Returns false if the CTA aborted, in all of them or in none: any role may raise the flag at any time, so one
+// thread looks at it between the two barriers and the others take what it found.
+// `wrote_operand`: this CTA wrote activations that other CTAs read with TMA after the barrier, so its global writes are
+// ordered before the async proxy's reads.
 // The barrier after a projection publishes only fp32 partials, which are read with ordinary loads: there the
 // proxy fence is left out (with bulk copies of the weight ring in flight it took about 2 us per barrier).
 __device__ __forceinline__ bool grid_barrier(const MegaArgs& a, MegaSmem* sm, unsigned long long& epoch, int wtid,
@@ -203,13 +209,13 @@ __device__ __forceinline__ bool grid_barrier(const MegaArgs& a, MegaSmem* sm, un
   ++epoch;
   if (wtid == 0) {
     const unsigned long long target = a.grid_base + epoch * gridDim.x;
-    if (!arrive_and_poll(a.grid_ctr, target, a.wait_limit, &sm->abort) && !sm->abort) {
-      atomicCAS(a.status, 0u, (uint32_t)kStatusGridBarrierTimeout);
-      sm->abort = 1;
+    if (!arrive_and_poll(a.grid_ctr, target, a.wait_limit, &sm->abort)) {
+      if (!sm->abort) atomicCAS(a.status, 0u, (uint32_t)kStatusGridBarrierTimeout);
+      sm->abort = sm->leave = 1;
     }
   }
   named_bar_workers();
-  return sm->abort == 0;
+  return sm->leave == 0;
 }
 
 // The stages between projections are chains of dependent L2 round trips (~0.7 us each), not bandwidth: the
@@ -1268,6 +1274,7 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
     sm->w_issued = 0;
     sm->act_epoch = 0;
     sm->abort = 0;
+    sm->leave = 0;
     fence_barrier_init();
     tma_prefetch_desc(&map_x);
     tma_prefetch_desc(&map_o);
@@ -1464,14 +1471,13 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
       mega_range(gs, part, it0, it1);
       long long it = it0;
       int seg_local = 0;
-      while (it < it1 && ok) {
+      while (it < it1) {
         const int tile = (int)(it / gs.kb);
         long long seg_end = (long long)(tile + 1) * gs.kb;
         if (seg_end > it1) seg_end = it1;
         const int buf = seg & 1;
-        ok = mega_wait(smem_u32(&sm->acc_full[buf]), (uint32_t)((seg >> 1) & 1), sm, a.status, kStatusEpilogueTimeout, a.wait_limit);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
+        const bool full = mega_wait(smem_u32(&sm->acc_full[buf]), (uint32_t)((seg >> 1) & 1), sm, a.status, kStatusEpilogueTimeout, a.wait_limit);
+        if (!__all_sync(0xffffffffu, full)) break;             // aborted: this warp goes on to the next grid barrier, where all leave
         tc_fence_after();
         const size_t slot = (size_t)part * gs.max_seg + seg_local;
         // batch rows held by this warp's lanes: 32 per lane quarter (16 with the 64-row instruction), on pairs as far as the
@@ -1537,14 +1543,11 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
         ++seg;
         ++seg_local;
       }
-      if (!ok) break;
       if (tracer) a.trace[tr++] = global_timer_ns();       // this CTA's accumulators drained
-      if constexpr (FLAG) {
-        ok = sm->abort == 0;
-      } else {
+      if constexpr (!FLAG) {
         ok = grid_barrier(a, sm, epoch, wtid, false);
+        if (!ok) break;
       }
-      if (!ok) break;
       if (tracer) a.trace[tr++] = global_timer_ns();       // every CTA's partials visible (FLAG: the stage looks for them)
       // ---- the stage that consumes the projection
       if (type == 0) {
@@ -1578,6 +1581,39 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
     if constexpr (PAIR) tmem_dealloc_pair(tmem_base, kTmemCols);
     else tmem_dealloc(tmem_base, kTmemCols);
   }
+}
+
+// Self-test of the workers' way out: eight worker warps that come to one grid barrier after the other at different times,
+// and a ninth warp that raises the abort flag in between, at another time in every CTA.  All eight must have passed the
+// same number of barriers; *torn counts the CTAs where they have not.
+constexpr int kLeaveSelftestThreads = kMegaWorkers + 32;
+__global__ void __launch_bounds__(kLeaveSelftestThreads, 1)
+leave_selftest_kernel(const __grid_constant__ MegaArgs a, uint32_t* torn) {
+  __shared__ MegaSmem smem;
+  MegaSmem* sm = &smem;
+  if (threadIdx.x == 0) sm->abort = sm->leave = 0;
+  __syncthreads();
+  const int wid = threadIdx.x >> 5;
+  auto pause = [](long long cycles) {
+    const long long t0 = clock64();
+    while (clock64() - t0 < cycles) { }
+  };
+  if (wid < 8) {
+    unsigned long long epoch = 0;
+    bool ok = true;
+    while (ok) {
+      pause(((unsigned)(wid * 5 + blockIdx.x) * 7u + (unsigned)epoch * 3u) % 8u * 150u);
+      ok = grid_barrier(a, sm, epoch, threadIdx.x, false);
+    }
+    if ((threadIdx.x & 31) == 0) sm->prefix[wid] = (int)epoch;
+  } else if (threadIdx.x == kMegaWorkers) {
+    pause(60000 + 37 * (long long)blockIdx.x);             // some dozens of barriers
+    sm->abort = 1;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int w = 1; w < 8; ++w)
+      if (sm->prefix[w] != sm->prefix[0]) { atomicAdd(torn, 1u); break; }
 }
 
 // Self-test of the bounded grid-wide wait, with nothing else in flight (no bulk copies, no tensor-core work): every

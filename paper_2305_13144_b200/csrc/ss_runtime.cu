@@ -1382,6 +1382,27 @@ int ss_set_wait_limit_ms(ss_ctx* c, int32_t ms) {
 int ss_selftest_wait_timeout(ss_ctx* c, int32_t limit_us) {
   if (!c || limit_us < 1 || limit_us > 1000000) return SS_ERR_ARG;
   if (c->in_batch) return SS_ERR_STATE;
+  // the workers of an abandoned step leave together
+  {
+    MegaArgs a{};
+    a.grid_ctr = c->grid_ctr;
+    a.grid_base = c->grid_epochs * (unsigned long long)c->n_sm;
+    a.status = c->status;
+    a.wait_limit = c->wait_limit;
+    uint32_t* torn = c->status + 1;
+    SS_CUDA(c, cudaMemsetAsync(torn, 0, 4, c->stream));
+    void* args[2] = {(void*)&a, (void*)&torn};
+    SS_CUDA(c, cudaLaunchCooperativeKernel((const void*)leave_selftest_kernel, dim3(c->n_sm), dim3(kLeaveSelftestThreads), args, 0, c->stream));
+    c->launches++;
+    SS_CUDA(c, cudaMemcpyAsync(c->pinned + 1, c->status, 8, cudaMemcpyDeviceToHost, c->stream));
+    SS_CUDA(c, cudaStreamSynchronize(c->stream));
+    const bool clean = c->pinned[1] == 0 && c->pinned[2] == 0;
+    reset_grid(c);
+    if (!clean) {
+      SS_CUDA(c, cudaMemsetAsync(c->status, 0, 4, c->stream));
+      return SS_OK;                    // an abort does not end as it should
+    }
+  }
   const long long limit = (long long)limit_us * c->clock_khz / 1000;
   unsigned long long base = c->grid_epochs * (unsigned long long)c->n_sm;
   unsigned long long* ctr = c->grid_ctr;

@@ -32,6 +32,16 @@ def test_wait_that_runs_out_is_reported_and_the_context_recovers():
     assert res["len"].tolist() == g.true_len.tolist()
 
 
+def test_workers_of_an_abandoned_step_leave_together():
+    """The abort flag goes up at another time in every CTA, between and inside the workers' barriers: all eight warps of a
+    CTA leave at the same one (the self-test reports a failure of its own otherwise)."""
+    from paper_2305_13144_b200 import api
+    shape = synth.TINY.with_layers(1)
+    eng = engine(shape, synth.make_weights(shape, seed=2))
+    for _ in range(20):
+        assert api.ss_selftest_wait_timeout(eng, 20) == api.SS_ERR_DEVICE_TIMEOUT
+
+
 def test_selftest_is_refused_while_a_batch_is_in_flight_and_limits_are_checked():
     from paper_2305_13144_b200 import api
     shape = synth.TINY.with_layers(1)
