@@ -116,6 +116,7 @@ struct MegaSmem {
   uint64_t empty[kMegaMaxStages];
   uint64_t acc_full[2];
   uint64_t acc_empty[2];
+  uint64_t mma_done;               // an abandoned step's last MMAs have ended
   uint32_t tmem_base;
   volatile int w_issued;           // ring iterations armed by the weight producer
   volatile int act_epoch;          // projections whose activation operand is complete
@@ -1271,6 +1272,7 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
       mbar_init(smem_u32(&sm->acc_empty[b]), PAIR ? 16 : 8);   // every worker warp (pairs: of both CTAs, used in the first)
     }
     for (int b = 0; b < 8 * kKvMaxPieces; ++b) mbar_init(smem_u32(&sm->kv_full[0][0] + b), 1);
+    mbar_init(smem_u32(&sm->mma_done), 1);
     sm->w_issued = 0;
     sm->act_epoch = 0;
     sm->abort = 0;
@@ -1438,6 +1440,14 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
           else umma_commit(smem_u32(&sm->acc_full[buf]));
           ++seg;
         }
+      }
+      if (!ok) {
+        // The step was abandoned, perhaps by another role right behind an issue: the MMAs in flight read the ring and write
+        // the accumulators, and get a bounded time to end before either is given up.
+        if constexpr (PAIR) umma_commit_pair(smem_u32(&sm->mma_done));
+        else umma_commit(smem_u32(&sm->mma_done));
+        const long long t0 = clock64();
+        while (!mbar_try_wait(smem_u32(&sm->mma_done), 0) && clock64() - t0 < 2000000LL) __nanosleep(100);
       }
     }
   } else if (warp >= 3) {
