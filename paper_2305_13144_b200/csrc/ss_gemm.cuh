@@ -50,14 +50,27 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Bounded wait: gives up after ~2 s of SM clock, records `code` and returns false.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t* status, uint32_t code) {
+// Bounded wait: gives up after `limit` SM cycles, records `code` and returns false.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t* status, uint32_t code, long long limit) {
   if (mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
   for (;;) {
     if (mbar_try_wait(bar, parity)) return true;
-    if (clock64() - t0 > 4000000000LL) {
+    if (clock64() - t0 > limit) {
       atomicCAS(status, 0u, code);
+      return false;
+    }
+  }
+}
+// Bounded wait, by one thread, for a word that another SM sets with release.
+__device__ __forceinline__ bool flag_wait(const uint32_t* flag, uint32_t* status, long long limit) {
+  const long long t0 = clock64();
+  for (;;) {
+    uint32_t f;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(f) : "l"(flag) : "memory");
+    if (f != 0u) return true;
+    if (clock64() - t0 > limit) {
+      atomicCAS(status, 0u, (uint32_t)kStatusFlagTimeout);
       return false;
     }
   }
@@ -346,7 +359,7 @@ gemm_wx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       for (int i = pre; i < n_it; ++i) {
         const long long it = it0 + i;
         const int tile = (int)(it / p.kb), kblk = (int)(it % p.kb);
-        if (!mbar_wait(smem_u32(&hdr->empty[stage]), phase ^ 1u, a.status, kStatusProducerTimeout)) break;
+        if (!mbar_wait(smem_u32(&hdr->empty[stage]), phase ^ 1u, a.status, kStatusProducerTimeout, a.wait_limit)) break;
         const uint32_t full = smem_u32(&hdr->full[stage]);
         mbar_expect_tx(full, stage_bytes);
         if (w_tiled) bulk_load(stage0 + stage * stage_bytes, w_block(tile, kblk), a_bytes, full, hint_w);
@@ -382,13 +395,13 @@ gemm_wx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         const int buf = seg & 1;
         const uint32_t use = (uint32_t)(seg >> 1);
         // wait until the epilogue has drained this accumulator buffer (first use passes at once)
-        ok = mbar_wait(smem_u32(&hdr->acc_empty[buf]), (use & 1u) ^ 1u, a.status, kStatusMmaTimeout);
+        ok = mbar_wait(smem_u32(&hdr->acc_empty[buf]), (use & 1u) ^ 1u, a.status, kStatusMmaTimeout, a.wait_limit);
         if (!ok) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(buf * p.NT);
         bool first = true;
         for (; it < seg_end; ++it) {
-          ok = mbar_wait(smem_u32(&hdr->full[stage]), phase, a.status, kStatusMmaTimeout);
+          ok = mbar_wait(smem_u32(&hdr->full[stage]), phase, a.status, kStatusMmaTimeout, a.wait_limit);
           if (!ok) break;
           tc_fence_after();
           const uint32_t sa = stage0 + stage * stage_bytes;
@@ -421,7 +434,7 @@ gemm_wx_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       if (seg_end > it1) seg_end = it1;
       const int buf = seg & 1;
       const uint32_t use = (uint32_t)(seg >> 1);
-      bool ok = mbar_wait(smem_u32(&hdr->acc_full[buf]), use & 1u, a.status, kStatusEpilogueTimeout);
+      bool ok = mbar_wait(smem_u32(&hdr->acc_full[buf]), use & 1u, a.status, kStatusEpilogueTimeout, a.wait_limit);
       ok = __all_sync(0xffffffffu, ok);           // warp-uniform, and reconverges the warp
       if (!ok) break;
       tc_fence_after();
@@ -696,7 +709,7 @@ gemm_wx_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
           phase = pre == p.stages ? 1u : 0u;
         }
         for (; i < s.k1; ++i, ++gi) {
-          if (gi >= p.stages && !(ok = mbar_wait(smem_u32(&hdr->empty[stage]), phase ^ 1u, a.status, kStatusProducerTimeout))) break;
+          if (gi >= p.stages && !(ok = mbar_wait(smem_u32(&hdr->empty[stage]), phase ^ 1u, a.status, kStatusProducerTimeout, a.wait_limit))) break;
           load_w(stage, i);
           load_x(stage, i);
           if (++stage == p.stages) { stage = 0; phase ^= 1u; }
@@ -711,6 +724,7 @@ gemm_wx_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
   } else if (warp == 1) {
     // ===================== MMA issuer (first CTA of the pair only) =====================
     if (lane == 0 && rank == 0) {
+      pdl_wait();                                        // the kernel in front does not count against the limit
       const uint32_t idesc = umma_idesc_bf16(p.NT, 256);
       int stage = 0;
       uint32_t phase = 0;
@@ -718,12 +732,12 @@ gemm_wx_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
       for (int r = 0; ok && walk.next(p, n_pairs, s); ++r) {
         const int buf = r & 1;
         // both CTAs' epilogues have drained this buffer (its first use passes at once)
-        ok = mbar_wait(smem_u32(&hdr->acc_empty[buf]), ((uint32_t)(r >> 1) & 1u) ^ 1u, a.status, kStatusMmaTimeout);
+        ok = mbar_wait(smem_u32(&hdr->acc_empty[buf]), ((uint32_t)(r >> 1) & 1u) ^ 1u, a.status, kStatusMmaTimeout, a.wait_limit);
         if (!ok) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(buf * kPairTokens);
         for (int i = s.k0; i < s.k1; ++i) {
-          ok = mbar_wait(smem_u32(&hdr->full[stage]), phase, a.status, kStatusMmaTimeout);
+          ok = mbar_wait(smem_u32(&hdr->full[stage]), phase, a.status, kStatusMmaTimeout, a.wait_limit);
           if (!ok) break;
           tc_fence_after();
           const uint32_t sa = stage0 + (uint32_t)stage * stage_bytes;
@@ -748,7 +762,7 @@ gemm_wx_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
       const int buf = r & 1;
       const int tok0 = s.tt * p.NT;
       const int n_valid = min(a.n_tok - tok0, p.NT);
-      bool ok = mbar_wait(smem_u32(&hdr->acc_full[buf]), (uint32_t)(r >> 1) & 1u, a.status, kStatusEpilogueTimeout);
+      bool ok = mbar_wait(smem_u32(&hdr->acc_full[buf]), (uint32_t)(r >> 1) & 1u, a.status, kStatusEpilogueTimeout, a.wait_limit);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
@@ -772,21 +786,8 @@ gemm_wx_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_cons
         if (s.k1 < p.kb) {
           // ranges behind this one until the unit's end
           while (PairWalk::pair_range(p, q + 1 + pp.n_more) < (s.unit + 1) * p.kb) ++pp.n_more;
-          if (lane == 0) {
-            for (int m = 1; m <= pp.n_more && ok; ++m) {
-              const long long t0 = clock64();
-              for (;;) {
-                uint32_t f;
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(f) : "l"(flag + m * 16) : "memory");
-                if (f != 0u) break;
-                if (clock64() - t0 > 4000000000LL) {
-                  atomicCAS(a.status, 0u, (uint32_t)kStatusFlagTimeout);
-                  ok = false;
-                  break;
-                }
-              }
-            }
-          }
+          if (lane == 0)
+            for (int m = 1; m <= pp.n_more && ok; ++m) ok = flag_wait(flag + m * 16, a.status, a.wait_limit);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           __syncwarp();                                     // lane 0's acquire holds for every lane's reads

@@ -37,6 +37,9 @@ enum : uint32_t {
   kStatusFlagTimeout = 6,
 };
 
+// SM cycles (about 2 s) that any wait inside a kernel may last unless ss_set_wait_limit_ms() says otherwise.
+constexpr long long kDefaultWaitLimit = 4000000000LL;
+
 // ---- GEMM:  D[n_out, tok] = W[n_out, K] . X[tok, K]^T  -------------------------------------
 // gemm_wx_kernel: the tile-iteration space (n_tiles x kb) is cut into `gridx` equal contiguous ranges, one per CTA (split
 // along K where a range ends inside a tile); every (CTA, tile) segment is written as an fp32 partial and the consumer
@@ -75,6 +78,7 @@ struct GemmArgs {
   void* kv_layer;              // the layer's pages
   size_t page_elems;
   uint32_t* status;
+  long long wait_limit;        // SM cycles after which a wait inside the kernel gives up
 };
 
 // Where the partial sums of one 128-row tile live: the first segment in slot `slot0`, the others

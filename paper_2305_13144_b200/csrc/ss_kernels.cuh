@@ -484,7 +484,7 @@ struct AttnPrefillSmem {
 template <int DH>
 __global__ void __launch_bounds__(128, 2)
 attn_prefill_kernel(const __grid_constant__ CUtensorMap map_qkv, const int32_t* __restrict__ cu_seqlens, bf16* __restrict__ out, int d,
-                    uint32_t* status) {
+                    uint32_t* status, long long limit) {
   constexpr int NB = DH / 64;                      // 64-column blocks per operand row
   constexpr uint32_t kTmemCols = 256;              // scores, then outputs
   extern __shared__ uint8_t smem_raw[];
@@ -539,7 +539,7 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap map_qkv, const int32_t* 
   uint32_t n_load = 0, n_mma = 0;
   bool ok = true;
   for (int kt0 = 0; kt0 < k_end; kt0 += kAttnTile) {
-    ok = mbar_wait(loaded, n_load++ & 1u, status, kStatusProducerTimeout);
+    ok = mbar_wait(loaded, n_load++ & 1u, status, kStatusProducerTimeout, limit);
     if (ok && threadIdx.x == 0) {
       tc_fence_after();
       const uint32_t idesc = umma_idesc_bf16(kAttnTile);
@@ -551,7 +551,7 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap map_qkv, const int32_t* 
       }
       umma_commit(mma_done);
     }
-    ok = ok && mbar_wait(mma_done, n_mma++ & 1u, status, kStatusMmaTimeout);
+    ok = ok && mbar_wait(mma_done, n_mma++ & 1u, status, kStatusMmaTimeout, limit);
     if (!__syncthreads_and(ok)) { ok = false; break; }
     tc_fence_after();
     // keys this row may see in the step: all, or up to its own position (rows beyond the prompt are never stored)
@@ -606,7 +606,7 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap map_qkv, const int32_t* 
                   smem_desc_mn_sw128(v_s + (uint32_t)(kk * 2048), kAttnBlock), idesc, kk ? 1u : 0u);
       umma_commit(mma_done);
     }
-    ok = mbar_wait(mma_done, n_mma++ & 1u, status, kStatusMmaTimeout);
+    ok = mbar_wait(mma_done, n_mma++ & 1u, status, kStatusMmaTimeout, limit);
     if (!__syncthreads_and(ok)) { ok = false; break; }
     if (threadIdx.x == 0 && kt0 + kAttnTile < k_end) load_kv(kt0 + kAttnTile, 0);
     tc_fence_after();

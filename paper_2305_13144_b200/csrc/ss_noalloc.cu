@@ -242,6 +242,7 @@ extern "C" int ss_logits_noalloc(const float* hidden, const void* norm_gain, con
   a.n_tok = n_rows;
   a.partial = partial;
   a.status = status;
+  a.wait_limit = kDefaultWaitLimit;
   if (launch_after(early, gemm_wx_kernel, dim3(p.gridx), dim3(kGemmThreads), (size_t)p.smem_bytes, st, mw, mx, a) != cudaSuccess) return SS_ERR_CUDA;
   SplitInfo sp;
   sp.gridx = p.gridx; sp.kb = p.kb; sp.max_seg = p.max_seg; sp.NT = p.NT; sp.total = total; sp.tiles = nullptr;

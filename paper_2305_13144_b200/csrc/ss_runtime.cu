@@ -130,7 +130,7 @@ struct ss_ctx {
   int n_sm = 0;
   bool use_pdl = true;
   bool trace_on = false;
-  long long wait_limit = 4000000000LL;   // SM cycles (about 2 s) any wait inside a kernel may last
+  long long wait_limit = kDefaultWaitLimit;   // SM cycles any wait inside a kernel may last
   int clock_khz = 1965000;
   int last_cuda = 0;
   int64_t launches = 0;
@@ -321,6 +321,7 @@ int run_gemm(ss_ctx* c, const uint8_t* w_tiled, const CUtensorMap& mx, const Gem
   a.n_tok = n_tok;
   a.partial = c->partial;
   a.status = c->status;
+  a.wait_limit = c->wait_limit;
   if ((size_t)p.gridx * p.max_seg * p.NT * 128 * sizeof(float) > c->partial_bytes) return SS_ERR_CAPACITY;
   // the weight tensor map is unused with tiled weights; the activation map stands in for it
   SS_CUDA(c, launch(c, gemm_wx_kernel, dim3(p.gridx), dim3(kGemmThreads), (size_t)p.smem_bytes, mx, mx, a));
@@ -362,6 +363,8 @@ int run_gemm_pair(ss_ctx* c, const CUtensorMap& mw, const CUtensorMap& mx, const
   a.p = p;
   a.partial = c->partial;
   a.pair_flag = c->pair_flag;
+  a.status = c->status;
+  a.wait_limit = c->wait_limit;
   SS_CUDA(c, launch(c, gemm_wx_pair_kernel, dim3(2 * a.p.gridx), dim3(kPairThreads), (size_t)a.p.smem_bytes, mw, mx, a));
   return SS_OK;
 }
@@ -673,16 +676,13 @@ int enqueue_prefill_chunk(ss_ctx* c, int s0, int s1, const int32_t* cu, int T) {
   qkv.tok_pos = c->d_tok_pos;
   qkv.tok_slot = c->d_tok_slot;
   qkv.page_elems = c->kv.page_elems;
-  qkv.status = c->status;
   GemmArgs res{}, glu{};
   res.mode = kGemmResidual;
   res.n_tok = T;
   res.residual = c->h;
-  res.status = c->status;
   glu.mode = kGemmSwiglu;
   glu.n_tok = T;
   glu.out = c->act;
-  glu.status = c->status;
   // more than one token tile of a pair: the paired kernel; up to it, the projections are split over the SMs along K too
   const bool pair = T > kShortTokens;
   const int shp[4][2] = {{3 * d, d}, {d, d}, {2 * F, d}, {d, F}};
@@ -698,9 +698,9 @@ int enqueue_prefill_chunk(ss_ctx* c, int s0, int s1, const int32_t* cu, int T) {
   auto attend = [&]() -> int {
     const dim3 ag(ceil_div(max_len, kAttnTile), H, nseq);
     if (Dh == 128)
-      SS_CUDA(c, launch(c, attn_prefill_kernel<128>, ag, dim3(128), (size_t)attn_prefill_smem<128>(), *mq, (const int32_t*)c->d_cu, c->attn_o, d, c->status));
+      SS_CUDA(c, launch(c, attn_prefill_kernel<128>, ag, dim3(128), (size_t)attn_prefill_smem<128>(), *mq, (const int32_t*)c->d_cu, c->attn_o, d, c->status, c->wait_limit));
     else
-      SS_CUDA(c, launch(c, attn_prefill_kernel<64>, ag, dim3(128), (size_t)attn_prefill_smem<64>(), *mq, (const int32_t*)c->d_cu, c->attn_o, d, c->status));
+      SS_CUDA(c, launch(c, attn_prefill_kernel<64>, ag, dim3(128), (size_t)attn_prefill_smem<64>(), *mq, (const int32_t*)c->d_cu, c->attn_o, d, c->status, c->wait_limit));
     return SS_OK;
   };
   const bf16* first_norm = m.n_layers ? c->layers[0].attn_norm : c->final_norm;

@@ -14,6 +14,8 @@
 
 #include <cuda_runtime.h>
 
+#include "ss_internal.h"
+
 namespace {
 struct Op {
   enum Kind { kCopy, kCopy2D, kSet, kKernel, kEvent } kind;
@@ -70,9 +72,12 @@ cudaError_t waited() {                    // the next wait reports an error, onc
   return e;
 }
 void add(Op op) { queue.push_back(std::move(op)); ++enqueued; }
-void add_kernel(const void* fn) {
+std::map<std::string, long long> wait_limits;            // what the prompt-pass kernels were last told, by name
+void add_kernel(const void* fn, void** args) {
   Op op{Op::kKernel};
   op.name = kernel_names()[fn];
+  if (op.name.find("gemm_wx") != std::string::npos) wait_limits[op.name] = ((const ss::GemmArgs*)args[2])->wait_limit;
+  if (op.name.find("attn_prefill") != std::string::npos) wait_limits[op.name] = *(const long long*)args[5];
   add(op);
 }
 int encode_tiled(...) { return 0; }
@@ -82,6 +87,12 @@ extern "C" {
 // ---- what a test asks
 int64_t fake_changed_sources() { return changed_sources; }
 void fake_fail_wait_behind(const char* part, int error) { bad_kernel = part; bad_kernel_error = (cudaError_t)error; }
+// The limit (SM cycles) that the last launch of the kernel was given, -1 if there was none.
+int64_t fake_wait_limit(const char* part) {
+  for (const auto& w : wait_limits)
+    if (w.first.find(part) != std::string::npos) return w.second;
+  return -1;
+}
 // Launches of kernels whose (mangled) name contains `part` that have not been executed.
 int64_t fake_pending(const char* part) {
   int64_t n = 0;
@@ -116,9 +127,9 @@ cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return c
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { *p = std::calloc(n, 1); return *p ? cudaSuccess : cudaErrorMemoryAllocation; }
 cudaError_t cudaFreeHost(void* p) { std::free(p); return cudaSuccess; }
 
-cudaError_t cudaLaunchKernel(const void* fn, dim3, dim3, void**, size_t, cudaStream_t) { add_kernel(fn); return cudaSuccess; }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t*, const void* fn, void**) { add_kernel(fn); return cudaSuccess; }
-cudaError_t cudaLaunchCooperativeKernel(const void* fn, dim3, dim3, void**, size_t, cudaStream_t) { add_kernel(fn); return cudaSuccess; }
+cudaError_t cudaLaunchKernel(const void* fn, dim3, dim3, void** args, size_t, cudaStream_t) { add_kernel(fn, args); return cudaSuccess; }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t*, const void* fn, void** args) { add_kernel(fn, args); return cudaSuccess; }
+cudaError_t cudaLaunchCooperativeKernel(const void* fn, dim3, dim3, void** args, size_t, cudaStream_t) { add_kernel(fn, args); return cudaSuccess; }
 cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) { *s = cudaStreamCaptureStatusNone; return cudaSuccess; }
 
 cudaError_t cudaMemcpyAsync(void* dst, const void* src, size_t n, cudaMemcpyKind kind, cudaStream_t) {

@@ -28,6 +28,7 @@ def fake(tmp_path_factory):
         L = api.lib()
         L.fake_changed_sources.restype = L.fake_pending.restype = C.c_int64
         L.fake_pending.argtypes = [C.c_char_p]
+        L.fake_wait_limit.restype, L.fake_wait_limit.argtypes = C.c_int64, [C.c_char_p]
         L.fake_fail_wait_behind.argtypes = [C.c_char_p, C.c_int]
         yield L
 
@@ -86,6 +87,21 @@ def test_prompt_pass_returns_behind_its_layers(fake):
     assert e.value.code == api.SS_ERR_CUDA and api.ss_last_cuda_error(eng) == 719
     api.ss_prefill(eng, toks, cu, None, 4)                 # the failed batch was released
     api.ss_release_batch(eng)
+    api.ss_destroy(eng)
+
+
+def test_the_wait_limit_reaches_the_prompt_pass(fake):
+    """Both GEMMs (chunks of up to 256 tokens and longer ones) and the attention."""
+    eng = _engine(fake, max_prefill=512)
+    for ms in (7, 50):
+        api.ss_set_wait_limit_ms(eng, ms)
+        for lens in ([20, 30], [60] * 6):
+            toks, cu = _batch(4, lens)
+            api.ss_prefill(eng, toks, cu, None, 4)
+            api.ss_release_batch(eng)
+        for kernel in (b"gemm_wx_kernel", b"gemm_wx_pair_kernel", b"attn_prefill"):
+            assert fake.fake_wait_limit(kernel) == ms * 1965000, kernel
+    api.ss_last_device_status(eng)
     api.ss_destroy(eng)
 
 
