@@ -230,46 +230,46 @@ __device__ __forceinline__ float ldcg_now(const float* p) {
   return v;
 }
 
-template <int N>
+// Partial sums, read past L1.  FLAG: words that one SM writes while another looks at them are read (and written, st_partial)
+// with relaxed accesses at gpu scope: a plain load need neither see a store ever nor read a word whole.  Nothing is ordered by
+// them and nothing has to be, since only the words themselves are used; so they clobber no memory either (with a clobber and a
+// predicate on every load 16 rows of the 7B shape, 32 layers, took 25340 us a call of 8 steps, without 25220, weak accesses 25190).
+template <bool FLAG, int N>
 __device__ __forceinline__ void ldcg_vec(const float* p, float (&x)[N]) {
-  static_assert(N == 2 || N == 4 || N == 8, "N");
-  if constexpr (N == 2) {
-    asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];" : "=f"(x[0]), "=f"(x[1]) : "l"(p));
-  } else {
-#pragma unroll
-    for (int i = 0; i < N; i += 4)
-      asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];"
-                   : "=f"(x[i]), "=f"(x[i + 1]), "=f"(x[i + 2]), "=f"(x[i + 3])
-                   : "l"(p + i));
-  }
+  static_assert(N == 2 || N == 4, "N");
+  if constexpr (FLAG && N == 2) asm volatile("ld.relaxed.gpu.global.v2.f32 {%0, %1}, [%2];" : "=f"(x[0]), "=f"(x[1]) : "l"(p));
+  else if constexpr (FLAG) asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]) : "l"(p));
+  else if constexpr (N == 2) asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];" : "=f"(x[0]), "=f"(x[1]) : "l"(p));
+  else asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]) : "l"(p));
 }
 
-// The same where `on`, zeros elsewhere: no branch, so that the loads of a sum stay together, and no traffic.  (With the last
+// Into the same registers where `on`.
+template <int N>
+__device__ __forceinline__ void ld_partial_if(const float* p, bool on, float (&x)[N]) {
+  static_assert(N == 2 || N == 4, "N");
+  if constexpr (N == 2)
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\t@p ld.relaxed.gpu.global.v2.f32 {%0, %1}, [%2];\n\t}"
+                 : "+f"(x[0]), "+f"(x[1]) : "l"(p), "r"((int)on));
+  else
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %5, 0;\n\t@p ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
+                 : "+f"(x[0]), "+f"(x[1]), "+f"(x[2]), "+f"(x[3]) : "l"(p), "r"((int)on));
+}
+
+// Where `on`, zeros elsewhere: no branch, so that the loads of a sum stay together, and no traffic.  (With the last
 // segment read again in the place of those that a tile has not: 7B shape, 4 layers, 1 / 16 / 256 rows 400 / 462 / 1066 us a
 // step, now 396.5 / 458 / 1030; residual stages of 256 rows on pairs, whose tiles have half of the segments, 8.5 -> 5.2 us.)
-template <int N>
+template <bool FLAG, int N>
 __device__ __forceinline__ void ldcg_vec_if(const float* p, bool on, float (&x)[N]) {
   static_assert(N == 2 || N == 4, "N");
 #pragma unroll
   for (int i = 0; i < N; ++i) x[i] = 0.f;
-  if constexpr (N == 2)
+  if constexpr (FLAG) ld_partial_if<N>(p, on, x);
+  else if constexpr (N == 2)
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\t@p ld.global.cg.v2.f32 {%0, %1}, [%2];\n\t}"
                  : "+f"(x[0]), "+f"(x[1]) : "l"(p), "r"((int)on));
   else
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %5, 0;\n\t@p ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
                  : "+f"(x[0]), "+f"(x[1]), "+f"(x[2]), "+f"(x[3]) : "l"(p), "r"((int)on));
-}
-
-// Again into the same registers, where `on`.
-template <int N>
-__device__ __forceinline__ void ldcg_vec_again(const float* p, bool on, float (&x)[N]) {
-  static_assert(N == 2 || N == 4, "N");
-  if constexpr (N == 2)
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\t@p ld.global.cg.v2.f32 {%0, %1}, [%2];\n\t}"
-                 : "+f"(x[0]), "+f"(x[1]) : "l"(p), "r"((int)on) : "memory");
-  else
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %5, 0;\n\t@p ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
-                 : "+f"(x[0]), "+f"(x[1]), "+f"(x[2]), "+f"(x[3]) : "l"(p), "r"((int)on) : "memory");
 }
 
 // ---- partial sums that announce themselves (FLAG: the kernel of up to 16 rows).  Between two uses a slot holds kNoPartial in
@@ -282,6 +282,9 @@ __device__ __forceinline__ void ldcg_vec_again(const float* p, bool on, float (&
 // 64 rows 483 / 536 / 603 / 616 with a barrier, 487 / 534 / 608 / 650 without.  Fewer polls are no way out: one missing segment
 // at a time 399 / 423 / 460 at 1 / 8 / 16 rows, a sleep of 64 or 100 ns between looks 427 / 446 / 490 and more.
 constexpr uint32_t kNoPartial = 0xffffffffu;        // a NaN that no instruction produces (results are 0x7fffffff)
+__device__ __forceinline__ void st_partial(float* p, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.relaxed.gpu.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(a), "r"(b), "r"(c), "r"(d));
+}
 template <int N>
 __device__ __forceinline__ bool no_partial(const float (&x)[N]) {
   bool m = false;
@@ -316,13 +319,13 @@ struct PartialLoads {
   float x[N];
   float u[BATCH][N];
 };
-template <int N, int BATCH>
+template <bool FLAG, int N, int BATCH>
 __device__ __forceinline__ void partials_issue(const MegaArgs& a, const MegaGemmShape& s, const int4 t, int n0, int tok, PartialLoads<N, BATCH>& q) {
   const size_t slot_stride = (size_t)a.NT * kTileN, cta_stride = slot_stride * s.max_seg;
   const size_t off = (size_t)tok * kTileN + (n0 % kTileN);
-  ldcg_vec<N>(s.partial + (size_t)t.x * slot_stride + off, q.x);
+  ldcg_vec<FLAG, N>(s.partial + (size_t)t.x * slot_stride + off, q.x);
 #pragma unroll
-  for (int j = 0; j < BATCH; ++j) ldcg_vec_if<N>(s.partial + (size_t)(t.y + j) * cta_stride + off, t.y + j <= t.z, q.u[j]);
+  for (int j = 0; j < BATCH; ++j) ldcg_vec_if<FLAG, N>(s.partial + (size_t)(t.y + j) * cta_stride + off, t.y + j <= t.z, q.u[j]);
 }
 template <bool FLAG, int N, int BATCH>
 __device__ __forceinline__ void partials_sum(const MegaArgs& a, MegaSmem* sm, const MegaGemmShape& s, const int4 t, int n0, int tok,
@@ -336,9 +339,9 @@ __device__ __forceinline__ void partials_sum(const MegaArgs& a, MegaSmem* sm, co
     if (more) {
       const long long t0 = clock64();
       do {
-        ldcg_vec_again<N>(s.partial + (size_t)t.x * slot_stride + off, no_partial<N>(q.x), q.x);
+        ld_partial_if<N>(s.partial + (size_t)t.x * slot_stride + off, no_partial<N>(q.x), q.x);
 #pragma unroll
-        for (int j = 0; j < BATCH; ++j) ldcg_vec_again<N>(s.partial + (size_t)(t.y + j) * cta_stride + off, no_partial<N>(q.u[j]), q.u[j]);
+        for (int j = 0; j < BATCH; ++j) ld_partial_if<N>(s.partial + (size_t)(t.y + j) * cta_stride + off, no_partial<N>(q.u[j]), q.u[j]);
         more = no_partial<N>(q.x);
 #pragma unroll
         for (int j = 0; j < BATCH; ++j) more |= no_partial<N>(q.u[j]);
@@ -354,7 +357,7 @@ __device__ __forceinline__ void partials_sum(const MegaArgs& a, MegaSmem* sm, co
   for (int c = t.y + BATCH; c <= t.z; c += BATCH) {
     float u[BATCH][N];
 #pragma unroll
-    for (int j = 0; j < BATCH; ++j) ldcg_vec_if<N>(s.partial + (size_t)(c + j) * cta_stride + off, c + j <= t.z, u[j]);
+    for (int j = 0; j < BATCH; ++j) ldcg_vec_if<FLAG, N>(s.partial + (size_t)(c + j) * cta_stride + off, c + j <= t.z, u[j]);
     if constexpr (FLAG) {
       const long long t0 = clock64();
       for (;;) {
@@ -363,7 +366,7 @@ __device__ __forceinline__ void partials_sum(const MegaArgs& a, MegaSmem* sm, co
         for (int j = 0; j < BATCH; ++j) more |= no_partial<N>(u[j]);
         if (!more || !partial_wait_on(a, sm, t0)) break;
 #pragma unroll
-        for (int j = 0; j < BATCH; ++j) ldcg_vec_again<N>(s.partial + (size_t)(c + j) * cta_stride + off, no_partial<N>(u[j]), u[j]);
+        for (int j = 0; j < BATCH; ++j) ld_partial_if<N>(s.partial + (size_t)(c + j) * cta_stride + off, no_partial<N>(u[j]), u[j]);
       }
     }
 #pragma unroll
@@ -377,7 +380,7 @@ template <bool FLAG, int N, int BATCH>
 __device__ __forceinline__ void sum_partials_cg(const MegaArgs& a, MegaSmem* sm, const MegaGemmShape& s, int n0, int tok, float (&x)[N]) {
   const int4 t = tile_seg(sm, s, n0);
   PartialLoads<N, BATCH> q;
-  partials_issue<N, BATCH>(a, s, t, n0, tok, q);
+  partials_issue<FLAG, N, BATCH>(a, s, t, n0, tok, q);
   partials_sum<FLAG, N, BATCH>(a, sm, s, t, n0, tok, q, x);
 }
 // The slots that this CTA wrote for a projection, empty again.
@@ -819,9 +822,9 @@ __device__ void stage_attention(const MegaArgs& a, MegaSmem* sm, AttnScratch* sc
       const int e0 = lane * EPL, nq = hd * DH + e0, nk = d + nq, nv = 2 * d + nq;
       const int4 tq = tile_seg(sm, gs, nq), tk = tile_seg(sm, gs, nk), tv = tile_seg(sm, gs, nv);
       PartialLoads<EPL, 4> lq, lk, lv;
-      partials_issue<EPL, 4>(a, gs, tq, nq, r, lq);
-      partials_issue<EPL, 4>(a, gs, tk, nk, r, lk);
-      partials_issue<EPL, 4>(a, gs, tv, nv, r, lv);
+      partials_issue<FLAG, EPL, 4>(a, gs, tq, nq, r, lq);
+      partials_issue<FLAG, EPL, 4>(a, gs, tk, nk, r, lk);
+      partials_issue<FLAG, EPL, 4>(a, gs, tv, nv, r, lv);
       // the two dimensions of a rotation are neighbours (in the weights, so here and in the cache)
       const float2* rp = a.rope + (size_t)pos * (DH / 2) + lane * (EPL / 2);
       float2 cs[EPL / 2];
@@ -1100,7 +1103,7 @@ __device__ void stage_swiglu(const MegaArgs& a, MegaSmem* sm, int wtid) {
     for (int k = 0; k < 4; ++k) {
       const int n = n0 + 128 * k < 2 * a.F ? n0 + 128 * k : 0;       // lanes beyond the last feature read the first ones, store nothing
       ts[k] = tile_seg(sm, gs, n);
-      partials_issue<4, 2>(a, gs, ts[k], n, r, q[k]);
+      partials_issue<FLAG, 4, 2>(a, gs, ts[k], n, r, q[k]);
     }
     const float inv = warp_row_inv_rms(a, r, lane);
 #pragma unroll
@@ -1145,7 +1148,7 @@ __device__ void stage_tile_argmax(const MegaArgs& a, MegaSmem* sm, int wtid) {
         const int r = min(2 * rg + k, a.B - 1);
         ss[k] = row_ss_issue(a, r, lane);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) partials_issue<4, 2>(a, gs, ts, v0 + 128 * h, r, q[k][h]);
+        for (int h = 0; h < 2; ++h) partials_issue<FLAG, 4, 2>(a, gs, ts, v0 + 128 * h, r, q[k][h]);
         gen[k] = a.st.gen[r] + 1;
         row_key[k] = a.st.row_key[r];
         skip[k] = a.st.eos_at[r] > 0 ? a.eos_id : -1;
@@ -1513,7 +1516,7 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
               if (tok < a.B) {
 #pragma unroll
                 for (int j = 0; j < 64; j += 4)
-                  *reinterpret_cast<uint4*>(dst + c + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                  st_partial(dst + c + j, v[j], v[j + 1], v[j + 2], v[j + 3]);
               }
             } else {
               // many rows: a lane holds one token's outputs, so direct 128-bit stores put every lane's 16 bytes
