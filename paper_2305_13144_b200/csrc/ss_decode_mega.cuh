@@ -1479,6 +1479,7 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
       const int type = gm == n_gemm - 1 ? 4 : (gm & 3);
       const int layer = gm >> 2;
       const MegaGemmShape& gs = a.shape[type];
+      float* const partial = gs.partial;
       // ---- drain this CTA's segments of projection gm into fp32 partials
       long long it0, it1;
       mega_range(gs, part, it0, it1);
@@ -1501,7 +1502,7 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
         if (per_q > 0 && tok0 < a.B) {                         // else no batch row in this warp's lanes (warp-uniform)
           const int tok = lane < per_q ? tok0 + lane : a.B;
           const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * kTileN + colhalf * 128);
-          float* dst = gs.partial + (slot * a.NT + tok) * kTileN + colhalf * 128;
+          float* dst = partial + (slot * a.NT + tok) * kTileN + colhalf * 128;
           // 64 columns per TMEM load: the last segment's drain is the serial tail of every projection
 #pragma unroll 1
           for (int c = 0; c < 128; c += 64) {
@@ -1538,7 +1539,7 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
                 for (int i = 0; i < cap_q / 8; ++i) {
                   const int tl = 8 * i + t_hi;
                   if (tl < per_q && tok0 + tl < a.B)
-                    *reinterpret_cast<uint4*>(gs.partial + (slot * a.NT + tok0 + tl) * kTileN + colhalf * 128 + c + sub * 16 + 4 * cg) =
+                    *reinterpret_cast<uint4*>(partial + (slot * a.NT + tok0 + tl) * kTileN + colhalf * 128 + c + sub * 16 + 4 * cg) =
                         *reinterpret_cast<const uint4*>(tr + tl * kDrainPad + 4 * cg);
                 }
                 __syncwarp();
