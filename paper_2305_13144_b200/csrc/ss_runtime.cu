@@ -346,16 +346,19 @@ GemmPlan plan_pair(int n_out, int K, int n_tok, int n_sm, size_t partial_bytes) 
   const int fit = (int)std::max<size_t>(1, kPairGroupBytes / tile_bytes);
   p.group = ceil_div(p.tok_tiles, ceil_div(p.tok_tiles, fit));
   const int n_units = (p.n_tiles / 2) * p.tok_tiles, n_pairs = n_sm / 2;
-  // Up to two token tiles the last round of pairs (all of o's and down's units at the 7B shape) is cut along K if it would
-  // leave a good part of the pairs without a unit: 300 / 400 tokens, 6 layers, 1470 / 1510 -> 1250 / 1400 us.  With more
-  // tiles the cut gains nothing (768 and 1024 tokens, 1850 and 2400 us either way: the power cap gives what idle pairs leave
-  // to the others), and cutting one full round more besides costs 5 to 13 % from 768 to 3200 tokens: pairs that are not at
-  // the same k-block share no weights.
+  // Up to two token tiles the last round of pairs (all of o's and down's units at the 7B shape) is cut along K where that
+  // shortens it.  It would last kb k-blocks and lasts kb * rest / n_pairs; a unit's owner then adds the n_pairs / rest - 1
+  // parts that others have of it, about ten k-blocks' time each, and as much is lost on the way.  Whole calls of 258 and 510
+  // tokens, always cut / never / by this line: d 1024, 4 layers, 508 / 408 / 408 and 629 / 449 / 449 us (eight units in nine
+  // parts each); 32 x 64 heads 605 / 564 / 540 and 717 / 604 / 596; 7B shape 864 / 1004 / 864 and 1002 / 1070 / 998; 13B
+  // shape, 2 layers, 1094 / 1205 / 1092 and 1308 / 1322 / 1308.  With more tiles the cut gains nothing (768 and 1024 tokens,
+  // 1850 and 2400 us either way: the power cap gives what idle pairs leave to the others), and cutting one full round more
+  // besides costs 5 to 13 % from 768 to 3200 tokens: pairs that are not at the same k-block share no weights.
   const int rest = n_units % n_pairs;
-  p.split_units = p.tok_tiles <= 2 && rest <= n_pairs * 85 / 100 ? rest : 0;
-  const long long total = (long long)p.split_units * p.kb;
-  p.ranges = (int)std::min<long long>(std::min<long long>(n_pairs, std::max(1LL, total / 4)), (long long)(partial_bytes / ((size_t)p.NT * 1024)));
-  if (p.ranges < 1) p.split_units = p.ranges = 0;
+  p.split_units = p.tok_tiles <= 2 && (long long)p.kb * (n_pairs - rest) * rest > 10LL * n_pairs * n_pairs ? rest : 0;
+  // (each of the ranges then has more than ten k-blocks)
+  p.ranges = p.split_units ? (int)std::min<size_t>(n_pairs, partial_bytes / ((size_t)p.NT * 1024)) : 0;
+  if (p.ranges < 1) p.split_units = 0;
   p.gridx = std::min(n_pairs, std::max(p.ranges, n_units - p.split_units));
   return p;
 }

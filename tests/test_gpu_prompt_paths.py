@@ -31,9 +31,12 @@ def test_prompt_lengths_and_paths(heads, head_dim, ffn, lens):
 
 
 @pytest.mark.parametrize("heads,ffn,lens", [
-    (4, 1000, [257]),                            # two token tiles of 160 (the second with 97), ranges of four k-blocks
-    (16, 264, [200, 100]),                       # 48 units of the q,k,v projection over 74 ranges: one to three parts each
-    (16, 5000, [256, 256]),                      # two full tiles of 256
+    (4, 1000, [257]),                            # two token tiles of 160 (the second with 97), nothing cut
+    (16, 264, [200, 100]),                       # q,k,v: 48 units for 74 pairs, not cut either
+    (16, 5000, [256, 256]),                      # two full tiles of 256; down: 16 units in four to six parts each
+    (24, 264, [200, 100]),                       # o: 24 units in three or four parts each, over two tiles of 160
+    (32, 2000, [130, 127]),                      # q,k,v: a full round of pairs, then 22 units in parts; o and gate/up too
+    (8, 16384, [300]),                           # down: 8 units of 256 k-blocks in nine or ten parts each
     (2, 16384, [425, 425, 424, 426]),            # seven token tiles, the down projection's in groups of four and three
 ])
 def test_cut_and_grouped_projections_of_the_paired_path(heads, ffn, lens):
