@@ -572,6 +572,14 @@ const void* mega_kernel_fn_dh(int rows, bool trace) {
 const void* mega_kernel_fn(int head_dim, int rows, bool trace) {
   return head_dim == 128 ? mega_kernel_fn_dh<128>(rows, trace) : mega_kernel_fn_dh<64>(rows, trace);
 }
+// Loads the instantiations that a context can launch (naming a kernel here costs its load): those of its head size, and the
+// ones with the trace when a trace is asked for.  With all sixteen the first context of a process took 14 ms longer.
+cudaError_t prepare_mega_kernels(int head_dim, bool trace) {
+  cudaError_t e = cudaSuccess;
+  for (int rows : {16, 64, 128, 256})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(mega_kernel_fn(head_dim, rows, trace), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  return e;
+}
 
 // ------------------------------------------------------------------------------------ decode step
 // One cooperative launch of the persistent kernel (see ss_decode_mega.cuh).
@@ -973,9 +981,7 @@ int ss_create(const ss_model_cfg* model, const ss_runtime_cfg* rt, void* dev_are
     e = cudaFuncSetAttribute(attn_prefill_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_prefill_smem<128>());
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(attn_prefill_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_prefill_smem<64>());
-  for (int v = 0; v < 16 && e == cudaSuccess; ++v)
-    e = cudaFuncSetAttribute(mega_kernel_fn((v & 1) ? 128 : 64, v < 4 ? 16 : 32 << (v >> 2), (v & 2) != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             227 * 1024);
+  if (e == cudaSuccess) e = prepare_mega_kernels(model->head_dim, false);
   if (e != cudaSuccess) {
     if (c->pinned) cudaFreeHost(c->pinned);
     if (c->up_sent) cudaEventDestroy(c->up_sent);
@@ -1423,6 +1429,7 @@ int ss_selftest_wait_timeout(ss_ctx* c, int32_t limit_us) {
 
 int ss_set_trace(ss_ctx* c, int32_t on) {
   if (!c) return SS_ERR_ARG;
+  if (on) SS_CUDA(c, prepare_mega_kernels(c->m.head_dim, true));
   c->trace_on = on != 0;
   return SS_OK;
 }

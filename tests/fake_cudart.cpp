@@ -9,6 +9,7 @@
 #include <cstring>
 #include <deque>
 #include <map>
+#include <set>
 #include <string>
 #include <vector>
 
@@ -72,6 +73,7 @@ cudaError_t waited() {                    // the next wait reports an error, onc
   return e;
 }
 void add(Op op) { queue.push_back(std::move(op)); ++enqueued; }
+std::set<std::string> loaded_kernels;                   // kernels that an attribute was set for (a real one is loaded by that)
 std::map<std::string, long long> wait_limits;            // what the prompt-pass kernels were last told, by name
 void add_kernel(const void* fn, void** args) {
   Op op{Op::kKernel};
@@ -92,6 +94,13 @@ int64_t fake_wait_limit(const char* part) {
   for (const auto& w : wait_limits)
     if (w.first.find(part) != std::string::npos) return w.second;
   return -1;
+}
+// Kernels loaded since the last call whose (mangled) name contains `part`.
+int64_t fake_loaded(const char* part) {
+  int64_t n = 0;
+  for (const std::string& k : loaded_kernels) n += k.find(part) != std::string::npos;
+  loaded_kernels.clear();
+  return n;
 }
 // Launches of kernels whose (mangled) name contains `part` that have not been executed.
 int64_t fake_pending(const char* part) {
@@ -123,7 +132,7 @@ cudaError_t cudaGetDriverEntryPoint(const char*, void** fn, unsigned long long, 
   *fn = (void*)&encode_tiled;
   return cudaSuccess;
 }
-cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaFuncSetAttribute(const void* fn, cudaFuncAttribute, int) { loaded_kernels.insert(kernel_names()[fn]); return cudaSuccess; }
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { *p = std::calloc(n, 1); return *p ? cudaSuccess : cudaErrorMemoryAllocation; }
 cudaError_t cudaFreeHost(void* p) { std::free(p); return cudaSuccess; }
 

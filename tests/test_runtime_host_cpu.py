@@ -28,6 +28,7 @@ def fake(tmp_path_factory):
         L = api.lib()
         L.fake_changed_sources.restype = L.fake_pending.restype = C.c_int64
         L.fake_pending.argtypes = [C.c_char_p]
+        L.fake_loaded.restype, L.fake_loaded.argtypes = C.c_int64, [C.c_char_p]
         L.fake_wait_limit.restype, L.fake_wait_limit.argtypes = C.c_int64, [C.c_char_p]
         L.fake_fail_wait_behind.argtypes = [C.c_char_p, C.c_int]
         yield L
@@ -102,6 +103,18 @@ def test_the_wait_limit_reaches_the_prompt_pass(fake):
         for kernel in (b"gemm_wx_kernel", b"gemm_wx_pair_kernel", b"attn_prefill"):
             assert fake.fake_wait_limit(kernel) == ms * 1965000, kernel
     api.ss_last_device_status(eng)
+    api.ss_destroy(eng)
+
+
+def test_a_context_loads_the_kernels_that_it_can_launch(fake):
+    """Four instantiations of the decode step (up to 16, 64, 128 and 256 rows of its head size), the traced ones when asked for."""
+    fake.fake_loaded(b"")
+    eng = _engine(fake)
+    assert fake.fake_loaded(b"decode_step_mega") == 4
+    api.ss_set_trace(eng, False)
+    assert fake.fake_loaded(b"decode_step_mega") == 0
+    api.ss_set_trace(eng, True)
+    assert fake.fake_loaded(b"decode_step_mega") == 4
     api.ss_destroy(eng)
 
 
