@@ -306,8 +306,9 @@ int ss_logits_noalloc(const float* hidden, const void* norm_gain, const void* lm
  * ss_set_wait_limit_ms() sets that limit (default about 2000 ms; 1..60000).
  * ss_selftest_wait_timeout() demonstrates the path without putting any work at risk: it launches a small kernel whose
  * warps are told to leave from between their barriers (all must leave at the same one), then one
- * in which every SM waits, for at most limit_us microseconds, for an arrival that never comes, and returns
- * what the runtime then reports -- SS_ERR_DEVICE_TIMEOUT when detection works.  SS_ERR_STATE while a batch is in
+ * in which every SM waits, for at most limit_us microseconds, for something that never comes (an arrival of another SM,
+ * partial sums, a barrier's completion, a flag: each on a quarter of the SMs), and returns what the runtime then
+ * reports -- SS_ERR_DEVICE_TIMEOUT when all of them were detected, SS_OK otherwise.  SS_ERR_STATE while a batch is in
  * flight.  Infrastructure, no passage of the paper. */
 int ss_set_wait_limit_ms(ss_ctx* ctx, int32_t ms);
 int ss_selftest_wait_timeout(ss_ctx* ctx, int32_t limit_us);

@@ -1630,15 +1630,42 @@ leave_selftest_kernel(const __grid_constant__ MegaArgs a, uint32_t* torn) {
       if (sm->prefix[w] != sm->prefix[0]) { atomicAdd(torn, 1u); break; }
 }
 
-// Self-test of the bounded grid-wide wait, with nothing else in flight (no bulk copies, no tensor-core work): every
-// CTA arrives on the counter and then waits for one arrival more than the grid can deliver.  The wait must run out
-// after `limit` cycles, record kStatusGridBarrierTimeout and let the kernel end normally.
+// Self-test of the bounded waits between SMs and on barriers, with nothing else in flight (no bulk copies, no tensor-core
+// work).  Every CTA has one of them, for something that never comes: an arrival more than the grid can deliver; partial sums
+// in an empty slot; the completion of a barrier that nobody arrives on; a flag that nobody sets.  Each must run out after
+// a.wait_limit cycles, record its status and let the kernel end normally; *ran_out gets a bit for each that did.
+constexpr uint32_t kWaitSelftests = 4;
 __global__ void __launch_bounds__(32)
-grid_wait_selftest_kernel(unsigned long long* ctr, unsigned long long base, long long limit, uint32_t* status) {
-  if (threadIdx.x == 0) {
-    const unsigned long long target = base + (unsigned long long)gridDim.x + 1ULL;
-    if (!arrive_and_poll(ctr, target, limit, nullptr)) atomicCAS(status, 0u, (uint32_t)kStatusGridBarrierTimeout);
+wait_selftest_kernel(const __grid_constant__ MegaArgs a, const uint32_t* flag, uint32_t* ran_out) {
+  __shared__ MegaSmem smem;
+  MegaSmem* sm = &smem;
+  const int lane = threadIdx.x;
+  const uint32_t which = blockIdx.x % kWaitSelftests, bar = smem_u32(&sm->acc_full[0]);
+  if (lane == 0) {
+    sm->abort = 0;
+    mbar_init(bar, 1);
+    fence_barrier_init();
   }
+  __syncwarp();
+  bool ended = false;
+  if (which == 1) {
+    PartialLoads<4, 2> q;
+    float x[4];
+    const int4 only_slot0 = make_int4(0, 1, 0, 0);
+    partials_issue<true, 4, 2>(a, a.shape[0], only_slot0, lane * 4, 0, q);
+    partials_sum<true, 4, 2>(a, sm, a.shape[0], only_slot0, lane * 4, 0, q, x);
+    ended = __all_sync(0xffffffffu, no_partial<4>(q.x));
+  } else if (lane == 0) {
+    if (which == 0) {
+      ended = !arrive_and_poll(a.grid_ctr, a.grid_base + (unsigned long long)gridDim.x + 1ULL, a.wait_limit, nullptr);
+      if (ended) atomicCAS(a.status, 0u, (uint32_t)kStatusGridBarrierTimeout);
+    } else if (which == 2) {
+      ended = !mega_wait(bar, 0, sm, a.status, kStatusMmaTimeout, a.wait_limit);
+    } else {
+      ended = !flag_wait(flag, a.status, a.wait_limit);
+    }
+  }
+  if (lane == 0 && ended) atomicOr(ran_out, 1u << which);
 }
 
 }  // namespace ss

@@ -1412,19 +1412,27 @@ int ss_selftest_wait_timeout(ss_ctx* c, int32_t limit_us) {
       return SS_OK;                    // an abort does not end as it should
     }
   }
-  const long long limit = (long long)limit_us * c->clock_khz / 1000;
-  unsigned long long base = c->grid_epochs * (unsigned long long)c->n_sm;
-  unsigned long long* ctr = c->grid_ctr;
-  uint32_t* status = c->status;
-  void* args[4] = {(void*)&ctr, (void*)&base, (void*)&limit, (void*)&status};
-  SS_CUDA(c, cudaLaunchCooperativeKernel((const void*)grid_wait_selftest_kernel, dim3(c->n_sm), dim3(32), args, 0, c->stream));
+  MegaArgs a{};
+  a.NT = 16;
+  a.shape[0].max_seg = 1;
+  a.shape[0].partial = c->part_dec[0];
+  a.grid_ctr = c->grid_ctr;
+  a.grid_base = c->grid_epochs * (unsigned long long)c->n_sm;
+  a.status = c->status;
+  a.wait_limit = (long long)limit_us * c->clock_khz / 1000;
+  const uint32_t* flag = c->pair_flag;
+  uint32_t* ran_out = c->status + 1;
+  SS_CUDA(c, cudaMemsetAsync(ran_out, 0, 4, c->stream));
+  void* args[3] = {(void*)&a, (void*)&flag, (void*)&ran_out};
+  SS_CUDA(c, cudaLaunchCooperativeKernel((const void*)wait_selftest_kernel, dim3(c->n_sm), dim3(32), args, 0, c->stream));
   c->launches++;
-  SS_CUDA(c, cudaMemcpyAsync(c->pinned + 1, c->status, 4, cudaMemcpyDeviceToHost, c->stream));
+  SS_CUDA(c, cudaMemcpyAsync(c->pinned + 1, c->status, 8, cudaMemcpyDeviceToHost, c->stream));
+  // what an abandoned step can leave behind: sums in the slots, flags up
+  SS_CUDA(c, cudaMemsetAsync(c->part_dec[0], 0, c->part_dec_bytes, c->stream));
+  SS_CUDA(c, cudaMemsetAsync(c->pair_flag, 1, (size_t)c->n_sm * 8 * sizeof(uint32_t), c->stream));
   SS_CUDA(c, cudaStreamSynchronize(c->stream));
-  if (c->pinned[1] != 0) return report_device_status(c, (uint32_t)c->pinned[1]);
-  // the wait came through although an arrival was missing: the counter no longer matches the epochs
-  reset_grid(c);
-  return SS_OK;
+  const int rc = report_device_status(c, (uint32_t)c->pinned[1]);          // clears all of it
+  return c->pinned[1] != 0 && (uint32_t)c->pinned[2] == (1u << kWaitSelftests) - 1 ? rc : SS_OK;
 }
 
 int ss_set_trace(ss_ctx* c, int32_t on) {

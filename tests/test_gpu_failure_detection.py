@@ -1,6 +1,6 @@
 """Failure detection on the GPU without a fault: a bounded wait that runs out must surface as
-SS_ERR_DEVICE_TIMEOUT and leave the context usable.  The wait that runs out belongs to a small self-test
-kernel (every SM waits at most a millisecond for an arrival that never comes; nothing else is in flight), not
+SS_ERR_DEVICE_TIMEOUT and leave the context usable.  The waits that run out belong to small self-test
+kernels (every SM waits at most a millisecond for something that never comes; nothing else is in flight), not
 to the decode kernel; nothing here traps, faults or hangs."""
 import numpy as np
 import pytest
@@ -40,6 +40,22 @@ def test_workers_of_an_abandoned_step_leave_together():
     eng = engine(shape, synth.make_weights(shape, seed=2))
     for _ in range(20):
         assert api.ss_selftest_wait_timeout(eng, 20) == api.SS_ERR_DEVICE_TIMEOUT
+
+
+def test_what_an_abandoned_step_leaves_behind_is_cleared():
+    """The self-test lets every kind of wait run out and leaves ordinary sums in the decode step's slots and the flags of
+    waiting partials up.  Behind it a prompt pass whose projections are cut along K (300 tokens, 24 heads) and a batch of
+    two rows, both of which would take these for their own."""
+    from paper_2305_13144_b200 import api
+    shape = synth.ModelShape(n_layers=1, d_model=3072, n_heads=24, head_dim=128, d_ffn=264, vocab=300)
+    w = synth.make_weights(shape, seed=35)
+    eng = engine(shape, w, max_ctx=256, max_prefill=512)
+    rng = np.random.default_rng(12)
+    prompts = [rng.integers(3, shape.vocab, size=n).tolist() for n in (200, 100)]
+    for _ in range(2):
+        assert api.ss_selftest_wait_timeout(eng, 100) == api.SS_ERR_DEVICE_TIMEOUT
+        el, eh, _ = teacher_forced(shape, w, prompts, [3, 3], 3, eng)
+        assert el <= LOGIT_TOL and eh <= HIDDEN_TOL, (el, eh)
 
 
 def test_selftest_is_refused_while_a_batch_is_in_flight_and_limits_are_checked():
