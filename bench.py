@@ -311,7 +311,9 @@ def stage_trace(eng, api, g, steps=60):
         acc[nm] = acc.get(nm, 0) + d
         cnt[nm] = cnt.get(nm, 0) + 1
     out = {"step_us": float(tr[-1]) / 1e3, "after_steps": steps,
-           "columns": ["projection_and_drain", "barrier", "following_stage", "barrier"]}
+           # up to 16 rows no barrier follows a projection: the stage waits for its partial sums itself
+           "columns": ["projection_and_drain", "barrier", "following_stage", "barrier"] if g.n > 16 else
+                      ["projection_and_drain", "no_barrier", "wait_and_following_stage", "barrier"]}
     for nm in acc:
         out[nm] = [round(float(x) / cnt[nm] / 1e3, 2) for x in acc[nm]]
     return out

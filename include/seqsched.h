@@ -320,7 +320,9 @@ int ss_set_trace(ss_ctx* ctx, int32_t on);
 /* Copies the time stamps (nanoseconds of the GPU's global timer) that CTA 0 took during the LAST decode step:
  * out[0] start, out[1] first operand ready, then for each projection in execution order
  * (qkv, o, gate/up, down per layer, LM head) four stamps: own accumulators drained, all partials
- * visible, own share of the following stage done, stage complete on every SM.
+ * visible, own share of the following stage done, stage complete on every SM.  Up to 16 rows there is no barrier
+ * behind a projection, the stage looks for its partial sums itself: the second stamp follows the first at once and the
+ * wait for other SMs is part of the stage.
  * out: host uint64 [cap]; n receives the number of stamps (2 + 4 * (4 * n_layers + 1));
  * SS_ERR_CAPACITY if cap is smaller, SS_ERR_STATE if tracing is off.  Synchronises the stream. */
 int ss_step_trace(ss_ctx* ctx, uint64_t* out, int32_t cap, int32_t* n);
