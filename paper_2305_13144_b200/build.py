@@ -9,7 +9,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libseqsched.so")
-SOURCES = ["ss_runtime.cu", "ss_noalloc.cu", "ss_sched.cpp"]
+SOURCES = ["ss_runtime.cu", "ss_mega_64.cu", "ss_mega_128.cu", "ss_noalloc.cu", "ss_sched.cpp"]
 HEADERS = ["ss_internal.h", "ss_gemm.cuh", "ss_kernels.cuh", "ss_decode_mega.cuh"]
 
 
@@ -25,7 +25,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    cmd = [nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
+    cmd = [nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "--threads", "3",
            "-shared", "-Xcompiler", "-fPIC",
            "-I", os.path.join(ROOT, "include"), "-I", CSRC]
     if verbose:

@@ -1194,7 +1194,7 @@ __device__ void stage_tile_argmax(const MegaArgs& a, MegaSmem* sm, int wtid) {
 }
 
 // ---- stage: final arg-max over tiles + row bookkeeping (one warp per row) -------------------------------
-__device__ void stage_final(const MegaArgs& a, int wtid) {
+static __device__ void stage_final(const MegaArgs& a, int wtid) {
   const int lane = wtid & 31, wid = wtid >> 5;
   for (int r = blockIdx.x * 8 + wid; r < a.B; r += gridDim.x * 8) {
     int tok = a.eos_id;
@@ -1597,11 +1597,22 @@ decode_step_mega_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_
   }
 }
 
+// The instantiation for batches of up to 16 / 64 / 128 / 256 rows, without or with the stage trace.
+template <int DH>
+const void* mega_kernel_of(int rows, bool trace) {
+  if (rows == 256) return trace ? (const void*)decode_step_mega_kernel<DH, 256, true> : (const void*)decode_step_mega_kernel<DH, 256, false>;
+  if (rows == 128) return trace ? (const void*)decode_step_mega_kernel<DH, 128, true> : (const void*)decode_step_mega_kernel<DH, 128, false>;
+  if (rows == 16) return trace ? (const void*)decode_step_mega_kernel<DH, 16, true> : (const void*)decode_step_mega_kernel<DH, 16, false>;
+  return trace ? (const void*)decode_step_mega_kernel<DH, 64, true> : (const void*)decode_step_mega_kernel<DH, 64, false>;
+}
+const void* mega_kernel_64(int rows, bool trace);          // ss_mega_64.cu
+const void* mega_kernel_128(int rows, bool trace);         // ss_mega_128.cu
+
 // Self-test of the workers' way out: eight worker warps that come to one grid barrier after the other at different times,
 // and a ninth warp that raises the abort flag in between, at another time in every CTA.  All eight must have passed the
 // same number of barriers; *torn counts the CTAs where they have not.
 constexpr int kLeaveSelftestThreads = kMegaWorkers + 32;
-__global__ void __launch_bounds__(kLeaveSelftestThreads, 1)
+static __global__ void __launch_bounds__(kLeaveSelftestThreads, 1)
 leave_selftest_kernel(const __grid_constant__ MegaArgs a, uint32_t* torn) {
   __shared__ MegaSmem smem;
   MegaSmem* sm = &smem;
@@ -1635,7 +1646,7 @@ leave_selftest_kernel(const __grid_constant__ MegaArgs a, uint32_t* torn) {
 // in an empty slot; the completion of a barrier that nobody arrives on; a flag that nobody sets.  Each must run out after
 // a.wait_limit cycles, record its status and let the kernel end normally; *ran_out gets a bit for each that did.
 constexpr uint32_t kWaitSelftests = 4;
-__global__ void __launch_bounds__(32)
+static __global__ void __launch_bounds__(32)
 wait_selftest_kernel(const __grid_constant__ MegaArgs a, const uint32_t* flag, uint32_t* ran_out) {
   __shared__ MegaSmem smem;
   MegaSmem* sm = &smem;

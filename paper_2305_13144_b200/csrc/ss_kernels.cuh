@@ -69,7 +69,7 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
 // source row goes in it: rows that one thread of an epilogue (or of the decode step) wants together become neighbours.
 //   half = 0: row r goes to row_off + r * step (step 1; 2 for gate and up, which alternate)
 //   half > 0: the two halves of every 2 * half rows alternate (q and k: the two dimensions of a rotation)
-__global__ void __launch_bounds__(256)
+static __global__ void __launch_bounds__(256)
 repack_weights_kernel(const uint4* __restrict__ src, long long rows, int K, uint8_t* __restrict__ dst, int row_off,
                       int kb, int half, int step) {
   const int chunks_per_row = K >> 3;
@@ -91,7 +91,7 @@ repack_weights_kernel(const uint4* __restrict__ src, long long rows, int K, uint
 // ------------------------------------------------------------------------------------ rotations
 // rope[pos][i] = (cos, sin) of pos * inv_freq[i]: grid (positions), block Dh / 2.  Filled once per context; the kernels
 // that rotate read it instead of evaluating a sine and a cosine per (token, head, pair).
-__global__ void rope_table_kernel(const float* __restrict__ inv_freq, float2* __restrict__ rope) {
+static __global__ void rope_table_kernel(const float* __restrict__ inv_freq, float2* __restrict__ rope) {
   float sn, cs;
   sincosf((float)blockIdx.x * inv_freq[threadIdx.x], &sn, &cs);
   rope[(size_t)blockIdx.x * blockDim.x + threadIdx.x] = make_float2(cs, sn);
@@ -126,7 +126,7 @@ __device__ __forceinline__ void store_normed(const float4 (&v)[kRowVec], int d4,
 }
 
 // h[t] = E[token]; x[t] = RMSNorm(h[t]) * g over T prompt tokens.
-__global__ void __launch_bounds__(256)
+static __global__ void __launch_bounds__(256)
 embed_rmsnorm_kernel(const int32_t* __restrict__ tokens, const bf16* __restrict__ E, const bf16* __restrict__ g, float* __restrict__ h,
                      bf16* __restrict__ x, int d, float eps, int vocab) {
   __shared__ float red[32];
@@ -199,7 +199,7 @@ __device__ __forceinline__ float decision_value(float logit, const SampleCfg& sc
 }
 
 constexpr int kArgmaxRows = 8;             // one after the other in a block: 100 rows by one block each took 92 us
-__global__ void __launch_bounds__(128)
+static __global__ void __launch_bounds__(128)
 lmhead_tile_argmax_kernel(const float* __restrict__ partial, SplitInfo sp, RowState st, float* __restrict__ dump_logits,
                           float* __restrict__ tile_val, int32_t* __restrict__ tile_idx, int B, int vocab, int n_tiles,
                           int eos_id, SampleCfg sc) {
@@ -244,7 +244,7 @@ lmhead_tile_argmax_kernel(const float* __restrict__ partial, SplitInfo sp, RowSt
 // One block of 1024 threads; warp w serves rows w, w+32, ...: final argmax over the vocabulary
 // tiles, then the row's state update.  is_prefill: the prompt has just been cached (ctx_len set
 // by the host) and this is generated token 1; otherwise the fed token becomes part of the cache.
-__global__ void __launch_bounds__(1024)
+static __global__ void __launch_bounds__(1024)
 bookkeeping_kernel(RowState st, const float* __restrict__ tile_val, const int32_t* __restrict__ tile_idx, int n_tiles,
                    const int32_t* __restrict__ forced, int32_t* __restrict__ next_tokens, int32_t* __restrict__ dump_choice,
                    int B, int eos_id, int is_prefill) {
@@ -296,7 +296,7 @@ bookkeeping_kernel(RowState st, const float* __restrict__ tile_val, const int32_
 
 // ------------------------------------------------------------------------------------ prompt-pass kernels
 // x[t] = RMSNorm(h[t]) * g over T tokens.
-__global__ void __launch_bounds__(256)
+static __global__ void __launch_bounds__(256)
 rmsnorm_kernel(const float* __restrict__ h, const bf16* __restrict__ g, bf16* __restrict__ x, int d, float eps) {
   __shared__ float red[32];
   pdl_launch_dependents();
@@ -312,7 +312,7 @@ rmsnorm_kernel(const float* __restrict__ h, const bf16* __restrict__ g, bf16* __
 }
 
 // Gather each sequence's last token: h_last[s] = h[last[s]]; x_last[s] = RMSNorm(h_last[s]) * g.
-__global__ void __launch_bounds__(256)
+static __global__ void __launch_bounds__(256)
 gather_last_rmsnorm_kernel(const float* __restrict__ h, const int32_t* __restrict__ last_tok, float* __restrict__ h_out,
                            const bf16* __restrict__ g, bf16* __restrict__ x_out, float* __restrict__ dump_hidden,
                            int d, float eps) {
@@ -364,7 +364,7 @@ __device__ __forceinline__ float4 sum_partials4(const float* __restrict__ partia
 }
 
 // grid (T, ceil(3d / 1024)), block 256
-__global__ void __launch_bounds__(256)
+static __global__ void __launch_bounds__(256)
 short_qkv_kernel(const float* __restrict__ partial, SplitInfo sp, GemmArgs a) {
   pdl_launch_dependents();
   const int t = blockIdx.x, n = (blockIdx.y * 256 + threadIdx.x) * 4;
@@ -389,7 +389,7 @@ short_qkv_kernel(const float* __restrict__ partial, SplitInfo sp, GemmArgs a) {
 
 // h[t] += projection; x[t] = RMSNorm(h[t]) * g.  grid (T), block 1024: few blocks, so every thread has only one or two
 // groups of four outputs, and what does not depend on the projection is read before the wait for it.
-__global__ void __launch_bounds__(1024)
+static __global__ void __launch_bounds__(1024)
 short_residual_kernel(const float* __restrict__ partial, SplitInfo sp, float* __restrict__ h, const bf16* __restrict__ g,
                       bf16* __restrict__ x, int d, float eps) {
   __shared__ float red[32];
@@ -431,7 +431,7 @@ short_residual_kernel(const float* __restrict__ partial, SplitInfo sp, float* __
 }
 
 // grid (T, ceil(2F / 1024)), block 256
-__global__ void __launch_bounds__(256)
+static __global__ void __launch_bounds__(256)
 short_swiglu_kernel(const float* __restrict__ partial, SplitInfo sp, bf16* __restrict__ act, int F) {
   pdl_launch_dependents();
   const int t = blockIdx.x, n = (blockIdx.y * 256 + threadIdx.x) * 4;

@@ -1,0 +1,9 @@
+// The decode step's instantiations for heads of 128: a module of its own, since the first kernel of a module that a process
+// launches loads all of it.  With all sixteen instantiations in one module the first context of a process took 22 ms, now 10.
+#include "ss_decode_mega.cuh"
+
+namespace ss {
+
+const void* mega_kernel_128(int rows, bool trace) { return mega_kernel_of<128>(rows, trace); }
+
+}  // namespace ss

@@ -562,18 +562,11 @@ double weight_bytes_per_step(const ss_model_cfg& m) {
 double kv_bytes_per_token(const ss_model_cfg& m) { return 2.0 * m.d_model * 2.0 * m.n_layers; }
 
 // The decode kernel's instantiations: head size 64 / 128, batches up to 16 / 64 / 128 / 256 rows, without / with the stage trace.
-template <int DH>
-const void* mega_kernel_fn_dh(int rows, bool trace) {
-  if (rows == 256) return trace ? (const void*)decode_step_mega_kernel<DH, 256, true> : (const void*)decode_step_mega_kernel<DH, 256, false>;
-  if (rows == 128) return trace ? (const void*)decode_step_mega_kernel<DH, 128, true> : (const void*)decode_step_mega_kernel<DH, 128, false>;
-  if (rows == 16) return trace ? (const void*)decode_step_mega_kernel<DH, 16, true> : (const void*)decode_step_mega_kernel<DH, 16, false>;
-  return trace ? (const void*)decode_step_mega_kernel<DH, 64, true> : (const void*)decode_step_mega_kernel<DH, 64, false>;
-}
 const void* mega_kernel_fn(int head_dim, int rows, bool trace) {
-  return head_dim == 128 ? mega_kernel_fn_dh<128>(rows, trace) : mega_kernel_fn_dh<64>(rows, trace);
+  return head_dim == 128 ? mega_kernel_128(rows, trace) : mega_kernel_64(rows, trace);
 }
-// Loads the instantiations that a context can launch (naming a kernel here costs its load): those of its head size, and the
-// ones with the trace when a trace is asked for.  With all sixteen the first context of a process took 14 ms longer.
+// Loads the instantiations that a context can launch: those of its head size, and the ones with the trace when a trace is
+// asked for.
 cudaError_t prepare_mega_kernels(int head_dim, bool trace) {
   cudaError_t e = cudaSuccess;
   for (int rows : {16, 64, 128, 256})
