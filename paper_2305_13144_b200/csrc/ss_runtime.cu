@@ -586,7 +586,8 @@ int enqueue_decode_step(ss_ctx* c, const ss_step_opts* opts, int32_t* next_token
   // pair's MMAs (two CTAs, 32 KiB of weights) pace the stream; where it streams few, the drains weigh more and pairs have
   // half of the segments.  72 / 112 / 128 rows, one CTA and pairs, us a step of 4 layers: 7B shape (83 blocks) 570 / - / 792
   // and 650 / - / 830; d 3072 (47) 416 / 578 / 562 and 432 / 570 / 548; d 2560 (33) 383 / 513 / 522 and 371 / 470 / 456; 32 x
-  // 64 heads (21) 331 / 450 / 456 and 316 / 400 / 398.  Up to 64 rows one CTA: 48 rows of 32 x 64 heads 290 and 306.
+  // 64 heads (21) 331 / 450 / 456 and 316 / 400 / 398.  (The line goes by the blocks alone: between 40 and 50 of them pairs are
+  // 1 to 3 % ahead from 112 rows on and 4 % behind at 72.)  Up to 64 rows one CTA: 48 rows of 32 x 64 heads 290 and 306.
   const double layer_blocks = (4.0 * d * d + 3.0 * d * F) * 2 / kBlockBytes / c->n_sm;
   const int kernel_rows = NT <= 16 ? 16 : NT <= 64 ? 64 : (NT <= 128 && layer_blocks > 40) ? 128 : 256;
   const bool pair = kernel_rows == 256, flagged = kernel_rows == 16;
